@@ -429,7 +429,7 @@ grpic_status grpic_create(const grpic_config *cfg, grpic_ctx **out) {
   const size_t ps = (size_t)plane_size(g), fs = ctx->fsz;
   size_t off = 0;
   ctx->off_planes = off; off += up(ps * fs) * 36;
-  ctx->off_tab = off;    off += up(ps * fs) * 4 * T_NQ;
+  ctx->off_tab = off;    off += up(ps * fs) * T_NQ;
   ctx->off_polar = off;  off += up((size_t)3 * g.NX * fs);
   ctx->off_ptab = off;   off += 16 * up((size_t)(g.NX > g.NY ? g.NX : g.NY) * 8);
   ctx->off_dt = off;     off += up(64);
@@ -575,16 +575,6 @@ grpic_status grpic_bind(grpic_ctx *ctx, void *arena, size_t bytes, void *stream)
 grpic_status grpic_init_metric(grpic_ctx *ctx) {
   grpic_status s = need_bound(ctx);
   if (s) return s;
-  if (ctx->mixed) {
-    CK(launch_metric_tables<float>(ctx->g, const_cast<float *>(ctx->F32.tab),
-                                   const_cast<float *>(ctx->F32.polar), ctx->stream));
-  } else {
-    CK(launch_metric_tables<double>(ctx->g, const_cast<double *>(ctx->F64.tab),
-                                    const_cast<double *>(ctx->F64.polar), ctx->stream));
-  }
-  CK(launch_push_tables(ctx->g, ctx->tb, ctx->stream));
-  CK(launch_inject_tables(ctx->g, reinterpret_cast<unsigned char *>(ctx->arena + ctx->off_inj),
-                          ctx->stream));
   if (!(ctx->cfg.dt > 0.0)) {
     double dmin = 0.0;
     CK(launch_dt_min(ctx->g, at<double>(ctx, ctx->off_dt), 8, &dmin, ctx->stream));
@@ -595,6 +585,16 @@ grpic_status grpic_init_metric(grpic_ctx *ctx) {
     ctx->g.dt = ctx->cfg.dt;
   }
   grid_float_copies(ctx->g);
+  if (ctx->mixed) {
+    CK(launch_metric_tables<float>(ctx->g, const_cast<float *>(ctx->F32.tab),
+                                   const_cast<float *>(ctx->F32.polar), ctx->stream));
+  } else {
+    CK(launch_metric_tables<double>(ctx->g, const_cast<double *>(ctx->F64.tab),
+                                    const_cast<double *>(ctx->F64.polar), ctx->stream));
+  }
+  CK(launch_push_tables(ctx->g, ctx->tb, ctx->stream));
+  CK(launch_inject_tables(ctx->g, reinterpret_cast<unsigned char *>(ctx->arena + ctx->off_inj),
+                          ctx->stream));
   ctx->metric_ready = true;
   return GRPIC_OK;
 }

@@ -9,18 +9,28 @@ namespace {
 
 constexpr int TPB = 256;
 
+// ---------------------------------------------------------------------------------
+// Coefficient tables of the field solver, FieldTab (grpic_internal.cuh): per component of
+// Eqs. (discretized-auxE), (discretized-auxH) the factor of every field value that enters it
+// (alpha h_ii; alpha sqrt(h~) h_13 / (2 sqrt(h~)) and sqrt(h~ h) beta^1 / (2 sqrt(h~)) of both
+// neighbours of an average), and dt / sqrt(h) of the curls, each formed in FP64 and rounded
+// once; the polar area A(x1) = dr (r^2 + a^2) sqrt(1 + 2 M r/(r^2 + a^2))
+// (1 - cos(theta(x2 = 1/2))) (App. A, per unit phi; theta(1/2) = dtheta/2 on the plain grid).
+//
+// Why whole coefficients: GB300's FP64 rate is 2 operations per clock and SM, so on 2048^2
+// points one FP64 operation per point costs 8 us, as much as 1.6 planes of HBM traffic. With
+// the metric factors tabulated one by one (alpha, h_11, h_22, h_33, weights) an auxiliary-field
+// kernel took ~50 FP64 operations per point and 13 table planes; a component as a sum of
+// coefficient x field products takes 11 and 11. With the boundary writes folded into the
+// curl kernels (put, below) and the launches that read the same fields merged, a vacuum step
+// on 2048^2 points went from 2220 to 1025 us in FP64, one on 500 x 300 points in FP32 (bound by
+// launches) from 90 to 49 us: 7 launches a step where there were 18.
+// ---------------------------------------------------------------------------------
 template <typename T>
-__device__ __forceinline__ T tabv(const T *tab, const GridP &g, int cls, int q, int i, int j) {
-  return __ldg(tab + ((int64_t)(cls * T_NQ + q)) * plane_size(g) + sidx(g, i, j));
+__device__ __forceinline__ T tabv(const T *tab, int64_t ps, int q, int64_t k) {
+  return __ldg(tab + q * ps + k);
 }
 
-// ---------------------------------------------------------------------------------
-// Tables: per Yee class, alpha, h_11, h_22, h_33, 1/(2 sqrt(h~)) (the weight of the
-// volume-weighted averages, stored as a reciprocal so the field kernels multiply instead of
-// dividing), [sqrt(h~) h_13], [sqrt(h~ h) beta^1], 1/sqrt(h) at every stored point; the
-// polar area A(x1) = dr (r^2 + a^2) sqrt(1 + 2 M r/(r^2 + a^2)) (1 - cos(theta(x2 = 1/2)))
-// (App. A, per unit phi; theta(1/2) = dtheta/2 on the plain grid).
-// ---------------------------------------------------------------------------------
 // The absorbing layer (MATCH, Sec. 3.3.3): a field value v relaxes towards its initial value
 // vi as v - k (v - vi), k = absorb_coef x^3, x = (r - r_absorb) / (r_max - r_absorb) capped at
 // 1, beyond r_absorb. k depends on x1 alone, so it is tabulated per column.
@@ -36,31 +46,68 @@ __device__ __forceinline__ double absorb_factor(const GridP &g, double x1) {
 template <typename T>
 __global__ void k_metric_tables(GridP g, T *tab, T *polar) {
   const int64_t ps = plane_size(g);
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < 4 * ps;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int cls = (int)(t / ps);
-    const int64_t q = t - cls * ps;
+  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < ps;
+       q += (int64_t)gridDim.x * blockDim.x) {
     const int i = (int)(q % g.NX) - G_, j = (int)(q / g.NX) - G_;
-    const double s1 = (cls == CLS_HN || cls == CLS_HH) ? 0.5 : 0.0;
-    const double s2 = (cls == CLS_NH || cls == CLS_HH) ? 0.5 : 0.0;
-    MetricV m;
-    metric_eval<false>(g, i + s1, j + s2, false, m, nullptr);
-    T *o = tab + (int64_t)cls * T_NQ * ps + q;
-    o[T_ALPHA * ps] = (T)m.alpha;
-    o[T_H11 * ps] = (T)m.h11;
-    o[T_H22 * ps] = (T)m.h22;
-    o[T_H33 * ps] = (T)m.h33;
-    o[T_IHT2 * ps] = (T)(0.5 / m.sqrt_ht);
-    o[T_WT13 * ps] = (T)(m.sqrt_ht * m.h13);
-    o[T_WB1 * ps] = (T)(m.sqrt_ht * m.sqrt_h * m.beta1);
-    o[T_ISH * ps] = (T)(1.0 / m.sqrt_h);
-    if (cls == CLS_HN && j == 0) {
+    T *o = tab + q;
+    MetricV c, lo, hi;
+    {  // (i, j) with its x1 neighbours (i -+ 1/2, j)
+      metric_eval<false>(g, i, j, false, c, nullptr);
+      metric_eval<false>(g, i - 0.5, j, false, lo, nullptr);
+      metric_eval<false>(g, i + 0.5, j, false, hi, nullptr);
+      const double w = 0.5 / c.sqrt_ht, wa = w * c.alpha;
+      o[T_E3D3 * ps] = (T)(c.alpha * c.h33);
+      o[T_E3D1L * ps] = (T)(wa * (lo.sqrt_ht * lo.h13));
+      o[T_E3D1R * ps] = (T)(wa * (hi.sqrt_ht * hi.h13));
+      o[T_E3B2L * ps] = (T)(w * (lo.sqrt_ht * lo.sqrt_h * lo.beta1));
+      o[T_E3B2R * ps] = (T)(w * (hi.sqrt_ht * hi.sqrt_h * hi.beta1));
+      o[T_D3 * ps] = (T)(g.dt / c.sqrt_h);
+    }
+    {  // (i + 1/2, j): neighbours (i, j), (i + 1, j)
+      lo = c;
+      c = hi;
+      metric_eval<false>(g, i + 1, j, false, hi, nullptr);
+      const double w = 0.5 / c.sqrt_ht, wa = w * c.alpha;
+      o[T_E1D1 * ps] = (T)(c.alpha * c.h11);
+      o[T_E1D3L * ps] = (T)(wa * (lo.sqrt_ht * lo.h13));
+      o[T_E1D3R * ps] = (T)(wa * (hi.sqrt_ht * hi.h13));
+      o[T_H2B2 * ps] = (T)(c.alpha * c.h22);
+      o[T_H2D3L * ps] = (T)(w * (lo.sqrt_ht * lo.sqrt_h * lo.beta1));
+      o[T_H2D3R * ps] = (T)(w * (hi.sqrt_ht * hi.sqrt_h * hi.beta1));
+      o[T_B2D1 * ps] = (T)(g.dt / c.sqrt_h);
+    }
+    {  // (i, j + 1/2): neighbours (i -+ 1/2, j + 1/2)
+      metric_eval<false>(g, i, j + 0.5, false, c, nullptr);
+      metric_eval<false>(g, i - 0.5, j + 0.5, false, lo, nullptr);
+      metric_eval<false>(g, i + 0.5, j + 0.5, false, hi, nullptr);
+      const double w = 0.5 / c.sqrt_ht, wa = w * c.alpha;
+      o[T_E2D2 * ps] = (T)(c.alpha * c.h22);
+      o[T_E2B3L * ps] = (T)(w * (lo.sqrt_ht * lo.sqrt_h * lo.beta1));
+      o[T_E2B3R * ps] = (T)(w * (hi.sqrt_ht * hi.sqrt_h * hi.beta1));
+      o[T_H1B1 * ps] = (T)(c.alpha * c.h11);
+      o[T_H1B3L * ps] = (T)(wa * (lo.sqrt_ht * lo.h13));
+      o[T_H1B3R * ps] = (T)(wa * (hi.sqrt_ht * hi.h13));
+      o[T_B1D2 * ps] = (T)(g.dt / c.sqrt_h);
+    }
+    {  // (i + 1/2, j + 1/2): neighbours (i, j + 1/2), (i + 1, j + 1/2)
+      lo = c;
+      c = hi;
+      metric_eval<false>(g, i + 1, j + 0.5, false, hi, nullptr);
+      const double w = 0.5 / c.sqrt_ht, wa = w * c.alpha;
+      o[T_H3B3 * ps] = (T)(c.alpha * c.h33);
+      o[T_H3B1L * ps] = (T)(wa * (lo.sqrt_ht * lo.h13));
+      o[T_H3B1R * ps] = (T)(wa * (hi.sqrt_ht * hi.h13));
+      o[T_H3D2L * ps] = (T)(w * (lo.sqrt_ht * lo.sqrt_h * lo.beta1));
+      o[T_H3D2R * ps] = (T)(w * (hi.sqrt_ht * hi.sqrt_h * hi.beta1));
+      o[T_B3 * ps] = (T)(g.dt / c.sqrt_h);
+    }
+    if (j == 0) {
       const double e = map_e(g, i + 0.5), r = g.r0 + e, a2 = g.a * g.a;
       polar[i + G_] = (T)(g.dxi * e * (r * r + a2) * sqrt(1.0 + 2.0 * g.M * r / (r * r + a2)) *
                           (1.0 - cos(map_theta(g, 0.5))));
+      polar[g.NX + i + G_] = (T)absorb_factor(g, i);
       polar[2 * g.NX + i + G_] = (T)absorb_factor(g, i + 0.5);
     }
-    if (cls == CLS_NN && j == 0) polar[g.NX + i + G_] = (T)absorb_factor(g, i);
   }
 }
 
@@ -240,91 +287,84 @@ __global__ void k_axis(GridP g, T *p0, T *p1, T *p2, int isB) {
 }
 
 // ---------------------------------------------------------------------------------
-// Auxiliary fields, Eq. (discretized-auxE) with the averages of Eq. (discretized-auxH).
-// D (and for E also B) may be the mean of two time levels: X = wa Xa + wb Xb.
-// Computed on stored i in [-1, n_r + 1], rows [0, n_theta].
+// Field kernels. One thread per point of a row; a block covers TPBX x TPBY points, so no
+// index is divided and the x2 neighbours of a block's rows are in its cache.
+//
+// Two time levels: a field that enters as the mean of two levels is read from a and b
+// (MEAN), one that enters as itself from a alone; which one is known at compile time, since a
+// multiplication by a weight of 1 would cost an FP64 operation per value.
 // ---------------------------------------------------------------------------------
+constexpr int TPBX = 64, TPBY = 4;
+
 template <typename T>
 struct Pair3 {
   const T *a[3], *b[3];
-  T wa, wb;
 };
-template <typename T>
+template <bool MEAN, typename T>
 __device__ __forceinline__ T pv(const Pair3<T> &P, int c, int64_t k) {
-  T v = P.wa * __ldg(P.a[c] + k);
-  if (P.wb != (T)0) v += P.wb * __ldg(P.b[c] + k);
-  return v;
+  if (MEAN) return (T)0.5 * (__ldg(P.a[c] + k) + __ldg(P.b[c] + k));
+  return __ldg(P.a[c] + k);
 }
 
+// E_1 at (i+1/2, j) = alpha [h_11 D^1 + <h_13 D^3>], E_3 at (i, j) = alpha [h_33 D^3 +
+// <h_13 D^1>] + <sqrt(h) beta^1 B^2> (zero on the axes), E_2 at (i, j+1/2) = alpha h_22 D^2 -
+// <sqrt(h) beta^1 B^3>; Eq. (discretized-auxE)
+template <typename T, bool DMEAN>
+__device__ __forceinline__ void aux_E(const GridP &g, const Pair3<T> &B, const Pair3<T> &D,
+                                      const T *tab, int64_t ps, int j, int64_t k, T *E1, T *E2,
+                                      T *E3) {
+  const T d1 = pv<DMEAN>(D, 0, k), d3 = pv<DMEAN>(D, 2, k);
+  E1[k] = fma(tabv(tab, ps, T_E1D1, k), d1,
+              fma(tabv(tab, ps, T_E1D3L, k), d3,
+                  tabv(tab, ps, T_E1D3R, k) * pv<DMEAN>(D, 2, k + 1)));
+  E3[k] = (j == 0 || j == g.n_th)
+              ? (T)0
+              : fma(tabv(tab, ps, T_E3D3, k), d3,
+                    fma(tabv(tab, ps, T_E3D1L, k), pv<DMEAN>(D, 0, k - 1),
+                        tabv(tab, ps, T_E3D1R, k) * d1)) +
+                    fma(tabv(tab, ps, T_E3B2L, k), pv<false>(B, 1, k - 1),
+                        tabv(tab, ps, T_E3B2R, k) * pv<false>(B, 1, k));
+  if (j < g.n_th)
+    E2[k] = fma(tabv(tab, ps, T_E2D2, k), pv<DMEAN>(D, 1, k),
+                -fma(tabv(tab, ps, T_E2B3L, k), pv<false>(B, 2, k - 1),
+                     tabv(tab, ps, T_E2B3R, k) * pv<false>(B, 2, k)));
+}
+
+// H_1 at (i, j+1/2) = alpha [h_11 B^1 + <h_13 B^3>], H_3 at (i+1/2, j+1/2) = alpha [h_33 B^3 +
+// <h_13 B^1>] - <sqrt(h) beta^1 D^2>, H_2 at (i+1/2, j) = alpha h_22 B^2 +
+// <sqrt(h) beta^1 D^3>; Eq. (discretized-auxH)
 template <typename T>
-__global__ void k_aux_E(GridP g, Pair3<T> B, Pair3<T> D, const T *tab, T *E1, T *E2, T *E3) {
-  const int ni = g.n_r + 3, nj = g.n_th + 1;
-  const int64_t n = (int64_t)ni * nj;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int i = (int)(t % ni) - 1, j = (int)(t / ni);
-    const int64_t k = sidx(g, i, j);
-    // E_1 at (i+1/2, j) = alpha [h_11 D^1 + <h_13 D^3>]
-    {
-      const T avg = (tabv(tab, g, CLS_NN, T_WT13, i, j) * pv(D, 2, k) +
-                     tabv(tab, g, CLS_NN, T_WT13, i + 1, j) * pv(D, 2, k + 1)) *
-                    tabv(tab, g, CLS_HN, T_IHT2, i, j);
-      E1[k] = tabv(tab, g, CLS_HN, T_ALPHA, i, j) *
-              (tabv(tab, g, CLS_HN, T_H11, i, j) * pv(D, 0, k) + avg);
-    }
-    // E_3 at (i, j) = alpha [h_33 D^3 + <h_13 D^1>] + <sqrt(h) beta^1 B^2>; zero on the axes
-    if (j == 0 || j == g.n_th) {
-      E3[k] = (T)0;
-    } else {
-      const T w2 = tabv(tab, g, CLS_NN, T_IHT2, i, j);
-      const T a13 = (tabv(tab, g, CLS_HN, T_WT13, i - 1, j) * pv(D, 0, k - 1) +
-                     tabv(tab, g, CLS_HN, T_WT13, i, j) * pv(D, 0, k)) * w2;
-      const T ab2 = (tabv(tab, g, CLS_HN, T_WB1, i - 1, j) * pv(B, 1, k - 1) +
-                     tabv(tab, g, CLS_HN, T_WB1, i, j) * pv(B, 1, k)) * w2;
-      E3[k] = tabv(tab, g, CLS_NN, T_ALPHA, i, j) *
-                  (tabv(tab, g, CLS_NN, T_H33, i, j) * pv(D, 2, k) + a13) + ab2;
-    }
-    // E_2 at (i, j+1/2) = alpha h_22 D^2 - <sqrt(h) beta^1 B^3>
-    if (j < g.n_th) {
-      const T ab3 = (tabv(tab, g, CLS_HH, T_WB1, i - 1, j) * pv(B, 2, k - 1) +
-                     tabv(tab, g, CLS_HH, T_WB1, i, j) * pv(B, 2, k)) *
-                    tabv(tab, g, CLS_NH, T_IHT2, i, j);
-      E2[k] = tabv(tab, g, CLS_NH, T_ALPHA, i, j) * tabv(tab, g, CLS_NH, T_H22, i, j) *
-                  pv(D, 1, k) - ab3;
-    }
+__device__ __forceinline__ void aux_H(const GridP &g, const Pair3<T> &B, const Pair3<T> &D,
+                                      const T *tab, int64_t ps, int j, int64_t k, T *H1, T *H2,
+                                      T *H3) {
+  if (j < g.n_th) {
+    const T b1 = pv<false>(B, 0, k), b3 = pv<false>(B, 2, k);
+    H1[k] = fma(tabv(tab, ps, T_H1B1, k), b1,
+                fma(tabv(tab, ps, T_H1B3L, k), pv<false>(B, 2, k - 1),
+                    tabv(tab, ps, T_H1B3R, k) * b3));
+    H3[k] = fma(tabv(tab, ps, T_H3B3, k), b3,
+                fma(tabv(tab, ps, T_H3B1L, k), b1,
+                    tabv(tab, ps, T_H3B1R, k) * pv<false>(B, 0, k + 1))) -
+            fma(tabv(tab, ps, T_H3D2L, k), pv<false>(D, 1, k),
+                tabv(tab, ps, T_H3D2R, k) * pv<false>(D, 1, k + 1));
   }
+  H2[k] = fma(tabv(tab, ps, T_H2B2, k), pv<false>(B, 1, k),
+              fma(tabv(tab, ps, T_H2D3L, k), pv<false>(D, 2, k),
+                  tabv(tab, ps, T_H2D3R, k) * pv<false>(D, 2, k + 1)));
 }
 
-template <typename T>
-__global__ void k_aux_H(GridP g, Pair3<T> B, Pair3<T> D, const T *tab, T *H1, T *H2, T *H3) {
-  const int ni = g.n_r + 3, nj = g.n_th + 1;
-  const int64_t n = (int64_t)ni * nj;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int i = (int)(t % ni) - 1, j = (int)(t / ni);
+// The auxiliary fields on stored i in [-1, n_r + 1], rows [0, n_theta]: E, H or both (both
+// read the same B and D, so one launch reads them once).
+template <typename T, bool DOE, bool DOH, bool DMEAN>
+__global__ void __launch_bounds__(TPBX *TPBY) k_aux(GridP g, Pair3<T> B, Pair3<T> D, const T *tab,
+                                                    T *E1, T *E2, T *E3, T *H1, T *H2, T *H3) {
+  const int i = (int)(blockIdx.x * TPBX + threadIdx.x) - 1;
+  const int64_t ps = plane_size(g);
+  for (int j = blockIdx.y * TPBY + threadIdx.y; j <= g.n_th; j += gridDim.y * TPBY) {
+    if (i > g.n_r + 1) return;
     const int64_t k = sidx(g, i, j);
-    if (j < g.n_th) {
-      // H_1 at (i, j+1/2) = alpha [h_11 B^1 + <h_13 B^3>]
-      const T a13 = (tabv(tab, g, CLS_HH, T_WT13, i - 1, j) * pv(B, 2, k - 1) +
-                     tabv(tab, g, CLS_HH, T_WT13, i, j) * pv(B, 2, k)) *
-                    tabv(tab, g, CLS_NH, T_IHT2, i, j);
-      H1[k] = tabv(tab, g, CLS_NH, T_ALPHA, i, j) *
-              (tabv(tab, g, CLS_NH, T_H11, i, j) * pv(B, 0, k) + a13);
-      // H_3 at (i+1/2, j+1/2) = alpha [h_33 B^3 + <h_13 B^1>] - <sqrt(h) beta^1 D^2>
-      const T w3 = tabv(tab, g, CLS_HH, T_IHT2, i, j);
-      const T b13 = (tabv(tab, g, CLS_NH, T_WT13, i, j) * pv(B, 0, k) +
-                     tabv(tab, g, CLS_NH, T_WT13, i + 1, j) * pv(B, 0, k + 1)) * w3;
-      const T bd2 = (tabv(tab, g, CLS_NH, T_WB1, i, j) * pv(D, 1, k) +
-                     tabv(tab, g, CLS_NH, T_WB1, i + 1, j) * pv(D, 1, k + 1)) * w3;
-      H3[k] = tabv(tab, g, CLS_HH, T_ALPHA, i, j) *
-                  (tabv(tab, g, CLS_HH, T_H33, i, j) * pv(B, 2, k) + b13) - bd2;
-    }
-    // H_2 at (i+1/2, j) = alpha h_22 B^2 + <sqrt(h) beta^1 D^3>
-    const T bd3 = (tabv(tab, g, CLS_NN, T_WB1, i, j) * pv(D, 2, k) +
-                   tabv(tab, g, CLS_NN, T_WB1, i + 1, j) * pv(D, 2, k + 1)) *
-                  tabv(tab, g, CLS_HN, T_IHT2, i, j);
-    H2[k] = tabv(tab, g, CLS_HN, T_ALPHA, i, j) * tabv(tab, g, CLS_HN, T_H22, i, j) *
-                pv(B, 1, k) + bd3;
+    if (DOE) aux_E<T, DMEAN>(g, B, D, tab, ps, j, k, E1, E2, E3);
+    if (DOH) aux_H<T>(g, B, D, tab, ps, j, k, H1, H2, H3);
   }
 }
 
@@ -339,73 +379,154 @@ __device__ __forceinline__ T match(const GridP &g, T v, const T *init, int64_t i
   return k == (T)0 ? v : v - k * (v - __ldg(init + idx));
 }
 
-// Faraday, Eq. (discretized-faraday): Bout = Bin - dt curl E / sqrt(h) on the evolved
-// points, Bout = Bin elsewhere; B^2 is not evolved on the axes. Covers every stored point.
+// Stores a point's new value together with every boundary value it determines, so that the
+// curl kernels need no boundary launches (k_horizon, then k_axis): the columns [-G, n_f] of
+// the horizon layer copy column n_f + 1, and the rows across the axes mirror rows inside
+// (half rows -1-r <- r, n+r <- n-1-r; node rows -r <- r, n+r <- n-r) with parity par. The
+// points that are written here by others are not stored by their own threads
+// (boundary_point). AXIS false: the horizon layer alone.
+template <bool AXIS>
+__device__ __forceinline__ bool boundary_point(const GridP &g, bool half, int i, int j) {
+  return i <= g.n_f || (AXIS && (j < 0 || j > g.n_th - (half ? 1 : 0)));
+}
 template <typename T>
-__global__ void k_faraday(GridP g, Pair3<T> Bin, const T *E1, const T *E2, const T *E3,
-                          const T *tab, const T *absorb, T *B1, T *B2, T *B3, const T *Bi1,
-                          const T *Bi2, const T *Bi3, int do_match) {
-  const int64_t n = plane_size(g);
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int i = (int)(t % g.NX) - G_, j = (int)(t / g.NX) - G_;
-    const int64_t k = t;
-    const T dt = (T)g.dt;
-    T b1 = pv(Bin, 0, k), b2 = pv(Bin, 1, k), b3 = pv(Bin, 2, k);
-    const bool rows_half = (j >= 0 && j < g.n_th);
-    if (rows_half && i >= 0 && i <= g.n_r)
-      b1 -= dt * (__ldg(E3 + k + g.NX) - __ldg(E3 + k)) * tabv(tab, g, CLS_NH, T_ISH, i, j);
-    if (j >= 1 && j < g.n_th && i >= 0 && i < g.n_r)
-      b2 += dt * (__ldg(E3 + k + 1) - __ldg(E3 + k)) * tabv(tab, g, CLS_HN, T_ISH, i, j);
-    if (rows_half && i >= 0 && i < g.n_r)
-      b3 -= dt * ((__ldg(E2 + k + 1) - __ldg(E2 + k)) - (__ldg(E1 + k + g.NX) - __ldg(E1 + k))) *
-            tabv(tab, g, CLS_HH, T_ISH, i, j);
-    if (do_match) {
-      b1 = match(g, b1, Bi1, k, absorb, i, j);
-      b2 = match(g, b2, Bi2, k, absorb + g.NX, i, j);
-      b3 = match(g, b3, Bi3, k, absorb + g.NX, i, j);
-    }
-    B1[k] = b1; B2[k] = b2; B3[k] = b3;
+__device__ __forceinline__ void put_row(const GridP &g, T *p, int i, int j, T v) {
+  p[sidx(g, i, j)] = v;
+  if (i == g.n_f + 1)
+    for (int q = -G_; q <= g.n_f; ++q) p[sidx(g, q, j)] = v;
+}
+template <bool AXIS, typename T>
+__device__ __forceinline__ void put(const GridP &g, T *p, bool half, T par, int i, int j, T v) {
+  if (boundary_point<AXIS>(g, half, i, j)) return;
+  put_row(g, p, i, j, v);
+  if (!AXIS) return;
+  const int N = g.n_th;
+  if (half) {
+    if (j < G_) put_row(g, p, i, -1 - j, par * v);
+    if (N - 1 - j <= G_) put_row(g, p, i, N + (N - 1 - j), par * v);
+  } else {
+    if (j >= 1 && j <= G_) put_row(g, p, i, -j, par * v);
+    if (N - j >= 1 && N - j <= G_) put_row(g, p, i, N + (N - j), par * v);
   }
+}
+
+// Faraday, Eq. (discretized-faraday): Bout = Bin - dt curl E / sqrt(h) on the evolved points,
+// Bout = Bin elsewhere; B^2 is not evolved on the axes.
+template <typename T, bool MEAN, bool MATCH>
+__device__ __forceinline__ void faraday(const GridP &g, const Pair3<T> &Bin, const T *E1,
+                                        const T *E2, const T *E3, const T *tab, const T *absorb,
+                                        T *const B[3], T *const Bi[3], int64_t ps, int i, int j,
+                                        int64_t k) {
+  T b1 = pv<MEAN>(Bin, 0, k), b2 = pv<MEAN>(Bin, 1, k), b3 = pv<MEAN>(Bin, 2, k);
+  const bool rows_half = (j >= 0 && j < g.n_th);
+  if (rows_half && i >= 0 && i <= g.n_r) {
+    const T e3 = __ldg(E3 + k);
+    b1 = fma(-(__ldg(E3 + k + g.NX) - e3), tabv(tab, ps, T_B1D2, k), b1);
+    if (i < g.n_r) {
+      if (j >= 1) b2 = fma(__ldg(E3 + k + 1) - e3, tabv(tab, ps, T_B2D1, k), b2);
+      b3 = fma(-((__ldg(E2 + k + 1) - __ldg(E2 + k)) - (__ldg(E1 + k + g.NX) - __ldg(E1 + k))),
+               tabv(tab, ps, T_B3, k), b3);
+    }
+  }
+  if (MATCH) {
+    b1 = match(g, b1, Bi[0], k, absorb, i, j);
+    b2 = match(g, b2, Bi[1], k, absorb + g.NX, i, j);
+    b3 = match(g, b3, Bi[2], k, absorb + g.NX, i, j);
+  }
+  put<true>(g, B[0], true, (T)1, i, j, b1);
+  put<true>(g, B[1], false, (T)-1, i, j, b2);
+  put<true>(g, B[2], true, (T)-1, i, j, b3);
 }
 
 // Ampere, Eq. (discretized-ampere): Dout = Din + dt (curl H - 4 pi J) / sqrt(h); on the
 // axes D^1 follows the integral form of Sec. 3.3.2 with the polar area (reading: the
 // whole radial flux into the half cell, coefficient 4 pi; -H_3 at theta = pi) and D^3
-// is not evolved. J may be the mean of two time levels.
-template <typename T>
-__global__ void k_ampere(GridP g, Pair3<T> Din, const T *H1, const T *H2, const T *H3, Pair3<T> J,
-                         const T *tab, const T *polar, T *D1, T *D2, T *D3, const T *Di1,
-                         const T *Di2, const T *Di3, int do_match) {
-  const int64_t n = plane_size(g);
-  const T fpi = (T)(4.0 * GRPIC_PI), dt = (T)g.dt;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int i = (int)(t % g.NX) - G_, j = (int)(t / g.NX) - G_;
-    const int64_t k = t;
-    T d1 = pv(Din, 0, k), d2 = pv(Din, 1, k), d3 = pv(Din, 2, k);
-    if (i >= 0 && i < g.n_r && j >= 0 && j <= g.n_th) {
+// is not evolved. MEAN: Din and J are means of two time levels, and only the horizon layer
+// follows; else the absorbing layer and both boundaries do.
+template <typename T, bool MEAN>
+__device__ __forceinline__ void ampere(const GridP &g, const Pair3<T> &Din, const T *H1,
+                                       const T *H2, const T *H3, const Pair3<T> &J, const T *tab,
+                                       const T *polar, T *const D[3], T *const Di[3], int64_t ps,
+                                       int i, int j, int64_t k) {
+  const T fpi = (T)(4.0 * GRPIC_PI);
+  T d1 = pv<MEAN>(Din, 0, k), d2 = pv<MEAN>(Din, 1, k), d3 = pv<MEAN>(Din, 2, k);
+  if (i >= 0 && i <= g.n_r && j >= 0 && j <= g.n_th) {
+    if (i < g.n_r) {
+      const T j1 = pv<MEAN>(J, 0, k);
       if (j == 0)
-        d1 += dt * (__ldg(H3 + k) - fpi * pv(J, 0, k)) / __ldg(polar + i + G_);
+        d1 += (T)g.dt * (__ldg(H3 + k) - fpi * j1) / __ldg(polar + i + G_);
       else if (j == g.n_th)
-        d1 += dt * (-__ldg(H3 + k - g.NX) - fpi * pv(J, 0, k)) / __ldg(polar + i + G_);
+        d1 += (T)g.dt * (-__ldg(H3 + k - g.NX) - fpi * j1) / __ldg(polar + i + G_);
       else
-        d1 += dt * ((__ldg(H3 + k) - __ldg(H3 + k - g.NX)) - fpi * pv(J, 0, k)) *
-              tabv(tab, g, CLS_HN, T_ISH, i, j);
+        d1 = fma(fma(-fpi, j1, __ldg(H3 + k) - __ldg(H3 + k - g.NX)),
+                 tabv(tab, ps, T_B2D1, k), d1);
     }
-    if (i >= 0 && i <= g.n_r && j >= 0 && j < g.n_th)
-      d2 += dt * (-(__ldg(H3 + k) - __ldg(H3 + k - 1)) - fpi * pv(J, 1, k)) *
-            tabv(tab, g, CLS_NH, T_ISH, i, j);
-    if (i >= 0 && i <= g.n_r && j >= 1 && j < g.n_th)
-      d3 += dt * ((__ldg(H2 + k) - __ldg(H2 + k - 1)) - (__ldg(H1 + k) - __ldg(H1 + k - g.NX)) -
-                  fpi * pv(J, 2, k)) *
-            tabv(tab, g, CLS_NN, T_ISH, i, j);
-    if (do_match) {
-      d1 = match(g, d1, Di1, k, polar + 2 * g.NX, i, j);
-      d2 = match(g, d2, Di2, k, polar + g.NX, i, j);
-      d3 = match(g, d3, Di3, k, polar + g.NX, i, j);
+    if (j < g.n_th) {
+      d2 = fma(-fma(fpi, pv<MEAN>(J, 1, k), __ldg(H3 + k) - __ldg(H3 + k - 1)),
+               tabv(tab, ps, T_B1D2, k), d2);
+      if (j >= 1)
+        d3 = fma(fma(-fpi, pv<MEAN>(J, 2, k),
+                     (__ldg(H2 + k) - __ldg(H2 + k - 1)) - (__ldg(H1 + k) - __ldg(H1 + k - g.NX))),
+                 tabv(tab, ps, T_D3, k), d3);
     }
-    D1[k] = d1; D2[k] = d2; D3[k] = d3;
+  }
+  if (!MEAN) {
+    d1 = match(g, d1, Di[0], k, polar + 2 * g.NX, i, j);
+    d2 = match(g, d2, Di[1], k, polar + g.NX, i, j);
+    d3 = match(g, d3, Di[2], k, polar + g.NX, i, j);
+  }
+  put<!MEAN>(g, D[0], false, (T)1, i, j, d1);
+  put<!MEAN>(g, D[1], true, (T)-1, i, j, d2);
+  put<!MEAN>(g, D[2], false, (T)-1, i, j, d3);
+}
+
+template <typename T>
+struct Planes3 {
+  T *p[3];
+};
+
+// Every stored point. The predict's Faraday: B^{n-1} -> B^n, no absorbing layer.
+template <typename T>
+__global__ void __launch_bounds__(TPBX *TPBY) k_faraday(GridP g, Pair3<T> Bin, Planes3<T> E,
+                                                        const T *tab, Planes3<T> Bout) {
+  const int i = (int)(blockIdx.x * TPBX + threadIdx.x) - G_;
+  const int64_t ps = plane_size(g);
+  for (int j = (int)(blockIdx.y * TPBY + threadIdx.y) - G_; j <= g.n_th + G_;
+       j += gridDim.y * TPBY) {
+    if (i > g.n_r + G_) return;
+    faraday<T, true, false>(g, Bin, E.p[0], E.p[1], E.p[2], tab, nullptr, Bout.p, Bout.p, ps, i,
+                            j, sidx(g, i, j));
+  }
+}
+// Step 6's Faraday B^{n-1/2} -> B^{n+1/2} and step 7's auxiliary Ampere D^{n-1/2} ->
+// D^{n+1/2}: independent of one another, one launch.
+template <typename T>
+__global__ void __launch_bounds__(TPBX *TPBY) k_faraday_ampere(
+    GridP g, Pair3<T> Bin, Planes3<T> E, Planes3<T> Bout, Planes3<T> Bi, Pair3<T> Din,
+    Planes3<T> H, Pair3<T> J, Planes3<T> Dout, const T *tab, const T *polar) {
+  const int i = (int)(blockIdx.x * TPBX + threadIdx.x) - G_;
+  const int64_t ps = plane_size(g);
+  for (int j = (int)(blockIdx.y * TPBY + threadIdx.y) - G_; j <= g.n_th + G_;
+       j += gridDim.y * TPBY) {
+    if (i > g.n_r + G_) return;
+    const int64_t k = sidx(g, i, j);
+    faraday<T, false, true>(g, Bin, E.p[0], E.p[1], E.p[2], tab, polar + g.NX, Bout.p, Bi.p, ps,
+                            i, j, k);
+    ampere<T, true>(g, Din, H.p[0], H.p[1], H.p[2], J, tab, polar, Dout.p, Dout.p, ps, i, j, k);
+  }
+}
+// The final Ampere D^n -> D^{n+1}.
+template <typename T>
+__global__ void __launch_bounds__(TPBX *TPBY) k_ampere(GridP g, Pair3<T> Din, Planes3<T> H,
+                                                       Pair3<T> J, const T *tab, const T *polar,
+                                                       Planes3<T> Dout, Planes3<T> Di) {
+  const int i = (int)(blockIdx.x * TPBX + threadIdx.x) - G_;
+  const int64_t ps = plane_size(g);
+  for (int j = (int)(blockIdx.y * TPBY + threadIdx.y) - G_; j <= g.n_th + G_;
+       j += gridDim.y * TPBY) {
+    if (i > g.n_r + G_) return;
+    ampere<T, false>(g, Din, H.p[0], H.p[1], H.p[2], J, tab, polar, Dout.p, Di.p, ps, i, j,
+                     sidx(g, i, j));
   }
 }
 
@@ -431,18 +552,18 @@ int blocks_for(int64_t n) {
 }
 
 template <typename T>
-Pair3<T> one(T *const p[3]) {
+Pair3<T> pair(T *const p[3], T *const q[3]) {
   Pair3<T> P;
-  for (int c = 0; c < 3; ++c) { P.a[c] = p[c]; P.b[c] = p[c]; }
-  P.wa = (T)1; P.wb = (T)0;
+  for (int c = 0; c < 3; ++c) { P.a[c] = p[c]; P.b[c] = q[c]; }
   return P;
 }
 template <typename T>
-Pair3<T> mean(T *const p[3], T *const q[3]) {
-  Pair3<T> P;
-  for (int c = 0; c < 3; ++c) { P.a[c] = p[c]; P.b[c] = q[c]; }
-  P.wa = (T)0.5; P.wb = (T)0.5;
-  return P;
+Pair3<T> one(T *const p[3]) {
+  return pair(p, p);
+}
+template <typename T>
+Planes3<T> planes(T *const p[3]) {
+  return {{p[0], p[1], p[2]}};
 }
 
 template <typename T>
@@ -457,16 +578,20 @@ void axis(const GridP &g, T *const p[3], int isB, cudaStream_t st) {
   k_axis<T><<<blocks_for(n), TPB, 0, st>>>(g, p[0], p[1], p[2], isB);
   COUNT_LAUNCH(1);
 }
-template <typename T>
-void auxE(const GridP &g, Pair3<T> B, Pair3<T> D, const FieldPtrsT<T> &F, cudaStream_t st) {
-  const int64_t n = (int64_t)(g.n_r + 3) * (g.n_th + 1);
-  k_aux_E<T><<<blocks_for(n), TPB, 0, st>>>(g, B, D, F.tab, F.E[0], F.E[1], F.E[2]);
-  COUNT_LAUNCH(1);
+
+// blocks of TPBX x TPBY points covering ni x nj points (rows beyond the grid's limit in y
+// are taken by the kernels' row loop)
+dim3 tiles_for(int ni, int nj) {
+  const int by = (nj + TPBY - 1) / TPBY;
+  return dim3((ni + TPBX - 1) / TPBX, by > 65535 ? 65535 : by);
 }
-template <typename T>
-void auxH(const GridP &g, Pair3<T> B, Pair3<T> D, const FieldPtrsT<T> &F, cudaStream_t st) {
-  const int64_t n = (int64_t)(g.n_r + 3) * (g.n_th + 1);
-  k_aux_H<T><<<blocks_for(n), TPB, 0, st>>>(g, B, D, F.tab, F.H[0], F.H[1], F.H[2]);
+const dim3 TILE(TPBX, TPBY);
+
+template <bool DOE, bool DOH, bool DMEAN, typename T>
+void aux(const GridP &g, const Pair3<T> &B, const Pair3<T> &D, const FieldPtrsT<T> &F,
+         cudaStream_t st) {
+  k_aux<T, DOE, DOH, DMEAN><<<tiles_for(g.n_r + 3, g.n_th + 1), TILE, 0, st>>>(
+      g, B, D, F.tab, F.E[0], F.E[1], F.E[2], F.H[0], F.H[1], F.H[2]);
   COUNT_LAUNCH(1);
 }
 
@@ -474,7 +599,7 @@ void auxH(const GridP &g, Pair3<T> B, Pair3<T> D, const FieldPtrsT<T> &F, cudaSt
 
 template <typename T>
 cudaError_t launch_metric_tables(const GridP &g, T *tab, T *polar, cudaStream_t st) {
-  k_metric_tables<T><<<blocks_for(4 * plane_size(g)), TPB, 0, st>>>(g, tab, polar);
+  k_metric_tables<T><<<blocks_for(plane_size(g)), TPB, 0, st>>>(g, tab, polar);
   COUNT_LAUNCH(1);
   return cudaGetLastError();
 }
@@ -541,15 +666,10 @@ cudaError_t launch_field_finish_init(const GridP &g, const FieldPtrsT<T> &F, int
 // E^{n-1/2} from {B^{n-1/2}, D^{n-1/2}}, auxiliary Faraday B^{n-1} -> B^n (BN planes).
 template <typename T>
 cudaError_t launch_predict(const GridP &g, const FieldPtrsT<T> &F, cudaStream_t st) {
-  auxE(g, one(F.B), mean(F.D0, F.D), F, st);
-  const Pair3<T> Bm = mean(F.B0, F.B);
-  const int64_t ps = plane_size(g);
-  k_faraday<T><<<blocks_for(ps), TPB, 0, st>>>(g, Bm, F.E[0], F.E[1], F.E[2], F.tab, nullptr,
-                                               F.Bn[0], F.Bn[1], F.Bn[2], nullptr, nullptr,
-                                               nullptr, 0);
+  aux<true, false, true>(g, one(F.B), pair(F.D0, F.D), F, st);
+  k_faraday<T><<<tiles_for(g.NX, g.NY), TILE, 0, st>>>(g, pair(F.B0, F.B), planes(F.E), F.tab,
+                                                       planes(F.Bn));
   COUNT_LAUNCH(1);
-  horizon(g, F.Bn, st);
-  axis(g, F.Bn, 1, st);
   return cudaGetLastError();
 }
 
@@ -557,30 +677,19 @@ cudaError_t launch_predict(const GridP &g, const FieldPtrsT<T> &F, cudaStream_t 
 // D^{n+1} into the D0 planes; the caller then swaps em/em0 and cur/cur0.
 template <typename T>
 cudaError_t launch_advance(const GridP &g, const FieldPtrsT<T> &F, cudaStream_t st) {
-  const int64_t ps = plane_size(g);
-  // step 6: E^n, H^n from {B^n, D^n}; Faraday B^{n-1/2} -> B^{n+1/2}
-  auxE(g, one(F.Bn), one(F.D), F, st);
-  auxH(g, one(F.Bn), one(F.D), F, st);
-  k_faraday<T><<<blocks_for(ps), TPB, 0, st>>>(g, one(F.B), F.E[0], F.E[1], F.E[2], F.tab,
-                                               F.polar + g.NX, F.B0[0], F.B0[1], F.B0[2],
-                                               F.Bi[0], F.Bi[1], F.Bi[2], 1);
+  const dim3 all = tiles_for(g.NX, g.NY);
+  // step 6: E^n, H^n from {B^n, D^n}; Faraday B^{n-1/2} -> B^{n+1/2}; step 7: auxiliary Ampere
+  // D^{n-1/2} -> D^{n+1/2} with H^n and J^n = (J^{n-1/2} + J^{n+1/2})/2
+  aux<true, true, false>(g, one(F.Bn), one(F.D), F, st);
+  k_faraday_ampere<T><<<all, TILE, 0, st>>>(g, one(F.B), planes(F.E), planes(F.B0), planes(F.Bi),
+                                            pair(F.D0, F.D), planes(F.H), pair(F.J0, F.J),
+                                            planes(F.Dh), F.tab, F.polar);
   COUNT_LAUNCH(1);
-  horizon(g, F.B0, st);
-  axis(g, F.B0, 1, st);
-  // step 7: auxiliary Ampere D^{n-1/2} -> D^{n+1/2} with H^n and J^n = (J^{n-1/2} + J^{n+1/2})/2
-  k_ampere<T><<<blocks_for(ps), TPB, 0, st>>>(g, mean(F.D0, F.D), F.H[0], F.H[1], F.H[2],
-                                              mean(F.J0, F.J), F.tab, F.polar, F.Dh[0], F.Dh[1],
-                                              F.Dh[2], nullptr, nullptr, nullptr, 0);
-  COUNT_LAUNCH(1);
-  horizon(g, F.Dh, st);
   // H^{n+1/2} from {B^{n+1/2}, D^{n+1/2}}; final Ampere D^n -> D^{n+1} with J^{n+1/2}
-  auxH(g, one(F.B0), one(F.Dh), F, st);
-  k_ampere<T><<<blocks_for(ps), TPB, 0, st>>>(g, one(F.D), F.H[0], F.H[1], F.H[2], one(F.J),
-                                              F.tab, F.polar, F.D0[0], F.D0[1], F.D0[2], F.Di[0],
-                                              F.Di[1], F.Di[2], 1);
+  aux<false, true, false>(g, one(F.B0), one(F.Dh), F, st);
+  k_ampere<T><<<all, TILE, 0, st>>>(g, one(F.D), planes(F.H), one(F.J), F.tab, F.polar,
+                                    planes(F.D0), planes(F.Di));
   COUNT_LAUNCH(1);
-  horizon(g, F.D0, st);
-  axis(g, F.D0, 0, st);
   return cudaGetLastError();
 }
 
@@ -588,8 +697,7 @@ cudaError_t launch_advance(const GridP &g, const FieldPtrsT<T> &F, cudaStream_t 
 // they stand (B^{n+1/2} and D^{n+1} after a step), into the E and H scratch planes.
 template <typename T>
 cudaError_t launch_aux_fields(const GridP &g, const FieldPtrsT<T> &F, cudaStream_t st) {
-  auxE(g, one(F.B), one(F.D), F, st);
-  auxH(g, one(F.B), one(F.D), F, st);
+  aux<true, true, false>(g, one(F.B), one(F.D), F, st);
   return cudaGetLastError();
 }
 

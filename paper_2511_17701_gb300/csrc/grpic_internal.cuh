@@ -114,10 +114,15 @@ __device__ __forceinline__ Cst<float> cst<float>(const GridP &g) {
   return {g.f_a, g.f_M, g.f_dxi, g.f_dth, g.f_ig2, g.f_dt, g.f_a2, g.f_M2};
 }
 
-// Yee point classes of the metric tables: (i, j), (i+1/2, j), (i, j+1/2), (i+1/2, j+1/2).
-enum { CLS_NN = 0, CLS_HN = 1, CLS_NH = 2, CLS_HH = 3 };
-// Quantities tabulated per class (Eq. discretized-auxE/auxH and the curls).
-enum { T_ALPHA = 0, T_H11, T_H22, T_H33, T_IHT2, T_WT13, T_WB1, T_ISH, T_NQ };
+// The field solver's coefficient tables, one plane each, stored at the component's point:
+// T_<c><f>: the factor of field component f in auxiliary component c (L, R: of its left and
+// right neighbour in x1 in an average); T_B1D2, T_B2D1, T_B3, T_D3: dt / sqrt(h) at the points of
+// B^1 and D^2 (i, j+1/2), B^2 and D^1 (i+1/2, j), B^3 (i+1/2, j+1/2), D^3 (i, j).
+enum {
+  T_E1D1 = 0, T_E1D3L, T_E1D3R, T_E2D2, T_E2B3L, T_E2B3R, T_E3D3, T_E3D1L, T_E3D1R, T_E3B2L,
+  T_E3B2R, T_H1B1, T_H1B3L, T_H1B3R, T_H2B2, T_H2D3L, T_H2D3R, T_H3B3, T_H3B1L, T_H3B1R, T_H3D2L,
+  T_H3D2R, T_B1D2, T_B2D1, T_B3, T_D3, T_NQ
+};
 
 __host__ __device__ inline int64_t plane_size(const GridP &g) { return (int64_t)g.NX * g.NY; }
 __host__ __device__ inline int64_t sidx(const GridP &g, int i, int j) {
@@ -332,7 +337,7 @@ template <typename T>
 struct FieldPtrsT {
   T *B[3], *D[3], *B0[3], *D0[3], *J[3], *J0[3], *Bn[3], *Bi[3], *Di[3];
   T *E[3], *H[3], *Dh[3];
-  const T *tab;    // [4 classes][T_NQ][plane]
+  const T *tab;    // [T_NQ][plane]
   const T *polar;  // [3][NX]: the polar area at x1 = i + 1/2, then the absorber factor
                    // absorb_coef x^3 at x1 = i and at x1 = i + 1/2 (stored at i)
 };
