@@ -29,45 +29,70 @@ __host__ __device__ constexpr DF dfc(double x) {
   return DF((float)x, (float)(x - (double)(float)x));
 }
 
+// The roundings below are explicit (__fadd_rn, __fmul_rn): a compiler that contracted a
+// product into a following sum would break the error terms.
 // s + e = a + b exactly (Knuth's two-sum)
 __device__ __forceinline__ DF two_sum(float a, float b) {
-  const float s = a + b, bb = s - a;
-  return DF(s, (a - (s - bb)) + (b - bb));
+  const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+  return DF(s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb)));
 }
 // s + e = a + b exactly when |a| >= |b| (or a = 0)
 __device__ __forceinline__ DF fast_two_sum(float a, float b) {
-  const float s = a + b;
-  return DF(s, b - (s - a));
+  const float s = __fadd_rn(a, b);
+  return DF(s, __fsub_rn(b, __fsub_rn(s, a)));
 }
 
+// The sum's high parts are added exactly, the low parts rounded: the error is within about
+// 2^-47 (|a| + |b|), 11 instructions (20 for a bound relative to |a + b|, which no use needs:
+// the terms that cancel here do so mildly).
 __device__ __forceinline__ DF operator+(DF a, DF b) {
   const DF s = two_sum(a.hi, b.hi);
-  const DF t = two_sum(a.lo, b.lo);
-  const DF u = fast_two_sum(s.hi, s.lo + t.hi);
-  return fast_two_sum(u.hi, u.lo + t.lo);
+  return fast_two_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo)));
 }
 __device__ __forceinline__ DF operator-(DF a) { return DF(-a.hi, -a.lo); }
 __device__ __forceinline__ DF operator-(DF a, DF b) { return a + (-b); }
 __device__ __forceinline__ DF operator*(DF a, DF b) {
-  const float p = a.hi * b.hi;
+  const float p = __fmul_rn(a.hi, b.hi);
   float e = fmaf(a.hi, b.hi, -p);  // the product's rounding error, exactly
   e = fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, e));
   return fast_two_sum(p, e);
 }
-__device__ __forceinline__ DF fma_(DF a, DF b, DF c) { return a * b + c; }
+// a b + c without normalising the product first
+__device__ __forceinline__ DF fma_(DF a, DF b, DF c) {
+  const float p = __fmul_rn(a.hi, b.hi);
+  float e = fmaf(a.hi, b.hi, -p);
+  e = fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, e));
+  const DF s = two_sum(p, c.hi);
+  return fast_two_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(e, c.lo)));
+}
+// a times a power of two (exact)
+__device__ __forceinline__ DF df_scale(DF a, float p2) { return DF(a.hi * p2, a.lo * p2); }
 
-// 1/b: the FP32 reciprocal refined by one Newton step in pairs (the error squares: 2^-44)
+// 1/b: the FP32 reciprocal r (within 2 ulp) refined in pairs, r (1 + e + e^2) with
+// e = 1 - b r (|e| < 2^-21, so the third order is below 2^-63)
 __device__ __forceinline__ DF df_rcp(DF b) {
-  const DF r(__fdividef(1.0f, b.hi));
-  const DF e = DF(1.0f) - b * r;
-  return r + r * e;
+  const float r = __fdividef(1.0f, b.hi);
+  const float p = __fmul_rn(b.hi, r);
+  // 1 - b r: 1 - p is exact (p within 2^-21 of 1), the other terms are small
+  const DF e = two_sum(__fsub_rn(1.0f, p), -fmaf(b.lo, r, fmaf(b.hi, r, -p)));
+  const float q = __fmul_rn(r, e.hi);
+  const float ql = fmaf(r, e.hi, -q) + r * fmaf(e.hi, e.hi, e.lo);
+  const DF s = fast_two_sum(r, q);
+  return fast_two_sum(s.hi, __fadd_rn(s.lo, ql));
 }
 __device__ __forceinline__ DF operator/(DF a, DF b) { return a * df_rcp(b); }
-// 1/sqrt(x): the FP32 value refined by one Newton step in pairs, r + r (1 - x r^2) / 2
+// 1/sqrt(x): the FP32 value r refined in pairs, r (1 + e/2 + 3 e^2 / 8) with e = 1 - x r^2
+// (|e| < 2^-20, so the third order is below 2^-61)
 __device__ __forceinline__ DF df_rsqrt(DF x) {
-  const DF r(rsqrtf(x.hi));
-  const DF e = DF(1.0f) - x * (r * r);
-  return r + r * DF(0.5f * e.hi, 0.5f * e.lo);
+  const float r = rsqrtf(x.hi);
+  const float y = __fmul_rn(r, r);
+  const DF xr = x * DF(y, fmaf(r, r, -y));
+  const DF e = two_sum(__fsub_rn(1.0f, xr.hi), -xr.lo);
+  const float h = 0.5f * r;
+  const float q = __fmul_rn(h, e.hi);
+  const float ql = fmaf(h, e.hi, -q) + h * fmaf(0.75f * e.hi, e.hi, e.lo);
+  const DF s = fast_two_sum(r, q);
+  return fast_two_sum(s.hi, __fadd_rn(s.lo, ql));
 }
 __device__ __forceinline__ DF rsqrt_(DF x) { return df_rsqrt(x); }
 

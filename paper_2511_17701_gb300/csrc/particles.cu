@@ -769,6 +769,12 @@ __device__ __forceinline__ void push64(const GridP &g, const FieldPtrsT<T> &F,
   if (DEPOSIT) deposit64(g, F, s.qc * (double)s.w[k], i1, i2, x1, x2, j1, j2, xb1, xb2, v3);
 }
 
+}  // namespace
+
+#include "push_inc.cuh"
+
+namespace {
+
 // =================================================================================
 // FP32 routine (mixed precision, particles off the horizon and axis guard zones).
 // Positions stay cell + offset: every coordinate is handled relative to the start cell,
@@ -1197,12 +1203,15 @@ __device__ __forceinline__ int guard_zone(const PushTables &tb, const GridP &g, 
 // Bound by the FP64 pipe; on 67 M particles of the 2048^2 workload 3 resident blocks per SM
 // (166 registers, no spills) measured 85.4 ms per launch against 86.9 ms with 4 (128
 // registers, spills) and 89.3 ms with 5 (96 registers).
-template <bool DEPOSIT, bool Q>
+// INC: the increment form (push_inc.cuh) for the particles it covers. A warp in which one
+// particle does not fit goes to push64 as a whole, so that no warp runs both for long.
 #ifndef GRPIC_PUSH64_MIN_BLOCKS  // resident blocks per SM the fused FP64 kernel is built for
 #define GRPIC_PUSH64_MIN_BLOCKS 3
 #endif
-__global__ void __launch_bounds__(TPB, DEPOSIT ? GRPIC_PUSH64_MIN_BLOCKS : 3) k_push(GridP g, FieldPtrsT<double> F, PushTables tb,
-                                              SpeciesDevT<double> s, unsigned long long *diag) {
+template <bool DEPOSIT, bool Q, bool INC>
+__global__ void __launch_bounds__(TPB, GRPIC_PUSH64_MIN_BLOCKS)
+    k_push(GridP g, FieldPtrsT<double> F, PushTables tb, SpeciesDevT<double> s,
+           unsigned long long *diag) {
   const int64_t n = *s.n;
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
        k += (int64_t)gridDim.x * blockDim.x) {
@@ -1214,8 +1223,17 @@ __global__ void __launch_bounds__(TPB, DEPOSIT ? GRPIC_PUSH64_MIN_BLOCKS : 3) k_
       if (tag != 0) s.tag[k] = 0;
       continue;
     }
+    if (INC && __all_sync(__activemask(), inc_fit(g, F, tb, s, k)) &&
+        push_inc<DEPOSIT>(g, F, tb, s, k, diag))
+      continue;
     push64<Q, double, DEPOSIT>(g, F, tb, s, k, diag);
   }
+}
+
+// Whether a run's FP64 pushes may take the increment form: the refined iterations on the
+// plain grid, with rows away from the axes clear of the small-angle clamp.
+bool inc_applies(const GridP &g) {
+  return !g.qks && g.iter_tol > 0.0 && g.n_iter >= 2 && g.small_angle < g.dth;
 }
 
 // Mixed path, classification: zone 1 and zone 2 particles are appended to their lists
@@ -1684,8 +1702,14 @@ cudaError_t push_impl(const GridP &g, const FieldPtrsT<T> &F, SpeciesDevT<T> s,
   if constexpr (sizeof(T) == 8) {
     if (!main_stage) return cudaSuccess;  // the FP64 path has no guard stage
     if (ps.t0) cudaEventRecord(ps.t0, ps.main);
-    if (deposit) k_push<true, Q><<<blocks_for(n_bound), TPB, 0, ps.main>>>(g, F, tb, s, diag);
-    else k_push<false, Q><<<blocks_for(n_bound), TPB, 0, ps.main>>>(g, F, tb, s, diag);
+    const int b = blocks_for(n_bound);
+    if (!Q && inc_applies(g)) {
+      if (deposit) k_push<true, false, true><<<b, TPB, 0, ps.main>>>(g, F, tb, s, diag);
+      else k_push<false, false, true><<<b, TPB, 0, ps.main>>>(g, F, tb, s, diag);
+    } else {
+      if (deposit) k_push<true, Q, false><<<b, TPB, 0, ps.main>>>(g, F, tb, s, diag);
+      else k_push<false, Q, false><<<b, TPB, 0, ps.main>>>(g, F, tb, s, diag);
+    }
     if (ps.t1) cudaEventRecord(ps.t1, ps.main);
     COUNT_LAUNCH(1);
   } else {
