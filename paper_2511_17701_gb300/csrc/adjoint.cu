@@ -16,8 +16,13 @@
 // differentiation through the iterations: at the fixed point t* = G(t*, p),
 // dt* = (I - dG/dt)^{-1} (dG/dp) dp. The Jacobians of a segment are formed while its states
 // are recomputed and kept in scratch memory for the reverse sweep.
+//
+// Both passes run a step in the increment form of inc.cuh where it applies: the state's
+// increment and J - 1, which are small against the state and 1, in pairs of floats, added in
+// FP64. The general FP64 form (step_values, step_jacobian) takes the rest.
 #include "dual.cuh"
 #include "grpic_internal.cuh"
+#include "inc.cuh"
 #include "pusher.cuh"
 
 namespace {
@@ -141,7 +146,7 @@ struct StepVals {
   bool ok;       // finite and inside 0 <= x1 < n_r, 0 <= x2 <= n_th
 };
 
-__device__ __forceinline__ void step_values(const GridP &g, const FieldPtrsT<double> &F,
+__device__ __noinline__ void step_values(const GridP &g, const FieldPtrsT<double> &F,
                                             const double st[6], double scale, double qm,
                                             int n_iter, StepVals &sv, Frame<double> &fr) {
   const double x[2] = {st[0], st[1]}, u[3] = {st[3], st[4], st[5]};
@@ -200,7 +205,7 @@ __device__ __forceinline__ void inv_i_minus(const double A[2][2], double M[2][2]
 // The step's Jacobian at st: J[r][c] = d(output r)/d(input c), outputs x1, x2, phi, u1, u2,
 // u3 after the step, inputs x1, x2, u1, u2, u3, scale (the phi column is the unit vector).
 constexpr int JC = 6;  // stored input columns
-__device__ void step_jacobian(const GridP &g, const FieldPtrsT<double> &F, const double st[6],
+__device__ __noinline__ void step_jacobian(const GridP &g, const FieldPtrsT<double> &F, const double st[6],
                               double scale, double qm, const StepVals &sv,
                               const Frame<double> &fr, double J[6][JC]) {
   // the implicit-function theorem's matrices: (I - dG/dt)^{-1} of the geodesic map at its fixed
@@ -321,12 +326,309 @@ __device__ void step_jacobian(const GridP &g, const FieldPtrsT<double> &F, const
   }
 }
 
-__global__ void __launch_bounds__(TPB_ADJ) k_adj_forward(GridP g, FieldPtrsT<double> F, int64_t n,
-                                                        double qm, double scale, int n_steps,
-                                                        int every, int n_iter,
-                                                        const double *__restrict__ st0,
-                                                        double *__restrict__ out,
-                                                        double *__restrict__ ckpt) {
+// ---------------------------------------------------------------------------------
+// A step in the increment form. GB300's FP64 pipe bounded both passes (~1800 FP64 operations
+// per particle-step forward, ~5500 backward, most of them exp and sincos per iterate and the
+// metric's derivatives in duals); here FP64 is left with one or two evaluations of the
+// coordinate map and the additions to the state. 65,536 orbits on 512^2, 100 steps forward and
+// back: 106.3 -> 28.1 ms, the gradients' error against FP64 references 1.2e-14 -> 1.1e-14. The
+// backward kernel is bound by the latency of its pair arithmetic at 8 warps per SM (255
+// registers, spills).
+// ---------------------------------------------------------------------------------
+constexpr int INC_MIN_ITER = 16;   // iteration counts below are taken literally (general form)
+constexpr float INC_ADJ_TOL = 1e-16f;
+
+struct AdjStep {
+  int i1, i2;
+  DF o1, o2;            // x^n in its cell
+  DF r, s, c;           // there
+  Local<DF> L;
+  DF V[6];              // B, D at x^n, unit amplitude
+  DF eB1[3], eD1[3];    // e B, e D in the tetrad frame at unit amplitude, e = qm alpha dt/4
+  DF eB[3], eD[3];      // at the amplitude
+  DF u[3], u1[3], dg[2], u2[3], un[3];  // u^n, after the first EM half step, the geodesic
+                        // substep's increment, after it, u^{n+1}
+  double u64[3], x64[2], v3, mid[2];    // u^{n+1}, x^{n+1}, dphi/dt; the midpoint's offsets
+};
+
+// The values of a step; false: not covered by the increment form.
+__device__ __forceinline__ bool adj_inc_step(const GridP &g, const FieldPtrsT<double> &F,
+                                             const PushTables &tb, const IncC &k,
+                                             const double st[6], DF scale, DF qm, int n_iter,
+                                             AdjStep &a) {
+  const double f1 = floor(st[0]), f2 = floor(st[1]);
+  a.i1 = (int)f1;
+  a.i2 = (int)f2;
+  if (!(a.i1 >= 0 && a.i1 < g.n_r && a.i2 >= 2 && a.i2 < g.n_th - 2)) return false;
+  const double dx1 = st[0] - f1, dx2 = st[1] - f2;
+  a.o1 = df_of(dx1);
+  a.o2 = df_of(dx2);
+  if (!inc_point(k, tb, a.i1, a.i2, a.o1, a.o2, a.r, a.s, a.c)) return false;
+  inc_local(k, a.r, a.s, a.c, a.L);
+  IncLerp l;
+  inc_lerp(a.i1, a.i2, a.o1, a.o2, l);
+  a.V[0] = inc_interp(F.B[0], g.NX, l, 0, 1);
+  a.V[1] = inc_interp(F.B[1], g.NX, l, 1, 0);
+  a.V[2] = inc_interp(F.B[2], g.NX, l, 1, 1);
+  a.V[3] = inc_interp(F.D[0], g.NX, l, 1, 0);
+  a.V[4] = inc_interp(F.D[1], g.NX, l, 0, 1);
+  a.V[5] = inc_interp(F.D[2], g.NX, l, 0, 0);
+  vec_hat(a.L, a.V, a.eB1);
+  vec_hat(a.L, a.V + 3, a.eD1);
+  const DF e = df_scale(qm * a.L.alpha * k.dt, 0.25f);
+  DF du[3] = {DF(0.0f), DF(0.0f), DF(0.0f)};
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    a.eB1[q] = e * a.eB1[q];
+    a.eD1[q] = e * a.eD1[q];
+    a.eB[q] = scale * a.eB1[q];
+    a.eD[q] = scale * a.eD1[q];
+    a.u[q] = df_of(st[3 + q]);
+  }
+  if (!inc_boris(a.L, a.eD, a.eB, a.u, du)) return false;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) a.u1[q] = a.u[q] + du[q];
+  GeoInc<DF> m;
+  geo_inc_setup(k, a.L, a.u1, 1.0f, m);
+  if (!geo_inc_solve(m, n_iter, INC_ADJ_TOL, a.dg[0], a.dg[1])) return false;
+  du[0] = du[0] + a.dg[0];
+  du[1] = du[1] + a.dg[1];
+  a.u2[0] = a.u[0] + du[0];
+  a.u2[1] = a.u[1] + du[1];
+  a.u2[2] = a.u1[2];
+  if (!inc_boris(a.L, a.eD, a.eB, a.u2, du)) return false;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    a.un[q] = a.u[q] + du[q];
+    a.u64[q] = st[3 + q] + df_to_double(du[q]);
+  }
+  double t1, t2;
+  if (!inc_coord<true>(g, k, tb, n_iter, INC_ADJ_TOL, a.i1, a.i2, dx1, dx2, a.o1, a.o2, a.u64,
+                       a.un, 1.0, 1.0f, t1, t2, a.v3))
+    return false;
+  a.mid[0] = 0.5 * (dx1 + t1);
+  a.mid[1] = 0.5 * (dx2 + t2);
+  a.x64[0] = f1 + t1;
+  a.x64[1] = f2 + t2;
+  return finite64(a.u64[0]) && finite64(a.u64[1]) && finite64(a.u64[2]);
+}
+
+// a field component at x^n with its derivatives along x1, x2 (V: its value)
+__device__ __forceinline__ D2F adj_interp_d(const double *__restrict__ pl, int NX, const IncLerp &l,
+                                            int h1, int h2, DF V) {
+  const double *p = pl + (int64_t)(l.j[h2] + G_) * NX + (l.i[h1] + G_);
+  const DF p00 = df_of(__ldg(p)), p10 = df_of(__ldg(p + 1));
+  const DF p01 = df_of(__ldg(p + NX)), p11 = df_of(__ldg(p + NX + 1));
+  const DF x0 = p10 - p00, x1 = p11 - p01, y0 = p01 - p00;
+  const DF xy = x1 - x0;
+  return D2F(V, fma_(l.w2[h2], xy, x0), fma_(l.w1[h1], xy, y0));
+}
+
+// The momentum's derivative along two directions: du' of u^{n+1} - u^n for metric values L
+// (M: DF, or D2F where the directions move x^n), u and the fields with their derivatives.
+// K: the geodesic substep's (I - A)^{-1}; G3 = its map's derivative with respect to u_3.
+template <typename M>
+__device__ __forceinline__ void adj_momentum_d(const IncC &k, const Local<M> &L, const D2F eD[3],
+                                               const D2F eB[3], const D2F u[3], const AdjStep &a,
+                                               const DF K[2][2], D2F du[3]) {
+  D2F h[3], x[3];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) du[q] = D2F(0.0f);
+  inc_boris_core(L, eD, eB, u, du, h, x);
+  D2F v[3] = {u[0] + du[0], u[1] + du[1], u[2] + du[2]};
+  {
+    GeoInc<D2F> m;
+    geo_inc_setup(k, L, v, 1.0f, m);
+    D2F n0, n1;
+    geo_inc_apply(m, a.dg[0], a.dg[1], n0, n1);
+    // implicit-function theorem at the fixed point
+    du[0].d0 = du[0].d0 + fma_(K[0][0], n0.d0, K[0][1] * n1.d0);
+    du[0].d1 = du[0].d1 + fma_(K[0][0], n0.d1, K[0][1] * n1.d1);
+    du[1].d0 = du[1].d0 + fma_(K[1][0], n0.d0, K[1][1] * n1.d0);
+    du[1].d1 = du[1].d1 + fma_(K[1][0], n0.d1, K[1][1] * n1.d1);
+  }
+#pragma unroll
+  for (int q = 0; q < 3; ++q) v[q] = D2F(a.u2[q], u[q].d0 + du[q].d0, u[q].d1 + du[q].d1);
+  inc_boris_core(L, eD, eB, v, du, h, x);
+}
+
+// (I - A)^{-1}
+__device__ __forceinline__ void adj_inv(const DF A[2][2], DF K[2][2]) {
+  const DF p = DF(1.0f) - A[0][0], q = DF(1.0f) - A[1][1];
+  const DF id = df_rcp(fma_(p, q, -(A[0][1] * A[1][0])));
+  K[0][0] = q * id;
+  K[0][1] = A[0][1] * id;
+  K[1][0] = A[1][0] * id;
+  K[1][1] = p * id;
+}
+
+// A step's derivatives in scratch memory: entry (row, column) of rows x1, x2, phi, u1, u2, u3
+// and columns x1, x2, u1, u2, u3, scale at w[(row * JC + column) n], either J - 1 as pairs (lo,
+// hi) or J as doubles; which one is the lowest bit of entry (0, 0): clear for pairs, set for
+// doubles (half an ulp of that one entry).
+__device__ __forceinline__ float2 adj_pack(DF a, bool first) {
+  return make_float2(first ? __uint_as_float(__float_as_uint(a.lo) & ~1u) : a.lo, a.hi);
+}
+
+__device__ __forceinline__ void adj_inc_jacobian(const GridP &g, const FieldPtrsT<double> &F,
+                                                 const PushTables &tb, const IncC &k, DF scale,
+                                                 DF qm, const AdjStep &a, double *wd, int64_t n) {
+  float2 *w = reinterpret_cast<float2 *>(wd);
+  // the coordinate map's velocity (inc_velocity's grouping) at the midpoint: its derivatives
+  // along x (Vx) and along u (Vu): with P_j = half of dX/du_j, V_j + beta_j = G P_j and
+  // dV_j/du_k = G (c_jk - P_j P_k / N), N = m2 Sigma + X
+  DF Vx[3][2], Vu[3][3], Mx[2][2];
+  {
+    DF r, s, c;
+    inc_point(k, tb, a.i1, a.i2, df_of(a.mid[0]), df_of(a.mid[1]), r, s, c);
+    const D2F R(r, k.dxi * r, DF(0.0f)), S(s, DF(0.0f), c * k.dth), C(c, DF(0.0f), -(s * k.dth));
+    const D2F s2 = S * S, r2 = R * R, f = k.dxi * R;
+    const D2F Sig = fma_(k.a2, C * C, r2), M2r = df_scale(k.M * R, 2.0f), S2 = Sig + M2r;
+    const D2F Rr = r2 + k.a2, A = fma_(Rr, Rr, -(k.a2 * s2 * (Rr - M2r)));
+    const D2F fs = f * s2, iQ = df_rcp(S2 * fs), iS2 = iQ * fs, T = iQ * S2;
+    const D2F fi = T * s2, w0 = a.un[0] * fi, AS = A * iS2, is2 = T * f;
+    const DF au = k.a * a.un[2], kk = k.ig2 * a.un[1];
+    const D2F I = fma_(AS, w0, D2F(au)), z = a.un[2] * is2;
+    const D2F X = fma_(w0, I + au, fma_(a.un[2], z, D2F(kk * a.un[1])));
+    const D2F G = df_rsqrt(S2 * (Sig + X));
+    const D2F P0 = fi * I, P2 = fma_(k.a, w0, z);
+    const D2F V0 = fma_(G, P0, -(M2r * iS2 * fi)), V1 = G * kk, V2 = G * P2;
+    Vx[0][0] = V0.d0; Vx[0][1] = V0.d1;
+    Vx[1][0] = V1.d0; Vx[1][1] = V1.d1;
+    Vx[2][0] = V2.d0; Vx[2][1] = V2.d1;
+    const DF iN = G.v * G.v * S2.v;
+    const DF q0 = P0.v * iN, q1 = kk * iN, q2 = P2.v * iN;
+    Vu[0][0] = G.v * (fi.v * fi.v * AS.v - q0 * P0.v);
+    Vu[1][1] = G.v * (k.ig2 - q1 * kk);
+    Vu[2][2] = G.v * (is2.v - q2 * P2.v);
+    Vu[0][1] = Vu[1][0] = -(G.v * (q0 * kk));
+    Vu[0][2] = Vu[2][0] = G.v * (k.a * fi.v - q0 * P2.v);
+    Vu[1][2] = Vu[2][1] = -(G.v * (q1 * P2.v));
+    const DF h = df_scale(k.dt, 0.5f);
+    const DF B[2][2] = {{h * Vx[0][0], h * Vx[0][1]}, {h * Vx[1][0], h * Vx[1][1]}};
+    adj_inv(B, Mx);
+  }
+  DF K[2][2];
+  {
+    GeoInc<DF> m;
+    geo_inc_setup(k, a.L, a.u1, 1.0f, m);
+    DF A[2][2];
+    geo_inc_jacobian(m, a.dg[0], a.dg[1], A);
+    adj_inv(A, K);
+  }
+  // a column: the increments' derivatives from that of u^{n+1} (seed + du') and x^n (xs)
+  auto column = [&](int col, const DF du[3], const DF seed[3], DF xs0, DF xs1) {
+    const DF p0 = seed[0] + du[0], p1 = seed[1] + du[1], p2 = seed[2] + du[2];
+    DF v[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+      v[q] = fma_(Vu[q][0], p0, fma_(Vu[q][1], p1, fma_(Vu[q][2], p2, fma_(Vx[q][0], xs0, Vx[q][1] * xs1))));
+    const DF y0 = k.dt * fma_(Mx[0][0], v[0], Mx[0][1] * v[1]);
+    const DF y1 = k.dt * fma_(Mx[1][0], v[0], Mx[1][1] * v[1]);
+    // dphi/dt moves with the midpoint, x + y/2
+    const DF ph = k.dt * (v[2] + df_scale(fma_(Vx[2][0], y0, Vx[2][1] * y1), 0.5f));
+    const DF o[6] = {y0, y1, ph, du[0], du[1], du[2]};
+#pragma unroll
+    for (int q = 0; q < 6; ++q)
+      w[(int64_t)(q * JC + col) * n] = adj_pack(o[q], q == 0 && col == 0);
+  };
+  const DF zero(0.0f), one(1.0f);
+  {  // x1, x2: metric, tetrads and fields move
+    const D2F R(a.r, k.dxi * a.r, zero), S(a.s, zero, a.c * k.dth), C(a.c, zero, -(a.s * k.dth));
+    Local<D2F> L;
+    inc_local(k, R, S, C, L);
+    D2F eB[3], eD[3];
+    {
+      IncLerp l;
+      inc_lerp(a.i1, a.i2, a.o1, a.o2, l);
+      const D2F V[6] = {adj_interp_d(F.B[0], g.NX, l, 0, 1, a.V[0]),
+                        adj_interp_d(F.B[1], g.NX, l, 1, 0, a.V[1]),
+                        adj_interp_d(F.B[2], g.NX, l, 1, 1, a.V[2]),
+                        adj_interp_d(F.D[0], g.NX, l, 1, 0, a.V[3]),
+                        adj_interp_d(F.D[1], g.NX, l, 0, 1, a.V[4]),
+                        adj_interp_d(F.D[2], g.NX, l, 0, 0, a.V[5])};
+      vec_hat(L, V, eB);
+      vec_hat(L, V + 3, eD);
+      const D2F e = df_scale(scale * qm * k.dt, 0.25f) * L.alpha;
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        eB[q] = e * eB[q];
+        eD[q] = e * eD[q];
+      }
+    }
+    const D2F u[3] = {D2F(a.u[0]), D2F(a.u[1]), D2F(a.u[2])};
+    D2F du[3];
+    adj_momentum_d(k, L, eD, eB, u, a, K, du);
+    const DF s0[3] = {zero, zero, zero};
+    const DF c0[3] = {du[0].d0, du[1].d0, du[2].d0}, c1[3] = {du[0].d1, du[1].d1, du[2].d1};
+    column(0, c0, s0, one, zero);
+    column(1, c1, s0, zero, one);
+  }
+#pragma unroll 1
+  for (int half = 0; half < 2; ++half) {  // (u1, u2), then (u3, scale)
+    const bool first = half == 0;
+    const DF on = first ? one : zero, off = first ? zero : one;
+    D2F eB[3], eD[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      eB[q] = D2F(a.eB[q], zero, off * a.eB1[q]);
+      eD[q] = D2F(a.eD[q], zero, off * a.eD1[q]);
+    }
+    const D2F u[3] = {D2F(a.u[0], on, zero), D2F(a.u[1], zero, on), D2F(a.u[2], off, zero)};
+    D2F du[3];
+    adj_momentum_d(k, a.L, eD, eB, u, a, K, du);
+    const DF s0[3] = {on, zero, off}, s1[3] = {zero, on, zero};
+    const DF c0[3] = {du[0].d0, du[1].d0, du[2].d0}, c1[3] = {du[0].d1, du[1].d1, du[2].d1};
+    column(2 + 2 * half, c0, s0, zero, zero);
+    column(3 + 2 * half, c1, s1, zero, zero);
+  }
+}
+
+// One step forward from st in either form; false: the particle left the domain
+template <bool INC>
+__device__ __forceinline__ bool adj_advance(const GridP &g, const FieldPtrsT<double> &F,
+                                            const PushTables &tb, const IncC &k, double scale,
+                                            DF scale_df, double qm, DF qm_df, int n_iter,
+                                            double st[6], double *w, int64_t n) {
+  if (INC) {
+    AdjStep a;
+    if (adj_inc_step(g, F, tb, k, st, scale_df, qm_df, n_iter, a)) {
+      const bool ok = a.x64[0] >= 0.0 && a.x64[0] < g.n_r && a.x64[1] >= 0.0 && a.x64[1] <= g.n_th;
+      if (!ok) return false;
+      if (w) adj_inc_jacobian(g, F, tb, k, scale_df, qm_df, a, w, n);
+      st[0] = a.x64[0];
+      st[1] = a.x64[1];
+      st[2] = fma(g.dt, a.v3, st[2]);
+      st[3] = a.u64[0];
+      st[4] = a.u64[1];
+      st[5] = a.u64[2];
+      return true;
+    }
+  }
+  StepVals sv;
+  Frame<double> fr;
+  step_values(g, F, st, scale, qm, n_iter, sv, fr);
+  if (!sv.ok) return false;
+  if (w) {
+    double J[6][JC];
+    step_jacobian(g, F, st, scale, qm, sv, fr, J);
+    for (int r = 0; r < 6; ++r)
+      for (int c = 0; c < JC; ++c) w[(int64_t)(r * JC + c) * n] = J[r][c];
+    w[0] = __longlong_as_double(__double_as_longlong(J[0][0]) | 1ll);
+  }
+  st[0] = sv.xn[0]; st[1] = sv.xn[1]; st[2] = sv.phin;
+  st[3] = sv.un[0]; st[4] = sv.un[1]; st[5] = sv.un[2];
+  return true;
+}
+
+template <bool INC>
+__global__ void __launch_bounds__(TPB_ADJ) k_adj_forward(
+    const __grid_constant__ GridP g, const __grid_constant__ FieldPtrsT<double> F,
+    const __grid_constant__ PushTables tb, int64_t n, double qm, double scale, int n_steps,
+    int every, int n_iter, const double *__restrict__ st0, double *__restrict__ out,
+    double *__restrict__ ckpt) {
+  const IncC kc = inc_c(g);
+  const DF sd = df_of(scale), qd = df_of(qm);
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
        k += (int64_t)gridDim.x * blockDim.x) {
     double st[6];
@@ -338,24 +640,65 @@ __global__ void __launch_bounds__(TPB_ADJ) k_adj_forward(GridP g, FieldPtrsT<dou
         for (int q = 0; q < 6; ++q) c[q * n + k] = bad ? NAN : st[q];
       }
       if (bad) continue;
-      StepVals sv;
-      Frame<double> fr;
-      step_values(g, F, st, scale, qm, n_iter, sv, fr);
-      if (!sv.ok) {
-        bad = true;
-        continue;
-      }
-      st[0] = sv.xn[0]; st[1] = sv.xn[1]; st[2] = sv.phin;
-      st[3] = sv.un[0]; st[4] = sv.un[1]; st[5] = sv.un[2];
+      bad = !adj_advance<INC>(g, F, tb, kc, scale, sd, qm, qd, n_iter, st, nullptr, n);
     }
     for (int q = 0; q < 6; ++q) out[q * n + k] = bad ? NAN : st[q];
   }
 }
 
+// lambda <- J^T lambda and the scale's derivative. With J - 1 in pairs: lambda += (J - 1)^T
+// lambda, the products in pairs on lambda scaled by the power of two that brings its largest
+// entry near 1 (any magnitude keeps its bits), the sums in FP64.
+__device__ __forceinline__ void adj_reverse(const double *w, int64_t n, double lam[6],
+                                            double &gs) {
+  // inputs x1, x2, u1, u2, u3 are state rows 0, 1, 3, 4, 5; phi passes through
+  const int row[5] = {0, 1, 3, 4, 5};
+  if (__double_as_longlong(w[0]) & 1ll) {
+    double nl[JC] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    for (int r = 0; r < 6; ++r)
+#pragma unroll
+      for (int c = 0; c < JC; ++c) nl[c] = fma(w[(int64_t)(r * JC + c) * n], lam[r], nl[c]);
+#pragma unroll
+    for (int c = 0; c < 5; ++c) lam[row[c]] = nl[c];
+    gs += nl[5];
+    return;
+  }
+  unsigned top = 0;
+#pragma unroll
+  for (int q = 0; q < 6; ++q)
+    top = max(top, ((unsigned)__double2hiint(lam[q]) >> 20) & 0x7ffu);
+  const unsigned tc = min(max(top, 1u), 2045u);
+  const double down = __hiloint2double((int)((2046u - tc) << 20), 0);  // 2^(1023 - tc)
+  const double up = __hiloint2double((int)(tc << 20), 0);              // 2^(tc - 1023)
+  DF l[6];
+#pragma unroll
+  for (int q = 0; q < 6; ++q) l[q] = df_of(lam[q] * down);
+  DF nl[JC];
+#pragma unroll
+  for (int c = 0; c < JC; ++c) nl[c] = DF(0.0f);
+#pragma unroll
+  for (int r = 0; r < 6; ++r)
+#pragma unroll
+    for (int c = 0; c < JC; ++c) {
+      const float2 v = reinterpret_cast<const float2 *>(w)[(int64_t)(r * JC + c) * n];
+      nl[c] = fma_(DF(v.y, v.x), l[r], nl[c]);
+    }
+  const bool lost = top == 0x7ffu;  // infinities and NaN stay such
+#pragma unroll
+  for (int c = 0; c < 5; ++c)
+    lam[row[c]] = lost ? lam[row[c]] + NAN : fma(df_to_double(nl[c]), up, lam[row[c]]);
+  gs = lost ? NAN : fma(df_to_double(nl[5]), up, gs);
+}
+
+template <bool INC>
 __global__ void __launch_bounds__(TPB_ADJ) k_adj_backward(
-    GridP g, FieldPtrsT<double> F, int64_t n, double qm, double scale, double gfac, int n_steps,
-    int every, int n_iter, const double *__restrict__ ckpt, const double *__restrict__ gout,
-    double *__restrict__ gin, double *__restrict__ gscale, double *__restrict__ scratch) {
+    const __grid_constant__ GridP g, const __grid_constant__ FieldPtrsT<double> F,
+    const __grid_constant__ PushTables tb, int64_t n, double qm, double scale, double gfac,
+    int n_steps, int every, int n_iter, const double *__restrict__ ckpt,
+    const double *__restrict__ gout, double *__restrict__ gin, double *__restrict__ gscale,
+    double *__restrict__ scratch) {
+  const IncC kc = inc_c(g);
+  const DF sd = df_of(scale), qd = df_of(qm);
   const int n_seg = (n_steps + every - 1) / every;
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
        k += (int64_t)gridDim.x * blockDim.x) {
@@ -377,36 +720,12 @@ __global__ void __launch_bounds__(TPB_ADJ) k_adj_backward(
         break;
       }
       // recompute the segment from its checkpoint, keeping each step's Jacobian
-      for (int j = 0; j < len; ++j) {
-        StepVals sv;
-        Frame<double> fr;
-        step_values(g, F, st, scale, qm, n_iter, sv, fr);
-        if (!sv.ok) {
-          bad = true;
-          break;
-        }
-        double J[6][JC];
-        step_jacobian(g, F, st, scale, qm, sv, fr, J);
-        double *w = scratch + (int64_t)j * 6 * JC * n + k;
-        for (int r = 0; r < 6; ++r)
-          for (int cc = 0; cc < JC; ++cc) w[(int64_t)(r * JC + cc) * n] = J[r][cc];
-        st[0] = sv.xn[0]; st[1] = sv.xn[1]; st[2] = sv.phin;
-        st[3] = sv.un[0]; st[4] = sv.un[1]; st[5] = sv.un[2];
-      }
+      double *w = scratch + k;
+      for (int j = 0; j < len && !bad; ++j)
+        bad = !adj_advance<INC>(g, F, tb, kc, scale, sd, qm, qd, n_iter, st,
+                                w + (int64_t)j * 6 * JC * n, n);
       // reverse sweep: lambda_n = J_n^T lambda_{n+1}
-      for (int j = len - 1; j >= 0 && !bad; --j) {
-        const double *w = scratch + (int64_t)j * 6 * JC * n + k;
-        double nl[JC] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-        for (int r = 0; r < 6; ++r)
-          for (int cc = 0; cc < JC; ++cc) nl[cc] = fma(w[(int64_t)(r * JC + cc) * n], lam[r], nl[cc]);
-        // inputs x1, x2, u1, u2, u3 map to state rows 0, 1, 3, 4, 5; phi passes through
-        lam[0] = nl[0];
-        lam[1] = nl[1];
-        lam[3] = nl[2];
-        lam[4] = nl[3];
-        lam[5] = nl[4];
-        gs += nl[5];
-      }
+      for (int j = len - 1; j >= 0 && !bad; --j) adj_reverse(w + (int64_t)j * 6 * JC * n, n, lam, gs);
     }
     // a particle that reached a boundary has no gradient: zero where its cotangent was zero
     // (it does not enter the loss), NaN otherwise
@@ -439,26 +758,35 @@ int adj_blocks(int64_t n) {
 
 }  // namespace
 
-cudaError_t launch_adjoint_forward(const GridP &g, const FieldPtrsT<double> &F, int64_t n,
-                                   double qm, double scale, int n_steps, int every, int n_iter,
-                                   const double *st0, double *out, double *ckpt,
-                                   cudaStream_t st) {
+// Whether the increment form may take steps: rows away from the axes clear of the
+// small-angle clamp, and an iteration limit that is one (the general form takes a small one
+// literally).
+static bool adj_inc_applies(const GridP &g, int n_iter) {
+  return n_iter >= INC_MIN_ITER && g.small_angle < g.dth;
+}
+
+cudaError_t launch_adjoint_forward(const GridP &g, const FieldPtrsT<double> &F,
+                                   const PushTables &tb, int64_t n, double qm, double scale,
+                                   int n_steps, int every, int n_iter, const double *st0,
+                                   double *out, double *ckpt, cudaStream_t st) {
   if (n <= 0) return cudaGetLastError();
-  k_adj_forward<<<adj_blocks(n), TPB_ADJ, 0, st>>>(g, F, n, qm, scale, n_steps, every, n_iter,
-                                                   st0, out, ckpt);
+  const auto kernel = adj_inc_applies(g, n_iter) ? k_adj_forward<true> : k_adj_forward<false>;
+  kernel<<<adj_blocks(n), TPB_ADJ, 0, st>>>(g, F, tb, n, qm, scale, n_steps, every, n_iter, st0,
+                                            out, ckpt);
   COUNT_LAUNCH(1);
   return cudaGetLastError();
 }
 
-cudaError_t launch_adjoint_backward(const GridP &g, const FieldPtrsT<double> &F, int64_t n,
-                                    double qm, double scale, double gfac, int n_steps, int every,
-                                    int n_iter,
+cudaError_t launch_adjoint_backward(const GridP &g, const FieldPtrsT<double> &F,
+                                    const PushTables &tb, int64_t n, double qm, double scale,
+                                    double gfac, int n_steps, int every, int n_iter,
                                     const double *ckpt, const double *gout, double *gin,
                                     double *gscale_pp, double *gscale_sum, double *scratch,
                                     cudaStream_t st) {
   if (n <= 0) return cudaMemsetAsync(gscale_sum, 0, sizeof(double), st);
-  k_adj_backward<<<adj_blocks(n), TPB_ADJ, 0, st>>>(g, F, n, qm, scale, gfac, n_steps, every,
-                                                    n_iter, ckpt, gout, gin, gscale_pp, scratch);
+  const auto kernel = adj_inc_applies(g, n_iter) ? k_adj_backward<true> : k_adj_backward<false>;
+  kernel<<<adj_blocks(n), TPB_ADJ, 0, st>>>(g, F, tb, n, qm, scale, gfac, n_steps, every, n_iter,
+                                            ckpt, gout, gin, gscale_pp, scratch);
   k_sum<<<1, 1024, 0, st>>>(gscale_pp, n, gscale_sum);
   COUNT_LAUNCH(2);
   return cudaGetLastError();

@@ -1172,7 +1172,7 @@ grpic_status grpic_adjoint_forward(grpic_ctx *ctx, int64_t n, double qm, double 
   if (s) return s;
   if (n > 0 && (!state0 || !state_out || (n_steps > 0 && !ckpt)))
     return fail(ctx, GRPIC_EINVAL, "null adjoint buffer");
-  CK(launch_adjoint_forward(ctx->g, ctx->F64, n, qm, b0 / ctx->field_b0, n_steps, ckpt_every,
+  CK(launch_adjoint_forward(ctx->g, ctx->F64, ctx->tb, n, qm, b0 / ctx->field_b0, n_steps, ckpt_every,
                             n_iter, state0, state_out, ckpt, ctx->stream));
   return GRPIC_OK;
 }
@@ -1187,7 +1187,7 @@ grpic_status grpic_adjoint_backward(grpic_ctx *ctx, int64_t n, double qm, double
                              (n_steps > 0 && (!ckpt || !scratch)))))
     return fail(ctx, GRPIC_EINVAL, "null adjoint buffer");
   // the kernels differentiate with respect to the field scale b0 / field_b0
-  CK(launch_adjoint_backward(ctx->g, ctx->F64, n, qm, b0 / ctx->field_b0, 1.0 / ctx->field_b0,
+  CK(launch_adjoint_backward(ctx->g, ctx->F64, ctx->tb, n, qm, b0 / ctx->field_b0, 1.0 / ctx->field_b0,
                              n_steps, ckpt_every, n_iter, ckpt, grad_out, grad_state0,
                              grad_b0_pp, grad_b0, scratch, ctx->stream));
   return GRPIC_OK;

@@ -456,11 +456,13 @@ template <typename T>
 cudaError_t launch_continuity(const GridP &g, const T *J1, const T *J2, const double *rho_prev,
                               const double *rho_new, const double *rho_abs, double *out,
                               cudaStream_t st);
-cudaError_t launch_adjoint_forward(const GridP &g, const FieldPtrsT<double> &F, int64_t n,
+cudaError_t launch_adjoint_forward(const GridP &g, const FieldPtrsT<double> &F,
+                                   const PushTables &tb, int64_t n,
                                    double qm, double scale, int n_steps, int every, int n_iter,
                                    const double *st0, double *out, double *ckpt,
                                    cudaStream_t st);
-cudaError_t launch_adjoint_backward(const GridP &g, const FieldPtrsT<double> &F, int64_t n,
+cudaError_t launch_adjoint_backward(const GridP &g, const FieldPtrsT<double> &F,
+                                    const PushTables &tb, int64_t n,
                                     double qm, double scale, double gfac, int n_steps, int every,
                                     int n_iter,
                                     const double *ckpt, const double *gout, double *gin,

@@ -1,442 +1,9 @@
-// push_inc.cuh -- the FP64 pusher's increment form (plain log-r grid), included by
-// particles.cu after the FP64 routine it stands in for.
-//
-// GB300 executes 2 FP64 operations per clock and SM against 128 FP32 ones, and the FP64
-// routine (push64) needs ~560 of them per particle. But everything a step computes for the
-// momentum ends in an increment that is a small part of u: u^{n+1} = u^n + du. An increment
-// of relative size eps, computed in pairs of floats (dfloat.cuh, relative error ~2^-47),
-// leaves an error of eps 2^-47 in u, which for eps <= 2^-5 is at or below FP64's own
-// rounding. So the metric and its derivatives at x^n, the tetrads, the field interpolation,
-// both Boris half steps and the geodesic substep are evaluated in float pairs, as
-// increments, and u^n + du is formed in FP64 by one addition per component. The coordinate
-// substep is not small against the offset it changes: its result is, as in push64, one FP64
-// evaluation of the map at the predictor's point.
-//
-// A particle that the bounds behind this do not cover (the axis rows, an increment above
-// 2^-5, an iteration that the predictor does not resolve, values outside the range of FP32)
-// is left to push64, untouched.
-//
-// Measured: a step of the 2048^2 workload (134 M particles) 173.6 -> 80.3 ms, of the 512^2 one
-// (16.8 M) 21.0 -> 11.0 ms. One push against 113-bit arithmetic, six grids from 64^2 to 2048^2
-// (60,000 particles each): rms errors of u 0.8-3.1e-16 of its rms (push64: 2.5-3.3e-16), of the
-// offsets 2.4-4.9e-17 (2.5-5.5e-17).
+// push_inc.cuh -- one particle of the FP64 path in the increment form (inc.cuh), included by
+// particles.cu.
 #pragma once
+#include "inc.cuh"
 
 namespace {
-
-constexpr float INC_MAX = 0x1p-5f;   // largest |increment| / max(1, |u|) of a Boris half step
-constexpr float INC_E = 0.055f;      // largest |offset of xi| of the radial series
-constexpr float INC_D = 0.035f;      // largest |offset of theta| of the angular series
-constexpr float INC_R = 1024.0f;     // largest r: r^-8 and its low parts stay in FP32's range
-
-__device__ __forceinline__ DF df2(const float2 v) { return DF(v.x, v.y); }
-
-// The grid's constants in pairs that the increment form reads
-struct IncC {
-  DF a, M, dxi, dth, ig2, dt, a2;
-};
-__device__ __forceinline__ IncC inc_c(const GridP &g) {
-  return {DF(g.d_a[0], g.d_a[1]),     DF(g.d_M[0], g.d_M[1]),   DF(g.d_dxi[0], g.d_dxi[1]),
-          DF(g.d_dth[0], g.d_dth[1]), DF(g.d_ig2[0], g.d_ig2[1]), DF(g.d_dt[0], g.d_dt[1]),
-          DF(g.d_a2[0], g.d_a2[1])};
-}
-
-// r, sin(theta), cos(theta) in pairs at x1 = i + o1, x2 = j + o2 from the tables of the
-// nearest cell corner. The series' leading terms are pairs, their tails (below 2^-24 of the
-// result's last bit but one) plain floats. Returns whether the offsets are in range.
-__device__ __forceinline__ bool inc_point(const IncC &k, const PushTables &tb, int i, int j, DF o1,
-                                          DF o2, DF &r, DF &s, DF &c) {
-  const int c1 = o1.hi >= 0.5f, c2 = o2.hi >= 0.5f;
-  const DF q1 = fast_two_sum(__fsub_rn(o1.hi, (float)c1), o1.lo);
-  const DF q2 = fast_two_sum(__fsub_rn(o2.hi, (float)c2), o2.lo);
-  const DF e = q1 * k.dxi, d = q2 * k.dth;
-  const float ef = e.hi;
-  // exp(e) = 1 + e + e^2/2 + e^3/6 + e^4 (1/24 + ...)
-  float t = fmaf(1.0f / 40320.0f, ef, 1.0f / 5040.0f);
-  t = fmaf(t, ef, 1.0f / 720.0f);
-  t = fmaf(t, ef, 1.0f / 120.0f);
-  DF x = dfc(1.0 / 24.0) + DF(t * ef);
-  x = fma_(x, e, dfc(1.0 / 6.0));
-  x = fma_(x, e, DF(0.5f));
-  x = fma_(x, e, DF(1.0f));
-  x = fma_(x, e, DF(1.0f));
-  r = df2(__ldg(tb.r_df + i + c1 + G_)) * x;
-  const DF q = d * d;
-  const float qf = q.hi;
-  t = fmaf(1.0f / 362880.0f, qf, -1.0f / 5040.0f);
-  t = fmaf(t, qf, 1.0f / 120.0f);
-  const DF se = fma_((dfc(-1.0 / 6.0) + DF(t * qf)) * q, d, d);  // sin(d)
-  t = fmaf(1.0f / 40320.0f, qf, -1.0f / 720.0f);
-  t = fmaf(t, qf, 1.0f / 24.0f);
-  const DF ce = fma_(DF(-0.5f) + DF(t * qf), q, DF(1.0f));  // cos(d)
-  const DF s0 = df2(__ldg(tb.s_df + j + c2 + G_)), c0 = df2(__ldg(tb.c_df + j + c2 + G_));
-  s = fma_(s0, ce, c0 * se);
-  c = fma_(c0, ce, -(s0 * se));
-  return fabsf(ef) <= INC_E && fabsf(d.hi) <= INC_D && o1.hi >= 0.0f && o1.hi <= 1.0f &&
-         o2.hi >= 0.0f && o2.hi <= 1.0f && r.hi <= INC_R;
-}
-
-// Metric, its derivatives and the tetrad coefficients at x^n in pairs: the quantities of
-// local_full, written so that each takes few operations (one reciprocal, three reciprocal
-// square roots: of Sigma, Sigma + 2 M r and A).
-__device__ __forceinline__ void inc_local(const IncC &k, DF r, DF s, DF c, Local<DF> &L) {
-  const DF s2 = s * s, r2 = r * r, f = k.dxi * r, sc = s * c;
-  const DF Sig = fma_(k.a2, c * c, r2);
-  const DF Mr = k.M * r, M2r = df_scale(Mr, 2.0f);
-  const DF S2 = Sig + M2r;
-  const DF R = r2 + k.a2, Del = R - M2r, as2 = k.a2 * s2;
-  const DF A = fma_(R, R, -(as2 * Del));
-  const DF P = Sig * S2, Pf = P * f;
-  const DF iQ = df_rcp(Pf * s2);
-  const DF iu = iQ * s2, is2 = iQ * Pf;
-  const DF iP = iu * f, fi = iu * P;
-  const DF iSig = iP * S2, iS2 = iP * Sig;
-  const DF rSig = df_rsqrt(Sig), rS2 = df_rsqrt(S2), rA = df_rsqrt(A);
-  const DF qSig = Sig * rSig, qS2 = S2 * rS2;
-  Geo<DF> &o = L.G;
-  const DF fi2 = fi * fi, AP = A * iP;
-  o.opz = S2 * iSig;
-  o.H11 = AP * fi2;
-  o.H13 = k.a * iSig * fi;
-  o.H22 = iSig * k.ig2;
-  o.H33 = iSig * is2;
-  o.beta1 = M2r * iS2 * fi;
-  L.alpha = qSig * rS2;
-  const DF dxS = df_scale(r * f, 2.0f), a2sc = k.a2 * sc * k.dth, deS = df_scale(a2sc, -2.0f);
-  const DF qS = dxS * iSig, qe = deS * iSig, Mf = k.M * f;
-  const DF ipf = iP * fi2;
-  // d(A)/dx1 = 2 f (2 r R - a^2 s^2 (r - M)), d(P)/dx1 = dxS S2 + Sigma (dxS + 2 M f)
-  const DF dxA = df_scale(f * fma_(df_scale(r, 2.0f), R, -(as2 * (r - k.M))), 2.0f);
-  const DF dxP = fma_(dxS, S2, Sig * (dxS + df_scale(Mf, 2.0f)));
-  L.d1H11 = fma_(ipf, dxA - AP * dxP, -(df_scale(k.dxi, 2.0f) * o.H11));
-  L.d2H11 = ipf * deS * (Del - AP * (S2 + Sig));
-  L.d1H22 = -(qS * o.H22);
-  L.d2H22 = -(qe * o.H22);
-  L.d1H33 = -(qS * o.H33);
-  L.d2H33 = -((qe + df_scale(sc * is2 * k.dth, 2.0f)) * o.H33);
-  L.d1H13 = -((qS + k.dxi) * o.H13);
-  L.d2H13 = -(qe * o.H13);
-  const DF fsr = fma_(f, Sig, -(r * dxS)), rde = Mr * deS;
-  const DF ia = iP * L.alpha;
-  L.d1alpha = -(k.M * fsr * ia);
-  L.d2alpha = rde * ia;
-  const DF w = df_scale(fi * iS2 * iS2, 2.0f);
-  L.d1beta1 = fma_(w * k.M, fsr, -(k.dxi * o.beta1));
-  L.d2beta1 = -(w * rde);
-  L.rH11 = f * qSig * qS2 * rA;
-  L.sH11 = fi * (rSig * rS2) * (A * rA);
-  L.rh22 = rSig * (k.ig2 * k.dth);
-  L.sh22 = qSig * k.dth;
-  const DF sA = s * rSig;
-  L.rh33 = qSig * rA * (s * is2);
-  L.sh33 = sA * (A * rA);
-  const DF faS = f * k.a * S2;
-  L.k13 = -(faS * sA * rA);
-  L.m13 = -(faS * (rA * rA));
-}
-
-// The geodesic substep as a map of the increment d = t - u: the same equation as GeoMap,
-// d -> G(u + d) - u. R: DF or float (the predictor, from the pairs' high parts).
-template <typename R>
-struct GeoInc {
-  R u0, u1, c0, c1, e1, e2, f1, f2, D1a, D1b, D2a, D2b, hdt;
-  R H11, H22, d1H11, d1H22, d2H11, d2H22;
-};
-__device__ __forceinline__ float half_(float a) { return 0.5f * a; }
-__device__ __forceinline__ DF half_(DF a) { return df_scale(a, 0.5f); }
-template <typename R>
-__device__ __forceinline__ void geo_inc_apply(const GeoInc<R> &m, R d0, R d1, R &n0, R &n1) {
-  const R b0 = m.u0 + half_(d0), b1 = m.u1 + half_(d1);
-  const R b1s = b1 * b1;
-  const R q = fma_(b0, fma_(m.H11, b0, m.c1), fma_(m.H22, b1s, m.c0));  // gamma_bar^2
-  const R ig = rsqrt_(q);
-  const R gb = q * ig, ha = m.hdt * ig;
-  const R k1 = fma_(b0, fma_(m.d1H11, b0, m.e2), fma_(m.d1H22, b1s, m.e1));
-  const R k2 = fma_(b0, fma_(m.d2H11, b0, m.f2), fma_(m.d2H22, b1s, m.f1));
-  n0 = fma_(b0, m.D1b, -fma_(gb, m.D1a, ha * k1));
-  n1 = fma_(b0, m.D2b, -fma_(gb, m.D2a, ha * k2));
-}
-// the map's Jacobian (GeoMap::jacobian in b = u + d/2)
-__device__ __forceinline__ void geo_inc_jacobian(const GeoInc<float> &m, float d0, float d1,
-                                                 float J[2][2]) {
-  const float b0 = fmaf(0.5f, d0, m.u0), b1 = fmaf(0.5f, d1, m.u1), b1s = b1 * b1;
-  const float q = fmaf(b0, fmaf(m.H11, b0, m.c1), fmaf(m.H22, b1s, m.c0));
-  const float ig = rsqrtf(q), ha = m.hdt * ig;
-  const float k1 = fmaf(b0, fmaf(m.d1H11, b0, m.e2), fmaf(m.d1H22, b1s, m.e1));
-  const float k2 = fmaf(b0, fmaf(m.d2H11, b0, m.f2), fmaf(m.d2H22, b1s, m.f1));
-  const float q0 = fmaf(2.0f * m.H11, b0, m.c1), q1 = 2.0f * m.H22 * b1;
-  const float hg = 0.5f * ig, hh = -0.5f * ha * ig * ig;
-  const float g0 = hg * q0, g1 = hg * q1, a0 = hh * q0, a1 = hh * q1;
-  J[0][0] = 0.5f * (m.D1b - g0 * m.D1a - a0 * k1 - ha * fmaf(2.0f * m.d1H11, b0, m.e2));
-  J[0][1] = 0.5f * (-g1 * m.D1a - a1 * k1 - ha * (2.0f * m.d1H22 * b1));
-  J[1][0] = 0.5f * (m.D2b - g0 * m.D2a - a0 * k2 - ha * fmaf(2.0f * m.d2H11, b0, m.f2));
-  J[1][1] = 0.5f * (-g1 * m.D2a - a1 * k2 - ha * (2.0f * m.d2H22 * b1));
-}
-// whether the method's n_iter iterations come within a tenth of tol of the fixed point
-// (method_converges on FP32 values)
-__device__ __forceinline__ bool inc_converges(float d1, const float J[2][2], int n_iter, float tol,
-                                              float scale) {
-  const float rho = spectral_radius(J);
-  if (!(rho < 0.25f)) return false;
-  return !(rho > 0.0f) ||
-         d1 * exp2f((float)n_iter * log2f(rho)) <= 0.1f * tol * fmaxf(1.0f, scale);
-}
-
-// du += the geodesic substep's increment from u; false: not resolved here. The FP32 map gives
-// the increment to FP32 rounding, one evaluation in pairs there and one Newton step with the
-// FP32 Jacobian J, d + (I - J)^{-1} r = G + M J r with r = G - d and M = (I - J)^{-1}, leave
-// an error of |J| 2^-24 |r|, far below the pairs' rounding of d.
-__device__ __forceinline__ bool inc_geodesic(const GridP &g, const IncC &k, const Local<DF> &L,
-                                             const DF u[3], float m2, DF &du0, DF &du1) {
-  GeoInc<DF> m;
-  const DF uu = u[2] * u[2], u2x2 = df_scale(u[2], 2.0f);
-  const Geo<DF> &o = L.G;
-  m.u0 = u[0];
-  m.u1 = u[1];
-  m.c0 = fma_(o.H33, uu, DF(m2));
-  m.c1 = o.H13 * u2x2;
-  m.e1 = L.d1H33 * uu;
-  m.e2 = L.d1H13 * u2x2;
-  m.f1 = L.d2H33 * uu;
-  m.f2 = L.d2H13 * u2x2;
-  m.D1a = k.dt * L.d1alpha;
-  m.D1b = k.dt * L.d1beta1;
-  m.D2a = k.dt * L.d2alpha;
-  m.D2b = k.dt * L.d2beta1;
-  m.hdt = df_scale(k.dt * L.alpha, 0.5f);
-  m.H11 = o.H11;
-  m.H22 = o.H22;
-  m.d1H11 = L.d1H11;
-  m.d1H22 = L.d1H22;
-  m.d2H11 = L.d2H11;
-  m.d2H22 = L.d2H22;
-  const GeoInc<float> mf = {m.u0.hi,  m.u1.hi,  m.c0.hi,  m.c1.hi,  m.e1.hi,    m.e2.hi,   m.f1.hi,
-                            m.f2.hi,  m.D1a.hi, m.D1b.hi, m.D2a.hi, m.D2b.hi,   m.hdt.hi,  m.H11.hi,
-                            m.H22.hi, m.d1H11.hi, m.d1H22.hi, m.d2H11.hi, m.d2H22.hi};
-  float p0 = 0.0f, p1 = 0.0f, first = 0.0f;
-  for (int it = 0; it < g.n_iter; ++it) {
-    float n0, n1;
-    geo_inc_apply(mf, p0, p1, n0, n1);
-    const float d = fmaxf(fabsf(n0 - p0), fabsf(n1 - p1));
-    if (it == 0) first = d;
-    p0 = n0;
-    p1 = n1;
-    if (d <= 0x1p-20f * fmaxf(fabsf(n0), fabsf(n1))) break;
-  }
-  DF n0, n1;
-  geo_inc_apply(m, DF(p0), DF(p1), n0, n1);
-  float J[2][2];
-  geo_inc_jacobian(mf, p0, p1, J);
-  const float r0 = (n0 - DF(p0)).hi, r1 = (n1 - DF(p1)).hi;
-  const float w0 = fmaf(J[0][0], r0, J[0][1] * r1), w1 = fmaf(J[1][0], r0, J[1][1] * r1);
-  const float a = 1.0f - J[0][0], d = 1.0f - J[1][1];
-  const float idet = __fdividef(1.0f, fmaf(a, d, -J[0][1] * J[1][0]));
-  n0 = n0 + DF(idet * fmaf(d, w0, J[0][1] * w1));
-  n1 = n1 + DF(idet * fmaf(J[1][0], w0, a * w1));
-  const float us = fmaxf(fabsf(m.u0.hi), fabsf(m.u1.hi));
-  const float ds = fmaxf(fabsf(n0.hi), fabsf(n1.hi));
-  // (a NaN anywhere makes one of the comparisons false)
-  if (!(fabsf(r0) + fabsf(r1) <= fmaf(0x1p-16f, ds, 0x1p-40f) && ds <= INC_MAX * fmaxf(1.0f, us)))
-    return false;
-  if (!inc_converges(first, J, g.n_iter, g.f_iter_tol, us)) return false;
-  du0 = du0 + n0;
-  du1 = du1 + n1;
-  return true;
-}
-
-// One Boris half step's increment of the covariant u, added to du (u = u^n + du in pairs):
-// u' - u = 2 e D + s (p x t) in the tetrad frame (boris), with eD = e D, eB = e B given.
-// False: above INC_MAX.
-__device__ __forceinline__ bool inc_boris(const Local<DF> &L, const DF eD[3], const DF eB[3],
-                                          const DF u[3], DF du[3]) {
-  const DF h0 = L.sH11 * fma_(-L.m13, u[2], u[0]), h1 = u[1] * L.rh22, h2 = u[2] * L.rh33;
-  const DF m0 = h0 + eD[0], m1 = h1 + eD[1], m2 = h2 + eD[2];
-  const DF ig = df_rsqrt(fma_(m0, m0, fma_(m1, m1, fma_(m2, m2, DF(1.0f)))));
-  const DF t0 = eB[0] * ig, t1 = eB[1] * ig, t2 = eB[2] * ig;
-  const DF sf = df_scale(df_rcp(fma_(t0, t0, fma_(t1, t1, fma_(t2, t2, DF(1.0f))))), 2.0f);
-  const DF p0 = fma_(m1, t2, fma_(-m2, t1, m0));
-  const DF p1 = fma_(m2, t0, fma_(-m0, t2, m1));
-  const DF p2 = fma_(m0, t1, fma_(-m1, t0, m2));
-  const DF x0 = fma_(sf, fma_(p1, t2, -(p2 * t1)), df_scale(eD[0], 2.0f));
-  const DF x1 = fma_(sf, fma_(p2, t0, -(p0 * t2)), df_scale(eD[1], 2.0f));
-  const DF x2 = fma_(sf, fma_(p0, t1, -(p1 * t0)), df_scale(eD[2], 2.0f));
-  const float xx = fmaf(x0.hi, x0.hi, fmaf(x1.hi, x1.hi, x2.hi * x2.hi));
-  const float hh = fmaf(h0.hi, h0.hi, fmaf(h1.hi, h1.hi, h2.hi * h2.hi));
-  if (!(xx <= INC_MAX * INC_MAX * fmaxf(1.0f, hh) && hh < 0x1p60f)) return false;
-  du[0] = du[0] + fma_(x0, L.rH11, L.k13 * x2);
-  du[1] = fma_(L.sh22, x1, du[1]);
-  du[2] = fma_(L.sh33, x2, du[2]);
-  return true;
-}
-
-// bilinear interpolation in pairs at the cell-relative offsets (o1, o2) of cell (i1, i2) for
-// a component offset by h1/2, h2/2 (w: the weights of both kinds per direction, c: their cells)
-struct IncLerp {
-  int i[2], j[2];
-  DF w1[2], w2[2];
-};
-__device__ __forceinline__ void inc_lerp(int i1, int i2, DF o1, DF o2, IncLerp &l) {
-  l.i[0] = i1;
-  l.j[0] = i2;
-  l.w1[0] = o1;
-  l.w2[0] = o2;
-  const bool b1 = o1.hi < 0.5f, b2 = o2.hi < 0.5f;
-  l.i[1] = i1 - (b1 ? 1 : 0);
-  l.j[1] = i2 - (b2 ? 1 : 0);
-  l.w1[1] = o1 + DF(b1 ? 0.5f : -0.5f);
-  l.w2[1] = o2 + DF(b2 ? 0.5f : -0.5f);
-}
-__device__ __forceinline__ DF inc_interp(const double *__restrict__ pl, int NX, const IncLerp &l,
-                                         int h1, int h2) {
-  const double *p = pl + (int64_t)(l.j[h2] + G_) * NX + (l.i[h1] + G_);
-  const DF p00 = df_of(__ldg(p)), p10 = df_of(__ldg(p + 1));
-  const DF p01 = df_of(__ldg(p + NX)), p11 = df_of(__ldg(p + NX + 1));
-  const DF a = fma_(l.w1[h1], p10 - p00, p00), b = fma_(l.w1[h1], p11 - p01, p01);
-  return fma_(l.w2[h2], b - a, a);
-}
-
-// The coordinate map of Eq. (discretized-geodesic-x) at a point, from r, sin, cos there:
-// with w0 = u_1 / f (f = dr/dx1), k = h-tilde^22 u_2 = u_2 / dtheta^2 and
-//   I = A w0 / S2 + a u_3,  X = w0 (I + a u_3) + k u_2 + u_3^2 / sin^2,
-//   G = (S2 (m2 Sigma + X))^(-1/2)  [= alpha / (gamma Sigma)],   S2 = Sigma + 2 M r,
-// V^1 = (G I - 2 M r / S2) / f, V^2 = G k, dphi/dt = G (a w0 + u_3 / sin^2): the metric's
-// products regrouped so that no 1/Sigma is needed (one reciprocal, of S2 f sin^2).
-template <typename R>
-struct Vel {
-  R v1, v2, v3;
-};
-__device__ __forceinline__ Vel<DF> inc_velocity(const IncC &k, DF r, DF s, DF c, const DF u[3],
-                                                float m2) {
-  const DF s2 = s * s, r2 = r * r, f = k.dxi * r;
-  const DF Sig = fma_(k.a2, c * c, r2), M2r = df_scale(k.M * r, 2.0f), S2 = Sig + M2r;
-  const DF Rr = r2 + k.a2, A = fma_(Rr, Rr, -(k.a2 * s2 * (Rr - M2r)));
-  const DF fs = f * s2, iQ = df_rcp(S2 * fs), iS2 = iQ * fs;
-  const DF fi = iQ * S2 * s2, w0 = u[0] * fi, au = k.a * u[2];
-  const DF I = fma_(A * iS2, w0, au), kk = k.ig2 * u[1];
-  const DF z = u[2] * (iQ * S2 * f);
-  const DF X = fma_(w0, I + au, fma_(kk, u[1], u[2] * z));
-  const DF Gf = df_rsqrt(S2 * (m2 != 0.0f ? Sig + X : X));
-  return {fi * fma_(Gf, I, -(M2r * iS2)), Gf * kk, Gf * fma_(k.a, w0, z)};
-}
-
-// The FP64 evaluation of the map t -> dx + dt V((x^n + t)/2) that the result comes from: r
-// from the nearest corner's table, theta formed as map_theta forms it and its offset from the
-// corner's theta exact (as local_rsc), then inc_velocity's grouping: ~80 FP64 operations.
-__device__ __forceinline__ void inc_coord64(const GridP &g, const PushTables &tb, int i1, int i2,
-                                            double dx1, double dx2, const double u[3], double m2,
-                                            double t1, double t2, double &n1, double &n2,
-                                            double &v3) {
-  const double o1 = 0.5 * __dadd_rn(dx1, t1), o2 = 0.5 * __dadd_rn(dx2, t2);
-  const int c1 = gt_pos(o1, 0.5), c2 = gt_pos(o2, 0.5);
-  const double e = (o1 - (c1 ? 1.0 : 0.0)) * g.dxi;
-  double ex;
-  if (abs_le(e, (double)INC_E)) {
-    double p = 1.0 / 40320.0;
-    p = fma(p, e, 1.0 / 5040.0);
-    p = fma(p, e, 1.0 / 720.0);
-    p = fma(p, e, 1.0 / 120.0);
-    p = fma(p, e, 1.0 / 24.0);
-    p = fma(p, e, 1.0 / 6.0);
-    p = fma(p, e, 0.5);
-    p = fma(p, e, 1.0);
-    ex = __ldg(tb.r64 + i1 + c1 + G_) * fma(p, e, 1.0);
-  } else {
-    ex = map_e(g, (double)i1 + o1);
-  }
-  const double th = __dmul_rn(__dadd_rn((double)i2, o2), g.dth);
-  const double d = th - __ldg(tb.th64 + i2 + c2 + G_);
-  double s, c;
-  if (abs_le(d, (double)INC_D)) {
-    const double q = d * d;
-    double sp = fma(-1.0 / 5040.0, q, 1.0 / 120.0);
-    sp = fma(sp, q, -1.0 / 6.0);
-    const double se = fma(sp * q, d, d);
-    double cp = fma(1.0 / 40320.0, q, -1.0 / 720.0);
-    cp = fma(cp, q, 1.0 / 24.0);
-    cp = fma(cp, q, -0.5);
-    const double ce = fma(cp, q, 1.0);
-    const double s0 = __ldg(tb.s64 + i2 + c2 + G_), c0 = __ldg(tb.c64 + i2 + c2 + G_);
-    s = fma(s0, ce, c0 * se);
-    c = fma(c0, ce, -s0 * se);
-  } else {
-    sincos(th, &s, &c);
-  }
-  const double s2 = s * s, r2 = ex * ex, f = g.dxi * ex;
-  const double Sig = fma(g.a2, c * c, r2), M2r = g.M2 * ex, S2 = Sig + M2r;
-  const double Rr = r2 + g.a2, A = fma(Rr, Rr, -(g.a2 * s2 * (Rr - M2r)));
-  const double fs = f * s2, iQ = rcp_nr(S2 * fs), iS2 = iQ * fs, T = iQ * S2;
-  const double fi = T * s2, w0 = u[0] * fi, au = g.a * u[2];
-  const double I = fma(A * iS2, w0, au), kk = g.ig2 * u[1];
-  const double z = u[2] * (T * f);
-  const double X = fma(w0, I + au, fma(kk, u[1], u[2] * z));
-  const double Gf = rsqrt(S2 * fma(m2, Sig, X));
-  n1 = fma(g.dt * fi, fma(Gf, I, -(M2r * iS2)), dx1);
-  n2 = fma(g.dt * Gf, kk, dx2);
-  v3 = Gf * fma(g.a, w0, z);
-}
-
-// The coordinate substep: as coord_refined (FP32 predictor, one step in pairs, FP64
-// evaluations until the stop rule holds), the FP32 and pair maps in inc_velocity's grouping.
-__device__ __forceinline__ bool inc_coord(const GridP &g, const IncC &k, const PushTables &tb,
-                                          int i1, int i2, double dx1, double dx2, DF o1, DF o2,
-                                          const double u[3], const DF ud[3], double m2, float m2f,
-                                          double &t1, double &t2, double &v3) {
-  const float uf[3] = {ud[0].hi, ud[1].hi, ud[2].hi};
-  const float a1 = o1.hi, a2 = o2.hi, dt = g.f_dt;
-  const float au = g.f_a * uf[2], kk = g.f_ig2 * uf[1], ku = kk * uf[1];
-  float p1 = a1, p2 = a2, first = 0.0f, d_prev = 0.0f;
-  for (int it = 0; it < g.n_iter; ++it) {
-    Pt<float> pf;
-    rsc32<false>(g, tb, i1, i2, 0.5f * (a1 + p1), 0.5f * (a2 + p2), pf);
-    const float s2 = pf.s * pf.s, r2 = pf.r * pf.r, M2r = g.f_M2 * pf.r;
-    const float Sig = fmaf(g.f_a2, pf.c * pf.c, r2), S2 = Sig + M2r, Rr = r2 + g.f_a2;
-    const float A = fmaf(Rr, Rr, -(g.f_a2 * s2 * (Rr - M2r)));
-    const float fs = pf.f * s2, iQ = __fdividef(1.0f, S2 * fs), iS2 = iQ * fs, T = iQ * S2;
-    const float fi = T * s2, w0 = uf[0] * fi, I = fmaf(A * iS2, w0, au), z = uf[2] * (T * pf.f);
-    const float X = fmaf(w0, I + au, fmaf(uf[2], z, ku));
-    const float Gf = rsqrtf(S2 * fmaf(m2f, Sig, X));
-    const float n1 = fmaf(dt * fi, fmaf(Gf, I, -(M2r * iS2)), a1), n2 = fmaf(dt * Gf, kk, a2);
-    const float d = fmaxf(fabsf(n1 - p1), fabsf(n2 - p2));
-    if (it == 0) first = d;
-    const bool fixed = (n1 == p1 && n2 == p2) || settled32_rate(d, d_prev);
-    d_prev = d;
-    p1 = n1;
-    p2 = n2;
-    if (fixed) break;
-  }
-  if (!(p1 > -1.0f && p1 < 2.0f && p2 > -1.0f && p2 < 2.0f)) return false;
-  float J[2][2];
-  {
-    Pt<float> pf;
-    rsc32<false>(g, tb, i1, i2, 0.5f * (a1 + p1), 0.5f * (a2 + p2), pf);
-    Local<float> Lf;
-    local_full<false>(g, pf, Lf);
-    coord_jacobian(g, Lf, uf, m2f, J);
-  }
-  double s1, s2;
-  {
-    const DF h1 = df_scale(o1 + DF(p1), 0.5f), h2 = df_scale(o2 + DF(p2), 0.5f);
-    DF r, s, c;
-    // (the midpoint lies within half a cell of the cell: the nearest corner's offset is at
-    // most half a cell there too)
-    inc_point(k, tb, i1, i2, h1, h2, r, s, c);
-    const Vel<DF> v = inc_velocity(k, r, s, c, ud, m2f);
-    DF s1d, s2d;
-    newton_df(J, DF(p1), DF(p2), fma_(k.dt, v.v1, o1), fma_(k.dt, v.v2, o2), s1d, s2d);
-    s1 = df_to_double(s1d);
-    s2 = df_to_double(s2d);
-  }
-  if (!(finite64(s1) && finite64(s2))) return false;
-  bool conv = false;
-  for (int it = 1; it < g.n_iter && !conv; ++it) {
-    inc_coord64(g, tb, i1, i2, dx1, dx2, u, m2, s1, s2, t1, t2, v3);
-    conv = converged(t1, s1, g.f_iter_tol) && converged(t2, s2, g.f_iter_tol);
-    s1 = t1;
-    s2 = t2;
-  }
-  const float scale = fmaxf(fabsf(f32_trunc(t1)), fabsf(f32_trunc(t2)));
-  return conv && scale < 2.0f && inc_converges(first, J, g.n_iter, g.f_iter_tol, scale);
-}
 
 // An FP32 estimate of whether a Boris half step stays below INC_MAX (fields of one node, no
 // interpolation): where it does not, the warp goes to push64 at once. Only speed depends on it.
@@ -528,7 +95,8 @@ __device__ __forceinline__ bool push_inc(const GridP &g, const FieldPtrsT<double
                         u64[2] + df_to_double(du[2])};
   const DF ud[3] = {u[0] + du[0], u[1] + du[1], u[2] + du[2]};
   double t1, t2, v3;
-  if (!inc_coord(g, k, tb, i1, i2, dx1, dx2, o1, o2, un, ud, s.m2, em ? 1.0f : 0.0f, t1, t2, v3))
+  if (!inc_coord<false>(g, k, tb, g.n_iter, g.f_iter_tol, i1, i2, dx1, dx2, o1, o2, un, ud, s.m2,
+                        em ? 1.0f : 0.0f, t1, t2, v3))
     return false;
   if (!(finite64(un[0]) && finite64(un[1]) && finite64(un[2]))) return false;
   const int c1 = inc_cell(t1), c2 = inc_cell(t2);
