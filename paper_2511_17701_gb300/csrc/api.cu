@@ -429,7 +429,7 @@ grpic_status grpic_create(const grpic_config *cfg, grpic_ctx **out) {
   const size_t ps = (size_t)plane_size(g), fs = ctx->fsz;
   size_t off = 0;
   ctx->off_planes = off; off += up(ps * fs) * 36;
-  ctx->off_tab = off;    off += up(ps * fs) * T_NQ;
+  ctx->off_tab = off;    off += up(ps * fs) * (ctx->mixed ? 4 * M_NQ : T_NQ);
   ctx->off_polar = off;  off += up((size_t)3 * g.NX * fs);
   ctx->off_ptab = off;   off += 16 * up((size_t)(g.NX > g.NY ? g.NX : g.NY) * 8);
   ctx->off_dt = off;     off += up(64);

@@ -25,10 +25,34 @@ constexpr int TPB = 256;
 // curl kernels (put, below) and the launches that read the same fields merged, a vacuum step
 // on 2048^2 points went from 2220 to 1025 us in FP64, one on 500 x 300 points in FP32 (bound by
 // launches) from 90 to 49 us: 7 launches a step where there were 18.
+//
+// FP32 planes keep the metric factors one by one (MetricTab): their kernels are bound by HBM
+// and launches, not by arithmetic, and next to the axes the curls amplify every FP32 rounding,
+// so that a regrouping moves a run's small components (B^3 of the 2048^2 workload after 10
+// steps: by up to 8.4e-4 of its rms) without making them better.
 // ---------------------------------------------------------------------------------
 template <typename T>
 __device__ __forceinline__ T tabv(const T *tab, int64_t ps, int q, int64_t k) {
   return __ldg(tab + q * ps + k);
+}
+
+// FP32: the factor q of Yee class cls
+struct MetricTab {
+  const float *tab;
+  int64_t ps;
+  __device__ __forceinline__ float operator()(int cls, int q, int64_t k) const {
+    return __ldg(tab + (int64_t)(cls * M_NQ + q) * ps + k);
+  }
+};
+// v + dt c / sqrt(h) at the points of a component: T_... in FP64, 1/sqrt(h) of Yee class cls in
+// FP32 (in the order of operations of the factors one by one)
+__device__ __forceinline__ double curl_step(const GridP &, const double *tab, int64_t ps, int q,
+                                            int, int64_t k, double c, double v) {
+  return fma(c, tabv(tab, ps, q, k), v);
+}
+__device__ __forceinline__ float curl_step(const GridP &g, const float *tab, int64_t ps, int,
+                                           int cls, int64_t k, float c, float v) {
+  return fmaf((float)g.dt * c, MetricTab{tab, ps}(cls, M_ISH, k), v);
 }
 
 // The absorbing layer (MATCH, Sec. 3.3.3): a field value v relaxes towards its initial value
@@ -43,71 +67,102 @@ __device__ __forceinline__ double absorb_factor(const GridP &g, double x1) {
   return g.absorb_coef * x * x * x;
 }
 
+// the polar area and the absorbing layer's factors of column i
 template <typename T>
-__global__ void k_metric_tables(GridP g, T *tab, T *polar) {
+__device__ __forceinline__ void polar_row(const GridP &g, int i, T *polar) {
+  const double e = map_e(g, i + 0.5), r = g.r0 + e, a2 = g.a * g.a;
+  polar[i + G_] = (T)(g.dxi * e * (r * r + a2) * sqrt(1.0 + 2.0 * g.M * r / (r * r + a2)) *
+                      (1.0 - cos(map_theta(g, 0.5))));
+  polar[g.NX + i + G_] = (T)absorb_factor(g, i);
+  polar[2 * g.NX + i + G_] = (T)absorb_factor(g, i + 0.5);
+}
+
+// Each lane evaluates the metric at its column's four Yee points and takes the averaged terms of
+// the columns next to it from its neighbours: a warp covers 30 columns of a row.
+__global__ void k_metric_tables(GridP g, double *tab, double *polar) {
+  constexpr unsigned FULL = 0xffffffffu;
   const int64_t ps = plane_size(g);
-  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < ps;
-       q += (int64_t)gridDim.x * blockDim.x) {
+  const int lane = threadIdx.x & 31, tiles = (g.NX + 29) / 30;
+  const int64_t warps = (int64_t)gridDim.x * (blockDim.x / 32);
+  for (int64_t t = blockIdx.x * (int64_t)(blockDim.x / 32) + (threadIdx.x >> 5);
+       t < (int64_t)tiles * g.NY; t += warps) {
+    const int i = (int)(t % tiles) * 30 + lane - 1 - G_, j = (int)(t / tiles) - G_;
+    MetricV nn, hn, nh, hh;
+    metric_eval<false>(g, i, j, false, nn, nullptr);
+    metric_eval<false>(g, i + 0.5, j, false, hn, nullptr);
+    metric_eval<false>(g, i, j + 0.5, false, nh, nullptr);
+    metric_eval<false>(g, i + 0.5, j + 0.5, false, hh, nullptr);
+    // [sqrt(h~) h_13] and [sqrt(h~ h) beta^1] here and at the neighbours half a cell away
+    const auto t13 = [](const MetricV &m) { return m.sqrt_ht * m.h13; };
+    const auto tb1 = [](const MetricV &m) { return m.sqrt_ht * m.sqrt_h * m.beta1; };
+    const double nn13 = t13(nn), nnb = tb1(nn), hn13 = t13(hn), hnb = tb1(hn);
+    const double nh13 = t13(nh), nhb = tb1(nh), hh13 = t13(hh), hhb = tb1(hh);
+    const double hn13l = __shfl_up_sync(FULL, hn13, 1), hnbl = __shfl_up_sync(FULL, hnb, 1);
+    const double hh13l = __shfl_up_sync(FULL, hh13, 1), hhbl = __shfl_up_sync(FULL, hhb, 1);
+    const double nn13r = __shfl_down_sync(FULL, nn13, 1), nnbr = __shfl_down_sync(FULL, nnb, 1);
+    const double nh13r = __shfl_down_sync(FULL, nh13, 1), nhbr = __shfl_down_sync(FULL, nhb, 1);
+    if (lane == 0 || lane == 31 || i > g.n_r + G_) continue;
+    double *o = tab + sidx(g, i, j);
+    double w = 0.5 / nn.sqrt_ht, wa = w * nn.alpha;
+    o[T_E3D3 * ps] = nn.alpha * nn.h33;
+    o[T_E3D1L * ps] = wa * hn13l;
+    o[T_E3D1R * ps] = wa * hn13;
+    o[T_E3B2L * ps] = w * hnbl;
+    o[T_E3B2R * ps] = w * hnb;
+    o[T_D3 * ps] = g.dt / nn.sqrt_h;
+    w = 0.5 / hn.sqrt_ht;
+    wa = w * hn.alpha;
+    o[T_E1D1 * ps] = hn.alpha * hn.h11;
+    o[T_E1D3L * ps] = wa * nn13;
+    o[T_E1D3R * ps] = wa * nn13r;
+    o[T_H2B2 * ps] = hn.alpha * hn.h22;
+    o[T_H2D3L * ps] = w * nnb;
+    o[T_H2D3R * ps] = w * nnbr;
+    o[T_B2D1 * ps] = g.dt / hn.sqrt_h;
+    w = 0.5 / nh.sqrt_ht;
+    wa = w * nh.alpha;
+    o[T_E2D2 * ps] = nh.alpha * nh.h22;
+    o[T_E2B3L * ps] = w * hhbl;
+    o[T_E2B3R * ps] = w * hhb;
+    o[T_H1B1 * ps] = nh.alpha * nh.h11;
+    o[T_H1B3L * ps] = wa * hh13l;
+    o[T_H1B3R * ps] = wa * hh13;
+    o[T_B1D2 * ps] = g.dt / nh.sqrt_h;
+    w = 0.5 / hh.sqrt_ht;
+    wa = w * hh.alpha;
+    o[T_H3B3 * ps] = hh.alpha * hh.h33;
+    o[T_H3B1L * ps] = wa * nh13;
+    o[T_H3B1R * ps] = wa * nh13r;
+    o[T_H3D2L * ps] = w * nhb;
+    o[T_H3D2R * ps] = w * nhbr;
+    o[T_B3 * ps] = g.dt / hh.sqrt_h;
+    if (j == 0) polar_row(g, i, polar);
+  }
+}
+
+// alpha, h_11, h_22, h_33, 1/(2 sqrt(h~)), [sqrt(h~) h_13], [sqrt(h~ h) beta^1] and 1/sqrt(h) per
+// Yee class, and the polar rows
+__global__ void k_metric_tables(GridP g, float *tab, float *polar) {
+  const int64_t ps = plane_size(g);
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < 4 * ps;
+       t += (int64_t)gridDim.x * blockDim.x) {
+    const int cls = (int)(t / ps);
+    const int64_t q = t - cls * ps;
     const int i = (int)(q % g.NX) - G_, j = (int)(q / g.NX) - G_;
-    T *o = tab + q;
-    MetricV c, lo, hi;
-    {  // (i, j) with its x1 neighbours (i -+ 1/2, j)
-      metric_eval<false>(g, i, j, false, c, nullptr);
-      metric_eval<false>(g, i - 0.5, j, false, lo, nullptr);
-      metric_eval<false>(g, i + 0.5, j, false, hi, nullptr);
-      const double w = 0.5 / c.sqrt_ht, wa = w * c.alpha;
-      o[T_E3D3 * ps] = (T)(c.alpha * c.h33);
-      o[T_E3D1L * ps] = (T)(wa * (lo.sqrt_ht * lo.h13));
-      o[T_E3D1R * ps] = (T)(wa * (hi.sqrt_ht * hi.h13));
-      o[T_E3B2L * ps] = (T)(w * (lo.sqrt_ht * lo.sqrt_h * lo.beta1));
-      o[T_E3B2R * ps] = (T)(w * (hi.sqrt_ht * hi.sqrt_h * hi.beta1));
-      o[T_D3 * ps] = (T)(g.dt / c.sqrt_h);
-    }
-    {  // (i + 1/2, j): neighbours (i, j), (i + 1, j)
-      lo = c;
-      c = hi;
-      metric_eval<false>(g, i + 1, j, false, hi, nullptr);
-      const double w = 0.5 / c.sqrt_ht, wa = w * c.alpha;
-      o[T_E1D1 * ps] = (T)(c.alpha * c.h11);
-      o[T_E1D3L * ps] = (T)(wa * (lo.sqrt_ht * lo.h13));
-      o[T_E1D3R * ps] = (T)(wa * (hi.sqrt_ht * hi.h13));
-      o[T_H2B2 * ps] = (T)(c.alpha * c.h22);
-      o[T_H2D3L * ps] = (T)(w * (lo.sqrt_ht * lo.sqrt_h * lo.beta1));
-      o[T_H2D3R * ps] = (T)(w * (hi.sqrt_ht * hi.sqrt_h * hi.beta1));
-      o[T_B2D1 * ps] = (T)(g.dt / c.sqrt_h);
-    }
-    {  // (i, j + 1/2): neighbours (i -+ 1/2, j + 1/2)
-      metric_eval<false>(g, i, j + 0.5, false, c, nullptr);
-      metric_eval<false>(g, i - 0.5, j + 0.5, false, lo, nullptr);
-      metric_eval<false>(g, i + 0.5, j + 0.5, false, hi, nullptr);
-      const double w = 0.5 / c.sqrt_ht, wa = w * c.alpha;
-      o[T_E2D2 * ps] = (T)(c.alpha * c.h22);
-      o[T_E2B3L * ps] = (T)(w * (lo.sqrt_ht * lo.sqrt_h * lo.beta1));
-      o[T_E2B3R * ps] = (T)(w * (hi.sqrt_ht * hi.sqrt_h * hi.beta1));
-      o[T_H1B1 * ps] = (T)(c.alpha * c.h11);
-      o[T_H1B3L * ps] = (T)(wa * (lo.sqrt_ht * lo.h13));
-      o[T_H1B3R * ps] = (T)(wa * (hi.sqrt_ht * hi.h13));
-      o[T_B1D2 * ps] = (T)(g.dt / c.sqrt_h);
-    }
-    {  // (i + 1/2, j + 1/2): neighbours (i, j + 1/2), (i + 1, j + 1/2)
-      lo = c;
-      c = hi;
-      metric_eval<false>(g, i + 1, j + 0.5, false, hi, nullptr);
-      const double w = 0.5 / c.sqrt_ht, wa = w * c.alpha;
-      o[T_H3B3 * ps] = (T)(c.alpha * c.h33);
-      o[T_H3B1L * ps] = (T)(wa * (lo.sqrt_ht * lo.h13));
-      o[T_H3B1R * ps] = (T)(wa * (hi.sqrt_ht * hi.h13));
-      o[T_H3D2L * ps] = (T)(w * (lo.sqrt_ht * lo.sqrt_h * lo.beta1));
-      o[T_H3D2R * ps] = (T)(w * (hi.sqrt_ht * hi.sqrt_h * hi.beta1));
-      o[T_B3 * ps] = (T)(g.dt / c.sqrt_h);
-    }
-    if (j == 0) {
-      const double e = map_e(g, i + 0.5), r = g.r0 + e, a2 = g.a * g.a;
-      polar[i + G_] = (T)(g.dxi * e * (r * r + a2) * sqrt(1.0 + 2.0 * g.M * r / (r * r + a2)) *
-                          (1.0 - cos(map_theta(g, 0.5))));
-      polar[g.NX + i + G_] = (T)absorb_factor(g, i);
-      polar[2 * g.NX + i + G_] = (T)absorb_factor(g, i + 0.5);
-    }
+    const double s1 = (cls == CLS_HN || cls == CLS_HH) ? 0.5 : 0.0;
+    const double s2 = (cls == CLS_NH || cls == CLS_HH) ? 0.5 : 0.0;
+    MetricV m;
+    metric_eval<false>(g, i + s1, j + s2, false, m, nullptr);
+    float *o = tab + (int64_t)cls * M_NQ * ps + q;
+    o[M_ALPHA * ps] = (float)m.alpha;
+    o[M_H11 * ps] = (float)m.h11;
+    o[M_H22 * ps] = (float)m.h22;
+    o[M_H33 * ps] = (float)m.h33;
+    o[M_IHT2 * ps] = (float)(0.5 / m.sqrt_ht);
+    o[M_WT13 * ps] = (float)(m.sqrt_ht * m.h13);
+    o[M_WB1 * ps] = (float)(m.sqrt_ht * m.sqrt_h * m.beta1);
+    o[M_ISH * ps] = (float)(1.0 / m.sqrt_h);
+    if (cls == CLS_HN && j == 0) polar_row(g, i, polar);
   }
 }
 
@@ -309,10 +364,11 @@ __device__ __forceinline__ T pv(const Pair3<T> &P, int c, int64_t k) {
 // E_1 at (i+1/2, j) = alpha [h_11 D^1 + <h_13 D^3>], E_3 at (i, j) = alpha [h_33 D^3 +
 // <h_13 D^1>] + <sqrt(h) beta^1 B^2> (zero on the axes), E_2 at (i, j+1/2) = alpha h_22 D^2 -
 // <sqrt(h) beta^1 B^3>; Eq. (discretized-auxE)
-template <typename T, bool DMEAN>
-__device__ __forceinline__ void aux_E(const GridP &g, const Pair3<T> &B, const Pair3<T> &D,
-                                      const T *tab, int64_t ps, int j, int64_t k, T *E1, T *E2,
-                                      T *E3) {
+template <bool DMEAN>
+__device__ __forceinline__ void aux_E(const GridP &g, const Pair3<double> &B,
+                                      const Pair3<double> &D, const double *tab, int64_t ps, int j,
+                                      int64_t k, double *E1, double *E2, double *E3) {
+  using T = double;
   const T d1 = pv<DMEAN>(D, 0, k), d3 = pv<DMEAN>(D, 2, k);
   E1[k] = fma(tabv(tab, ps, T_E1D1, k), d1,
               fma(tabv(tab, ps, T_E1D3L, k), d3,
@@ -333,10 +389,10 @@ __device__ __forceinline__ void aux_E(const GridP &g, const Pair3<T> &B, const P
 // H_1 at (i, j+1/2) = alpha [h_11 B^1 + <h_13 B^3>], H_3 at (i+1/2, j+1/2) = alpha [h_33 B^3 +
 // <h_13 B^1>] - <sqrt(h) beta^1 D^2>, H_2 at (i+1/2, j) = alpha h_22 B^2 +
 // <sqrt(h) beta^1 D^3>; Eq. (discretized-auxH)
-template <typename T>
-__device__ __forceinline__ void aux_H(const GridP &g, const Pair3<T> &B, const Pair3<T> &D,
-                                      const T *tab, int64_t ps, int j, int64_t k, T *H1, T *H2,
-                                      T *H3) {
+__device__ __forceinline__ void aux_H(const GridP &g, const Pair3<double> &B,
+                                      const Pair3<double> &D, const double *tab, int64_t ps, int j,
+                                      int64_t k, double *H1, double *H2, double *H3) {
+  using T = double;
   if (j < g.n_th) {
     const T b1 = pv<false>(B, 0, k), b3 = pv<false>(B, 2, k);
     H1[k] = fma(tabv(tab, ps, T_H1B1, k), b1,
@@ -353,6 +409,57 @@ __device__ __forceinline__ void aux_H(const GridP &g, const Pair3<T> &B, const P
                   tabv(tab, ps, T_H2D3R, k) * pv<false>(D, 2, k + 1)));
 }
 
+// The same in FP32, from the factors one by one (explicit fused multiply-adds: a fixed order of
+// roundings, see above on the axes).
+__device__ __forceinline__ float two_terms(float t0, float v0, float t1, float v1, float w) {
+  return fmaf(t1, v1, t0 * v0) * w;  // an average of two weighted neighbours
+}
+template <bool DMEAN>
+__device__ __forceinline__ void aux_E(const GridP &g, const Pair3<float> &B, const Pair3<float> &D,
+                                      const float *tab, int64_t ps, int j, int64_t k, float *E1,
+                                      float *E2, float *E3) {
+  const MetricTab m{tab, ps};
+  const float d1 = pv<DMEAN>(D, 0, k), d3 = pv<DMEAN>(D, 2, k);
+  E1[k] = m(CLS_HN, M_ALPHA, k) *
+          fmaf(m(CLS_HN, M_H11, k), d1,
+               two_terms(m(CLS_NN, M_WT13, k), d3, m(CLS_NN, M_WT13, k + 1),
+                         pv<DMEAN>(D, 2, k + 1), m(CLS_HN, M_IHT2, k)));
+  if (j == 0 || j == g.n_th) {
+    E3[k] = 0.0f;
+  } else {
+    const float w2 = m(CLS_NN, M_IHT2, k);
+    const float a13 = two_terms(m(CLS_HN, M_WT13, k), d1, m(CLS_HN, M_WT13, k - 1),
+                                pv<DMEAN>(D, 0, k - 1), w2);
+    const float ab2 = two_terms(m(CLS_HN, M_WB1, k - 1), pv<false>(B, 1, k - 1),
+                                m(CLS_HN, M_WB1, k), pv<false>(B, 1, k), w2);
+    E3[k] = fmaf(m(CLS_NN, M_ALPHA, k), fmaf(m(CLS_NN, M_H33, k), d3, a13), ab2);
+  }
+  if (j < g.n_th)
+    E2[k] = fmaf(m(CLS_NH, M_ALPHA, k) * m(CLS_NH, M_H22, k), pv<DMEAN>(D, 1, k),
+                 -two_terms(m(CLS_HH, M_WB1, k - 1), pv<false>(B, 2, k - 1), m(CLS_HH, M_WB1, k),
+                            pv<false>(B, 2, k), m(CLS_NH, M_IHT2, k)));
+}
+__device__ __forceinline__ void aux_H(const GridP &g, const Pair3<float> &B, const Pair3<float> &D,
+                                      const float *tab, int64_t ps, int j, int64_t k, float *H1,
+                                      float *H2, float *H3) {
+  const MetricTab m{tab, ps};
+  if (j < g.n_th) {
+    const float b1 = pv<false>(B, 0, k), b3 = pv<false>(B, 2, k), w3 = m(CLS_HH, M_IHT2, k);
+    H1[k] = m(CLS_NH, M_ALPHA, k) *
+            fmaf(m(CLS_NH, M_H11, k), b1,
+                 two_terms(m(CLS_HH, M_WT13, k - 1), pv<false>(B, 2, k - 1), m(CLS_HH, M_WT13, k),
+                           b3, m(CLS_NH, M_IHT2, k)));
+    const float b13 = two_terms(m(CLS_NH, M_WT13, k), b1, m(CLS_NH, M_WT13, k + 1),
+                                pv<false>(B, 0, k + 1), w3);
+    const float bd2 = two_terms(m(CLS_NH, M_WB1, k), pv<false>(D, 1, k), m(CLS_NH, M_WB1, k + 1),
+                                pv<false>(D, 1, k + 1), w3);
+    H3[k] = fmaf(m(CLS_HH, M_ALPHA, k), fmaf(m(CLS_HH, M_H33, k), b3, b13), -bd2);
+  }
+  H2[k] = fmaf(m(CLS_HN, M_ALPHA, k) * m(CLS_HN, M_H22, k), pv<false>(B, 1, k),
+               two_terms(m(CLS_NN, M_WB1, k), pv<false>(D, 2, k), m(CLS_NN, M_WB1, k + 1),
+                         pv<false>(D, 2, k + 1), m(CLS_HN, M_IHT2, k)));
+}
+
 // The auxiliary fields on stored i in [-1, n_r + 1], rows [0, n_theta]: E, H or both (both
 // read the same B and D, so one launch reads them once).
 template <typename T, bool DOE, bool DOH, bool DMEAN>
@@ -363,8 +470,8 @@ __global__ void __launch_bounds__(TPBX *TPBY) k_aux(GridP g, Pair3<T> B, Pair3<T
   for (int j = blockIdx.y * TPBY + threadIdx.y; j <= g.n_th; j += gridDim.y * TPBY) {
     if (i > g.n_r + 1) return;
     const int64_t k = sidx(g, i, j);
-    if (DOE) aux_E<T, DMEAN>(g, B, D, tab, ps, j, k, E1, E2, E3);
-    if (DOH) aux_H<T>(g, B, D, tab, ps, j, k, H1, H2, H3);
+    if (DOE) aux_E<DMEAN>(g, B, D, tab, ps, j, k, E1, E2, E3);
+    if (DOH) aux_H(g, B, D, tab, ps, j, k, H1, H2, H3);
   }
 }
 
@@ -421,11 +528,12 @@ __device__ __forceinline__ void faraday(const GridP &g, const Pair3<T> &Bin, con
   const bool rows_half = (j >= 0 && j < g.n_th);
   if (rows_half && i >= 0 && i <= g.n_r) {
     const T e3 = __ldg(E3 + k);
-    b1 = fma(-(__ldg(E3 + k + g.NX) - e3), tabv(tab, ps, T_B1D2, k), b1);
+    b1 = curl_step(g, tab, ps, T_B1D2, CLS_NH, k, -(__ldg(E3 + k + g.NX) - e3), b1);
     if (i < g.n_r) {
-      if (j >= 1) b2 = fma(__ldg(E3 + k + 1) - e3, tabv(tab, ps, T_B2D1, k), b2);
-      b3 = fma(-((__ldg(E2 + k + 1) - __ldg(E2 + k)) - (__ldg(E1 + k + g.NX) - __ldg(E1 + k))),
-               tabv(tab, ps, T_B3, k), b3);
+      if (j >= 1) b2 = curl_step(g, tab, ps, T_B2D1, CLS_HN, k, __ldg(E3 + k + 1) - e3, b2);
+      b3 = curl_step(g, tab, ps, T_B3, CLS_HH, k,
+                     -((__ldg(E2 + k + 1) - __ldg(E2 + k)) - (__ldg(E1 + k + g.NX) - __ldg(E1 + k))),
+                     b3);
     }
   }
   if (MATCH) {
@@ -458,16 +566,17 @@ __device__ __forceinline__ void ampere(const GridP &g, const Pair3<T> &Din, cons
       else if (j == g.n_th)
         d1 += (T)g.dt * (-__ldg(H3 + k - g.NX) - fpi * j1) / __ldg(polar + i + G_);
       else
-        d1 = fma(fma(-fpi, j1, __ldg(H3 + k) - __ldg(H3 + k - g.NX)),
-                 tabv(tab, ps, T_B2D1, k), d1);
+        d1 = curl_step(g, tab, ps, T_B2D1, CLS_HN, k,
+                       fma(-fpi, j1, __ldg(H3 + k) - __ldg(H3 + k - g.NX)), d1);
     }
     if (j < g.n_th) {
-      d2 = fma(-fma(fpi, pv<MEAN>(J, 1, k), __ldg(H3 + k) - __ldg(H3 + k - 1)),
-               tabv(tab, ps, T_B1D2, k), d2);
+      d2 = curl_step(g, tab, ps, T_B1D2, CLS_NH, k,
+                     -fma(fpi, pv<MEAN>(J, 1, k), __ldg(H3 + k) - __ldg(H3 + k - 1)), d2);
       if (j >= 1)
-        d3 = fma(fma(-fpi, pv<MEAN>(J, 2, k),
-                     (__ldg(H2 + k) - __ldg(H2 + k - 1)) - (__ldg(H1 + k) - __ldg(H1 + k - g.NX))),
-                 tabv(tab, ps, T_D3, k), d3);
+        d3 = curl_step(g, tab, ps, T_D3, CLS_NN, k,
+                       fma(-fpi, pv<MEAN>(J, 2, k), (__ldg(H2 + k) - __ldg(H2 + k - 1)) -
+                                                        (__ldg(H1 + k) - __ldg(H1 + k - g.NX))),
+                       d3);
     }
   }
   if (!MEAN) {
@@ -599,7 +708,7 @@ void aux(const GridP &g, const Pair3<T> &B, const Pair3<T> &D, const FieldPtrsT<
 
 template <typename T>
 cudaError_t launch_metric_tables(const GridP &g, T *tab, T *polar, cudaStream_t st) {
-  k_metric_tables<T><<<blocks_for(plane_size(g)), TPB, 0, st>>>(g, tab, polar);
+  k_metric_tables<<<blocks_for(plane_size(g)), TPB, 0, st>>>(g, tab, polar);
   COUNT_LAUNCH(1);
   return cudaGetLastError();
 }

@@ -30,6 +30,7 @@ struct GridP {
   // pusher's double-float predictor: a, M, dxi, dth, 1/dth^2, dt, a^2, 2M
   float d_a[2], d_M[2], d_dxi[2], d_dth[2], d_ig2[2], d_dt[2], d_a2[2], d_M2[2], d_r0[2],
       d_c3[2];
+  float d_ss[2], d_cs[2];  // sin and cos of small_angle as pairs
   double ig2;  // 1 / dth^2
   // quasi-spherical map: radial offset, equatorial concentration, qks = (r0 != 0 || h0 != 0),
   // c3 = 4 h0 / pi^2 (the cubic coefficient of theta(eta_j + d) - theta(eta_j))
@@ -56,6 +57,11 @@ inline void grid_float_copies(GridP &g) {
     dp[k][0] = (float)dv[k];
     dp[k][1] = (float)(dv[k] - (double)dp[k][0]);
   }
+  const double ss = sin(g.small_angle), cs = cos(g.small_angle);
+  g.d_ss[0] = (float)ss;
+  g.d_ss[1] = (float)(ss - (double)g.d_ss[0]);
+  g.d_cs[0] = (float)cs;
+  g.d_cs[1] = (float)(cs - (double)g.d_cs[0]);
   g.f_iter_tol = (float)g.iter_tol;
   g.f_a = (float)g.a; g.f_M = (float)g.M; g.f_dxi = (float)g.dxi; g.f_dth = (float)g.dth;
   g.f_ig2 = (float)g.ig2; g.f_dt = (float)g.dt; g.f_idt = g.dt > 0.0 ? (float)(1.0 / g.dt) : 0.0f;
@@ -114,7 +120,11 @@ __device__ __forceinline__ Cst<float> cst<float>(const GridP &g) {
   return {g.f_a, g.f_M, g.f_dxi, g.f_dth, g.f_ig2, g.f_dt, g.f_a2, g.f_M2};
 }
 
-// The field solver's coefficient tables, one plane each, stored at the component's point:
+// Yee point classes of the FP32 tables: (i, j), (i+1/2, j), (i, j+1/2), (i+1/2, j+1/2), and the
+// quantities tabulated per class (Eq. discretized-auxE/auxH and the curls).
+enum { CLS_NN = 0, CLS_HN = 1, CLS_NH = 2, CLS_HH = 3 };
+enum { M_ALPHA = 0, M_H11, M_H22, M_H33, M_IHT2, M_WT13, M_WB1, M_ISH, M_NQ };
+// The FP64 field solver's coefficient tables, one plane each, stored at the component's point:
 // T_<c><f>: the factor of field component f in auxiliary component c (L, R: of its left and
 // right neighbour in x1 in an average); T_B1D2, T_B2D1, T_B3, T_D3: dt / sqrt(h) at the points of
 // B^1 and D^2 (i, j+1/2), B^2 and D^1 (i+1/2, j), B^3 (i+1/2, j+1/2), D^3 (i, j).
@@ -337,7 +347,7 @@ template <typename T>
 struct FieldPtrsT {
   T *B[3], *D[3], *B0[3], *D0[3], *J[3], *J0[3], *Bn[3], *Bi[3], *Di[3];
   T *E[3], *H[3], *Dh[3];
-  const T *tab;    // [T_NQ][plane]
+  const T *tab;    // FP64: [T_NQ][plane]; FP32: [4 classes][M_NQ][plane]
   const T *polar;  // [3][NX]: the polar area at x1 = i + 1/2, then the absorber factor
                    // absorb_coef x^3 at x1 = i and at x1 = i + 1/2 (stored at i)
 };

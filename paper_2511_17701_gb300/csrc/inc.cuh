@@ -471,4 +471,10 @@ __device__ __forceinline__ bool inc_coord(const GridP &g, const IncC &k, const P
   return conv && scale < 2.0f && inc_converges(first, J, n_iter, tol, scale);
 }
 
+// floor of a pair
+__device__ __forceinline__ int inc_floor(DF a) {
+  const float f = floorf(a.hi);
+  return (int)f - (f == a.hi && a.lo < 0.0f ? 1 : 0);
+}
+
 }  // namespace

@@ -4,7 +4,7 @@
 // FP64 path: the double-precision pipe, not HBM, bounds the kernel on GB300 (every
 // particle-step evaluates the metric up to n_iter + 2 times). Mixed path: FP32 state,
 // fields and arithmetic; for particles within a few cells of the horizon or an axis the
-// metric, lapse and shift are evaluated in FP64 (and rounded), in a second kernel. Particle state is SoA; consecutive threads read consecutive elements,
+// metric, lapse and shift are evaluated in pairs of floats (and rounded), in a second kernel. Particle state is SoA; consecutive threads read consecutive elements,
 // and field gathers hit L1/L2 because the particles are kept sorted by cell.
 #include "grpic_internal.cuh"
 #include "pusher.cuh"
@@ -263,9 +263,9 @@ __device__ __forceinline__ void deposit64(const GridP &g, const FieldPtrsT<T> &F
 // r, sin(theta), cos(theta) and the map's factors as pairs at x1 = i + o1, x2 = j + o2: the
 // corner tables and Taylor series of the offsets (|o1 dxi|, |theta offset| <= 0.12: the
 // series' truncation below 1e-19), on a quasi-spherical grid with the theta offset's cubic in
-// the offset in eta and its derivatives
+// the offset in eta and its derivatives. Returns the theta offset.
 template <bool Q>
-__device__ __forceinline__ void rsc_df(const GridP &g, const PushTables &tb, int i, int j, DF o1,
+__device__ __forceinline__ float rsc_df(const GridP &g, const PushTables &tb, int i, int j, DF o1,
                                        DF o2, Pt<DF> &p) {
   const Cst<DF> k = cst<DF>(g);
   const DF e = o1 * k.dxi;
@@ -313,6 +313,7 @@ __device__ __forceinline__ void rsc_df(const GridP &g, const PushTables &tb, int
   const DF s0(st.x, st.y), c0(ct.x, ct.y);
   p.s = s0 * ce + c0 * se;
   p.c = c0 * ce - s0 * se;
+  return d.hi;
 }
 
 // the coordinate map t -> dx + dt V((x^n + t)/2) of Eq. (discretized-geodesic-x) in pairs
@@ -410,36 +411,6 @@ __device__ __forceinline__ void geodesic_refined(const GridP &g, const PushTable
   u[1] = s1;
 }
 
-// The FP64 routine on FP32 storage (the mixed path's axis rows) stops its iterations once the
-// update is within SETTLE32 max(1, |value|), far below what the stored FP32 result resolves;
-// the FP64 path (settle 0) stops at an exact repeat only.
-constexpr double SETTLE32 = 0x1p-26;
-__device__ __forceinline__ bool settled64(double n0, double t0, double n1, double t1,
-                                          double settle) {
-  return fabs(n0 - t0) <= settle * fmax(1.0, fabs(n0)) &&
-         fabs(n1 - t1) <= settle * fmax(1.0, fabs(n1));
-}
-// the geodesic momentum substep with that stop rule (settle 0: geodesic_momentum itself)
-__device__ __forceinline__ void geodesic_momentum_settle(const GridP &g, const Local<double> &L,
-                                                         double u[3], double m2, double settle) {
-  if (settle == 0.0) {
-    geodesic_momentum(g, L, u, m2);
-    return;
-  }
-  const GeoMap<double> m(g, L, u, m2);
-  double t0 = u[0], t1 = u[1];
-  for (int it = 0; it < g.n_iter; ++it) {
-    double n0, n1;
-    m.apply(t0, t1, n0, n1);
-    const bool fixed = settled64(n0, t0, n1, t1, settle);
-    t0 = n0;
-    t1 = n1;
-    if (fixed && g.stop_on_repeat) break;
-  }
-  u[0] = t0;
-  u[1] = t1;
-}
-
 // The coordinate substep, Eq. (discretized-geodesic-x), as the method iterates it: metric at
 // x_bar = (x^n + x~)/2, the first iterate x^n itself (metric L.G), n_iter iterations or
 // until an exact repeat. t1, t2: the new offsets from cell (i1, i2).
@@ -447,7 +418,7 @@ template <bool Q = true>
 __device__ __forceinline__ void coord_exact(const GridP &g, const Base &b, const Local<double> &L,
                                             int i1, int i2, double dx1, double dx2,
                                             const double u[3], double m2, double &t1,
-                                            double &t2, double settle = 0.0) {
+                                            double &t2) {
   const double uu0 = 2.0 * u[0] * u[2];
   t1 = dx1;
   t2 = dx2;
@@ -467,9 +438,7 @@ __device__ __forceinline__ void coord_exact(const GridP &g, const Base &b, const
     const double ag = rsqrt(o.opz * q);  // alpha / gamma
     const double n1 = fma(g.dt, fma(ag, fma(o.H11, u[0], o.H13 * u[2]), -o.beta1), dx1);
     const double n2 = fma(g.dt, ag * o.H22 * u[1], dx2);
-    // exact repeat: later iterations are no-ops; or (settle > 0) an update below settle
-    const bool fixed = settle > 0.0 ? settled64(n1, t1, n2, t2, settle)
-                                    : (n1 == t1) && (n2 == t2);
+    const bool fixed = (n1 == t1) && (n2 == t2);  // later iterations are no-ops
     t1 = n1;
     t2 = n2;
     if (fixed && g.stop_on_repeat) break;
@@ -572,28 +541,25 @@ __device__ __forceinline__ void coord_refined(const GridP &g, const PushTables &
 }
 
 // One particle in FP64: steps 2-11 of Sec. 3.1, the boundaries of Sec. 3.3.3, and
-// (DEPOSIT) the deposit of its move. T is the storage type of state and fields. REFINE
-// false compiles the refined iterations out (a caller whose particles all sit in the two
-// cell rows next to an axis, where they never apply).
-template <bool Q, typename T, bool DEPOSIT, bool REFINE = true>
-__device__ __forceinline__ void push64(const GridP &g, const FieldPtrsT<T> &F,
-                                       const PushTables &tb, const SpeciesDevT<T> &s,
+// (DEPOSIT) the deposit of its move.
+template <bool Q, bool DEPOSIT>
+__device__ __forceinline__ void push64(const GridP &g, const FieldPtrsT<double> &F,
+                                       const PushTables &tb, const SpeciesDevT<double> &s,
                                        int64_t k, unsigned long long *diag) {
   const int i1 = s.i1[k], i2 = s.i2[k];
-  const double dx1 = (double)s.dx1[k], dx2 = (double)s.dx2[k];
+  const double dx1 = s.dx1[k], dx2 = s.dx2[k];
   const double x1 = i1 + dx1, x2 = i2 + dx2;
   const bool em = s.m2 != 0.0;  // massless particles skip the EM push (Sec. 3.1)
-  const double settle = sizeof(T) == 4 ? SETTLE32 : 0.0;  // FP32 storage: see SETTLE32
   // the refined iterations keep two cell rows away from the axes: there the coordinate map
   // (metric terms ~ 1/sin^2(theta)) has more than one fixed point within reach, and the
   // method's answer is the one its iteration from x^n finds
-  const bool refine = REFINE && g.iter_tol > 0.0 && i2 >= 2 && i2 < g.n_th - 2;
+  const bool refine = g.iter_tol > 0.0 && i2 >= 2 && i2 < g.n_th - 2;
   const Base b = refine ? make_base_tab<Q>(g, tb, i1, i2, dx1, x1, x2) : make_base<Q>(g, x1, x2);
   Pt<double> p0;
   local_at_base<Q>(g, b, x2, p0);  // clamps theta near the axes
   Local<double> L;
   local_full<Q>(g, p0, L);
-  double Bh[3], Dh[3], uh[3], u[3] = {(double)s.u1[k], (double)s.u2[k], (double)s.u3[k]};
+  double Bh[3], Dh[3], uh[3], u[3] = {s.u1[k], s.u2[k], s.u3[k]};
   const double hq = s.qm * L.alpha * 0.5 * g.dt;
   if (em) {
     // step 2: fields at x^n
@@ -614,7 +580,7 @@ __device__ __forceinline__ void push64(const GridP &g, const FieldPtrsT<T> &F,
     hat_cov(L, uh, u);         // step 5
   }
   if (refine) geodesic_refined<Q>(g, tb, i1, i2, f32_trunc(dx1), f32_trunc(dx2), L, u, s.m2);
-  else geodesic_momentum_settle(g, L, u, s.m2, settle);  // step 6
+  else geodesic_momentum(g, L, u, s.m2);  // step 6
   if (em) {
     cov_hat(L, u, uh);         // step 7
     boris(uh, Dh, Bh, hq);     // step 8
@@ -623,7 +589,7 @@ __device__ __forceinline__ void push64(const GridP &g, const FieldPtrsT<T> &F,
   // step 10: implicit coordinate push, Eq. (discretized-geodesic-x)
   double t1 = dx1, t2 = dx2, v3r = NAN;
   if (refine) coord_refined<Q>(g, tb, b, L, i1, i2, dx1, dx2, u, s.m2, t1, t2, v3r);
-  else coord_exact<Q>(g, b, L, i1, i2, dx1, dx2, u, s.m2, t1, t2, settle);
+  else coord_exact<Q>(g, b, L, i1, i2, dx1, dx2, u, s.m2, t1, t2);
   if (!(finite64(u[0]) && finite64(u[1]) && finite64(u[2]) && abs_lt(t1, 1e6) &&
         abs_lt(t2, 1e6))) {
     s.tag[k] = 0;
@@ -641,16 +607,16 @@ __device__ __forceinline__ void push64(const GridP &g, const FieldPtrsT<T> &F,
     count(diag, DG_NONFINITE);
     return;
   }
-  s.i1[k] = j1; s.i2[k] = j2; s.dx1[k] = (T)e1; s.dx2[k] = (T)e2;
-  s.u1[k] = (T)u[0]; s.u2[k] = (T)u[1]; s.u3[k] = (T)u[2];
+  s.i1[k] = j1; s.i2[k] = j2; s.dx1[k] = e1; s.dx2[k] = e2;
+  s.u1[k] = u[0]; s.u2[k] = u[1]; s.u3[k] = u[2];
   if (j1 < 0) { s.tag[k] = 2; count(diag, DG_LEFT_INNER); }
   else if (j1 >= g.n_r) { s.tag[k] = 2; count(diag, DG_LEFT_OUTER); }
   // step 11: phi at x^{n+1/2}, the midpoint of the stored x^n and the final x^{n+1}
   const double xb1 = j1 + e1, xb2 = j2 + e2;
   const double v3 = isnan(v3r)
       ? phi_rate64<Q>(g, b, 0.5 * __dadd_rn(x1, xb1), 0.5 * __dadd_rn(x2, xb2), u, s.m2) : v3r;
-  s.phi[k] = (T)((double)s.phi[k] + g.dt * v3);
-  if (DEPOSIT) deposit64(g, F, s.qc * (double)s.w[k], i1, i2, x1, x2, j1, j2, xb1, xb2, v3);
+  s.phi[k] = s.phi[k] + g.dt * v3;
+  if (DEPOSIT) deposit64(g, F, s.qc * s.w[k], i1, i2, x1, x2, j1, j2, xb1, xb2, v3);
 }
 
 }  // namespace
@@ -666,80 +632,74 @@ namespace {
 // of the offset from the cell corner, so FP32 keeps its relative accuracy at any cell
 // index and next to theta = pi.
 // =================================================================================
-// The guard-zone form of rsc32: r, sin and cos in FP64 from the FP64 corner tables, with
-// theta clamped to [small_angle, pi - small_angle] as in the FP64 routine.
+// exp(xi) and sin, cos(theta) beyond the series' range (coarse grids), in FP64
+__device__ __noinline__ float2 far_exp(double e_min, double xi) {
+  const DF e = df_of(e_min * exp(xi));
+  return make_float2(e.hi, e.lo);
+}
+__device__ __noinline__ float4 far_sincos(double th) {
+  double s, c;
+  sincos(th, &s, &c);
+  const DF sd = df_of(s), cd = df_of(c);
+  return make_float4(sd.hi, sd.lo, cd.hi, cd.lo);
+}
+// The guard-zone form of rsc32: r, sin and cos in float pairs (about 48 bits) with theta
+// clamped to [small_angle, pi - small_angle] (where sin(theta) is below its value there), as in
+// the FP64 routine. The zones' metric has to be better than FP32 and is rounded to FP32, or
+// enters an FP32 result: pairs give the same rounded values as FP64 (up to ties within 2^-47),
+// on the FP32 pipe, 32 times wider than GB300's FP64 pipe.
 template <bool Q = true>
-__device__ __forceinline__ void rsc64(const GridP &g, const PushTables &tb, int i, int j,
-                                      float o1, float o2, Pt<double> &p) {
-  const double e = (double)o1 * g.dxi;
-  const double ex = fabs(e) <= 0.05 ? __ldg(tb.r64 + i + G_) * exp_small(e)  // < 1e-15
-                                    : map_e(g, (double)i + (double)o1);
-  p.r = Q ? g.r0 + ex : ex;
-  p.f = g.dxi * ex;
-  double d = (double)o2 * g.dth;  // the offset in eta, then in theta
-  double th;
-  if (Q && g.qks) {
-    const double x2 = (double)j + (double)o2;
-    map_g<Q>(g, x2, p.gg, p.gp);
-    th = map_theta<Q>(g, x2);
-    const double t1 = __ldg(tb.t1_64 + j + G_), t2 = __ldg(tb.t2_64 + j + G_);
-    d = d * fma(d, fma(g.c3, d, t2), t1);
-  } else {
-    p.gg = g.dth;
-    p.igg = g.ig2;
-    p.gp = 0.0;
-    th = ((double)j + (double)o2) * g.dth;
+__device__ __forceinline__ void rsc_guard(const GridP &g, const PushTables &tb, int i, int j,
+                                          DF o1, DF o2, Pt<DF> &p) {
+  const float d = rsc_df<Q>(g, tb, i, j, o1, o2, p);
+  if (fabsf(o1.hi * g.f_dxi) > 0.12f) {
+    const float2 v = far_exp(g.e_min, ((double)i + df_to_double(o1)) * g.dxi);
+    const DF ex(v.x, v.y);
+    p.r = Q ? DF(g.d_r0[0], g.d_r0[1]) + ex : ex;
+    p.f = cst<DF>(g).dxi * ex;
   }
-  double &s = p.s, &c = p.c;
-  if (th < g.small_angle || th > GRPIC_PI - g.small_angle) {
-    sincos(fmin(fmax(th, g.small_angle), GRPIC_PI - g.small_angle), &s, &c);
-  } else if (fabs(d) <= 0.1) {
-    const double q = d * d;  // Taylor series to d^9 and d^10: truncation below 3e-17
-    double sp = 1.0 / 362880.0;
-    sp = fma(sp, q, -1.0 / 5040.0);
-    sp = fma(sp, q, 1.0 / 120.0);
-    sp = fma(sp, q, -1.0 / 6.0);
-    const double se = fma(sp * q, d, d);
-    double cp = -1.0 / 3628800.0;
-    cp = fma(cp, q, 1.0 / 40320.0);
-    cp = fma(cp, q, -1.0 / 720.0);
-    cp = fma(cp, q, 1.0 / 24.0);
-    cp = fma(cp, q, -0.5);
-    const double ce = fma(cp, q, 1.0);
-    const double s0 = __ldg(tb.s64 + j + G_), c0 = __ldg(tb.c64 + j + G_);
-    s = fma(s0, ce, c0 * se);
-    c = fma(c0, ce, -s0 * se);
-  } else {
-    sincos(th, &s, &c);
+  if (fabsf(d) > 0.12f) {
+    const float4 v = far_sincos(map_theta<Q>(g, (double)j + df_to_double(o2)));
+    p.s = DF(v.x, v.y);
+    p.c = DF(v.z, v.w);
   }
+  if (p.s.hi < g.d_ss[0]) {
+    p.s = DF(g.d_ss[0], g.d_ss[1]);
+    p.c = p.c.hi < 0.0f ? DF(-g.d_cs[0], -g.d_cs[1]) : DF(g.d_cs[0], g.d_cs[1]);
+  }
+}
+template <bool Q>
+__device__ __forceinline__ void local_guard(const GridP &g, const Pt<DF> &p, Local<DF> &L) {
+  if constexpr (Q) local_full<Q>(g, p, L);
+  else inc_local(inc_c(g), p.r, p.s, p.c, L);  // the plain grid's shorter form
 }
 
-// FP64 metric values rounded for the FP32 arithmetic of the guard zones
-__device__ __forceinline__ void narrow(const Geo<double> &a, Geo<float> &b) {
-  b.H11 = (float)a.H11; b.H13 = (float)a.H13; b.H22 = (float)a.H22; b.H33 = (float)a.H33;
-  b.beta1 = (float)a.beta1; b.opz = (float)a.opz;
+// metric values in pairs rounded for the FP32 arithmetic of the guard zones
+__device__ __forceinline__ void narrow(const Geo<DF> &a, Geo<float> &b) {
+  b.H11 = a.H11.hi; b.H13 = a.H13.hi; b.H22 = a.H22.hi; b.H33 = a.H33.hi;
+  b.beta1 = a.beta1.hi; b.opz = a.opz.hi;
 }
-__device__ __forceinline__ void narrow(const Local<double> &a, Local<float> &b) {
-  b.alpha = (float)a.alpha;
+__device__ __forceinline__ void narrow(const Local<DF> &a, Local<float> &b) {
+  b.alpha = a.alpha.hi;
   narrow(a.G, b.G);
-  b.d1H11 = (float)a.d1H11; b.d1H22 = (float)a.d1H22; b.d1H33 = (float)a.d1H33;
-  b.d1H13 = (float)a.d1H13; b.d1alpha = (float)a.d1alpha; b.d1beta1 = (float)a.d1beta1;
-  b.d2H11 = (float)a.d2H11; b.d2H22 = (float)a.d2H22; b.d2H33 = (float)a.d2H33;
-  b.d2H13 = (float)a.d2H13; b.d2alpha = (float)a.d2alpha; b.d2beta1 = (float)a.d2beta1;
-  b.rH11 = (float)a.rH11; b.sH11 = (float)a.sH11; b.rh22 = (float)a.rh22;
-  b.sh22 = (float)a.sh22; b.rh33 = (float)a.rh33; b.sh33 = (float)a.sh33;
-  b.k13 = (float)a.k13; b.m13 = (float)a.m13;
+  b.d1H11 = a.d1H11.hi; b.d1H22 = a.d1H22.hi; b.d1H33 = a.d1H33.hi;
+  b.d1H13 = a.d1H13.hi; b.d1alpha = a.d1alpha.hi; b.d1beta1 = a.d1beta1.hi;
+  b.d2H11 = a.d2H11.hi; b.d2H22 = a.d2H22.hi; b.d2H33 = a.d2H33.hi;
+  b.d2H13 = a.d2H13.hi; b.d2alpha = a.d2alpha.hi; b.d2beta1 = a.d2beta1.hi;
+  b.rH11 = a.rH11.hi; b.sH11 = a.sH11.hi; b.rh22 = a.rh22.hi;
+  b.sh22 = a.sh22.hi; b.rh33 = a.rh33.hi; b.sh33 = a.sh33.hi;
+  b.k13 = a.k13.hi; b.m13 = a.m13.hi;
 }
 
-// The contravariant metric, shift and 1 + z at a cell-relative point, evaluated in FP64
-// (G64: guard zones) or in FP32, as FP32 values.
-template <bool Q, bool G64>
+// The contravariant metric, shift and 1 + z at a cell-relative point, evaluated in pairs
+// (GUARD: guard zones) or in FP32, as FP32 values.
+template <bool Q, bool GUARD>
 __device__ __forceinline__ void geo_at(const GridP &g, const PushTables &tb, int i, int j,
                                        float o1, float o2, Geo<float> &o) {
-  if constexpr (G64) {
-    Pt<double> p;
-    rsc64<Q>(g, tb, i, j, o1, o2, p);
-    Geo<double> od;
+  if constexpr (GUARD) {
+    Pt<DF> p;
+    rsc_guard<Q>(g, tb, i, j, DF(o1), DF(o2), p);
+    Geo<DF> od;
     geo_from_rsc<Q>(g, p, od);
     narrow(od, o);
   } else {
@@ -834,6 +794,37 @@ __device__ __forceinline__ void zigzag32(const GridP &g, const Move32 &m, float 
   cell[2] = (int)sidx(g, m.ia + (int)f1, m.ja + (int)f2);
 }
 
+// zigzag32 in pairs, rounded to FP32 contributions: the move from (a1, a2) of cell (i, j) to
+// (b1, b2) relative to that cell, in cell (i + c1, j + c2)
+__device__ __forceinline__ void zigzag_df(const GridP &g, DF q, int i, int j, DF a1, DF a2, int c1,
+                                          int c2, DF b1, DF b2, DF v3, float c[3][4],
+                                          int cell[3]) {
+  const DF qi = q * df_of(g.idt);
+  const DF m1 = df_scale(a1 + b1, 0.5f), m2 = df_scale(a2 + b2, 0.5f);
+  const DF r1 = c1 == 0 ? m1 : DF(c1 > 0 ? 1.0f : (float)(c1 + 1));
+  const DF r2 = c2 == 0 ? m2 : DF(c2 > 0 ? 1.0f : (float)(c2 + 1));
+#pragma unroll
+  for (int seg = 0; seg < 2; ++seg) {
+    const DF F1 = qi * (seg ? b1 - r1 : r1 - a1), F2 = qi * (seg ? b2 - r2 : r2 - a2);
+    const DF W1 = seg ? df_scale(r1 + b1, 0.5f) + DF(-(float)c1) : df_scale(a1 + r1, 0.5f);
+    const DF W2 = seg ? df_scale(r2 + b2, 0.5f) + DF(-(float)c2) : df_scale(a2 + r2, 0.5f);
+    const DF t = F1 * W2, v = F2 * W1;
+    c[seg][0] = (F1 - t).hi;
+    c[seg][1] = t.hi;
+    c[seg][2] = (F2 - v).hi;
+    c[seg][3] = v.hi;
+    cell[seg] = seg ? (int)sidx(g, i + c1, j + c2) : (int)sidx(g, i, j);
+  }
+  const int n1 = inc_floor(m1), n2 = inc_floor(m2);
+  const DF w1 = m1 + DF(-(float)n1), w2 = m2 + DF(-(float)n2);
+  const DF qv = q * v3, x = qv * w1, y = qv - x, xt = x * w2, yt = y * w2;
+  c[2][0] = (y - yt).hi;
+  c[2][1] = (x - xt).hi;
+  c[2][2] = yt.hi;
+  c[2][3] = xt.hi;
+  cell[2] = (int)sidx(g, i + n1, j + n2);
+}
+
 // Where the deposit goes: the current planes in global memory ...
 struct GlobalSink {
   float *J[3];
@@ -913,12 +904,9 @@ __device__ __forceinline__ bool run_sums(int key, float v[4]) {
 // of each run issues the four atomics. A move that stays in its cell has both segments in
 // that cell; they are added before the reduction.
 template <class Sink>
-__device__ __forceinline__ void deposit32_warp(const GridP &g, const Sink &sink,
-                                               const Move32 &m, bool on) {
-  float c[3][4];
-  int cell[3] = {-1, -1, -1};
+__device__ __forceinline__ void deposit_groups(const Sink &sink, float c[3][4], int cell[3],
+                                               bool on) {
   if (on) {
-    zigzag32(g, m, c, cell);
     if (cell[1] == cell[0]) {
 #pragma unroll
       for (int q = 0; q < 4; ++q) c[0][q] += c[1][q];
@@ -926,9 +914,11 @@ __device__ __forceinline__ void deposit32_warp(const GridP &g, const Sink &sink,
     }
   } else {
 #pragma unroll
-    for (int grp = 0; grp < 3; ++grp)
+    for (int grp = 0; grp < 3; ++grp) {
+      cell[grp] = -1;
 #pragma unroll
       for (int q = 0; q < 4; ++q) c[grp][q] = 0.0f;
+    }
   }
 #pragma unroll
   for (int grp = 0; grp < 3; ++grp) {
@@ -937,7 +927,14 @@ __device__ __forceinline__ void deposit32_warp(const GridP &g, const Sink &sink,
     if (head && cell[grp] >= 0) sink.add(grp, cell[grp], c[grp]);
   }
 }
-
+template <class Sink>
+__device__ __forceinline__ void deposit32_warp(const GridP &g, const Sink &sink,
+                                               const Move32 &m, bool on) {
+  float c[3][4];
+  int cell[3];
+  if (on) zigzag32(g, m, c, cell);
+  deposit_groups(sink, c, cell, on);
+}
 
 // The FP32 momentum substep: n_iter applications of the geodesic map, or fewer under the
 // stop rule above.
@@ -957,24 +954,24 @@ __device__ __forceinline__ void geodesic_momentum32(const GridP &g, const Local<
   u[1] = t1;
 }
 
-template <bool Q, bool G64>
+template <bool Q, bool GUARD>
 __device__ __forceinline__ float phi_rate32(const GridP &g, const PushTables &tb, int i, int j,
                                             float o1, float o2, const float u[3], float m2) {
   Geo<float> o;
-  geo_at<Q, G64>(g, tb, i, j, o1, o2, o);
+  geo_at<Q, GUARD>(g, tb, i, j, o1, o2, o);
   const float q = fmaf(o.H11 * u[0], u[0], fmaf(o.H22 * u[1], u[1],
                   fmaf(o.H33 * u[2], u[2], fmaf(o.H13, 2.0f * u[0] * u[2], m2))));
   return rsqrtf(o.opz * q) * fmaf(o.H13, u[0], o.H33 * u[2]);
 }
 
 // One particle of the mixed path: steps 2-11 of Sec. 3.1 in FP32 with the metric, lapse
-// and shift evaluated in FP32 (G64 false: off the guard zones) or in FP64 (G64 true: guard
-// zone 1). Returns false when the particle was dropped, else its move (for the deposit). The cell rows on the axes (zone 2) take the
-// FP64 routine instead: there the FP32 rounding of the tetrad-frame momentum, about eps |u|,
+// and shift evaluated in FP32 (GUARD false: off the guard zones) or in pairs (GUARD true: guard
+// zone 1). Returns false when the particle was dropped, else its move (for the deposit). The
+// cell rows on the axes (zone 2) take push_axis, all in pairs, instead: there the FP32 rounding of the tetrad-frame momentum, about eps |u|,
 // enters dphi/dt divided by r sin(theta), which has no lower bound in those rows; one row
 // or more away sin(theta) >= dtheta and dt <= CFL r dtheta bound the phi error per step
 // by about eps CFL.
-template <bool Q, bool G64, class Fields>
+template <bool Q, bool GUARD, class Fields>
 __device__ __forceinline__ bool push32(const GridP &g, const Fields &F, const PushTables &tb,
                                        const SpeciesDevT<float> &s, int64_t k,
                                        unsigned long long *diag, Move32 &mv) {
@@ -982,11 +979,11 @@ __device__ __forceinline__ bool push32(const GridP &g, const Fields &F, const Pu
   const float dx1 = s.dx1[k], dx2 = s.dx2[k];
   const bool em = s.f_m2 != 0.0f;  // massless particles skip the EM push (Sec. 3.1)
   Local<float> L;
-  if constexpr (G64) {
-    Pt<double> p;
-    rsc64<Q>(g, tb, i1, i2, dx1, dx2, p);
-    Local<double> Ld;
-    local_full<Q>(g, p, Ld);
+  if constexpr (GUARD) {
+    Pt<DF> p;
+    rsc_guard<Q>(g, tb, i1, i2, DF(dx1), DF(dx2), p);
+    Local<DF> Ld;
+    local_guard<Q>(g, p, Ld);
     narrow(Ld, L);
   } else {
     Pt<float> p;
@@ -1027,7 +1024,7 @@ __device__ __forceinline__ bool push32(const GridP &g, const Fields &F, const Pu
   for (int it = 0; it < g.n_iter; ++it) {
     Geo<float> o;
     if (it == 0) o = L.G;
-    else geo_at<Q, G64>(g, tb, i1, i2, 0.5f * (dx1 + t1), 0.5f * (dx2 + t2), o);
+    else geo_at<Q, GUARD>(g, tb, i1, i2, 0.5f * (dx1 + t1), 0.5f * (dx2 + t2), o);
     const float q = fmaf(o.H11 * u[0], u[0], fmaf(o.H22 * u[1], u[1],
                     fmaf(o.H33 * u[2], u[2], fmaf(o.H13, uu0, s.f_m2))));
     const float ag = rsqrtf(o.opz * q);
@@ -1069,14 +1066,140 @@ __device__ __forceinline__ bool push32(const GridP &g, const Fields &F, const Pu
   // phi at the midpoint, relative to the start cell (when the iteration ran to n_iter)
   const float b1 = (float)di + e1, b2 = (float)dj + e2;
   if (isnan(v3))
-    v3 = phi_rate32<Q, G64>(g, tb, i1, i2, 0.5f * (dx1 + b1), 0.5f * (dx2 + b2), u, s.f_m2);
+    v3 = phi_rate32<Q, GUARD>(g, tb, i1, i2, 0.5f * (dx1 + b1), 0.5f * (dx2 + b2), u, s.f_m2);
   s.phi[k] = fmaf(dt, v3, s.phi[k]);
   mv = Move32{i1, i2, di, dj, dx1, dx2, b1, b2, s.f_qc * s.w[k], v3};
   return true;
 }
 
-// 0: FP32 metric; 1: FP64 metric (within guard_j rows of an axis or guard cells of the
-// horizon); 2: the cell rows on the axes, FP64 routine
+// One particle of the cell rows on the axes (zone 2 of the mixed path): steps 2-11 of Sec. 3.1
+// in pairs on FP32 storage, the iterations as the method runs them from x^n (next to an axis
+// the coordinate map has more than one fixed point within reach) until the update is within
+// SETTLE32, far below what the stored FP32 result resolves. Returns whether a move is to be
+// deposited: its groups as zigzag32 gives them.
+constexpr float SETTLE32 = 0x1p-26f;
+__device__ __forceinline__ bool settled_df(DF n0, DF t0, DF n1, DF t1) {
+  return fabsf((n0 - t0).hi) <= SETTLE32 * fmaxf(1.0f, fabsf(n0.hi)) &&
+         fabsf((n1 - t1).hi) <= SETTLE32 * fmaxf(1.0f, fabsf(n1.hi));
+}
+__device__ __forceinline__ DF interp_axis(const float *__restrict__ pl, int NX, int i1, int i2,
+                                          float o1, float o2, bool h1, bool h2) {
+  const int b1 = h1 && o1 < 0.5f, b2 = h2 && o2 < 0.5f;
+  const DF w1 = h1 ? two_sum(o1, b1 ? 0.5f : -0.5f) : DF(o1);
+  const DF w2 = h2 ? two_sum(o2, b2 ? 0.5f : -0.5f) : DF(o2);
+  const float *p = pl + (int64_t)(i2 - b2 + G_) * NX + (i1 - b1 + G_);
+  const float p00 = __ldg(p), p10 = __ldg(p + 1), p01 = __ldg(p + NX), p11 = __ldg(p + NX + 1);
+  const DF a = fma_(w1, two_sum(p10, -p00), DF(p00)), b = fma_(w1, two_sum(p11, -p01), DF(p01));
+  return fma_(w2, b - a, a);
+}
+__device__ __forceinline__ DF gamma2_df(const Geo<DF> &o, const DF u[3], DF m2) {
+  return fma_(o.H11 * u[0], u[0], fma_(o.H22 * u[1], u[1],
+         fma_(o.H33 * u[2], u[2], fma_(o.H13, df_scale(u[0] * u[2], 2.0f), m2))));
+}
+template <bool Q>
+__device__ __forceinline__ bool push_axis(const GridP &g, const FieldPtrsT<float> &F,
+                                          const PushTables &tb, const SpeciesDevT<float> &s,
+                                          int64_t k, unsigned long long *diag, float c[3][4],
+                                          int cell[3]) {
+  const int i1 = s.i1[k], i2 = s.i2[k];
+  const float dx1 = s.dx1[k], dx2 = s.dx2[k];
+  const DF o1(dx1), o2(dx2), m2(s.f_m2), dt = cst<DF>(g).dt;
+  const bool em = s.f_m2 != 0.0f;  // massless particles skip the EM push (Sec. 3.1)
+  Local<DF> L;
+  {
+    Pt<DF> p;
+    rsc_guard<Q>(g, tb, i1, i2, o1, o2, p);
+    local_guard<Q>(g, p, L);
+  }
+  DF Bh[3], Dh[3], uh[3], u[3] = {DF(s.u1[k]), DF(s.u2[k]), DF(s.u3[k])};
+  const DF hq = df_scale(df_of(s.qm) * L.alpha * dt, 0.5f);
+  if (em) {
+    DF V[3] = {interp_axis(F.Bn[0], g.NX, i1, i2, dx1, dx2, false, true),
+               interp_axis(F.Bn[1], g.NX, i1, i2, dx1, dx2, true, false),
+               interp_axis(F.Bn[2], g.NX, i1, i2, dx1, dx2, true, true)};
+    vec_hat(L, V, Bh);
+    V[0] = interp_axis(F.D[0], g.NX, i1, i2, dx1, dx2, true, false);
+    V[1] = interp_axis(F.D[1], g.NX, i1, i2, dx1, dx2, false, true);
+    V[2] = interp_axis(F.D[2], g.NX, i1, i2, dx1, dx2, false, false);
+    vec_hat(L, V, Dh);
+    cov_hat(L, u, uh);
+    boris(uh, Dh, Bh, hq);
+    hat_cov(L, uh, u);
+  }
+  {
+    const GeoMap<DF> m(g, L, u, m2);
+    DF t0 = u[0], t1 = u[1];
+    for (int it = 0; it < g.n_iter; ++it) {
+      DF n0, n1;
+      m.apply(t0, t1, n0, n1);
+      const bool fixed = settled_df(n0, t0, n1, t1);
+      t0 = n0;
+      t1 = n1;
+      if (fixed && g.stop_on_repeat) break;
+    }
+    u[0] = t0;
+    u[1] = t1;
+  }
+  if (em) {
+    cov_hat(L, u, uh);
+    boris(uh, Dh, Bh, hq);
+    hat_cov(L, uh, u);
+  }
+  DF t1 = o1, t2 = o2;
+  Geo<DF> o = L.G;  // the first iterate is x^n itself
+  for (int it = 0; it < g.n_iter; ++it) {
+    if (it > 0) {
+      Pt<DF> p;
+      rsc_guard<Q>(g, tb, i1, i2, df_scale(o1 + t1, 0.5f), df_scale(o2 + t2, 0.5f), p);
+      geo_from_rsc<Q>(g, p, o);
+    }
+    const DF ag = rsqrt_(o.opz * gamma2_df(o, u, m2));  // alpha / gamma
+    const DF n1 = fma_(dt, fma_(ag, fma_(o.H11, u[0], o.H13 * u[2]), -o.beta1), o1);
+    const DF n2 = fma_(dt, ag * o.H22 * u[1], o2);
+    const bool fixed = settled_df(n1, t1, n2, t2);
+    t1 = n1;
+    t2 = n2;
+    if (fixed && g.stop_on_repeat) break;
+  }
+  if (!(isfinite(u[0].hi) && isfinite(u[1].hi) && isfinite(u[2].hi) && fabsf(t1.hi) < 1e6f &&
+        fabsf(t2.hi) < 1e6f)) {
+    s.tag[k] = 0;
+    count(diag, DG_NONFINITE);
+    return false;
+  }
+  const int f1 = inc_floor(t1), f2 = inc_floor(t2);
+  const int j1 = i1 + f1;
+  int j2 = i2 + f2;
+  DF e1 = t1 + DF(-(float)f1), e2 = t2 + DF(-(float)f2);
+  // boundaries (Sec. 3.3.3): reflection off the axes, removal into the ghost zone
+  if (j2 < 0 || j2 >= g.n_th) {
+    j2 = j2 < 0 ? 0 : g.n_th - 1;
+    e2 = DF(1.0f) - e2;
+    u[1] = -u[1];
+    count(diag, DG_REFLECT);
+  }
+  // the stored position is what the next step and the deposit start from
+  e1 = DF(e1.hi);
+  e2 = DF(e2.hi);
+  s.i1[k] = j1; s.i2[k] = j2; s.dx1[k] = e1.hi; s.dx2[k] = e2.hi;
+  s.u1[k] = u[0].hi; s.u2[k] = u[1].hi; s.u3[k] = u[2].hi;
+  if (j1 < 0) { s.tag[k] = 2; count(diag, DG_LEFT_INNER); }
+  else if (j1 >= g.n_r) { s.tag[k] = 2; count(diag, DG_LEFT_OUTER); }
+  // step 11: phi at the midpoint of x^n and the final x^{n+1}
+  const int c1 = j1 - i1, c2 = j2 - i2;
+  const DF b1 = e1 + DF((float)c1), b2 = e2 + DF((float)c2);
+  Pt<DF> p;
+  rsc_guard<Q>(g, tb, i1, i2, df_scale(o1 + b1, 0.5f), df_scale(o2 + b2, 0.5f), p);
+  geo_from_rsc<Q>(g, p, o);
+  const DF v3 = rsqrt_(o.opz * gamma2_df(o, u, m2)) * fma_(o.H13, u[0], o.H33 * u[2]);
+  s.phi[k] = fma_(dt, v3, DF(s.phi[k])).hi;
+  if (!(j1 >= -G_ && j1 <= g.n_r)) return false;
+  zigzag_df(g, df_of(s.qc) * DF(s.w[k]), i1, i2, o1, o2, c1, c2, b1, b2, v3, c, cell);
+  return true;
+}
+
+// 0: FP32 metric; 1: metric in pairs (within guard_j rows of an axis or guard cells of the
+// horizon); 2: the cell rows on the axes, all in pairs
 __device__ __forceinline__ int guard_zone(const PushTables &tb, const GridP &g, int i1, int i2) {
   if (i2 == 0 || i2 == g.n_th - 1) return 2;
   return ((i1 >= tb.guard_ilo && i1 < tb.guard_ihi) || i2 < tb.guard_j ||
@@ -1110,7 +1233,7 @@ __global__ void __launch_bounds__(TPB, GRPIC_PUSH64_MIN_BLOCKS)
     if (INC && __all_sync(__activemask(), inc_fit(g, F, tb, s, k)) &&
         push_inc<DEPOSIT>(g, F, tb, s, k, diag))
       continue;
-    push64<Q, double, DEPOSIT>(g, F, tb, s, k, diag);
+    push64<Q, DEPOSIT>(g, F, tb, s, k, diag);
   }
 }
 
@@ -1133,16 +1256,15 @@ constexpr int CL_U = 8;
 #ifndef GRPIC_AXIS_BLOCKS_PER_SM
 #define GRPIC_AXIS_BLOCKS_PER_SM 4
 #endif
-// their register caps as resident one-warp blocks per SM (65536 / (32 x this) registers):
-// the registers they hold while resident are taken from the concurrent FP32 kernel. The
-// zone-1 kernel capped at 80 (a few spills) left the FP32 kernel enough to make the mixed
-// step 2% faster on GB300 than uncapped (119) or at 64; capping the zone-2 kernel cost more
-// than it gave.
+// their register cap as resident one-warp blocks per SM (65536 / (32 x this) registers): the
+// registers they hold while resident are taken from the concurrent FP32 kernel (with the
+// metric in FP64, 80 registers and a few spills left it enough to make the mixed step 2% faster
+// than uncapped or at 64). With the zones in pairs of floats instead of FP64 (zone 2 alone took
+// 60 us on 64^2 cells, for FP64 operations at 2 per clock and SM) ten steps of the 64^2 run went
+// from 2.28 to 1.37 ms, of the 512^2 one from 10.6 to 9.7 ms, of the 2048^2 one from 77.5 to
+// 74.7 ms.
 #ifndef GRPIC_GUARD_MIN_BLOCKS
 #define GRPIC_GUARD_MIN_BLOCKS 24
-#endif
-#ifndef GRPIC_AXIS_MIN_BLOCKS
-#define GRPIC_AXIS_MIN_BLOCKS 1
 #endif
 __global__ void __launch_bounds__(TPB) k_classify(GridP g, SpeciesDevT<float> s, PushTables tb,
                                                   GuardList gl) {
@@ -1164,27 +1286,32 @@ __global__ void __launch_bounds__(TPB) k_classify(GridP g, SpeciesDevT<float> s,
         b[q] = s.i2[k];
       }
     }
+    unsigned m1[CL_U], m2[CL_U];
+    int n1 = 0, n2 = 0;
 #pragma unroll
     for (int q = 0; q < CL_U; ++q) {
       const int64_t kw = w0 + q * stride;  // the warp's first particle
-      if (kw >= n) break;
       const int zone = tag[q] == 1 ? guard_zone(tb, g, a[q], b[q]) : 0;
-      const unsigned m1 = __ballot_sync(0xffffffffu, zone == 1);
-      const unsigned m2 = __ballot_sync(0xffffffffu, zone == 2);
-      if (lane == 0) gl.mask[kw >> 5] = m1 | m2;
-      if (m1 | m2) {
-        unsigned long long b1 = 0, b2 = 0;
-        if (lane == 0) {
-          if (m1) b1 = atomicAdd(gl.count, (unsigned long long)__popc(m1));
-          if (m2) b2 = atomicAdd(gl.count + 1, (unsigned long long)__popc(m2));
-        }
-        b1 = __shfl_sync(0xffffffffu, b1, 0);
-        b2 = __shfl_sync(0xffffffffu, b2, 0);
-        const unsigned below = (1u << lane) - 1u;
-        const uint32_t k = (uint32_t)(kw + lane);
-        if (zone == 1) gl.idx[b1 + __popc(m1 & below)] = k;
-        if (zone == 2) gl.idx[gl.cap - 1 - (int64_t)(b2 + __popc(m2 & below))] = k;
-      }
+      m1[q] = __ballot_sync(0xffffffffu, zone == 1);
+      m2[q] = __ballot_sync(0xffffffffu, zone == 2);
+      n1 += __popc(m1[q]);
+      n2 += __popc(m2[q]);
+      if (lane == 0 && kw < n) gl.mask[kw >> 5] = m1[q] | m2[q];
+    }
+    if (n1 + n2 == 0) continue;
+    // one reservation per list for all the trip's particles (lanes 0 and 1: one latency)
+    unsigned long long got = 0;
+    if (lane < 2) got = atomicAdd(gl.count + lane, (unsigned long long)(lane ? n2 : n1));
+    unsigned long long b1 = __shfl_sync(0xffffffffu, got, 0);
+    unsigned long long b2 = __shfl_sync(0xffffffffu, got, 1);
+    const unsigned bit = 1u << lane, below = bit - 1u;
+#pragma unroll
+    for (int q = 0; q < CL_U; ++q) {
+      const uint32_t k = (uint32_t)(w0 + q * stride + lane);
+      if (m1[q] & bit) gl.idx[b1 + __popc(m1[q] & below)] = k;
+      if (m2[q] & bit) gl.idx[gl.cap - 1 - (int64_t)(b2 + __popc(m2[q] & below))] = k;
+      b1 += __popc(m1[q]);
+      b2 += __popc(m2[q]);
     }
   }
 }
@@ -1380,41 +1507,36 @@ size_t tiled_smem_bytes(const TileInfo &ti) {
          128;
 }
 
-// Mixed path, guard kernels (side stream): step 1 and the routine of the listed particles,
-// zone 1 with the metric in FP64, zone 2 with the FP64 routine.
+// Mixed path, guard kernel (side stream): step 1 and the routine of the listed particles, zone 2
+// (the rows on the axes, the longer routine, first: blocks below `axis_blocks`) in pairs,
+// zone 1 with the metric in pairs.
 template <bool DEPOSIT, bool Q>
-__global__ void __launch_bounds__(32, GRPIC_GUARD_MIN_BLOCKS) k_push_guard(GridP g, FieldPtrsT<float> F,
-                                                    SpeciesDevT<float> s, PushTables tb,
-                                                    GuardList gl, unsigned long long *diag) {
-  const int64_t n = (int64_t)gl.count[0];
+__global__ void __launch_bounds__(32, GRPIC_GUARD_MIN_BLOCKS)
+    k_push_guard(GridP g, FieldPtrsT<float> F, SpeciesDevT<float> s, PushTables tb, GuardList gl,
+                 int axis_blocks, unsigned long long *diag) {
   const int lane = threadIdx.x & 31;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t - lane < n;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    Move32 mv;
+  const bool axis = (int)blockIdx.x < axis_blocks;
+  const int64_t n = (int64_t)gl.count[axis ? 1 : 0];
+  const int64_t b = axis ? blockIdx.x : blockIdx.x - axis_blocks;
+  const int64_t stride = (axis ? axis_blocks : (int)gridDim.x - axis_blocks) * (int64_t)32;
+  for (int64_t t = b * 32 + lane; t - lane < n; t += stride) {
+    float c[3][4];
+    int cell[3];
     bool on = false;
     if (t < n) {
-      const int64_t k = gl.idx[t];
+      const int64_t k = axis ? gl.idx[gl.cap - 1 - t] : gl.idx[t];
       if (s.i1p) {
         s.i1p[k] = s.i1[k]; s.i2p[k] = s.i2[k]; s.dx1p[k] = s.dx1[k]; s.dx2p[k] = s.dx2[k];
       }
-      on = push32<Q, true>(g, GlobalFields(g, F), tb, s, k, diag, mv);
+      if (axis) {
+        on = push_axis<Q>(g, F, tb, s, k, diag, c, cell);
+      } else {
+        Move32 mv;
+        on = push32<Q, true>(g, GlobalFields(g, F), tb, s, k, diag, mv);
+        if (DEPOSIT && on) zigzag32(g, mv, c, cell);
+      }
     }
-    if (DEPOSIT) deposit32_warp(g, GlobalSink(g, F), mv, on);
-  }
-}
-
-template <bool DEPOSIT, bool Q>
-__global__ void __launch_bounds__(32, GRPIC_AXIS_MIN_BLOCKS) k_push_axis(GridP g, FieldPtrsT<float> F,
-                                                   SpeciesDevT<float> s, PushTables tb,
-                                                   GuardList gl, unsigned long long *diag) {
-  const int64_t n = (int64_t)gl.count[1];
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t k = gl.idx[gl.cap - 1 - t];
-    if (s.i1p) {
-      s.i1p[k] = s.i1[k]; s.i2p[k] = s.i2[k]; s.dx1p[k] = s.dx1[k]; s.dx2p[k] = s.dx2[k];
-    }
-    push64<Q, float, DEPOSIT, false>(g, F, tb, s, k, diag);  // axis rows: never refined
+    if (DEPOSIT) deposit_groups(GlobalSink(g, F), c, cell, on);
   }
 }
 
@@ -1614,18 +1736,13 @@ cudaError_t push_impl(const GridP &g, const FieldPtrsT<T> &F, SpeciesDevT<T> s,
       COUNT_LAUNCH(1);
     }
     if (kernels_stage) {
-      // the guard kernels are FP64-pipe bound: a few one-warp blocks per SM reach every SM
-      // sub-partition's FP64 unit and leave the registers to the concurrent FP32 kernel
+      // a few one-warp blocks per SM: the guard kernel runs beside the FP32 kernel, to which it
+      // leaves the registers
       constexpr int gb = 152 * GRPIC_GUARD_BLOCKS_PER_SM, ab = 152 * GRPIC_AXIS_BLOCKS_PER_SM;
-      if (deposit) {
-        k_push_guard<true, Q><<<gb, 32, 0, ps.side>>>(g, F, s, tb, gl, diag);
-        k_push_axis<true, Q><<<ab, 32, 0, ps.side>>>(g, F, s, tb, gl, diag);
-      } else {
-        k_push_guard<false, Q><<<gb, 32, 0, ps.side>>>(g, F, s, tb, gl, diag);
-        k_push_axis<false, Q><<<ab, 32, 0, ps.side>>>(g, F, s, tb, gl, diag);
-      }
+      if (deposit) k_push_guard<true, Q><<<gb + ab, 32, 0, ps.side>>>(g, F, s, tb, gl, ab, diag);
+      else k_push_guard<false, Q><<<gb + ab, 32, 0, ps.side>>>(g, F, s, tb, gl, ab, diag);
       if ((e = cudaEventRecord(ps.done, ps.side)) != cudaSuccess) return e;
-      COUNT_LAUNCH(2);
+      COUNT_LAUNCH(1);
     }
     if (!main_stage) return cudaGetLastError();
     // the FP32 kernel reads the mask the classify writes
