@@ -85,7 +85,11 @@ __device__ __forceinline__ double map_theta(const GridP &g, double x2) {
   const double q = __dmul_rn(__dmul_rn(__dmul_rn(__dmul_rn(2.0, g.h0), eta),
                                        __dadd_rn(GRPIC_PI, -__dmul_rn(2.0, eta))),
                              __dadd_rn(GRPIC_PI, -eta));
-  return __dadd_rn(eta, __ddiv_rn(q, __dmul_rn(GRPIC_PI, GRPIC_PI)));
+  // q / pi^2, correctly rounded without a division: from the correctly rounded reciprocal the
+  // quotient's residual is exact and one correction rounds right (Markstein's theorem)
+  constexpr double b = GRPIC_PI * GRPIC_PI, y = 1.0 / b;
+  const double q0 = __dmul_rn(q, y);
+  return __dadd_rn(eta, __fma_rn(__fma_rn(-q0, b, q), y, q0));
 }
 // g = deta (1 + 2 h0 + 12 h0 (eta/pi)(eta/pi - 1)), gp = deta^2 12 h0 (2 eta/pi^2 - 1/pi)
 template <bool Q = true>

@@ -150,18 +150,45 @@ __device__ __forceinline__ void local_rsc(const GridP &g, const Base &b, double 
   }
 }
 
-// dphi/dt = alpha/gamma h^{3j} u_j at (x1t, x2t) (Eq. discretized-geodesic-x-phi; q times
-// it is J^3 / sqrt(h) w, Sec. 3.2); alpha/gamma = 1/sqrt((1+z) gamma^2).
+// The coordinate velocities of Eqs. (discretized-geodesic-x) and (-x-phi) at a point, the
+// metric's products regrouped as in inc_velocity (inc.cuh), so that they take 45 FP64
+// operations instead of the ~70 of the metric first and the velocities from it
+// (geo_from_rsc): photons on a quasi-spherical grid, 10^6 x 4 pushes, 10.05 -> 8.92 ms (with
+// the tetrads left out for photons and x^n from the corner tables).
+template <bool Q = true>
+__device__ __forceinline__ void velocity64(const GridP &g, const Pt<double> &p, const double u[3],
+                                           double m2, double &v1, double &v2, double &v3) {
+  const double s2 = p.s * p.s, r2 = p.r * p.r, f = p.f;
+  const double Sig = fma(g.a2, p.c * p.c, r2), M2r = g.M2 * p.r, S2 = Sig + M2r;
+  const double Rr = r2 + g.a2, A = fma(Rr, Rr, -(g.a2 * s2 * (Rr - M2r)));
+  const double fs = f * s2, X0 = S2 * fs;
+  double iQ, igg;
+  if (Q && g.qks) {
+    const double g2 = p.gg * p.gg, iX = rcp_nr(X0 * g2);
+    iQ = iX * g2;
+    igg = iX * X0;
+  } else {
+    iQ = rcp_nr(X0);
+    igg = p.igg;
+  }
+  const double iS2 = iQ * fs, T = iQ * S2, fi = T * s2, w0 = u[0] * fi, au = g.a * u[2];
+  const double I = fma(A * iS2, w0, au), kk = igg * u[1], z = u[2] * (T * f);
+  const double X = fma(w0, I + au, fma(kk, u[1], u[2] * z));
+  const double G = rsqrt(S2 * fma(m2, Sig, X));  // alpha / (gamma Sigma)
+  v1 = fi * fma(G, I, -(M2r * iS2));
+  v2 = G * kk;
+  v3 = G * fma(g.a, w0, z);
+}
+
+// dphi/dt at (x1t, x2t); q times it is J^3 / sqrt(h) w (Sec. 3.2)
 template <bool Q = true>
 __device__ __forceinline__ double phi_rate64(const GridP &g, const Base &b, double x1t,
                                              double x2t, const double u[3], double m2) {
   Pt<double> p;
   local_rsc<Q>(g, b, x1t, x2t, p);
-  Geo<double> o;
-  geo_from_rsc<Q>(g, p, o);
-  const double q = fma(o.H11 * u[0], u[0], fma(o.H22 * u[1], u[1], fma(o.H33 * u[2], u[2],
-                   fma(2.0 * o.H13 * u[0], u[2], m2))));
-  return rsqrt(o.opz * q) * fma(o.H13, u[0], o.H33 * u[2]);
+  double v1, v2, v3;
+  velocity64<Q>(g, p, u, m2, v1, v2, v3);
+  return v3;
 }
 
 // Bilinear interpolation at code position (x1, x2) of planes whose Yee location is offset by
@@ -419,25 +446,25 @@ __device__ __forceinline__ void coord_exact(const GridP &g, const Base &b, const
                                             int i1, int i2, double dx1, double dx2,
                                             const double u[3], double m2, double &t1,
                                             double &t2) {
-  const double uu0 = 2.0 * u[0] * u[2];
   t1 = dx1;
   t2 = dx2;
   for (int it = 0; it < g.n_iter; ++it) {
-    Geo<double> o;
+    double v1, v2, v3;
     if (it == 0) {
-      o = L.G;
+      const Geo<double> &o = L.G;
+      const double q = fma(o.H11 * u[0], u[0], fma(o.H22 * u[1], u[1],
+                       fma(o.H33 * u[2], u[2], fma(o.H13, 2.0 * u[0] * u[2], m2))));
+      const double ag = rsqrt(o.opz * q);  // alpha / gamma
+      v1 = fma(ag, fma(o.H11, u[0], o.H13 * u[2]), -o.beta1);
+      v2 = ag * o.H22 * u[1];
     } else {
       Pt<double> p;
       // x_bar = i + (dx + x~)/2, rounded in that order
       local_rsc<Q>(g, b, __dadd_rn((double)i1, 0.5 * __dadd_rn(dx1, t1)),
                    __dadd_rn((double)i2, 0.5 * __dadd_rn(dx2, t2)), p);
-      geo_from_rsc<Q>(g, p, o);
+      velocity64<Q>(g, p, u, m2, v1, v2, v3);
     }
-    const double q = fma(o.H11 * u[0], u[0], fma(o.H22 * u[1], u[1],
-                     fma(o.H33 * u[2], u[2], fma(o.H13, uu0, m2))));
-    const double ag = rsqrt(o.opz * q);  // alpha / gamma
-    const double n1 = fma(g.dt, fma(ag, fma(o.H11, u[0], o.H13 * u[2]), -o.beta1), dx1);
-    const double n2 = fma(g.dt, ag * o.H22 * u[1], dx2);
+    const double n1 = fma(g.dt, v1, dx1), n2 = fma(g.dt, v2, dx2);
     const bool fixed = (n1 == t1) && (n2 == t2);  // later iterations are no-ops
     t1 = n1;
     t2 = n2;
@@ -455,14 +482,10 @@ __device__ __forceinline__ void coord_map64(const GridP &g, const Base &b, int i
   Pt<double> p;
   local_rsc<Q>(g, b, __dadd_rn((double)i1, 0.5 * __dadd_rn(dx1, t1)),
                __dadd_rn((double)i2, 0.5 * __dadd_rn(dx2, t2)), p);
-  Geo<double> o;
-  geo_from_rsc<Q>(g, p, o);
-  const double q = fma(o.H11 * u[0], u[0], fma(o.H22 * u[1], u[1],
-                   fma(o.H33 * u[2], u[2], fma(o.H13, 2.0 * u[0] * u[2], m2))));
-  const double ag = rsqrt(o.opz * q);
-  n1 = fma(g.dt, fma(ag, fma(o.H11, u[0], o.H13 * u[2]), -o.beta1), dx1);
-  n2 = fma(g.dt, ag * o.H22 * u[1], dx2);
-  v3 = ag * fma(o.H13, u[0], o.H33 * u[2]);  // Eq. (discretized-geodesic-x-phi) at x_bar
+  double v1, v2;
+  velocity64<Q>(g, p, u, m2, v1, v2, v3);  // v3: Eq. (discretized-geodesic-x-phi) at x_bar
+  n1 = fma(g.dt, v1, dx1);
+  n2 = fma(g.dt, v2, dx2);
 }
 
 // the coordinate substep's refined iterations; t1, t2: the new offsets from cell (i1, i2)
@@ -553,12 +576,13 @@ __device__ __forceinline__ void push64(const GridP &g, const FieldPtrsT<double> 
   // the refined iterations keep two cell rows away from the axes: there the coordinate map
   // (metric terms ~ 1/sin^2(theta)) has more than one fixed point within reach, and the
   // method's answer is the one its iteration from x^n finds
-  const bool refine = g.iter_tol > 0.0 && i2 >= 2 && i2 < g.n_th - 2;
-  const Base b = refine ? make_base_tab<Q>(g, tb, i1, i2, dx1, x1, x2) : make_base<Q>(g, x1, x2);
+  const bool inner = i2 >= 2 && i2 < g.n_th - 2 && i1 >= 0 && i1 < g.n_r;
+  const bool refine = g.iter_tol > 0.0 && inner;
+  const Base b = inner ? make_base_tab<Q>(g, tb, i1, i2, dx1, x1, x2) : make_base<Q>(g, x1, x2);
   Pt<double> p0;
   local_at_base<Q>(g, b, x2, p0);  // clamps theta near the axes
   Local<double> L;
-  local_full<Q>(g, p0, L);
+  local_full<Q>(g, p0, L, em);
   double Bh[3], Dh[3], uh[3], u[3] = {s.u1[k], s.u2[k], s.u3[k]};
   const double hq = s.qm * L.alpha * 0.5 * g.dt;
   if (em) {

@@ -127,8 +127,9 @@ __device__ __forceinline__ void geo_from_rsc(const GridP &g, const Pt<R> &p, Geo
   o.beta1 = M2 * r * iS2 * fi;
 }
 
-// The metric at x^n with the derivatives the momentum push needs, and the tetrad
-// coefficients; one division, four reciprocal square roots.
+// The metric at x^n with the derivatives the momentum push needs, and (tet) the tetrad
+// coefficients, which massless particles do without; one division, one or four reciprocal
+// square roots.
 template <typename R>
 struct Local {
   R alpha;
@@ -138,7 +139,8 @@ struct Local {
   R rH11, sH11, rh22, sh22, rh33, sh33, k13, m13;
 };
 template <bool Q = true, typename R>
-__device__ __forceinline__ void local_full(const GridP &g, const Pt<R> &p, Local<R> &L) {
+__device__ __forceinline__ void local_full(const GridP &g, const Pt<R> &p, Local<R> &L,
+                                           bool tet = true) {
   const Cst<R> k = cst<R>(g);
   const R a = k.a, M = k.M, a2 = k.a2, M2 = k.M2, gg = p.gg, dxi = k.dxi;
   const R r = p.r, s = p.s, c = p.c, r2 = r * r, s2 = s * s;
@@ -192,6 +194,7 @@ __device__ __forceinline__ void local_full(const GridP &g, const Pt<R> &p, Local
   L.d2alpha = M * r * deS * iSg2 * al3;
   L.d1beta1 = M2 * fi * fsr * iS2 * iS2 - dxi * o.beta1;
   L.d2beta1 = (R)-2 * M * fi * r * deS * iS2 * iS2;
+  if (!tet) return;
   const R h22 = gg * gg * Sig, h33 = A * s2 * iSig, h13 = -f * a * o.opz * s2;
   L.rH11 = rsqrt_(o.H11);
   L.sH11 = o.H11 * L.rH11;
