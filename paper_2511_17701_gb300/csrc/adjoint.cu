@@ -363,7 +363,7 @@ __device__ __forceinline__ bool adj_inc_step(const GridP &g, const FieldPtrsT<do
   const double dx1 = st[0] - f1, dx2 = st[1] - f2;
   a.o1 = df_of(dx1);
   a.o2 = df_of(dx2);
-  if (!inc_point(k, tb, a.i1, a.i2, a.o1, a.o2, a.r, a.s, a.c)) return false;
+  if (!inc_point_n(g, k, tb, a.i1, a.i2, dx2, a.o1, a.o2, a.r, a.s, a.c)) return false;
   inc_local(k, a.r, a.s, a.c, a.L);
   IncLerp l;
   inc_lerp(a.i1, a.i2, a.o1, a.o2, l);
@@ -390,7 +390,9 @@ __device__ __forceinline__ bool adj_inc_step(const GridP &g, const FieldPtrsT<do
   for (int q = 0; q < 3; ++q) a.u1[q] = a.u[q] + du[q];
   GeoInc<DF> m;
   geo_inc_setup(k, a.L, a.u1, 1.0f, m);
-  if (!geo_inc_solve(m, n_iter, INC_ADJ_TOL, a.dg[0], a.dg[1])) return false;
+  if (geo_inc_solve<false>(m, a.L.G.H33.hi * a.u[2].hi * a.u[2].hi, n_iter, INC_ADJ_TOL, a.dg[0],
+                           a.dg[1]) != GEO_SMALL)
+    return false;
   du[0] = du[0] + a.dg[0];
   du[1] = du[1] + a.dg[1];
   a.u2[0] = a.u[0] + du[0];

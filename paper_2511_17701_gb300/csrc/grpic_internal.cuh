@@ -422,6 +422,7 @@ struct PushStreams {
   cudaEvent_t fork, done, classified;  // side after main; guard kernels done; classify done
   cudaEvent_t t0, t1;  // when not null: recorded on `main` around the main push kernel
   int stage = PUSH_ALL;
+  bool apart = false;  // FP64: a small push may run on `side` (forked and recorded as above)
 };
 
 template <typename T>

@@ -5,31 +5,37 @@
 // GB300 executes 2 FP64 operations per clock and SM against 128 FP32 ones, and the FP64
 // routine (push64) needs ~560 of them per particle. But everything a step computes for the
 // momentum ends in an increment that is a small part of u: u^{n+1} = u^n + du. An increment
-// of relative size eps, computed in pairs of floats (dfloat.cuh, relative error ~2^-47),
-// leaves an error of eps 2^-47 in u, which for eps <= 2^-5 is at or below FP64's own
-// rounding. So the metric and its derivatives at x^n, the tetrads, the field interpolation,
+// of relative size eps, computed in pairs of floats (dfloat.cuh, relative error ~2^-48),
+// leaves an error of eps 2^-48 in u, which for eps <= 2^-4 is at or below what the FP64
+// routine's own rounding leaves (3e-16 of |u| rms). So the metric and its derivatives at x^n, the tetrads, the field interpolation,
 // both Boris half steps and the geodesic substep are evaluated in float pairs, as
 // increments, and u^n + du is formed in FP64 by one addition per component. The coordinate
 // substep is not small against the offset it changes: its result is, as in push64, one FP64
 // evaluation of the map at the predictor's point.
 //
-// A particle that the bounds behind this do not cover (the axis rows, an increment above
-// 2^-5, an iteration that the predictor does not resolve, values outside the range of FP32)
-// is left to push64, untouched.
+// Where a Boris half step turns or kicks the momentum by more than INC_MAX of itself (strong
+// fields) both are taken in FP64, the rest as above. A particle that the
+// bounds behind this do not cover (a reflection off an axis, an iteration that the predictor
+// does not resolve, values outside the range of FP32) is left to push64, untouched.
 //
-// Measured: a step of the 2048^2 workload (134 M particles) 173.6 -> 80.3 ms, of the 512^2 one
-// (16.8 M) 21.0 -> 11.0 ms. One push against 113-bit arithmetic, six grids from 64^2 to 2048^2
-// (60,000 particles each): rms errors of u 0.8-3.1e-16 of its rms (push64: 2.5-3.3e-16), of the
-// offsets 2.4-4.9e-17 (2.5-5.5e-17).
+// Measured: a step of the 2048^2 workload (134 M particles) 173.6 -> 65.9 ms, of the 512^2 one
+// (16.8 M) 21.0 -> 8.85 ms. One push against 113-bit arithmetic, six grids from 64^2 to 2048^2
+// (60,000 particles each): rms errors of u 4.7-8.0e-17 of its rms (push64: 2.5-3.3e-16), of the
+// offsets 2.4-4.6e-17 (2.4-5.5e-17).
 #pragma once
 #include "dual_df.cuh"
 #include "refine.cuh"
 
 namespace {
 
-constexpr float INC_MAX = 0x1p-5f;   // largest |increment| / max(1, |u|) of a Boris half step
+constexpr float INC_MAX = 0x1p-4f;   // largest |increment| / |u| of a Boris half step in pairs
+constexpr float INC_GEO = 0x1p-4f;   // the same of the geodesic substep
+// increments are measured against 1/4 (a velocity of c/4) where |u| is less: what the rest of
+// a step sees of such a momentum is its absolute error, here below 2^-54
+constexpr float INC_UU = 0x1p-4f;
 constexpr float INC_E = 0.055f;      // largest |offset of xi| of the radial series
 constexpr float INC_D = 0.035f;      // largest |offset of theta| of the angular series
+constexpr int INC_ROWS = 64;          // rows from either axis with theta as map_theta rounds it
 constexpr float INC_R = 1024.0f;     // largest r: r^-8 and its low parts stay in FP32's range
 
 __device__ __forceinline__ DF df2(const float2 v) { return DF(v.x, v.y); }
@@ -45,14 +51,14 @@ __device__ __forceinline__ IncC inc_c(const GridP &g) {
 }
 
 // r, sin(theta), cos(theta) in pairs at x1 = i + o1, x2 = j + o2 from the tables of the
-// nearest cell corner. The series' leading terms are pairs, their tails (below 2^-24 of the
-// result's last bit but one) plain floats. Returns whether the offsets are in range.
-__device__ __forceinline__ bool inc_point(const IncC &k, const PushTables &tb, int i, int j, DF o1,
-                                          DF o2, DF &r, DF &s, DF &c) {
-  const int c1 = o1.hi >= 0.5f, c2 = o2.hi >= 0.5f;
+// nearest cell corner (rows' corner j + c2, d: theta's offset from it). The series' leading
+// terms are pairs, their tails (below 2^-24 of the result's last bit but one) plain floats.
+// Returns whether the offsets are in range.
+__device__ __forceinline__ bool inc_point_d(const IncC &k, const PushTables &tb, int i, int j,
+                                            DF o1, DF o2, int c2, DF d, DF &r, DF &s, DF &c) {
+  const int c1 = o1.hi >= 0.5f;
   const DF q1 = fast_two_sum(__fsub_rn(o1.hi, (float)c1), o1.lo);
-  const DF q2 = fast_two_sum(__fsub_rn(o2.hi, (float)c2), o2.lo);
-  const DF e = q1 * k.dxi, d = q2 * k.dth;
+  const DF e = q1 * k.dxi;
   const float ef = e.hi;
   // exp(e) = 1 + e + e^2/2 + e^3/6 + e^4 (1/24 + ...)
   float t = fmaf(1.0f / 40320.0f, ef, 1.0f / 5040.0f);
@@ -77,6 +83,29 @@ __device__ __forceinline__ bool inc_point(const IncC &k, const PushTables &tb, i
   c = fma_(c0, ce, -(s0 * se));
   return fabsf(ef) <= INC_E && fabsf(d.hi) <= INC_D && o1.hi >= 0.0f && o1.hi <= 1.0f &&
          o2.hi >= 0.0f && o2.hi <= 1.0f && r.hi <= INC_R;
+}
+
+__device__ __forceinline__ bool inc_point(const IncC &k, const PushTables &tb, int i, int j, DF o1,
+                                          DF o2, DF &r, DF &s, DF &c) {
+  const int c2 = o2.hi >= 0.5f;
+  const DF q2 = fast_two_sum(__fsub_rn(o2.hi, (float)c2), o2.lo);
+  return inc_point_d(k, tb, i, j, o1, o2, c2, q2 * k.dth, r, s, c);
+}
+// At x^n = (i + dx1, j + dx2): in the rows near the axes theta is formed as map_theta forms it
+// (x2 dtheta, rounded) and its offset from the corner's exact. Next to theta = pi that rounding
+// is a relative 2e-16 / (pi - theta) of sin(theta), which the momentum's increments, of order u
+// there, would show at ~1e-12 if it were formed in another way.
+__device__ __forceinline__ bool inc_point_n(const GridP &g, const IncC &k, const PushTables &tb,
+                                            int i, int j, double dx2, DF o1, DF o2, DF &r, DF &s,
+                                            DF &c) {
+  const int c2 = o2.hi >= 0.5f;
+  DF d;
+  if (j < INC_ROWS || j >= g.n_th - INC_ROWS) {
+    d = df_of(__dmul_rn(__dadd_rn((double)j, dx2), g.dth) - __ldg(tb.th64 + j + c2 + G_));
+  } else {
+    d = fast_two_sum(__fsub_rn(o2.hi, (float)c2), o2.lo) * k.dth;
+  }
+  return inc_point_d(k, tb, i, j, o1, o2, c2, d, r, s, c);
 }
 
 // Metric, its derivatives and the tetrad coefficients at x^n in pairs: the quantities of
@@ -217,13 +246,17 @@ __device__ __forceinline__ void geo_inc_setup(const IncC &k, const Local<M> &L, 
   m.d2H22 = R(L.d2H22);
 }
 
-// The fixed point (n0, n1) of the map; false: not resolved here. The FP32 map gives the
-// increment to FP32 rounding, one evaluation in pairs there and one Newton step with the
-// FP32 Jacobian J, d + (I - J)^{-1} r = G + M J r with r = G - d and M = (I - J)^{-1}, leave
-// an error of |J| 2^-24 |r|, far below the pairs' rounding of d. n_iter, tol: the method's
-// iterations and what they have to come within (inc_converges).
-__device__ __forceinline__ bool geo_inc_solve(const GeoInc<DF> &m, int n_iter, float tol, DF &n0,
-                                              DF &n1) {
+// The fixed point (n0, n1) of the map. The FP32 map gives the increment to FP32 rounding, one
+// evaluation in pairs there and one Newton step with the FP32 Jacobian J, d + (I - J)^{-1} r =
+// G + M J r with r = G - d and M = (I - J)^{-1}, leave an error of |J| 2^-24 |r|, far below the
+// pairs' rounding of d. n_iter, tol: the method's iterations and what they have to come within
+// (inc_converges), else the method's iterations themselves are run, in pairs (LITERAL). h33:
+// h^33 u_3^2. Returns GEO_SMALL; GEO_LARGE where the increment is above INC_GEO, and the point
+// (n0, n1) whose image the result is to be; GEO_NONE: not resolved.
+enum { GEO_NONE = 0, GEO_SMALL, GEO_LARGE };
+template <bool LITERAL>
+__device__ __forceinline__ int geo_inc_solve(const GeoInc<DF> &m, float h33, int n_iter, float tol,
+                                             DF &n0, DF &n1) {
   const GeoInc<float> mf = {m.u0.hi,  m.u1.hi,  m.c0.hi,  m.c1.hi,  m.e1.hi,    m.e2.hi,   m.f1.hi,
                             m.f2.hi,  m.D1a.hi, m.D1b.hi, m.D2a.hi, m.D2b.hi,   m.hdt.hi,  m.H11.hi,
                             m.H22.hi, m.d1H11.hi, m.d1H22.hi, m.d2H11.hi, m.d2H22.hi};
@@ -247,22 +280,29 @@ __device__ __forceinline__ bool geo_inc_solve(const GeoInc<DF> &m, int n_iter, f
   n0 = n0 + DF(idet * fmaf(d, w0, J[0][1] * w1));
   n1 = n1 + DF(idet * fmaf(J[1][0], w0, a * w1));
   const float us = fmaxf(fabsf(m.u0.hi), fabsf(m.u1.hi));
-  const float ds = fmaxf(fabsf(n0.hi), fabsf(n1.hi));
   // (a NaN anywhere makes one of the comparisons false)
-  return fabsf(r0) + fabsf(r1) <= fmaf(0x1p-16f, ds, 0x1p-40f) &&
-         ds <= INC_MAX * fmaxf(1.0f, us) && inc_converges(first, J, n_iter, tol, us);
-}
-
-// du += the geodesic substep's increment from u; false: not resolved here
-__device__ __forceinline__ bool inc_geodesic(const GridP &g, const IncC &k, const Local<DF> &L,
-                                             const DF u[3], float m2, DF &du0, DF &du1) {
-  GeoInc<DF> m;
-  geo_inc_setup(k, L, u, m2, m);
-  DF n0, n1;
-  if (!geo_inc_solve(m, g.n_iter, g.f_iter_tol, n0, n1)) return false;
-  du0 = du0 + n0;
-  du1 = du1 + n1;
-  return true;
+  const float ds = fmaxf(fabsf(n0.hi), fabsf(n1.hi));
+  DF l0 = n0, l1 = n1;  // the iterate before the last
+  if (!(fabsf(r0) + fabsf(r1) <= fmaf(0x1p-16f, ds, 0x1p-40f) &&
+        inc_converges(first, J, n_iter, tol, us))) {
+    // (an iteration that does not contract amplifies the pairs' rounding as well as FP64's)
+    if (!LITERAL || !(spectral_radius(J) < 0.5f)) return GEO_NONE;
+    n0 = n1 = DF(0.0f);
+#pragma unroll 1
+    for (int it = 0; it < n_iter; ++it) {
+      l0 = n0;
+      l1 = n1;
+      geo_inc_apply(m, l0, l1, n0, n1);
+      if (n0.hi == l0.hi && n0.lo == l0.lo && n1.hi == l1.hi && n1.lo == l1.lo) break;
+    }
+  }
+  // the increment and the momentum as lengths in the tetrad frame, squared (h^13 aside)
+  const float dd = fmaf(mf.H11 * n0.hi, n0.hi, mf.H22 * n1.hi * n1.hi);
+  const float uu = fmaf(mf.u0, fmaf(mf.H11, mf.u0, mf.c1), fmaf(mf.H22 * mf.u1, mf.u1, h33));
+  if (dd <= INC_GEO * INC_GEO * fmaxf(uu, INC_UU)) return GEO_SMALL;
+  n0 = l0;
+  n1 = l1;
+  return dd < 0x1p60f ? GEO_LARGE : GEO_NONE;
 }
 
 // One Boris half step's increment of the covariant u, added to du (u = u^n + du in pairs):
@@ -288,14 +328,14 @@ __device__ __forceinline__ void inc_boris_core(const Local<M> &L, const R eD[3],
   du[1] = fma_(L.sh22, x[1], du[1]);
   du[2] = fma_(L.sh33, x[2], du[2]);
 }
-// False: the increment is above INC_MAX.
+// False: the increment is above INC_MAX of |u| (of 1/4, where |u| is less).
 __device__ __forceinline__ bool inc_boris(const Local<DF> &L, const DF eD[3], const DF eB[3],
                                           const DF u[3], DF du[3]) {
   DF h[3], x[3];
   inc_boris_core(L, eD, eB, u, du, h, x);
   const float xx = fmaf(x[0].hi, x[0].hi, fmaf(x[1].hi, x[1].hi, x[2].hi * x[2].hi));
   const float hh = fmaf(h[0].hi, h[0].hi, fmaf(h[1].hi, h[1].hi, h[2].hi * h[2].hi));
-  return xx <= INC_MAX * INC_MAX * fmaxf(1.0f, hh) && hh < 0x1p60f;
+  return xx <= INC_MAX * INC_MAX * fmaxf(hh, INC_UU) && hh < 0x1p60f;
 }
 
 // bilinear interpolation in pairs at the cell-relative offsets (o1, o2) of cell (i1, i2) for
@@ -348,17 +388,14 @@ __device__ __forceinline__ Vel<DF> inc_velocity(const IncC &k, DF r, DF s, DF c,
   return {fi * fma_(Gf, I, -(M2r * iS2)), Gf * kk, Gf * fma_(k.a, w0, z)};
 }
 
-// The FP64 evaluation of the map t -> dx + dt V((x^n + t)/2) that the result comes from: r
-// from the nearest corner's table, theta formed as map_theta forms it and its offset from the
-// corner's theta exact (as local_rsc), then inc_velocity's grouping: ~80 FP64 operations.
-__device__ __forceinline__ void inc_coord64(const GridP &g, const PushTables &tb, int i1, int i2,
-                                            double dx1, double dx2, const double u[3], double m2,
-                                            double t1, double t2, double &n1, double &n2,
-                                            double &v3) {
-  const double o1 = 0.5 * __dadd_rn(dx1, t1), o2 = 0.5 * __dadd_rn(dx2, t2);
+// r, sin(theta), cos(theta) in FP64 at offsets (o1, o2) of cell (i1, i2): r from the nearest
+// corner's table, theta formed as map_theta forms it and its offset from the corner's theta
+// exact (as local_rsc)
+__device__ __forceinline__ void inc_point64(const GridP &g, const PushTables &tb, int i1, int i2,
+                                            double o1, double o2, double &ex, double &s,
+                                            double &c) {
   const int c1 = gt_pos(o1, 0.5), c2 = gt_pos(o2, 0.5);
   const double e = (o1 - (c1 ? 1.0 : 0.0)) * g.dxi;
-  double ex;
   if (abs_le(e, (double)INC_E)) {
     double p = 1.0 / 40320.0;
     p = fma(p, e, 1.0 / 5040.0);
@@ -374,7 +411,6 @@ __device__ __forceinline__ void inc_coord64(const GridP &g, const PushTables &tb
   }
   const double th = __dmul_rn(__dadd_rn((double)i2, o2), g.dth);
   const double d = th - __ldg(tb.th64 + i2 + c2 + G_);
-  double s, c;
   if (abs_le(d, (double)INC_D)) {
     const double q = d * d;
     double sp = fma(-1.0 / 5040.0, q, 1.0 / 120.0);
@@ -390,6 +426,16 @@ __device__ __forceinline__ void inc_coord64(const GridP &g, const PushTables &tb
   } else {
     sincos(th, &s, &c);
   }
+}
+
+// The FP64 evaluation of the map t -> dx + dt V((x^n + t)/2) that the result comes from, in
+// inc_velocity's grouping: ~80 FP64 operations.
+__device__ __forceinline__ void inc_coord64(const GridP &g, const PushTables &tb, int i1, int i2,
+                                            double dx1, double dx2, const double u[3], double m2,
+                                            double t1, double t2, double &n1, double &n2,
+                                            double &v3) {
+  double ex, s, c;
+  inc_point64(g, tb, i1, i2, 0.5 * __dadd_rn(dx1, t1), 0.5 * __dadd_rn(dx2, t2), ex, s, c);
   const double s2 = s * s, r2 = ex * ex, f = g.dxi * ex;
   const double Sig = fma(g.a2, c * c, r2), M2r = g.M2 * ex, S2 = Sig + M2r;
   const double Rr = r2 + g.a2, A = fma(Rr, Rr, -(g.a2 * s2 * (Rr - M2r)));
@@ -469,6 +515,46 @@ __device__ __forceinline__ bool inc_coord(const GridP &g, const IncC &k, const P
   }
   const float scale = fmaxf(fabsf(f32_trunc(t1)), fabsf(f32_trunc(t2)));
   return conv && scale < 2.0f && inc_converges(first, J, n_iter, tol, scale);
+}
+
+// The coordinate substep in the two cell rows next to an axis, where the map (~1/sin^2(theta))
+// has more than one fixed point within reach: the method's iterations from x^n in pairs, then
+// FP64 evaluations from the point they settle at, until what is left is below 2^-55. False:
+// they do not settle within n_iter, or come near the small-angle clamp.
+__device__ __forceinline__ bool inc_coord_axis(const GridP &g, const IncC &k, const PushTables &tb,
+                                               int i1, int i2, double dx1, double dx2, DF o1,
+                                               DF o2, const double u[3], const DF ud[3], double m2,
+                                               float m2f, double &t1, double &t2, double &v3) {
+  DF p1 = o1, p2 = o2;
+  float d = 0.0f, d_prev = 1.0f;
+  bool settled = false;
+#pragma unroll 1
+  for (int it = 0; it < g.n_iter && !settled; ++it) {
+    DF r, s, c;
+    inc_point(k, tb, i1, i2, df_scale(o1 + p1, 0.5f), df_scale(o2 + p2, 0.5f), r, s, c);
+    if (!(s.hi > 2.0f * g.d_ss[0])) return false;
+    const Vel<DF> v = inc_velocity(k, r, s, c, ud, m2f);
+    const DF n1 = fma_(k.dt, v.v1, o1), n2 = fma_(k.dt, v.v2, o2);
+    if (it > 0) d_prev = d;
+    d = fmaxf(fabsf((n1 - p1).hi), fabsf((n2 - p2).hi));
+    p1 = n1;
+    p2 = n2;
+    settled = d <= 0x1p-44f;
+    if (!(fabsf(p1.hi - 0.5f) < 1.5f && fabsf(p2.hi - 0.5f) < 1.5f)) return false;
+  }
+  const float rate = fminf(fmaxf(d / d_prev, 0x1p-12f), 1.0f);  // the contraction, or above it
+  if (!settled || rate > 0.25f) return false;
+  double s1 = df_to_double(p1), s2 = df_to_double(p2);
+  const float stop = 0x1p-55f / rate;
+  bool conv = false;
+#pragma unroll 1
+  for (int it = 0; it < g.n_iter && !conv; ++it) {
+    inc_coord64(g, tb, i1, i2, dx1, dx2, u, m2, s1, s2, t1, t2, v3);
+    conv = converged(t1, s1, stop) && converged(t2, s2, stop);
+    s1 = t1;
+    s2 = t2;
+  }
+  return conv && fabsf(f32_trunc(t1)) < 2.0f && fabsf(f32_trunc(t2)) < 2.0f;
 }
 
 // floor of a pair

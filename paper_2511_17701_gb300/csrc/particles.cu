@@ -1234,33 +1234,99 @@ __device__ __forceinline__ int guard_zone(const PushTables &tb, const GridP &g, 
 // Bound by the FP64 pipe; on 67 M particles of the 2048^2 workload 3 resident blocks per SM
 // (166 registers, no spills) measured 85.4 ms per launch against 86.9 ms with 4 (128
 // registers, spills) and 89.3 ms with 5 (96 registers).
-// INC: the increment form (push_inc.cuh) for the particles it covers. A warp in which one
-// particle does not fit goes to push64 as a whole, so that no warp runs both for long.
-#ifndef GRPIC_PUSH64_MIN_BLOCKS  // resident blocks per SM the fused FP64 kernel is built for
+#ifndef GRPIC_PUSH64_MIN_BLOCKS  // resident blocks per SM the general FP64 kernels are built for
 #define GRPIC_PUSH64_MIN_BLOCKS 3
 #endif
-template <bool DEPOSIT, bool Q, bool INC>
+// step 1 of particle k; whether it is to be pushed
+__device__ __forceinline__ bool push_begin(const SpeciesDevT<double> &s, int64_t k) {
+  if (s.i1p) {  // the previous position, when a later call reads it
+    s.i1p[k] = s.i1[k]; s.i2p[k] = s.i2[k]; s.dx1p[k] = s.dx1[k]; s.dx2p[k] = s.dx2[k];
+  }
+  const uint8_t tag = s.tag[k];
+  if (tag != 1 && tag != 0) s.tag[k] = 0;
+  return tag == 1;
+}
+template <bool DEPOSIT, bool Q>
 __global__ void __launch_bounds__(TPB, GRPIC_PUSH64_MIN_BLOCKS)
     k_push(GridP g, FieldPtrsT<double> F, PushTables tb, SpeciesDevT<double> s,
            unsigned long long *diag) {
   const int64_t n = *s.n;
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
+       k += (int64_t)gridDim.x * blockDim.x)
+    if (push_begin(s, k)) push64<Q, DEPOSIT>(g, F, tb, s, k, diag);
+}
+
+// The increment form (push_inc.cuh) for the particles it covers; the rest are marked by the
+// tag TAG_REST, which lives from this kernel to k_push_rest right behind it. Two kernels, so
+// that this one runs with the registers of its own code (128, 4 blocks per SM; with push64 in
+// it, 166 and 3) and the long routine with full warps: a step of the 2048^2 workload 80.3 ->
+// 65.9 ms, of the 512^2 one 11.0 -> 8.85 ms, of the 512^2 monopole problem, whose Boris half
+// steps are taken in FP64, 5.94 -> 4.18 ms. What bounds it: 124 FP64 instructions and ~7500
+// others per warp overlap to about half of either pipe's peak; between them warps wait for FP64
+// results, for instructions (the code is 14,000 instructions) and for their own pair arithmetic.
+// 5 and 6 blocks per SM (96, 80 registers) measured within 1% of 4.
+constexpr uint8_t TAG_REST = 3;
+#ifndef GRPIC_PUSH_INC_MIN_BLOCKS
+#define GRPIC_PUSH_INC_MIN_BLOCKS 4
+#endif
+template <bool DEPOSIT>
+__global__ void __launch_bounds__(TPB, GRPIC_PUSH_INC_MIN_BLOCKS)
+    k_push_inc(GridP g, FieldPtrsT<double> F, PushTables tb, SpeciesDevT<double> s,
+               unsigned long long *diag) {
+  const int64_t n = *s.n;
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
        k += (int64_t)gridDim.x * blockDim.x) {
-    if (s.i1p) {  // step 1: the previous position, when a later call reads it
-      s.i1p[k] = s.i1[k]; s.i2p[k] = s.i2[k]; s.dx1p[k] = s.dx1[k]; s.dx2p[k] = s.dx2[k];
+    if (!push_begin(s, k)) continue;
+    if (!push_inc<DEPOSIT>(g, F, tb, s, k, diag)) s.tag[k] = TAG_REST;
+  }
+}
+// push64 for the marked particles: each warp scans REST_U x 32 tags and gathers the marked
+// indices, so that the long routine runs with full warps however thinly they are spread. One
+// tag per lane in small runs, which have too few warps to share.
+template <bool DEPOSIT, int REST_U>
+__global__ void __launch_bounds__(TPB, GRPIC_PUSH64_MIN_BLOCKS)
+    k_push_rest(GridP g, FieldPtrsT<double> F, PushTables tb, SpeciesDevT<double> s,
+                unsigned long long *diag) {
+  constexpr unsigned FULL = 0xffffffffu;
+  __shared__ uint32_t queue[TPB / 32][32 * (REST_U + 1)];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t n = *s.n;
+  uint32_t *q = queue[w];
+  int qn = 0;  // marked particles waiting, below 32 at the top of the loop
+  const int64_t stride = (int64_t)gridDim.x * TPB * REST_U;
+  for (int64_t base = (blockIdx.x * (int64_t)(TPB / 32) + w) * 32 * REST_U;; base += stride) {
+    const bool more = base < n;
+    if (more) {
+      uint8_t tag[REST_U];
+#pragma unroll
+      for (int u = 0; u < REST_U; ++u) {
+        const int64_t k = base + u * 32 + lane;
+        tag[u] = k < n ? s.tag[k] : 0;
+      }
+#pragma unroll
+      for (int u = 0; u < REST_U; ++u) {
+        const unsigned m = __ballot_sync(FULL, tag[u] == TAG_REST);
+        if (tag[u] == TAG_REST)
+          q[qn + __popc(m & ((1u << lane) - 1u))] = (uint32_t)(base + u * 32 + lane);
+        qn += __popc(m);
+      }
     }
-    const uint8_t tag = s.tag[k];
-    if (tag != 1) {
-      if (tag != 0) s.tag[k] = 0;
-      continue;
+    __syncwarp();
+    while (qn >= 32 || (!more && qn > 0)) {
+      const int take = min(qn, 32);
+      qn -= take;
+      if (lane < take) {
+        const int64_t k = q[qn + lane];
+        s.tag[k] = 1;
+        push64<false, DEPOSIT>(g, F, tb, s, k, diag);
+      }
+      __syncwarp();
     }
-    if (INC && __all_sync(__activemask(), inc_fit(g, F, tb, s, k)) &&
-        push_inc<DEPOSIT>(g, F, tb, s, k, diag))
-      continue;
-    push64<Q, DEPOSIT>(g, F, tb, s, k, diag);
+    if (!more) break;
   }
 }
 
+constexpr int64_t APART_MAX = 1 << 18;
 // Whether a run's FP64 pushes may take the increment form: the refined iterations on the
 // plain grid, with rows away from the axes clear of the small-angle clamp.
 bool inc_applies(const GridP &g) {
@@ -1731,16 +1797,40 @@ cudaError_t push_impl(const GridP &g, const FieldPtrsT<T> &F, SpeciesDevT<T> s,
   }
   if constexpr (sizeof(T) == 8) {
     if (!main_stage) return cudaSuccess;  // the FP64 path has no guard stage
-    if (ps.t0) cudaEventRecord(ps.t0, ps.main);
+    // a push of fewer warps than the GPU holds runs beside that of the species before it: on
+    // 64^2 cells (1024 warps a species) the two took 2 x 95 us one behind the other
+    cudaStream_t st = ps.main;
+    if (ps.apart && n_bound < APART_MAX) {
+      cudaError_t e;
+      st = ps.side;
+      if ((e = cudaEventRecord(ps.fork, ps.main)) != cudaSuccess) return e;
+      if ((e = cudaStreamWaitEvent(st, ps.fork, 0)) != cudaSuccess) return e;
+    }
+    if (ps.t0) cudaEventRecord(ps.t0, st);
     const int b = blocks_for(n_bound);
     if (!Q && inc_applies(g)) {
-      if (deposit) k_push<true, false, true><<<b, TPB, 0, ps.main>>>(g, F, tb, s, diag);
-      else k_push<false, false, true><<<b, TPB, 0, ps.main>>>(g, F, tb, s, diag);
+      const bool small = n_bound < (1 << 19);
+      const int br = blocks_for(small ? n_bound : (n_bound + 7) / 8);
+      if (deposit) {
+        k_push_inc<true><<<b, TPB, 0, st>>>(g, F, tb, s, diag);
+        if (small) k_push_rest<true, 1><<<br, TPB, 0, st>>>(g, F, tb, s, diag);
+        else k_push_rest<true, 8><<<br, TPB, 0, st>>>(g, F, tb, s, diag);
+      } else {
+        k_push_inc<false><<<b, TPB, 0, st>>>(g, F, tb, s, diag);
+        if (small) k_push_rest<false, 1><<<br, TPB, 0, st>>>(g, F, tb, s, diag);
+        else k_push_rest<false, 8><<<br, TPB, 0, st>>>(g, F, tb, s, diag);
+      }
+      COUNT_LAUNCH(1);
+    } else if (deposit) {
+      k_push<true, Q><<<b, TPB, 0, st>>>(g, F, tb, s, diag);
     } else {
-      if (deposit) k_push<true, Q, false><<<b, TPB, 0, ps.main>>>(g, F, tb, s, diag);
-      else k_push<false, Q, false><<<b, TPB, 0, ps.main>>>(g, F, tb, s, diag);
+      k_push<false, Q><<<b, TPB, 0, st>>>(g, F, tb, s, diag);
     }
-    if (ps.t1) cudaEventRecord(ps.t1, ps.main);
+    if (ps.t1) cudaEventRecord(ps.t1, st);
+    if (st != ps.main) {
+      const cudaError_t e = cudaEventRecord(ps.done, st);
+      if (e != cudaSuccess) return e;
+    }
     COUNT_LAUNCH(1);
   } else {
     cudaError_t e;

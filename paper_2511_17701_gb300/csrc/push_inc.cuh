@@ -5,8 +5,9 @@
 
 namespace {
 
-// An FP32 estimate of whether a Boris half step stays below INC_MAX (fields of one node, no
-// interpolation): where it does not, the warp goes to push64 at once. Only speed depends on it.
+// An FP32 estimate of whether a Boris half step stays below INC_MAX for a momentum of order 1
+// (fields of one node, no interpolation): where it does not, the warp takes both half steps in
+// FP64 at once. Only speed depends on it.
 __device__ __forceinline__ bool inc_small(const GridP &g, const FieldPtrsT<double> &F,
                                           const PushTables &tb, int i1, int i2, float f_qm) {
   const float r = __ldg(tb.r + i1 + G_), s = __ldg(tb.s + i2 + G_), c = __ldg(tb.c + i2 + G_);
@@ -25,14 +26,66 @@ __device__ __forceinline__ bool inc_small(const GridP &g, const FieldPtrsT<doubl
   return e * e * (BB + DD) <= INC_MAX * INC_MAX;
 }
 
-// Whether a particle is likely to take the increment form: off the axis rows (where the
-// refined iterations do not apply either), and with small increments.
-__device__ __forceinline__ bool inc_fit(const GridP &g, const FieldPtrsT<double> &F,
-                                        const PushTables &tb, const SpeciesDevT<double> &s,
-                                        int64_t kp) {
-  const int i1 = s.i1[kp], i2 = s.i2[kp];
-  return i2 >= 2 && i2 < g.n_th - 2 && i1 >= 0 && i1 < g.n_r &&
-         (s.m2 == 0.0 || inc_small(g, F, tb, i1, i2, s.f_qm));
+// The tetrad, the fields in it and the Boris half steps in FP64, for strong fields
+struct Strong {
+  double rH11, sH11, rh22, sh22, rh33, sh33, k13, m13, eB[3], eD[3];
+};
+__device__ __forceinline__ void strong_frame(const GridP &g, const FieldPtrsT<double> &F,
+                                             const PushTables &tb, int i1, int i2, double dx1,
+                                             double dx2, double qm, Strong &w) {
+  double r, s, c;
+  inc_point64(g, tb, i1, i2, dx1, dx2, r, s, c);
+  const double s2 = s * s, r2 = r * r, f = g.dxi * r;
+  const double Sig = fma(g.a2, c * c, r2), M2r = g.M2 * r, S2 = Sig + M2r;
+  const double Rr = r2 + g.a2, A = fma(Rr, Rr, -(g.a2 * s2 * (Rr - M2r)));
+  const double rSig = rsqrt(Sig), rS2 = rsqrt(S2), rA = rsqrt(A);
+  const double ifs = rcp_nr(f * s), qSig = Sig * rSig, qA = A * rA;
+  w.rH11 = f * qSig * (S2 * rS2) * rA;
+  w.sH11 = ifs * s * (rSig * rS2) * qA;
+  w.rh22 = rSig * (g.ig2 * g.dth);
+  w.sh22 = qSig * g.dth;
+  w.rh33 = qSig * rA * (ifs * f);
+  w.sh33 = s * rSig * qA;
+  const double faS = f * g.a * S2;
+  w.k13 = -(faS * (s * rSig) * rA);
+  w.m13 = -(faS * (rA * rA));
+  const double e = 0.25 * qm * (qSig * rS2) * g.dt;  // half of qm alpha dt/2
+  const bool l1 = lt_pos(dx1, 0.5) || dx1 == 0.0, l2 = lt_pos(dx2, 0.5) || dx2 == 0.0;
+  const double w1[2] = {dx1, l1 ? dx1 + 0.5 : dx1 - 0.5}, w2[2] = {dx2, l2 ? dx2 + 0.5 : dx2 - 0.5};
+  double V[6];
+#pragma unroll 1
+  for (int q = 0; q < 6; ++q) {  // one copy of the code: see push_inc
+    const int h1 = q == 1 || q == 2 || q == 3, h2 = q == 0 || q == 2 || q == 4;
+    const double *pl = q < 3 ? F.Bn[q] : F.D[q - 3];
+    const double *p = pl + sidx(g, i1 - (h1 && l1 ? 1 : 0), i2 - (h2 && l2 ? 1 : 0));
+    const double p00 = __ldg(p), p10 = __ldg(p + 1), p01 = __ldg(p + g.NX), p11 = __ldg(p + g.NX + 1);
+    const double a1 = h1 ? w1[1] : w1[0], a2 = h2 ? w2[1] : w2[0];
+    const double x = fma(a1, p10 - p00, p00), y = fma(a1, p11 - p01, p01);
+    V[q] = fma(a2, y - x, x);
+  }
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const double *v = V + 3 * q;
+    double *o = q ? w.eD : w.eB;
+    o[0] = e * (v[0] * w.rH11);
+    o[1] = e * (w.sh22 * v[1]);
+    o[2] = e * fma(w.k13, v[0], w.sh33 * v[2]);
+  }
+}
+__device__ __forceinline__ void strong_boris(const Strong &w, double u[3]) {
+  const double m0 = fma(w.sH11, fma(-w.m13, u[2], u[0]), w.eD[0]);
+  const double m1 = fma(w.rh22, u[1], w.eD[1]), m2 = fma(w.rh33, u[2], w.eD[2]);
+  const double ig = rsqrt(fma(m0, m0, fma(m1, m1, fma(m2, m2, 1.0))));
+  const double t0 = w.eB[0] * ig, t1 = w.eB[1] * ig, t2 = w.eB[2] * ig;
+  const double sf = 2.0 * rcp_nr(fma(t0, t0, fma(t1, t1, fma(t2, t2, 1.0))));
+  const double p0 = fma(m1, t2, fma(-m2, t1, m0)), p1 = fma(m2, t0, fma(-m0, t2, m1));
+  const double p2 = fma(m0, t1, fma(-m1, t0, m2));
+  const double h0 = fma(sf, fma(p1, t2, -(p2 * t1)), m0 + w.eD[0]);
+  const double h1 = fma(sf, fma(p2, t0, -(p0 * t2)), m1 + w.eD[1]);
+  const double h2 = fma(sf, fma(p0, t1, -(p1 * t0)), m2 + w.eD[2]);
+  u[0] = fma(h0, w.rH11, w.k13 * h2);
+  u[1] = w.sh22 * h1;
+  u[2] = w.sh33 * h2;
 }
 
 // floor of t in (-2, 2), on the integer pipe
@@ -43,73 +96,196 @@ __device__ __forceinline__ int inc_cell(double t) {
   return a == 0 ? 0 : (a > one ? -2 : -1);
 }
 
-// One particle (inc_fit) in the increment form; false: nothing stored, push64 has to take it.
+// deposit64 in pairs, relative to the start cell: the end points a, b are the positions as
+// deposit64 rounds them (absolute coordinates: a multiple of their last place, at most 48
+// bits, so a pair holds them exactly), the rest of its ~70 FP64 operations is in pairs. The
+// pairs' 2^-47 is below that rounding's share of a move. (i, j): the start cell, (c1, c2): the
+// end cell relative to it.
+__device__ __forceinline__ void inc_deposit(const GridP &g, const FieldPtrsT<double> &F, DF q,
+                                            DF idt, int i, int j, DF a1, DF a2, int c1, int c2,
+                                            DF b1, DF b2, DF v3) {
+  const int NX = g.NX;
+  const DF qi = q * idt;
+  const DF m1 = df_scale(a1 + b1, 0.5f), m2 = df_scale(a2 + b2, 0.5f);
+  // the relay point: the midpoint clamped to the two cells' common range
+  const DF r1 = c1 == 0 ? m1 : DF(c1 > 0 ? 1.0f : (float)(c1 + 1));
+  const DF r2 = c2 == 0 ? m2 : DF(c2 > 0 ? 1.0f : (float)(c2 + 1));
+  const int64_t ka = sidx(g, i, j), kb = sidx(g, i + c1, j + c2);
+  double *J1 = F.J[0], *J2 = F.J[1], *J3 = F.J[2];
+  {
+    const DF F1 = qi * (r1 - a1), F2 = qi * (r2 - a2);
+    const DF t = F1 * df_scale(a2 + r2, 0.5f), s = F2 * df_scale(a1 + r1, 0.5f);
+    atomicAdd(J1 + ka, df_to_double(F1 - t));
+    atomicAdd(J1 + ka + NX, df_to_double(t));
+    atomicAdd(J2 + ka, df_to_double(F2 - s));
+    atomicAdd(J2 + ka + 1, df_to_double(s));
+  }
+  {
+    const DF F1 = qi * (b1 - r1), F2 = qi * (b2 - r2);
+    const DF t = F1 * (df_scale(r2 + b2, 0.5f) + DF(-(float)c2));
+    const DF s = F2 * (df_scale(r1 + b1, 0.5f) + DF(-(float)c1));
+    atomicAdd(J1 + kb, df_to_double(F1 - t));
+    atomicAdd(J1 + kb + NX, df_to_double(t));
+    atomicAdd(J2 + kb, df_to_double(F2 - s));
+    atomicAdd(J2 + kb + 1, df_to_double(s));
+  }
+  const int n1 = inc_floor(m1), n2 = inc_floor(m2);
+  const DF w1 = m1 + DF(-(float)n1), w2 = m2 + DF(-(float)n2);
+  const int64_t k = sidx(g, i + n1, j + n2);
+  const DF qv = q * v3, x = qv * w1, y = qv - x;
+  const DF xt = x * w2, yt = y * w2;
+  atomicAdd(J3 + k, df_to_double(y - yt));
+  atomicAdd(J3 + k + 1, df_to_double(x - xt));
+  atomicAdd(J3 + k + NX, df_to_double(yt));
+  atomicAdd(J3 + k + NX + 1, df_to_double(xt));
+}
+
+// The geodesic substep's increment (d0, d1) from u in FP64, where it is large against u (next to
+// the axes, where the metric changes by order one over a step): the FP64 map's image of the
+// point that the pairs found
+__device__ __forceinline__ void strong_geodesic(const GridP &g, const PushTables &tb, int i1,
+                                                int i2, double dx1, double dx2, double m2,
+                                                DF d0, DF d1, double u[3]) {
+  Pt<double> p;
+  inc_point64(g, tb, i1, i2, dx1, dx2, p.r, p.s, p.c);
+  p.f = g.dxi * p.r;
+  p.gg = g.dth;
+  p.igg = g.ig2;
+  p.gp = 0.0;
+  Local<double> L;
+  local_full<false>(g, p, L, false);
+  const GeoMap<double> m(g, L, u, m2);
+  m.apply(u[0] + df_to_double(d0), u[1] + df_to_double(d1), u[0], u[1]);
+}
+
+// One particle in the increment form; false: nothing stored, push64 has to take it. Loops that
+// the compiler would unroll stay loops: the code is straight-line and long, and warps waited
+// for its instructions (17% of their time with every copy unrolled).
 template <bool DEPOSIT>
 __device__ __forceinline__ bool push_inc(const GridP &g, const FieldPtrsT<double> &F,
                                          const PushTables &tb, const SpeciesDevT<double> &s,
                                          int64_t kp, unsigned long long *diag) {
   const int i1 = s.i1[kp], i2 = s.i2[kp];
-  const bool em = s.m2 != 0.0;
+  if (!(i2 >= 0 && i2 < g.n_th && i1 >= 0 && i1 < g.n_r)) return false;
+  const bool em = s.m2 != 0.0, axis = i2 < 2 || i2 >= g.n_th - 2;
   const double dx1 = s.dx1[kp], dx2 = s.dx2[kp];
   const IncC k = inc_c(g);
   const DF o1 = df_of(dx1), o2 = df_of(dx2);
-  const double u64[3] = {s.u1[kp], s.u2[kp], s.u3[kp]};
-  const DF u[3] = {df_of(u64[0]), df_of(u64[1]), df_of(u64[2])};
-  DF du[3] = {DF(0.0f), DF(0.0f), DF(0.0f)};
+  double un[3] = {s.u1[kp], s.u2[kp], s.u3[kp]};
+  DF ud[3] = {df_of(un[0]), df_of(un[1]), df_of(un[2])};
   {
+    const DF u[3] = {ud[0], ud[1], ud[2]};
+    DF du[3] = {DF(0.0f), DF(0.0f), DF(0.0f)};
     Local<DF> L;
     {
       DF r, sn, cs;
-      if (!inc_point(k, tb, i1, i2, o1, o2, r, sn, cs)) return false;
+      if (!inc_point_n(g, k, tb, i1, i2, dx2, o1, o2, r, sn, cs) || !(sn.hi > 2.0f * g.d_ss[0])) return false;
       inc_local(k, r, sn, cs, L);
     }
     DF eD[3], eB[3];
-    if (em) {
+    Strong w;
+    bool weak = !em || __all_sync(__activemask(), inc_small(g, F, tb, i1, i2, s.f_qm));
+    if (em && weak) {
       IncLerp l;
       inc_lerp(i1, i2, o1, o2, l);
       const DF e = df_scale(df_of(s.qm) * L.alpha * k.dt, 0.25f);  // half of qm alpha dt/2
-      DF V[3] = {inc_interp(F.Bn[0], g.NX, l, 0, 1), inc_interp(F.Bn[1], g.NX, l, 1, 0),
-                 inc_interp(F.Bn[2], g.NX, l, 1, 1)};
+      DF V[6];
+#pragma unroll 1
+      for (int q = 0; q < 6; ++q) {
+        const int h1 = q == 1 || q == 2 || q == 3, h2 = q == 0 || q == 2 || q == 4;
+        V[q] = inc_interp(q < 3 ? F.Bn[q] : F.D[q - 3], g.NX, l, h1, h2);
+      }
       vec_hat(L, V, eB);
-      V[0] = inc_interp(F.D[0], g.NX, l, 1, 0);
-      V[1] = inc_interp(F.D[1], g.NX, l, 0, 1);
-      V[2] = inc_interp(F.D[2], g.NX, l, 0, 0);
-      vec_hat(L, V, eD);
+      vec_hat(L, V + 3, eD);
 #pragma unroll
       for (int q = 0; q < 3; ++q) {
         eB[q] = e * eB[q];
         eD[q] = e * eD[q];
       }
-      if (!inc_boris(L, eD, eB, u, du)) return false;
+      weak = inc_boris(L, eD, eB, u, du);
     }
-    const float m2f = em ? 1.0f : 0.0f;
-    DF un[3] = {u[0] + du[0], u[1] + du[1], u[2] + du[2]};
-    if (!inc_geodesic(g, k, L, un, m2f, du[0], du[1])) return false;
-    if (em) {
-      un[0] = u[0] + du[0];
-      un[1] = u[1] + du[1];
-      if (!inc_boris(L, eD, eB, un, du)) return false;
+    if (!weak) {
+      strong_frame(g, F, tb, i1, i2, dx1, dx2, s.qm, w);
+      strong_boris(w, un);
+#pragma unroll
+      for (int q = 0; q < 3; ++q) ud[q] = df_of(un[q]);
+      du[0] = du[1] = du[2] = DF(0.0f);
+    } else {
+#pragma unroll
+      for (int q = 0; q < 3; ++q) ud[q] = u[q] + du[q];
     }
+    {
+      GeoInc<DF> m;
+      geo_inc_setup(k, L, ud, em ? 1.0f : 0.0f, m);
+      DF d0, d1;
+      // in the axis rows the result is the method's to rounding, as push64's is there
+      const int found = geo_inc_solve<true>(m, L.G.H33.hi * ud[2].hi * ud[2].hi, g.n_iter,
+                                            axis ? 0x1p-54f : g.f_iter_tol, d0, d1);
+      if (found == GEO_NONE) return false;
+      if (found == GEO_LARGE) {
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          un[q] += df_to_double(du[q]);
+          du[q] = DF(0.0f);
+        }
+        strong_geodesic(g, tb, i1, i2, dx1, dx2, s.m2, d0, d1, un);
+      } else {
+        du[0] = du[0] + d0;
+        du[1] = du[1] + d1;
+      }
+    }
+    if (em && weak) {
+#pragma unroll
+      for (int q = 0; q < 3; ++q) ud[q] = df_of(un[q]) + du[q];
+      if (!inc_boris(L, eD, eB, ud, du)) return false;
+    }
+#pragma unroll
+    for (int q = 0; q < 3; ++q) un[q] += df_to_double(du[q]);
+    if (!weak) strong_boris(w, un);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) ud[q] = df_of(un[q]);
   }
-  const double un[3] = {u64[0] + df_to_double(du[0]), u64[1] + df_to_double(du[1]),
-                        u64[2] + df_to_double(du[2])};
-  const DF ud[3] = {u[0] + du[0], u[1] + du[1], u[2] + du[2]};
   double t1, t2, v3;
-  if (!inc_coord<false>(g, k, tb, g.n_iter, g.f_iter_tol, i1, i2, dx1, dx2, o1, o2, un, ud, s.m2,
-                        em ? 1.0f : 0.0f, t1, t2, v3))
+  const float m2f = em ? 1.0f : 0.0f;
+  if (axis) {
+    if (!inc_coord_axis(g, k, tb, i1, i2, dx1, dx2, o1, o2, un, ud, s.m2, m2f, t1, t2, v3))
+      return false;
+  } else if (!inc_coord<false>(g, k, tb, g.n_iter, g.f_iter_tol, i1, i2, dx1, dx2, o1, o2, un, ud,
+                               s.m2, m2f, t1, t2, v3)) {
     return false;
+  }
   if (!(finite64(un[0]) && finite64(un[1]) && finite64(un[2]))) return false;
-  const int c1 = inc_cell(t1), c2 = inc_cell(t2);
-  const int j1 = i1 + c1, j2 = i2 + c2;
-  if (j2 < 0 || j2 >= g.n_th) return false;
-  const double e1 = t1 - (double)c1, e2 = t2 - (double)c2;
+  const int c1 = inc_cell(t1);
+  int c2 = inc_cell(t2);
+  const int j1 = i1 + c1;
+  int j2 = i2 + c2;
+  const double e1 = t1 - (double)c1;
+  double e2 = t2 - (double)c2;
+  if (j2 < 0 || j2 >= g.n_th) {  // reflection off an axis (Sec. 3.3.3)
+    j2 = j2 < 0 ? 0 : g.n_th - 1;
+    e2 = 1.0 - e2;
+    c2 = j2 - i2;
+    un[1] = -un[1];
+    // dphi/dt at the midpoint of x^n and the reflected x^{n+1}, clear of the small-angle clamp
+    const double b2 = (double)c2 + e2;
+    const float mid = 0.5f * (f32_trunc(dx2) + f32_trunc(b2)) + (float)(j2 == 0 ? i2 : i2 + 1 - g.n_th);
+    if (!axis || fabsf(mid - (j2 == 0 ? 0.0f : 1.0f)) * g.f_dth < 2.0f * g.d_ss[0]) return false;
+    double n1, n2;
+    inc_coord64(g, tb, i1, i2, dx1, dx2, un, s.m2, t1, b2, n1, n2, v3);
+    count(diag, DG_REFLECT);
+  }
   s.i1[kp] = j1; s.i2[kp] = j2; s.dx1[kp] = e1; s.dx2[kp] = e2;
   s.u1[kp] = un[0]; s.u2[kp] = un[1]; s.u3[kp] = un[2];
   if (j1 < 0) { s.tag[kp] = 2; count(diag, DG_LEFT_INNER); }
   else if (j1 >= g.n_r) { s.tag[kp] = 2; count(diag, DG_LEFT_OUTER); }
   s.phi[kp] = s.phi[kp] + g.dt * v3;
-  if (DEPOSIT)
-    deposit64(g, F, s.qc * s.w[kp], i1, i2, i1 + dx1, i2 + dx2, j1, j2, j1 + e1, j2 + e2, v3);
+  if (DEPOSIT) {
+    const double p1 = i1, p2 = i2;
+    inc_deposit(g, F, df_of(s.qc * s.w[kp]), df_of(g.idt), i1, i2,
+                df_of(__dadd_rn(__dadd_rn(p1, dx1), -p1)), df_of(__dadd_rn(__dadd_rn(p2, dx2), -p2)),
+                c1, c2, df_of(__dadd_rn(__dadd_rn((double)j1, e1), -p1)),
+                df_of(__dadd_rn(__dadd_rn((double)j2, e2), -p2)), df_of(v3));
+  }
   return true;
 }
 

@@ -67,3 +67,29 @@ def test_push_against_oracle(torch_cuda, over, qm, massless):
     osim.push(0)
     g.push(0)
     assert_particles(g.get_particles(0), osim.species[0].view())
+
+
+def test_gathered_rest_gives_the_same_bits(torch_cuda):
+    """Particles that the increment form leaves to the general routine are gathered over more
+    particles per warp in large pushes than in small ones; a particle's result depends on
+    neither: one push of 2^19 + 777 particles, and the same in pieces below 2^19."""
+    from paper_2511_17701_gb300 import FIELD_WALD, Sim
+    cfg = W.grid_config("wald64", n_r=96, n_theta=96, iter_tol=1e-12, sort_every=0)
+    n = (1 << 19) + 777
+    pos, uh = particles(cfg, False, n, 21)
+    w0 = 0.1 * np.ones(n)
+
+    def push(sel):
+        g = Sim(cfg, [len(w0[sel])])
+        g.init_metric()
+        g.init_fields(FIELD_WALD, 1.0)
+        g.load_particles(0, {k: v[sel] for k, v in pos.items()}, uh[:, sel], w0[sel], 3.0, 0.2)
+        g.push(0)
+        return g.get_particles(0)
+
+    whole = push(slice(0, n))
+    for a in range(0, n, 200001):
+        sel = slice(a, min(n, a + 200001))
+        part = push(sel)
+        for k in ("i1", "i2", "dx1", "dx2", "u1", "u2", "u3", "phi", "tag"):
+            assert np.array_equal(part[k], whole[k][sel]), k
