@@ -331,9 +331,9 @@ __device__ __noinline__ void step_jacobian(const GridP &g, const FieldPtrsT<doub
 // per particle-step forward, ~5500 backward, most of them exp and sincos per iterate and the
 // metric's derivatives in duals); here FP64 is left with one or two evaluations of the
 // coordinate map and the additions to the state. 65,536 orbits on 512^2, 100 steps forward and
-// back: 106.3 -> 28.1 ms, the gradients' error against FP64 references 1.2e-14 -> 1.1e-14. The
-// backward kernel is bound by the latency of its pair arithmetic at 8 warps per SM (255
-// registers, spills).
+// back: 107 -> 29 ms, the gradients' error against FP64 references as before (4.3e-15, 4.2e-15).
+// The backward kernel waits for instructions and for its pair arithmetic at 8 warps per SM
+// (255 registers, spills).
 // ---------------------------------------------------------------------------------
 constexpr int INC_MIN_ITER = 16;   // iteration counts below are taken literally (general form)
 constexpr float INC_ADJ_TOL = 1e-16f;
@@ -367,12 +367,11 @@ __device__ __forceinline__ bool adj_inc_step(const GridP &g, const FieldPtrsT<do
   inc_local(k, a.r, a.s, a.c, a.L);
   IncLerp l;
   inc_lerp(a.i1, a.i2, a.o1, a.o2, l);
-  a.V[0] = inc_interp(F.B[0], g.NX, l, 0, 1);
-  a.V[1] = inc_interp(F.B[1], g.NX, l, 1, 0);
-  a.V[2] = inc_interp(F.B[2], g.NX, l, 1, 1);
-  a.V[3] = inc_interp(F.D[0], g.NX, l, 1, 0);
-  a.V[4] = inc_interp(F.D[1], g.NX, l, 0, 1);
-  a.V[5] = inc_interp(F.D[2], g.NX, l, 0, 0);
+#pragma unroll 1
+  for (int q = 0; q < 6; ++q) {
+    const int h1 = q == 1 || q == 2 || q == 3, h2 = q == 0 || q == 2 || q == 4;
+    a.V[q] = inc_interp(q < 3 ? F.B[q] : F.D[q - 3], g.NX, l, h1, h2);
+  }
   vec_hat(a.L, a.V, a.eB1);
   vec_hat(a.L, a.V + 3, a.eD1);
   const DF e = df_scale(qm * a.L.alpha * k.dt, 0.25f);
@@ -426,19 +425,20 @@ __device__ __forceinline__ D2F adj_interp_d(const double *__restrict__ pl, int N
   return D2F(V, fma_(l.w2[h2], xy, x0), fma_(l.w1[h1], xy, y0));
 }
 
-// The momentum's derivative along two directions: du' of u^{n+1} - u^n for metric values L
-// (M: DF, or D2F where the directions move x^n), u and the fields with their derivatives.
-// K: the geodesic substep's (I - A)^{-1}; G3 = its map's derivative with respect to u_3.
-template <typename M>
-__device__ __forceinline__ void adj_momentum_d(const IncC &k, const Local<M> &L, const D2F eD[3],
+// The momentum's derivative along two directions: du' of u^{n+1} - u^n for metric values L, u
+// and the fields with their derivatives. K: the geodesic substep's (I - A)^{-1}.
+__device__ __forceinline__ void adj_momentum_d(const IncC &k, const Local<D2F> &L, const D2F eD[3],
                                                const D2F eB[3], const D2F u[3], const AdjStep &a,
                                                const DF K[2][2], D2F du[3]) {
-  D2F h[3], x[3];
+  D2F h[3], x[3], v[3] = {u[0], u[1], u[2]};
 #pragma unroll
   for (int q = 0; q < 3; ++q) du[q] = D2F(0.0f);
-  inc_boris_core(L, eD, eB, u, du, h, x);
-  D2F v[3] = {u[0] + du[0], u[1] + du[1], u[2] + du[2]};
-  {
+#pragma unroll 1
+  for (int half = 0;; ++half) {
+    inc_boris_core(L, eD, eB, v, du, h, x);
+    if (half) return;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) v[q] = D2F(a.u1[q], u[q].d0 + du[q].d0, u[q].d1 + du[q].d1);
     GeoInc<D2F> m;
     geo_inc_setup(k, L, v, 1.0f, m);
     D2F n0, n1;
@@ -448,10 +448,9 @@ __device__ __forceinline__ void adj_momentum_d(const IncC &k, const Local<M> &L,
     du[0].d1 = du[0].d1 + fma_(K[0][0], n0.d1, K[0][1] * n1.d1);
     du[1].d0 = du[1].d0 + fma_(K[1][0], n0.d0, K[1][1] * n1.d0);
     du[1].d1 = du[1].d1 + fma_(K[1][0], n0.d1, K[1][1] * n1.d1);
-  }
 #pragma unroll
-  for (int q = 0; q < 3; ++q) v[q] = D2F(a.u2[q], u[q].d0 + du[q].d0, u[q].d1 + du[q].d1);
-  inc_boris_core(L, eD, eB, v, du, h, x);
+    for (int q = 0; q < 3; ++q) v[q] = D2F(a.u2[q], u[q].d0 + du[q].d0, u[q].d1 + du[q].d1);
+  }
 }
 
 // (I - A)^{-1}
@@ -518,71 +517,74 @@ __device__ __forceinline__ void adj_inc_jacobian(const GridP &g, const FieldPtrs
     geo_inc_jacobian(m, a.dg[0], a.dg[1], A);
     adj_inv(A, K);
   }
-  // a column: the increments' derivatives from that of u^{n+1} (seed + du') and x^n (xs)
-  auto column = [&](int col, const DF du[3], const DF seed[3], DF xs0, DF xs1) {
-    const DF p0 = seed[0] + du[0], p1 = seed[1] + du[1], p2 = seed[2] + du[2];
-    DF v[3];
-#pragma unroll
-    for (int q = 0; q < 3; ++q)
-      v[q] = fma_(Vu[q][0], p0, fma_(Vu[q][1], p1, fma_(Vu[q][2], p2, fma_(Vx[q][0], xs0, Vx[q][1] * xs1))));
-    const DF y0 = k.dt * fma_(Mx[0][0], v[0], Mx[0][1] * v[1]);
-    const DF y1 = k.dt * fma_(Mx[1][0], v[0], Mx[1][1] * v[1]);
-    // dphi/dt moves with the midpoint, x + y/2
-    const DF ph = k.dt * (v[2] + df_scale(fma_(Vx[2][0], y0, Vx[2][1] * y1), 0.5f));
-    const DF o[6] = {y0, y1, ph, du[0], du[1], du[2]};
-#pragma unroll
-    for (int q = 0; q < 6; ++q)
-      w[(int64_t)(q * JC + col) * n] = adj_pack(o[q], q == 0 && col == 0);
-  };
+  // Three pairs of columns, (x1, x2), (u1, u2), (u3, scale), through one copy of the code: the
+  // kernel waits for instructions more than for anything else, so that the metric's derivatives
+  // ride along as zeros in the second and third pass costs less than a second instance.
   const DF zero(0.0f), one(1.0f);
+  Local<D2F> L;
+  D2F eB[3], eD[3];
   {  // x1, x2: metric, tetrads and fields move
     const D2F R(a.r, k.dxi * a.r, zero), S(a.s, zero, a.c * k.dth), C(a.c, zero, -(a.s * k.dth));
-    Local<D2F> L;
     inc_local(k, R, S, C, L);
-    D2F eB[3], eD[3];
-    {
-      IncLerp l;
-      inc_lerp(a.i1, a.i2, a.o1, a.o2, l);
-      const D2F V[6] = {adj_interp_d(F.B[0], g.NX, l, 0, 1, a.V[0]),
-                        adj_interp_d(F.B[1], g.NX, l, 1, 0, a.V[1]),
-                        adj_interp_d(F.B[2], g.NX, l, 1, 1, a.V[2]),
-                        adj_interp_d(F.D[0], g.NX, l, 1, 0, a.V[3]),
-                        adj_interp_d(F.D[1], g.NX, l, 0, 1, a.V[4]),
-                        adj_interp_d(F.D[2], g.NX, l, 0, 0, a.V[5])};
-      vec_hat(L, V, eB);
-      vec_hat(L, V + 3, eD);
-      const D2F e = df_scale(scale * qm * k.dt, 0.25f) * L.alpha;
-#pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        eB[q] = e * eB[q];
-        eD[q] = e * eD[q];
-      }
-    }
-    const D2F u[3] = {D2F(a.u[0]), D2F(a.u[1]), D2F(a.u[2])};
-    D2F du[3];
-    adj_momentum_d(k, L, eD, eB, u, a, K, du);
-    const DF s0[3] = {zero, zero, zero};
-    const DF c0[3] = {du[0].d0, du[1].d0, du[2].d0}, c1[3] = {du[0].d1, du[1].d1, du[2].d1};
-    column(0, c0, s0, one, zero);
-    column(1, c1, s0, zero, one);
-  }
+    IncLerp l;
+    inc_lerp(a.i1, a.i2, a.o1, a.o2, l);
+    D2F V[6];
 #pragma unroll 1
-  for (int half = 0; half < 2; ++half) {  // (u1, u2), then (u3, scale)
-    const bool first = half == 0;
-    const DF on = first ? one : zero, off = first ? zero : one;
-    D2F eB[3], eD[3];
+    for (int q = 0; q < 6; ++q) {
+      const int h1 = q == 1 || q == 2 || q == 3, h2 = q == 0 || q == 2 || q == 4;
+      V[q] = adj_interp_d(q < 3 ? F.B[q] : F.D[q - 3], g.NX, l, h1, h2, a.V[q]);
+    }
+    vec_hat(L, V, eB);
+    vec_hat(L, V + 3, eD);
+    const D2F e = df_scale(scale * qm * k.dt, 0.25f) * L.alpha;
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
-      eB[q] = D2F(a.eB[q], zero, off * a.eB1[q]);
-      eD[q] = D2F(a.eD[q], zero, off * a.eD1[q]);
+      eB[q] = e * eB[q];
+      eD[q] = e * eD[q];
     }
-    const D2F u[3] = {D2F(a.u[0], on, zero), D2F(a.u[1], zero, on), D2F(a.u[2], off, zero)};
+  }
+#pragma unroll 1
+  for (int pass = 0; pass < 3; ++pass) {
+    const DF s0 = pass == 1 ? one : zero, s2 = pass == 2 ? one : zero;
+    if (pass == 1) {
+      D2F *m = reinterpret_cast<D2F *>(&L);
+      for (int q = 0; q < (int)(sizeof(L) / sizeof(D2F)); ++q) m[q].d0 = m[q].d1 = zero;
+    }
+    if (pass > 0)
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        eB[q].d0 = eD[q].d0 = zero;
+        eB[q].d1 = s2 * a.eB1[q];
+        eD[q].d1 = s2 * a.eD1[q];
+      }
+    // seeds of the first and second direction of the pass: u1, u2; u3, scale
+    const D2F u[3] = {D2F(a.u[0], s0, zero), D2F(a.u[1], zero, s0), D2F(a.u[2], s2, zero)};
     D2F du[3];
-    adj_momentum_d(k, a.L, eD, eB, u, a, K, du);
-    const DF s0[3] = {on, zero, off}, s1[3] = {zero, on, zero};
-    const DF c0[3] = {du[0].d0, du[1].d0, du[2].d0}, c1[3] = {du[0].d1, du[1].d1, du[2].d1};
-    column(2 + 2 * half, c0, s0, zero, zero);
-    column(3 + 2 * half, c1, s1, zero, zero);
+    adj_momentum_d(k, L, eD, eB, u, a, K, du);
+#pragma unroll 1
+    for (int d = 0; d < 2; ++d) {
+      // the increments' derivatives from that of u^{n+1} (seed + du') and of x^n (xs)
+      const int col = 2 * pass + d;
+      DF w3[3], p[3], v[3];
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        w3[q] = d ? du[q].d1 : du[q].d0;
+        p[q] = (d ? u[q].d1 : u[q].d0) + w3[q];
+      }
+      const DF xs0 = col == 0 ? one : zero, xs1 = col == 1 ? one : zero;
+#pragma unroll
+      for (int q = 0; q < 3; ++q)
+        v[q] = fma_(Vu[q][0], p[0], fma_(Vu[q][1], p[1], fma_(Vu[q][2], p[2],
+               fma_(Vx[q][0], xs0, Vx[q][1] * xs1))));
+      const DF y0 = k.dt * fma_(Mx[0][0], v[0], Mx[0][1] * v[1]);
+      const DF y1 = k.dt * fma_(Mx[1][0], v[0], Mx[1][1] * v[1]);
+      // dphi/dt moves with the midpoint, x + y/2
+      const DF ph = k.dt * (v[2] + df_scale(fma_(Vx[2][0], y0, Vx[2][1] * y1), 0.5f));
+      const DF o[6] = {y0, y1, ph, w3[0], w3[1], w3[2]};
+#pragma unroll
+      for (int q = 0; q < 6; ++q)
+        w[(int64_t)(q * JC + col) * n] = adj_pack(o[q], q == 0 && col == 0);
+    }
   }
 }
 
@@ -692,8 +694,23 @@ __device__ __forceinline__ void adj_reverse(const double *w, int64_t n, double l
   gs = lost ? NAN : fma(df_to_double(nl[5]), up, gs);
 }
 
+// The step's code (about 20,000 instructions) is larger than the instruction caches: warps that
+// wander through it apart from one another fetch it once each, and most of their time went to
+// waiting for instructions (7.0 of 10.9 cycles between issues). The barrier before each step
+// keeps a block's warps together, so that a fetch serves all of them; every thread reaches it,
+// particles or none. Together with one copy of the Jacobian's code for all columns: 39.6 ->
+// 31.0 ms for 65,536 orbits, 100 steps forward and back, events around repeated passes; 1 x 256,
+// 2 x 256 and 4 x 128 threads per SM measured 1 to 8% slower. Barriers inside the step as well
+// took twice as long (what a step keeps across them goes to local memory).
+#ifndef GRPIC_ADJ_BWD_TPB
+#define GRPIC_ADJ_BWD_TPB 128
+#endif
+#ifndef GRPIC_ADJ_BWD_BLOCKS
+#define GRPIC_ADJ_BWD_BLOCKS 2
+#endif
+constexpr int TPB_BWD = GRPIC_ADJ_BWD_TPB;
 template <bool INC>
-__global__ void __launch_bounds__(TPB_ADJ) k_adj_backward(
+__global__ void __launch_bounds__(TPB_BWD, GRPIC_ADJ_BWD_BLOCKS) k_adj_backward(
     const __grid_constant__ GridP g, const __grid_constant__ FieldPtrsT<double> F,
     const __grid_constant__ PushTables tb, int64_t n, double qm, double scale, double gfac,
     int n_steps, int every, int n_iter, const double *__restrict__ ckpt,
@@ -702,8 +719,9 @@ __global__ void __launch_bounds__(TPB_ADJ) k_adj_backward(
   const IncC kc = inc_c(g);
   const DF sd = df_of(scale), qd = df_of(qm);
   const int n_seg = (n_steps + every - 1) / every;
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
-       k += (int64_t)gridDim.x * blockDim.x) {
+  for (int64_t k0 = blockIdx.x * (int64_t)blockDim.x; k0 < n; k0 += (int64_t)gridDim.x * blockDim.x) {
+    const bool have = k0 + threadIdx.x < n;
+    const int64_t k = have ? k0 + threadIdx.x : n - 1;
     double lam[6];
     bool zero = true;
     for (int q = 0; q < 6; ++q) {
@@ -711,24 +729,25 @@ __global__ void __launch_bounds__(TPB_ADJ) k_adj_backward(
       zero = zero && lam[q] == 0.0;
     }
     double gs = 0.0;
-    bool bad = false;
-    for (int seg = n_seg - 1; seg >= 0 && !bad; --seg) {
+    bool bad = !have;
+    for (int seg = n_seg - 1; seg >= 0; --seg) {
       const int s0 = seg * every, len = min(n_steps, s0 + every) - s0;
       double st[6];
       const double *c = ckpt + (int64_t)seg * 6 * n;
       for (int q = 0; q < 6; ++q) st[q] = c[q * n + k];
-      if (!inside(g, st)) {
-        bad = true;
-        break;
-      }
+      bad = bad || !inside(g, st);
       // recompute the segment from its checkpoint, keeping each step's Jacobian
       double *w = scratch + k;
-      for (int j = 0; j < len && !bad; ++j)
-        bad = !adj_advance<INC>(g, F, tb, kc, scale, sd, qm, qd, n_iter, st,
-                                w + (int64_t)j * 6 * JC * n, n);
+      for (int j = 0; j < len; ++j) {
+        __syncthreads();
+        if (!bad)
+          bad = !adj_advance<INC>(g, F, tb, kc, scale, sd, qm, qd, n_iter, st,
+                                  w + (int64_t)j * 6 * JC * n, n);
+      }
       // reverse sweep: lambda_n = J_n^T lambda_{n+1}
       for (int j = len - 1; j >= 0 && !bad; --j) adj_reverse(w + (int64_t)j * 6 * JC * n, n, lam, gs);
     }
+    if (!have) continue;
     // a particle that reached a boundary has no gradient: zero where its cotangent was zero
     // (it does not enter the loss), NaN otherwise
     const double fill = zero ? 0.0 : NAN;
@@ -752,8 +771,8 @@ __global__ void __launch_bounds__(1024) k_sum(const double *__restrict__ x, int6
   if (threadIdx.x == 0) out[0] = red[0];
 }
 
-int adj_blocks(int64_t n) {
-  int64_t b = (n + TPB_ADJ - 1) / TPB_ADJ;
+int adj_blocks(int64_t n, int tpb) {
+  int64_t b = (n + tpb - 1) / tpb;
   const int64_t cap = 152 * 32;
   return (int)(b < 1 ? 1 : (b > cap ? cap : b));
 }
@@ -773,8 +792,8 @@ cudaError_t launch_adjoint_forward(const GridP &g, const FieldPtrsT<double> &F,
                                    double *out, double *ckpt, cudaStream_t st) {
   if (n <= 0) return cudaGetLastError();
   const auto kernel = adj_inc_applies(g, n_iter) ? k_adj_forward<true> : k_adj_forward<false>;
-  kernel<<<adj_blocks(n), TPB_ADJ, 0, st>>>(g, F, tb, n, qm, scale, n_steps, every, n_iter, st0,
-                                            out, ckpt);
+  kernel<<<adj_blocks(n, TPB_ADJ), TPB_ADJ, 0, st>>>(g, F, tb, n, qm, scale, n_steps, every,
+                                                     n_iter, st0, out, ckpt);
   COUNT_LAUNCH(1);
   return cudaGetLastError();
 }
@@ -787,8 +806,8 @@ cudaError_t launch_adjoint_backward(const GridP &g, const FieldPtrsT<double> &F,
                                     cudaStream_t st) {
   if (n <= 0) return cudaMemsetAsync(gscale_sum, 0, sizeof(double), st);
   const auto kernel = adj_inc_applies(g, n_iter) ? k_adj_backward<true> : k_adj_backward<false>;
-  kernel<<<adj_blocks(n), TPB_ADJ, 0, st>>>(g, F, tb, n, qm, scale, gfac, n_steps, every, n_iter,
-                                            ckpt, gout, gin, gscale_pp, scratch);
+  kernel<<<adj_blocks(n, TPB_BWD), TPB_BWD, 0, st>>>(g, F, tb, n, qm, scale, gfac, n_steps, every,
+                                                     n_iter, ckpt, gout, gin, gscale_pp, scratch);
   k_sum<<<1, 1024, 0, st>>>(gscale_pp, n, gscale_sum);
   COUNT_LAUNCH(2);
   return cudaGetLastError();
