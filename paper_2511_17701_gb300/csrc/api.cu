@@ -74,7 +74,8 @@ struct grpic_ctx {
   size_t need = 0;
   char *arena = nullptr;
   cudaStream_t stream = nullptr;
-  cudaStream_t side = nullptr;  // guard kernels of the mixed push
+  // species k's guard kernels (mixed push), or its whole push where that is small, on side[k % 2]
+  cudaStream_t side[2] = {};
   cudaEvent_t ev_fork[GRPIC_MAX_SPECIES] = {}, ev_done[GRPIC_MAX_SPECIES] = {};
   cudaEvent_t ev_class[GRPIC_MAX_SPECIES] = {};
   // grpic_step_host: copy streams, events and pinned counts, created on its first call;
@@ -267,8 +268,8 @@ cudaError_t do_push(grpic_ctx *c, FieldPtrsT<T> &F, int k, bool deposit, int sta
   SpeciesState &sp = c->sp[k];
   const std::pair<cudaEvent_t, cudaEvent_t> *kt =
       push_main_stage(stage) ? next_events(c, PH_KERNEL) : nullptr;
-  const PushStreams ps{c->stream, c->side, c->ev_fork[k], c->ev_done[k], c->ev_class[k],
-                       kt ? kt->first : nullptr, kt ? kt->second : nullptr, stage};
+  const PushStreams ps{c->stream, c->side[k & 1], c->ev_fork[k], c->ev_done[k], c->ev_class[k],
+                       kt ? kt->first : nullptr, kt ? kt->second : nullptr, stage, (k & 1) != 0};
   const int tr = c->cfg.tile_r, tt = c->cfg.tile_theta;
   const int ntr = (c->g.n_r + tr - 1) / tr, ntt = (c->g.n_th + tt - 1) / tt;
   TileInfo ti{};
@@ -296,11 +297,14 @@ cudaError_t do_push(grpic_ctx *c, FieldPtrsT<T> &F, int k, bool deposit, int sta
 }
 // the main stream waits for the guard kernels of species k (mixed path)
 cudaError_t join_push(grpic_ctx *c, int k) {
-  return c->mixed ? cudaStreamWaitEvent(c->stream, c->ev_done[k], 0) : cudaSuccess;
+  return cudaStreamWaitEvent(c->stream, c->ev_done[k], 0);
 }
 template <typename T>
 cudaError_t do_zero_J(grpic_ctx *c, FieldPtrsT<T> &F) {
-  const int64_t ps = plane_size(c->g);
+  const int64_t ps = plane_size(c->g), step = F.J[1] - F.J[0];
+  // the three planes lie one behind the other (up to their alignment): one launch
+  if (step >= ps && step < ps + 256 && F.J[2] - F.J[1] == step)
+    return launch_zero<T>(F.J[0], 2 * step + ps, c->stream);
   for (int i = 0; i < 3; ++i) {
     cudaError_t e = launch_zero<T>(F.J[i], ps, c->stream);
     if (e != cudaSuccess) return e;
@@ -541,15 +545,15 @@ grpic_status grpic_bind(grpic_ctx *ctx, void *arena, size_t bytes, void *stream)
       sp.tile_start = at<uint32_t>(ctx, sp.off_tiles);
       sp.tiles_valid = false;
     }
-    if (!ctx->side) {  // the guard kernels are the longer chain: higher priority
-      int lo = 0, hi = 0;
-      CK(cudaDeviceGetStreamPriorityRange(&lo, &hi));
-      CK(cudaStreamCreateWithPriority(&ctx->side, cudaStreamNonBlocking, hi));
-      for (int s = 0; s < GRPIC_MAX_SPECIES; ++s) {
-        CK(cudaEventCreateWithFlags(&ctx->ev_fork[s], cudaEventDisableTiming));
-        CK(cudaEventCreateWithFlags(&ctx->ev_done[s], cudaEventDisableTiming));
-        CK(cudaEventCreateWithFlags(&ctx->ev_class[s], cudaEventDisableTiming));
-      }
+  }
+  if (!ctx->side[0]) {  // the guard kernels are the longer chain: higher priority
+    int lo = 0, hi = 0;
+    CK(cudaDeviceGetStreamPriorityRange(&lo, &hi));
+    for (cudaStream_t &st : ctx->side) CK(cudaStreamCreateWithPriority(&st, cudaStreamNonBlocking, hi));
+    for (int s = 0; s < GRPIC_MAX_SPECIES; ++s) {
+      CK(cudaEventCreateWithFlags(&ctx->ev_fork[s], cudaEventDisableTiming));
+      CK(cudaEventCreateWithFlags(&ctx->ev_done[s], cudaEventDisableTiming));
+      CK(cudaEventCreateWithFlags(&ctx->ev_class[s], cudaEventDisableTiming));
     }
   }
   ctx->diag = at<unsigned long long>(ctx, ctx->off_diag);
@@ -911,7 +915,7 @@ cudaError_t push_range(grpic_ctx *c, int k, int64_t a, int64_t m, const int64_t 
   v.i1 += a; v.i2 += a; v.dx1 += a; v.dx2 += a; v.u1 += a; v.u2 += a; v.u3 += a;
   v.phi += a; v.w += a; v.tag += a; v.i1p += a; v.i2p += a; v.dx1p += a; v.dx2p += a;
   v.n = n_chunk;
-  const PushStreams ps{c->stream, c->side, c->ev_fork[k], c->ev_done[k], c->ev_class[k],
+  const PushStreams ps{c->stream, c->side[k & 1], c->ev_fork[k], c->ev_done[k], c->ev_class[k],
                        nullptr, nullptr, PUSH_ALL};
   TileInfo ti{};
   ti.tr = c->cfg.tile_r;
@@ -1278,9 +1282,11 @@ void grpic_destroy(grpic_ctx *ctx) {
       cudaEventDestroy(e.first);
       cudaEventDestroy(e.second);
     }
-  if (ctx->side) {
-    cudaStreamSynchronize(ctx->side);
-    cudaStreamDestroy(ctx->side);
+  if (ctx->side[0]) {
+    for (cudaStream_t st : ctx->side) {
+      cudaStreamSynchronize(st);
+      cudaStreamDestroy(st);
+    }
     for (int s = 0; s < GRPIC_MAX_SPECIES; ++s) {
       cudaEventDestroy(ctx->ev_fork[s]);
       cudaEventDestroy(ctx->ev_done[s]);
