@@ -349,7 +349,7 @@ __global__ void k_axis(GridP g, T *p0, T *p1, T *p2, int isB) {
 // (MEAN), one that enters as itself from a alone; which one is known at compile time, since a
 // multiplication by a weight of 1 would cost an FP64 operation per value.
 // ---------------------------------------------------------------------------------
-constexpr int TPBX = 64, TPBY = 4;
+constexpr int TPBX = 64, TPBY = 4;  // the largest block
 
 template <typename T>
 struct Pair3 {
@@ -359,6 +359,12 @@ template <bool MEAN, typename T>
 __device__ __forceinline__ T pv(const Pair3<T> &P, int c, int64_t k) {
   if (MEAN) return (T)0.5 * (__ldg(P.a[c] + k) + __ldg(P.b[c] + k));
   return __ldg(P.a[c] + k);
+}
+
+// v - 4 pi J
+template <bool MEAN, typename T>
+__device__ __forceinline__ T less_4pi_j(const Pair3<T> &J, int c, int64_t k, T v) {
+  return fma((T)(-4.0 * GRPIC_PI), pv<MEAN>(J, c, k), v);
 }
 
 // E_1 at (i+1/2, j) = alpha [h_11 D^1 + <h_13 D^3>], E_3 at (i, j) = alpha [h_33 D^3 +
@@ -465,9 +471,9 @@ __device__ __forceinline__ void aux_H(const GridP &g, const Pair3<float> &B, con
 template <typename T, bool DOE, bool DOH, bool DMEAN>
 __global__ void __launch_bounds__(TPBX *TPBY) k_aux(GridP g, Pair3<T> B, Pair3<T> D, const T *tab,
                                                     T *E1, T *E2, T *E3, T *H1, T *H2, T *H3) {
-  const int i = (int)(blockIdx.x * TPBX + threadIdx.x) - 1;
+  const int i = (int)(blockIdx.x * blockDim.x + threadIdx.x) - 1;
   const int64_t ps = plane_size(g);
-  for (int j = blockIdx.y * TPBY + threadIdx.y; j <= g.n_th; j += gridDim.y * TPBY) {
+  for (int j = blockIdx.y * blockDim.y + threadIdx.y; j <= g.n_th; j += gridDim.y * blockDim.y) {
     if (i > g.n_r + 1) return;
     const int64_t k = sidx(g, i, j);
     if (DOE) aux_E<DMEAN>(g, B, D, tab, ps, j, k, E1, E2, E3);
@@ -556,26 +562,24 @@ __device__ __forceinline__ void ampere(const GridP &g, const Pair3<T> &Din, cons
                                        const T *H2, const T *H3, const Pair3<T> &J, const T *tab,
                                        const T *polar, T *const D[3], T *const Di[3], int64_t ps,
                                        int i, int j, int64_t k) {
-  const T fpi = (T)(4.0 * GRPIC_PI);
   T d1 = pv<MEAN>(Din, 0, k), d2 = pv<MEAN>(Din, 1, k), d3 = pv<MEAN>(Din, 2, k);
   if (i >= 0 && i <= g.n_r && j >= 0 && j <= g.n_th) {
     if (i < g.n_r) {
-      const T j1 = pv<MEAN>(J, 0, k);
       if (j == 0)
-        d1 += (T)g.dt * (__ldg(H3 + k) - fpi * j1) / __ldg(polar + i + G_);
+        d1 += (T)g.dt * less_4pi_j<MEAN>(J, 0, k, __ldg(H3 + k)) / __ldg(polar + i + G_);
       else if (j == g.n_th)
-        d1 += (T)g.dt * (-__ldg(H3 + k - g.NX) - fpi * j1) / __ldg(polar + i + G_);
+        d1 += (T)g.dt * less_4pi_j<MEAN>(J, 0, k, -__ldg(H3 + k - g.NX)) / __ldg(polar + i + G_);
       else
         d1 = curl_step(g, tab, ps, T_B2D1, CLS_HN, k,
-                       fma(-fpi, j1, __ldg(H3 + k) - __ldg(H3 + k - g.NX)), d1);
+                       less_4pi_j<MEAN>(J, 0, k, __ldg(H3 + k) - __ldg(H3 + k - g.NX)), d1);
     }
     if (j < g.n_th) {
       d2 = curl_step(g, tab, ps, T_B1D2, CLS_NH, k,
-                     -fma(fpi, pv<MEAN>(J, 1, k), __ldg(H3 + k) - __ldg(H3 + k - 1)), d2);
+                     less_4pi_j<MEAN>(J, 1, k, __ldg(H3 + k - 1) - __ldg(H3 + k)), d2);
       if (j >= 1)
         d3 = curl_step(g, tab, ps, T_D3, CLS_NN, k,
-                       fma(-fpi, pv<MEAN>(J, 2, k), (__ldg(H2 + k) - __ldg(H2 + k - 1)) -
-                                                        (__ldg(H1 + k) - __ldg(H1 + k - g.NX))),
+                       less_4pi_j<MEAN>(J, 2, k, (__ldg(H2 + k) - __ldg(H2 + k - 1)) -
+                                                     (__ldg(H1 + k) - __ldg(H1 + k - g.NX))),
                        d3);
     }
   }
@@ -598,10 +602,10 @@ struct Planes3 {
 template <typename T>
 __global__ void __launch_bounds__(TPBX *TPBY) k_faraday(GridP g, Pair3<T> Bin, Planes3<T> E,
                                                         const T *tab, Planes3<T> Bout) {
-  const int i = (int)(blockIdx.x * TPBX + threadIdx.x) - G_;
+  const int i = (int)(blockIdx.x * blockDim.x + threadIdx.x) - G_;
   const int64_t ps = plane_size(g);
-  for (int j = (int)(blockIdx.y * TPBY + threadIdx.y) - G_; j <= g.n_th + G_;
-       j += gridDim.y * TPBY) {
+  for (int j = (int)(blockIdx.y * blockDim.y + threadIdx.y) - G_; j <= g.n_th + G_;
+       j += gridDim.y * blockDim.y) {
     if (i > g.n_r + G_) return;
     faraday<T, true, false>(g, Bin, E.p[0], E.p[1], E.p[2], tab, nullptr, Bout.p, Bout.p, ps, i,
                             j, sidx(g, i, j));
@@ -613,10 +617,10 @@ template <typename T>
 __global__ void __launch_bounds__(TPBX *TPBY) k_faraday_ampere(
     GridP g, Pair3<T> Bin, Planes3<T> E, Planes3<T> Bout, Planes3<T> Bi, Pair3<T> Din,
     Planes3<T> H, Pair3<T> J, Planes3<T> Dout, const T *tab, const T *polar) {
-  const int i = (int)(blockIdx.x * TPBX + threadIdx.x) - G_;
+  const int i = (int)(blockIdx.x * blockDim.x + threadIdx.x) - G_;
   const int64_t ps = plane_size(g);
-  for (int j = (int)(blockIdx.y * TPBY + threadIdx.y) - G_; j <= g.n_th + G_;
-       j += gridDim.y * TPBY) {
+  for (int j = (int)(blockIdx.y * blockDim.y + threadIdx.y) - G_; j <= g.n_th + G_;
+       j += gridDim.y * blockDim.y) {
     if (i > g.n_r + G_) return;
     const int64_t k = sidx(g, i, j);
     faraday<T, false, true>(g, Bin, E.p[0], E.p[1], E.p[2], tab, polar + g.NX, Bout.p, Bi.p, ps,
@@ -629,10 +633,10 @@ template <typename T>
 __global__ void __launch_bounds__(TPBX *TPBY) k_ampere(GridP g, Pair3<T> Din, Planes3<T> H,
                                                        Pair3<T> J, const T *tab, const T *polar,
                                                        Planes3<T> Dout, Planes3<T> Di) {
-  const int i = (int)(blockIdx.x * TPBX + threadIdx.x) - G_;
+  const int i = (int)(blockIdx.x * blockDim.x + threadIdx.x) - G_;
   const int64_t ps = plane_size(g);
-  for (int j = (int)(blockIdx.y * TPBY + threadIdx.y) - G_; j <= g.n_th + G_;
-       j += gridDim.y * TPBY) {
+  for (int j = (int)(blockIdx.y * blockDim.y + threadIdx.y) - G_; j <= g.n_th + G_;
+       j += gridDim.y * blockDim.y) {
     if (i > g.n_r + G_) return;
     ampere<T, false>(g, Din, H.p[0], H.p[1], H.p[2], J, tab, polar, Dout.p, Di.p, ps, i, j,
                      sidx(g, i, j));
@@ -688,18 +692,23 @@ void axis(const GridP &g, T *const p[3], int isB, cudaStream_t st) {
   COUNT_LAUNCH(1);
 }
 
-// blocks of TPBX x TPBY points covering ni x nj points (rows beyond the grid's limit in y
-// are taken by the kernels' row loop)
-dim3 tiles_for(int ni, int nj) {
-  const int by = (nj + TPBY - 1) / TPBY;
-  return dim3((ni + TPBX - 1) / TPBX, by > 65535 ? 65535 : by);
+// Blocks covering ni x nj points: TPBX x TPBY, or 32 x 2 on grids that would not give every SM
+// two of those (64^2 points were 19 blocks, 8 warps of FP64 work on each of 19 SMs); rows beyond
+// the grid's limit in y are taken by the kernels' row loop
+struct Tiles {
+  dim3 grid, block;
+};
+Tiles tiles_for(int ni, int nj) {
+  const bool few = (int64_t)ni * nj < 2 * 152 * TPBX * TPBY;
+  const int bx = few ? 32 : TPBX, by = few ? 2 : TPBY, ny = (nj + by - 1) / by;
+  return {dim3((ni + bx - 1) / bx, ny > 65535 ? 65535 : ny), dim3(bx, by)};
 }
-const dim3 TILE(TPBX, TPBY);
 
 template <bool DOE, bool DOH, bool DMEAN, typename T>
 void aux(const GridP &g, const Pair3<T> &B, const Pair3<T> &D, const FieldPtrsT<T> &F,
          cudaStream_t st) {
-  k_aux<T, DOE, DOH, DMEAN><<<tiles_for(g.n_r + 3, g.n_th + 1), TILE, 0, st>>>(
+  const Tiles t = tiles_for(g.n_r + 3, g.n_th + 1);
+  k_aux<T, DOE, DOH, DMEAN><<<t.grid, t.block, 0, st>>>(
       g, B, D, F.tab, F.E[0], F.E[1], F.E[2], F.H[0], F.H[1], F.H[2]);
   COUNT_LAUNCH(1);
 }
@@ -776,8 +785,8 @@ cudaError_t launch_field_finish_init(const GridP &g, const FieldPtrsT<T> &F, int
 template <typename T>
 cudaError_t launch_predict(const GridP &g, const FieldPtrsT<T> &F, cudaStream_t st) {
   aux<true, false, true>(g, one(F.B), pair(F.D0, F.D), F, st);
-  k_faraday<T><<<tiles_for(g.NX, g.NY), TILE, 0, st>>>(g, pair(F.B0, F.B), planes(F.E), F.tab,
-                                                       planes(F.Bn));
+  const Tiles all = tiles_for(g.NX, g.NY);
+  k_faraday<T><<<all.grid, all.block, 0, st>>>(g, pair(F.B0, F.B), planes(F.E), F.tab, planes(F.Bn));
   COUNT_LAUNCH(1);
   return cudaGetLastError();
 }
@@ -786,17 +795,17 @@ cudaError_t launch_predict(const GridP &g, const FieldPtrsT<T> &F, cudaStream_t 
 // D^{n+1} into the D0 planes; the caller then swaps em/em0 and cur/cur0.
 template <typename T>
 cudaError_t launch_advance(const GridP &g, const FieldPtrsT<T> &F, cudaStream_t st) {
-  const dim3 all = tiles_for(g.NX, g.NY);
+  const Tiles all = tiles_for(g.NX, g.NY);
   // step 6: E^n, H^n from {B^n, D^n}; Faraday B^{n-1/2} -> B^{n+1/2}; step 7: auxiliary Ampere
   // D^{n-1/2} -> D^{n+1/2} with H^n and J^n = (J^{n-1/2} + J^{n+1/2})/2
   aux<true, true, false>(g, one(F.Bn), one(F.D), F, st);
-  k_faraday_ampere<T><<<all, TILE, 0, st>>>(g, one(F.B), planes(F.E), planes(F.B0), planes(F.Bi),
+  k_faraday_ampere<T><<<all.grid, all.block, 0, st>>>(g, one(F.B), planes(F.E), planes(F.B0), planes(F.Bi),
                                             pair(F.D0, F.D), planes(F.H), pair(F.J0, F.J),
                                             planes(F.Dh), F.tab, F.polar);
   COUNT_LAUNCH(1);
   // H^{n+1/2} from {B^{n+1/2}, D^{n+1/2}}; final Ampere D^n -> D^{n+1} with J^{n+1/2}
   aux<false, true, false>(g, one(F.B0), one(F.Dh), F, st);
-  k_ampere<T><<<all, TILE, 0, st>>>(g, one(F.D), planes(F.H), one(F.J), F.tab, F.polar,
+  k_ampere<T><<<all.grid, all.block, 0, st>>>(g, one(F.D), planes(F.H), one(F.J), F.tab, F.polar,
                                     planes(F.D0), planes(F.Di));
   COUNT_LAUNCH(1);
   return cudaGetLastError();
