@@ -22,6 +22,10 @@
 namespace {
 
 constexpr int FT_X = 64, FT_Y = 32, F_MAXP = 8, F_TPB = 512;
+// The output tile of a block: FT_X x FT_Y, or FS_X x FS_Y on grids whose large tiles would leave
+// most SMs without one (64^2 points: 9 blocks, 22 us for 4 passes, of which all but the few SMs
+// in use see nothing); the small tiles' halo costs more arithmetic in all, but on idle SMs.
+constexpr int FS_X = 16, FS_Y = 8, FS_TPB = 128;
 
 template <typename T>
 struct FilterPlanes {
@@ -50,14 +54,15 @@ __device__ __forceinline__ int reflect_row(int j, int N, int half, float par, fl
 }
 
 template <typename T>
-size_t filter_smem(int P) {
-  return (size_t)2 * (FT_X + 2 * P) * (FT_Y + 2 * P) * sizeof(T);
+size_t filter_smem(int tx, int ty, int P) {
+  return (size_t)2 * (tx + 2 * P) * (ty + 2 * P) * sizeof(T);
 }
 
 template <typename T>
-__global__ void __launch_bounds__(F_TPB) k_filter(GridP g, FilterPlanes<T> fp, int P) {
+__global__ void __launch_bounds__(F_TPB) k_filter(GridP g, FilterPlanes<T> fp, int P, int tx,
+                                                  int ty) {
   extern __shared__ unsigned char f_smem[];
-  const int W = FT_X + 2 * P, H = FT_Y + 2 * P;
+  const int W = tx + 2 * P, H = ty + 2 * P;
   T *A = reinterpret_cast<T *>(f_smem), *Bt = A + W * H;  // values, x1 sums
   const int c = blockIdx.z;
   const T *in = fp.in[c];
@@ -65,7 +70,7 @@ __global__ void __launch_bounds__(F_TPB) k_filter(GridP g, FilterPlanes<T> fp, i
   const int half = fp.half[c];
   const float par = (float)fp.parity[c];
   const int N = g.n_th;
-  const int i0 = -G_ + (int)blockIdx.x * FT_X, j0 = -G_ + (int)blockIdx.y * FT_Y;  // stored
+  const int i0 = -G_ + (int)blockIdx.x * tx, j0 = -G_ + (int)blockIdx.y * ty;  // stored
   const int ilo = -G_, ihi = g.n_r + G_;
   // load the extended values of the tile and its halo; cells beyond the x1 range are zero
   for (int e = threadIdx.x; e < W * H; e += blockDim.x) {
@@ -103,13 +108,13 @@ __global__ void __launch_bounds__(F_TPB) k_filter(GridP g, FilterPlanes<T> fp, i
   T scale = (T)1;
   for (int p = 0; p < P; ++p) scale *= (T)0.0625;
   const int jmax = half ? N - 1 : N;
-  for (int e = threadIdx.x; e < FT_X * FT_Y; e += blockDim.x) {
-    const int ty = e / FT_X, tx = e - ty * FT_X;
-    const int i = i0 + tx, j = j0 + ty;
+  for (int e = threadIdx.x; e < tx * ty; e += blockDim.x) {
+    const int y = e / tx, x = e - y * tx;
+    const int i = i0 + x, j = j0 + y;
     if (i > ihi || j > N + G_) continue;
     T v = (T)0;
     if (j >= 0 && j <= jmax) {
-      v = A[(P + ty) * W + P + tx] * scale;
+      v = A[(P + y) * W + P + x] * scale;
       if (!half && (j == 0 || j == N)) v *= (T)0.5;
     }
     out[sidx(g, i, j)] = v;
@@ -122,12 +127,15 @@ cudaError_t filter_chunk(const GridP &g, const FilterPlanes<T> &fp, int n_comp, 
   static bool attr = false;  // per instantiation: opt in to the largest tile's shared memory
   if (!attr) {
     cudaError_t e = cudaFuncSetAttribute(k_filter<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)filter_smem<T>(F_MAXP));
+                                         (int)filter_smem<T>(FT_X, FT_Y, F_MAXP));
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  const dim3 grid((g.NX + FT_X - 1) / FT_X, (g.NY + FT_Y - 1) / FT_Y, n_comp);
-  k_filter<T><<<grid, F_TPB, filter_smem<T>(P), st>>>(g, fp, P);
+  const int64_t large = (int64_t)((g.NX + FT_X - 1) / FT_X) * ((g.NY + FT_Y - 1) / FT_Y) * n_comp;
+  const bool few = large < 152;
+  const int tx = few ? FS_X : FT_X, ty = few ? FS_Y : FT_Y;
+  const dim3 grid((g.NX + tx - 1) / tx, (g.NY + ty - 1) / ty, n_comp);
+  k_filter<T><<<grid, few ? FS_TPB : F_TPB, filter_smem<T>(tx, ty, P), st>>>(g, fp, P, tx, ty);
   COUNT_LAUNCH(1);
   return cudaGetLastError();
 }
