@@ -61,9 +61,10 @@ typedef enum { GRPIC_METRIC_KS0 = 0, GRPIC_METRIC_KS = 1 } grpic_metric_kind;
 typedef enum {
   GRPIC_FP64 = 0,  /* FP64 state, fields and arithmetic                                  */
   GRPIC_MIXED = 1  /* FP32 fields, momenta, offsets and currents (int32 cells); FP32
-                      arithmetic, with the metric, lapse and shift evaluated in FP64 for
-                      particles within fp64_guard_cells of the horizon or an axis, and
-                      the whole push in FP64 for particles in the cell rows on the axes */
+                      arithmetic, with the metric, lapse and shift evaluated in pairs of
+                      FP32 numbers (48 bits) for particles within fp64_guard_cells of the
+                      horizon or an axis, and the whole push in pairs for particles in the
+                      cell rows on the axes                                             */
 } grpic_precision;
 typedef enum {
   GRPIC_FIELD_ZERO = 0,     /* all fields zero                                    */
@@ -119,13 +120,13 @@ typedef struct {
   int full_iterations; /* 0: the implicit pushes stop once an iterate repeats bit for bit (every
                           later iteration would return the same bits, so the result equals the
                           n_iter result exactly), except in GRPIC_MIXED: its FP32 iterations
-                          stop once the update is within 2^-22 max(1, |value|), the FP64
-                          iterations of its axis rows (stored in FP32) within 2^-26 max(1,
+                          stop once the update is within 2^-22 max(1, |value|), the
+                          iterations of its axis rows (48 bits) within 2^-26 max(1,
                           |value|) (the remaining error, a fraction rho / (1 - rho) of that,
                           is below the rounding of the stored values); 1: always run n_iter
                           iterations                                                         */
   int fp64_guard_cells; /* GRPIC_MIXED: cells from the horizon and from each axis where the
-                           metric is evaluated in FP64 (default 4 when 0)                     */
+                           metric is evaluated in 48 bits (default 4 when 0)                  */
   int tiled_push;       /* GRPIC_MIXED: 1 = after a sort, push each sort tile in one CTA with
                            the fields of the tile and a 6-cell halo staged in shared memory and
                            the currents accumulated there (the window loaded by the CTA's
@@ -143,7 +144,10 @@ typedef struct {
                            until the update is at most iter_tol max(1, |value|) (at most n_iter
                            evaluations in all): the FP64 fixed point to about rho iter_tol
                            (rho < 1 the contraction of the iteration), in fewer FP64
-                           operations. Must be below 1e-6                                      */
+                           operations. On the plain log-r grid the momentum's increments (steps
+                           2 to 9) are formed in pairs of FP32 numbers (48 bits) where they are
+                           small against the momentum and added in FP64, which leaves a smaller
+                           error than FP64 throughout. Must be below 1e-6                      */
   double r0, h0;        /* quasi-spherical Kerr-Schild grid (App. A): r = r0 + exp(xi), xi
                            uniform in x1 (r0 < r_min); theta = eta + 2 h0 eta (pi - 2 eta)
                            (pi - eta) / pi^2, eta uniform in x2 (-1/2 < h0 < 1; h0 > 0 puts
@@ -210,9 +214,10 @@ GRPIC_API size_t grpic_arena_bytes(const grpic_ctx *ctx);
 /* (Memory and stream management, no counterpart in the paper.)
  * Binds the caller-owned device arena (>= grpic_arena_bytes, 256-byte aligned)
  * and the CUDA stream (cudaStream_t, NULL = legacy default) on the current device.
- * With GRPIC_MIXED the first bind also creates one internal stream and event pairs
- * (no device memory): the push forks the FP64 guard-zone kernels onto it and joins
- * them back to the bound stream before returning, so callers see one stream.
+ * The first bind also creates up to two internal streams and event pairs (no device
+ * memory): the mixed push forks its guard-zone kernels onto them, small FP64 pushes of every
+ * other species run there, and both join the bound stream before returning, so callers see
+ * one stream.
  * Errors: GRPIC_ENOMEM (too small), GRPIC_EINVAL (misaligned), GRPIC_ECUDA. */
 GRPIC_API grpic_status grpic_bind(grpic_ctx *ctx, void *arena, size_t bytes, void *stream);
 

@@ -297,6 +297,8 @@ cudaError_t do_push(grpic_ctx *c, FieldPtrsT<T> &F, int k, bool deposit, int sta
 }
 // the main stream waits for the guard kernels of species k (mixed path)
 cudaError_t join_push(grpic_ctx *c, int k) {
+  // an event that this push has not recorded is left alone (a stream capture would refuse it)
+  if (!c->mixed && !push_apart((k & 1) != 0, c->sp[k].n_bound)) return cudaSuccess;
   return cudaStreamWaitEvent(c->stream, c->ev_done[k], 0);
 }
 template <typename T>
@@ -546,10 +548,13 @@ grpic_status grpic_bind(grpic_ctx *ctx, void *arena, size_t bytes, void *stream)
       sp.tiles_valid = false;
     }
   }
-  if (!ctx->side[0]) {  // the guard kernels are the longer chain: higher priority
+  // the guard kernels are the longer chain: higher priority (FP64 runs of one species need no
+  // stream, others the second)
+  if (!ctx->side[1] && (ctx->mixed || ctx->cfg.n_species > 1)) {
     int lo = 0, hi = 0;
     CK(cudaDeviceGetStreamPriorityRange(&lo, &hi));
-    for (cudaStream_t &st : ctx->side) CK(cudaStreamCreateWithPriority(&st, cudaStreamNonBlocking, hi));
+    if (ctx->mixed) CK(cudaStreamCreateWithPriority(&ctx->side[0], cudaStreamNonBlocking, hi));
+    CK(cudaStreamCreateWithPriority(&ctx->side[1], cudaStreamNonBlocking, hi));
     for (int s = 0; s < GRPIC_MAX_SPECIES; ++s) {
       CK(cudaEventCreateWithFlags(&ctx->ev_fork[s], cudaEventDisableTiming));
       CK(cudaEventCreateWithFlags(&ctx->ev_done[s], cudaEventDisableTiming));
@@ -1282,17 +1287,17 @@ void grpic_destroy(grpic_ctx *ctx) {
       cudaEventDestroy(e.first);
       cudaEventDestroy(e.second);
     }
-  if (ctx->side[0]) {
-    for (cudaStream_t st : ctx->side) {
-      cudaStreamSynchronize(st);
-      cudaStreamDestroy(st);
-    }
+  for (cudaStream_t st : ctx->side) {
+    if (!st) continue;
+    cudaStreamSynchronize(st);
+    cudaStreamDestroy(st);
+  }
+  if (ctx->side[1])
     for (int s = 0; s < GRPIC_MAX_SPECIES; ++s) {
       cudaEventDestroy(ctx->ev_fork[s]);
       cudaEventDestroy(ctx->ev_done[s]);
       cudaEventDestroy(ctx->ev_class[s]);
     }
-  }
   delete ctx;
 }
 

@@ -417,6 +417,10 @@ __host__ __device__ inline bool push_classify_stage(int s) {
 __host__ __device__ inline bool push_guard_kernels_stage(int s) {
   return s == PUSH_ALL || s == PUSH_GUARD || s == PUSH_GUARD_KERNELS;
 }
+// whether an FP64 push that may run apart does: fewer particles than fill the GPU
+inline bool push_apart(bool may, int64_t n_bound) {
+  return may && n_bound > 0 && n_bound < (1 << 18);
+}
 struct PushStreams {
   cudaStream_t main, side;
   cudaEvent_t fork, done, classified;  // side after main; guard kernels done; classify done

@@ -389,10 +389,10 @@ __device__ __forceinline__ Vel<DF> inc_velocity(const IncC &k, DF r, DF s, DF c,
 }
 
 // r, sin(theta), cos(theta) in FP64 at offsets (o1, o2) of cell (i1, i2): r from the nearest
-// corner's table, theta formed as map_theta forms it and its offset from the corner's theta
-// exact (as local_rsc)
+// corner's table, theta formed from x2 = i2 + o2 as map_theta forms it and its offset from the
+// corner's theta exact (as local_rsc)
 __device__ __forceinline__ void inc_point64(const GridP &g, const PushTables &tb, int i1, int i2,
-                                            double o1, double o2, double &ex, double &s,
+                                            double o1, double o2, double x2, double &ex, double &s,
                                             double &c) {
   const int c1 = gt_pos(o1, 0.5), c2 = gt_pos(o2, 0.5);
   const double e = (o1 - (c1 ? 1.0 : 0.0)) * g.dxi;
@@ -409,7 +409,7 @@ __device__ __forceinline__ void inc_point64(const GridP &g, const PushTables &tb
   } else {
     ex = map_e(g, (double)i1 + o1);
   }
-  const double th = __dmul_rn(__dadd_rn((double)i2, o2), g.dth);
+  const double th = __dmul_rn(x2, g.dth);
   const double d = th - __ldg(tb.th64 + i2 + c2 + G_);
   if (abs_le(d, (double)INC_D)) {
     const double q = d * d;
@@ -435,7 +435,8 @@ __device__ __forceinline__ void inc_coord64(const GridP &g, const PushTables &tb
                                             double t1, double t2, double &n1, double &n2,
                                             double &v3) {
   double ex, s, c;
-  inc_point64(g, tb, i1, i2, 0.5 * __dadd_rn(dx1, t1), 0.5 * __dadd_rn(dx2, t2), ex, s, c);
+  const double o2 = 0.5 * __dadd_rn(dx2, t2);
+  inc_point64(g, tb, i1, i2, 0.5 * __dadd_rn(dx1, t1), o2, __dadd_rn((double)i2, o2), ex, s, c);
   const double s2 = s * s, r2 = ex * ex, f = g.dxi * ex;
   const double Sig = fma(g.a2, c * c, r2), M2r = g.M2 * ex, S2 = Sig + M2r;
   const double Rr = r2 + g.a2, A = fma(Rr, Rr, -(g.a2 * s2 * (Rr - M2r)));

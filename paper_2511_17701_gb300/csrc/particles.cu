@@ -1202,9 +1202,6 @@ __device__ __forceinline__ bool push_axis(const GridP &g, const FieldPtrsT<float
     u[1] = -u[1];
     count(diag, DG_REFLECT);
   }
-  // the stored position is what the next step and the deposit start from
-  e1 = DF(e1.hi);
-  e2 = DF(e2.hi);
   s.i1[k] = j1; s.i2[k] = j2; s.dx1[k] = e1.hi; s.dx2[k] = e2.hi;
   s.u1[k] = u[0].hi; s.u2[k] = u[1].hi; s.u3[k] = u[2].hi;
   if (j1 < 0) { s.tag[k] = 2; count(diag, DG_LEFT_INNER); }
@@ -1326,7 +1323,6 @@ __global__ void __launch_bounds__(TPB, GRPIC_PUSH64_MIN_BLOCKS)
   }
 }
 
-constexpr int64_t APART_MAX = 1 << 18;
 // Whether a run's FP64 pushes may take the increment form: the refined iterations on the
 // plain grid, with rows away from the axes clear of the small-angle clamp.
 bool inc_applies(const GridP &g) {
@@ -1800,7 +1796,7 @@ cudaError_t push_impl(const GridP &g, const FieldPtrsT<T> &F, SpeciesDevT<T> s,
     // a push of fewer warps than the GPU holds runs beside that of the species before it: on
     // 64^2 cells (1024 warps a species) the two took 2 x 95 us one behind the other
     cudaStream_t st = ps.main;
-    if (ps.apart && n_bound < APART_MAX) {
+    if (push_apart(ps.apart, n_bound)) {
       cudaError_t e;
       st = ps.side;
       if ((e = cudaEventRecord(ps.fork, ps.main)) != cudaSuccess) return e;

@@ -34,7 +34,7 @@ __device__ __forceinline__ void strong_frame(const GridP &g, const FieldPtrsT<do
                                              const PushTables &tb, int i1, int i2, double dx1,
                                              double dx2, double qm, Strong &w) {
   double r, s, c;
-  inc_point64(g, tb, i1, i2, dx1, dx2, r, s, c);
+  inc_point64(g, tb, i1, i2, dx1, dx2, __dadd_rn((double)i2, dx2), r, s, c);
   const double s2 = s * s, r2 = r * r, f = g.dxi * r;
   const double Sig = fma(g.a2, c * c, r2), M2r = g.M2 * r, S2 = Sig + M2r;
   const double Rr = r2 + g.a2, A = fma(Rr, Rr, -(g.a2 * s2 * (Rr - M2r)));
@@ -147,7 +147,7 @@ __device__ __forceinline__ void strong_geodesic(const GridP &g, const PushTables
                                                 int i2, double dx1, double dx2, double m2,
                                                 DF d0, DF d1, double u[3]) {
   Pt<double> p;
-  inc_point64(g, tb, i1, i2, dx1, dx2, p.r, p.s, p.c);
+  inc_point64(g, tb, i1, i2, dx1, dx2, __dadd_rn((double)i2, dx2), p.r, p.s, p.c);
   p.f = g.dxi * p.r;
   p.gg = g.dth;
   p.igg = g.ig2;
@@ -166,7 +166,9 @@ __device__ __forceinline__ bool push_inc(const GridP &g, const FieldPtrsT<double
                                          const PushTables &tb, const SpeciesDevT<double> &s,
                                          int64_t kp, unsigned long long *diag) {
   const int i1 = s.i1[kp], i2 = s.i2[kp];
-  if (!(i2 >= 0 && i2 < g.n_th && i1 >= 0 && i1 < g.n_r)) return false;
+  // (the row on the axis theta = pi: dphi/dt there follows every rounding of absolute positions
+  // that large, so push64's own sequence of them is kept)
+  if (!(i2 >= 0 && i2 < g.n_th - 1 && i1 >= 0 && i1 < g.n_r)) return false;
   const bool em = s.m2 != 0.0, axis = i2 < 2 || i2 >= g.n_th - 2;
   const double dx1 = s.dx1[kp], dx2 = s.dx2[kp];
   const IncC k = inc_c(g);
@@ -266,13 +268,26 @@ __device__ __forceinline__ bool push_inc(const GridP &g, const FieldPtrsT<double
     e2 = 1.0 - e2;
     c2 = j2 - i2;
     un[1] = -un[1];
-    // dphi/dt at the midpoint of x^n and the reflected x^{n+1}, clear of the small-angle clamp
+    // the midpoint of x^n and the reflected x^{n+1}, below, has to be clear of the small-angle clamp
     const double b2 = (double)c2 + e2;
     const float mid = 0.5f * (f32_trunc(dx2) + f32_trunc(b2)) + (float)(j2 == 0 ? i2 : i2 + 1 - g.n_th);
     if (!axis || fabsf(mid - (j2 == 0 ? 0.0f : 1.0f)) * g.f_dth < 2.0f * g.d_ss[0]) return false;
-    double n1, n2;
-    inc_coord64(g, tb, i1, i2, dx1, dx2, un, s.m2, t1, b2, n1, n2, v3);
     count(diag, DG_REFLECT);
+  }
+  if (axis) {
+    // dphi/dt varies by order one over the distance to the axis, which next to theta = pi makes
+    // it sensitive to how the midpoint is rounded: as push64 rounds it, from the absolute positions
+    const double p1 = i1, p2 = i2;
+    const double m1 = 0.5 * __dadd_rn(__dadd_rn(p1, dx1), __dadd_rn((double)j1, e1));
+    const double m2 = 0.5 * __dadd_rn(__dadd_rn(p2, dx2), __dadd_rn((double)j2, e2));
+    Pt<double> p;
+    inc_point64(g, tb, i1, i2, m1 - p1, m2 - p2, m2, p.r, p.s, p.c);
+    p.f = g.dxi * p.r;
+    p.gg = g.dth;
+    p.igg = g.ig2;
+    p.gp = 0.0;
+    double v1, v2;
+    velocity64<false>(g, p, un, s.m2, v1, v2, v3);
   }
   s.i1[kp] = j1; s.i2[kp] = j2; s.dx1[kp] = e1; s.dx2[kp] = e2;
   s.u1[kp] = un[0]; s.u2[kp] = un[1]; s.u3[kp] = un[2];
