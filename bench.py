@@ -42,7 +42,7 @@ METRIC = ("particle-steps/sec (push+deposit+field) & % HBM roofline, FP64 vs mix
 
 # Algorithmic bytes of one particle-step of the dominant kernel of each precision, as the
 # bench runs it (the fused push + deposit stores no previous positions):
-# FP64 k_push<deposit> reads i1, i2, dx1, dx2, u1, u2, u3, phi, w, tag (4+4+8+8+24+8+8+1 =
+# FP64 k_push_inc<deposit> reads i1, i2, dx1, dx2, u1, u2, u3, phi, w, tag (4+4+8+8+24+8+8+1 =
 # 65 B) and writes all of them but w (57 B): 122 B.
 FP64_BYTES_PER_PARTICLE_STEP = 65 + 57
 # Mixed k_push32<deposit>: FP32 offsets, momenta, phi and w and the guard bitmask read
@@ -55,24 +55,26 @@ GRID_BYTES_PER_CELL = {"fp64": 33 * 8, "mixed": 33 * 4}
 
 # Executed work and DRAM traffic per particle of the dominant kernels, from ncu captures of
 # the kernel sources whose digest is `src` (profiles/): FP64-pipe operations (DFMA + DMUL +
-# DADD thread instructions) of k_push<deposit>, warp instructions of k_push32<deposit>, and
+# DADD thread instructions) of k_push_inc<deposit>, warp instructions of k_push32<deposit>, and
 # dram__bytes_read.sum + dram__bytes_write.sum per particle. When the sources change the
 # counts are reported as stale and the traffic as null until they are captured again.
 KERNEL_COUNTS = {
-    "fp64": {"src": "396195e5c4b7c291",
-             "workload": "wald2048; operations from ncu --set full of one launch at 1 particle "
-                         "per cell per species (4,194,304 particles), DRAM bytes from a one-pass "
-                         "capture of a full launch (67,108,864 particles)",
-             "fp64_ops": 198.63 + 269.56 + 94.10, "flop": 2 * 198.63 + 269.56 + 94.10,
-             "dram_bytes": (4712624896 + 3813730816) / 67108864},
-    "mixed": {"src": "396195e5c4b7c291",
-              "workload": "wald2048; warp instructions from ncu --set full of one launch at 1 "
-                          "particle per cell per species, DRAM bytes from a one-pass capture of a "
-                          "full launch (67,108,864 particles)",
-              "warp_inst": 168257970 / 4194304,
+    "fp64": {"src": "23bfe67d759bc726",
+             "workload": "wald2048; operations from ncu of one launch at 1 particle per cell per "
+                         "species (4,194,304 particles), DRAM bytes from a one-pass capture of a "
+                         "full launch (67,108,864 particles)",
+             "fp64_ops": (189295783 + 151432644 + 146901615) / 4194304,
+             "flop": (189295783 + 151432644 + 2 * 146901615) / 4194304,
+             "dram_bytes": (4717784576 + 3834690560) / 67108864},
+    "mixed": {"src": "23bfe67d759bc726",
+              "workload": "wald2048; warp instructions from ncu of one launch at 1 particle per "
+                          "cell per species, DRAM bytes from a one-pass capture of a full launch "
+                          "(67,108,864 particles)",
+              "warp_inst": 163906694 / 4194304,
               "dram_bytes": (2653071872 + 2371053056) / 67108864},
 }
-KERNEL_SOURCES = ("particles.cu", "pusher.cuh", "dfloat.cuh", "grpic_internal.cuh")
+KERNEL_SOURCES = ("particles.cu", "push_inc.cuh", "inc.cuh", "refine.cuh", "pusher.cuh", "dfloat.cuh",
+                  "grpic_internal.cuh")
 
 
 def kernel_src_digest() -> str:
@@ -193,7 +195,7 @@ def allreduce_sum(ws, x, device):
 
 
 PRECISION_DESC = {"fp64": "FP64",
-                  "mixed": "mixed precision (FP32 state, fields and currents; FP64 metric "
+                  "mixed": "mixed precision (FP32 state, fields and currents; 48-bit metric "
                            "within 4 cells of the horizon and the axes)"}
 
 
@@ -517,7 +519,8 @@ def rooflines(out, precision, alu, args, photons=False):
                 "nominal_peak_at_sampled_clock": 2 * sms * mhz / 1e3 if (sms and mhz) else None,
                 "ops_per_particle": kc["fp64_ops"],
                 "tflops": parts * kc["flop"] / (kms * 1e-3) / 1e12,
-                "kernel": "k_push<deposit> (fused FP64 push + deposit)"}
+                "kernel": "k_push_inc<deposit> (fused FP64 push + deposit, momentum increments in "
+                          "float pairs) and k_push_rest"}
         bpp = FP64_BYTES_PER_PARTICLE_STEP
     else:
         ach = parts * kc["warp_inst"] / (kms * 1e-3) / 1e9
@@ -713,7 +716,7 @@ def run_gpu(args, ws, rank, local):
                 "value": main["value"], "unit": "particle-steps/s", "n_gpus": ws,
                 "steps": args.steps, "warmup": args.warmup, "ms_per_step": main["ms_per_step"],
                 "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-                "dtype": "f64" if precisions[0] == "fp64" else "f32 (f64 metric in the guard zones)",
+                "dtype": "f64" if precisions[0] == "fp64" else "f32 (48-bit metric in the guard zones)",
                 "data": "synthetic (seeded workload generator)",
                 "config": {"workload": main["workload"],
                            "sort_every": args.sort_every, "tile": args.tile,
