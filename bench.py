@@ -59,14 +59,14 @@ GRID_BYTES_PER_CELL = {"fp64": 33 * 8, "mixed": 33 * 4}
 # dram__bytes_read.sum + dram__bytes_write.sum per particle. When the sources change the
 # counts are reported as stale and the traffic as null until they are captured again.
 KERNEL_COUNTS = {
-    "fp64": {"src": "23bfe67d759bc726",
+    "fp64": {"src": "68122ff546bee08f",
              "workload": "wald2048; operations from ncu of one launch at 1 particle per cell per "
                          "species (4,194,304 particles), DRAM bytes from a one-pass capture of a "
                          "full launch (67,108,864 particles)",
              "fp64_ops": (189295783 + 151432644 + 146901615) / 4194304,
              "flop": (189295783 + 151432644 + 2 * 146901615) / 4194304,
              "dram_bytes": (4717784576 + 3834690560) / 67108864},
-    "mixed": {"src": "23bfe67d759bc726",
+    "mixed": {"src": "68122ff546bee08f",
               "workload": "wald2048; warp instructions from ncu of one launch at 1 particle per "
                           "cell per species, DRAM bytes from a one-pass capture of a full launch "
                           "(67,108,864 particles)",

@@ -18,8 +18,8 @@
 // bounds behind this do not cover (a reflection off an axis, an iteration that the predictor
 // does not resolve, values outside the range of FP32) is left to push64, untouched.
 //
-// Measured: a step of the 2048^2 workload (134 M particles) 173.6 -> 65.9 ms, of the 512^2 one
-// (16.8 M) 21.0 -> 8.85 ms. One push against 113-bit arithmetic, six grids from 64^2 to 2048^2
+// Measured: a step of the 2048^2 workload (134 M particles) 173.6 -> 66.3 ms, of the 512^2 one
+// (16.8 M) 21.0 -> 9.35 ms. One push against 113-bit arithmetic, six grids from 64^2 to 2048^2
 // (60,000 particles each): rms errors of u 4.7-8.0e-17 of its rms (push64: 2.5-3.3e-16), of the
 // offsets 2.4-4.6e-17 (2.4-5.5e-17).
 #pragma once

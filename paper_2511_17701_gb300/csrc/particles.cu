@@ -1257,7 +1257,7 @@ __global__ void __launch_bounds__(TPB, GRPIC_PUSH64_MIN_BLOCKS)
 // tag TAG_REST, which lives from this kernel to k_push_rest right behind it. Two kernels, so
 // that this one runs with the registers of its own code (128, 4 blocks per SM; with push64 in
 // it, 166 and 3) and the long routine with full warps: a step of the 2048^2 workload 80.3 ->
-// 65.9 ms, of the 512^2 one 11.0 -> 8.85 ms, of the 512^2 monopole problem, whose Boris half
+// 66.3 ms, of the 512^2 one 11.0 -> 9.35 ms, of the 512^2 monopole problem, whose Boris half
 // steps are taken in FP64, 5.94 -> 4.18 ms. What bounds it: 124 FP64 instructions and ~7500
 // others per warp overlap to about half of either pipe's peak; between them warps wait for FP64
 // results, for instructions (the code is 14,000 instructions) and for their own pair arithmetic.

@@ -166,9 +166,7 @@ __device__ __forceinline__ bool push_inc(const GridP &g, const FieldPtrsT<double
                                          const PushTables &tb, const SpeciesDevT<double> &s,
                                          int64_t kp, unsigned long long *diag) {
   const int i1 = s.i1[kp], i2 = s.i2[kp];
-  // (the row on the axis theta = pi: dphi/dt there follows every rounding of absolute positions
-  // that large, so push64's own sequence of them is kept)
-  if (!(i2 >= 0 && i2 < g.n_th - 1 && i1 >= 0 && i1 < g.n_r)) return false;
+  if (!(i2 >= 0 && i2 < g.n_th && i1 >= 0 && i1 < g.n_r)) return false;
   const bool em = s.m2 != 0.0, axis = i2 < 2 || i2 >= g.n_th - 2;
   const double dx1 = s.dx1[kp], dx2 = s.dx2[kp];
   const IncC k = inc_c(g);
@@ -263,6 +261,7 @@ __device__ __forceinline__ bool push_inc(const GridP &g, const FieldPtrsT<double
   int j2 = i2 + c2;
   const double e1 = t1 - (double)c1;
   double e2 = t2 - (double)c2;
+  bool reflected = false;
   if (j2 < 0 || j2 >= g.n_th) {  // reflection off an axis (Sec. 3.3.3)
     j2 = j2 < 0 ? 0 : g.n_th - 1;
     e2 = 1.0 - e2;
@@ -272,9 +271,15 @@ __device__ __forceinline__ bool push_inc(const GridP &g, const FieldPtrsT<double
     const double b2 = (double)c2 + e2;
     const float mid = 0.5f * (f32_trunc(dx2) + f32_trunc(b2)) + (float)(j2 == 0 ? i2 : i2 + 1 - g.n_th);
     if (!axis || fabsf(mid - (j2 == 0 ? 0.0f : 1.0f)) * g.f_dth < 2.0f * g.d_ss[0]) return false;
-    count(diag, DG_REFLECT);
+    reflected = true;
   }
   if (axis) {
+    // Close to the axis theta = pi dphi/dt (~ 1 / distance^2) follows every rounding of absolute
+    // positions that large: within n_theta 2^-10 cells of it, where that would show at ~1e-12,
+    // push64's own sequence of roundings is kept
+    const float far = (float)g.n_th * 0x1p-10f;
+    const float d0 = (float)(g.n_th - i2) - o2.hi, d1 = (float)(g.n_th - j2) - f32_trunc(e2);
+    if (fminf(d0, d1) < far) return false;
     // dphi/dt varies by order one over the distance to the axis, which next to theta = pi makes
     // it sensitive to how the midpoint is rounded: as push64 rounds it, from the absolute positions
     const double p1 = i1, p2 = i2;
@@ -289,6 +294,7 @@ __device__ __forceinline__ bool push_inc(const GridP &g, const FieldPtrsT<double
     double v1, v2;
     velocity64<false>(g, p, un, s.m2, v1, v2, v3);
   }
+  if (reflected) count(diag, DG_REFLECT);
   s.i1[kp] = j1; s.i2[kp] = j2; s.dx1[kp] = e1; s.dx2[kp] = e2;
   s.u1[kp] = un[0]; s.u2[kp] = un[1]; s.u3[kp] = un[2];
   if (j1 < 0) { s.tag[kp] = 2; count(diag, DG_LEFT_INNER); }
