@@ -1324,9 +1324,12 @@ __global__ void __launch_bounds__(TPB, GRPIC_PUSH64_MIN_BLOCKS)
 }
 
 // Whether a run's FP64 pushes may take the increment form: the refined iterations on the
-// plain grid, with rows away from the axes clear of the small-angle clamp.
+// plain grid, with rows away from the axes clear of the small-angle clamp, and a time step that
+// is far from the ends of a pair's range (2^-126, 2^128), as its products with velocities and
+// charges then are.
 bool inc_applies(const GridP &g) {
-  return !g.qks && g.iter_tol > 0.0 && g.n_iter >= 2 && g.small_angle < g.dth;
+  return !g.qks && g.iter_tol > 0.0 && g.n_iter >= 2 && g.small_angle < g.dth &&
+         g.dt >= 0x1p-40 && g.dt <= 0x1p40;
 }
 
 // Mixed path, classification: zone 1 and zone 2 particles are appended to their lists

@@ -96,14 +96,33 @@ __device__ __forceinline__ int inc_cell(double t) {
   return a == 0 ? 0 : (a > one ? -2 : -1);
 }
 
+// q = qc w of one particle. The unit of charge is the caller's, so q may lie anywhere in FP64's
+// range, far outside that of a pair: the deposit in pairs takes q's fraction, in [1, 2), and the
+// power of two goes back onto each contribution, exactly, on the integer pipe (add_scaled).
+// Whether q's exponent leaves room for that (and q is finite); zero does.
+__device__ __forceinline__ bool inc_charge(double q) {
+  const unsigned h = (unsigned)__double2hiint(q) & 0x7fffffffu, ex = h >> 20;
+  return (ex >= 1023u - 860u && ex <= 1023u + 900u) || (h | (unsigned)__double2loint(q)) == 0u;
+}
+// adds v 2^e, e in the upper word's exponent field; |v| is 0 or in [2^-126, 2^100]
+__device__ __forceinline__ void add_scaled(double *p, DF v, int e) {
+  const double x = df_to_double(v);
+  const int h = __double2hiint(x);
+  atomicAdd(p, (h << 1) == 0 ? x : __hiloint2double(h + e, __double2loint(x)));
+}
+
 // deposit64 in pairs, relative to the start cell: the end points a, b are the positions as
 // deposit64 rounds them (absolute coordinates: a multiple of their last place, at most 48
 // bits, so a pair holds them exactly), the rest of its ~70 FP64 operations is in pairs. The
 // pairs' 2^-47 is below that rounding's share of a move. (i, j): the start cell, (c1, c2): the
 // end cell relative to it.
-__device__ __forceinline__ void inc_deposit(const GridP &g, const FieldPtrsT<double> &F, DF q,
-                                            DF idt, int i, int j, DF a1, DF a2, int c1, int c2,
-                                            DF b1, DF b2, DF v3) {
+__device__ __forceinline__ void inc_deposit(const GridP &g, const FieldPtrsT<double> &F,
+                                            double charge, DF idt, int i, int j, DF a1, DF a2,
+                                            int c1, int c2, DF b1, DF b2, DF v3) {
+  const int qh = __double2hiint(charge);
+  const bool some = (qh << 1) != 0;
+  const int e = some ? (qh & 0x7ff00000) - 0x3ff00000 : 0;  // q = 2^e times its fraction
+  const DF q = df_of(__hiloint2double(some ? qh - e : qh, __double2loint(charge)));
   const int NX = g.NX;
   const DF qi = q * idt;
   const DF m1 = df_scale(a1 + b1, 0.5f), m2 = df_scale(a2 + b2, 0.5f);
@@ -115,29 +134,29 @@ __device__ __forceinline__ void inc_deposit(const GridP &g, const FieldPtrsT<dou
   {
     const DF F1 = qi * (r1 - a1), F2 = qi * (r2 - a2);
     const DF t = F1 * df_scale(a2 + r2, 0.5f), s = F2 * df_scale(a1 + r1, 0.5f);
-    atomicAdd(J1 + ka, df_to_double(F1 - t));
-    atomicAdd(J1 + ka + NX, df_to_double(t));
-    atomicAdd(J2 + ka, df_to_double(F2 - s));
-    atomicAdd(J2 + ka + 1, df_to_double(s));
+    add_scaled(J1 + ka, F1 - t, e);
+    add_scaled(J1 + ka + NX, t, e);
+    add_scaled(J2 + ka, F2 - s, e);
+    add_scaled(J2 + ka + 1, s, e);
   }
   {
     const DF F1 = qi * (b1 - r1), F2 = qi * (b2 - r2);
     const DF t = F1 * (df_scale(r2 + b2, 0.5f) + DF(-(float)c2));
     const DF s = F2 * (df_scale(r1 + b1, 0.5f) + DF(-(float)c1));
-    atomicAdd(J1 + kb, df_to_double(F1 - t));
-    atomicAdd(J1 + kb + NX, df_to_double(t));
-    atomicAdd(J2 + kb, df_to_double(F2 - s));
-    atomicAdd(J2 + kb + 1, df_to_double(s));
+    add_scaled(J1 + kb, F1 - t, e);
+    add_scaled(J1 + kb + NX, t, e);
+    add_scaled(J2 + kb, F2 - s, e);
+    add_scaled(J2 + kb + 1, s, e);
   }
   const int n1 = inc_floor(m1), n2 = inc_floor(m2);
   const DF w1 = m1 + DF(-(float)n1), w2 = m2 + DF(-(float)n2);
   const int64_t k = sidx(g, i + n1, j + n2);
   const DF qv = q * v3, x = qv * w1, y = qv - x;
   const DF xt = x * w2, yt = y * w2;
-  atomicAdd(J3 + k, df_to_double(y - yt));
-  atomicAdd(J3 + k + 1, df_to_double(x - xt));
-  atomicAdd(J3 + k + NX, df_to_double(yt));
-  atomicAdd(J3 + k + NX + 1, df_to_double(xt));
+  add_scaled(J3 + k, y - yt, e);
+  add_scaled(J3 + k + 1, x - xt, e);
+  add_scaled(J3 + k + NX, yt, e);
+  add_scaled(J3 + k + NX + 1, xt, e);
 }
 
 // The geodesic substep's increment (d0, d1) from u in FP64, where it is large against u (next to
@@ -167,6 +186,7 @@ __device__ __forceinline__ bool push_inc(const GridP &g, const FieldPtrsT<double
                                          int64_t kp, unsigned long long *diag) {
   const int i1 = s.i1[kp], i2 = s.i2[kp];
   if (!(i2 >= 0 && i2 < g.n_th && i1 >= 0 && i1 < g.n_r)) return false;
+  if (DEPOSIT && !inc_charge(s.qc * s.w[kp])) return false;
   const bool em = s.m2 != 0.0, axis = i2 < 2 || i2 >= g.n_th - 2;
   const double dx1 = s.dx1[kp], dx2 = s.dx2[kp];
   const IncC k = inc_c(g);
@@ -302,7 +322,7 @@ __device__ __forceinline__ bool push_inc(const GridP &g, const FieldPtrsT<double
   s.phi[kp] = s.phi[kp] + g.dt * v3;
   if (DEPOSIT) {
     const double p1 = i1, p2 = i2;
-    inc_deposit(g, F, df_of(s.qc * s.w[kp]), df_of(g.idt), i1, i2,
+    inc_deposit(g, F, s.qc * s.w[kp], df_of(g.idt), i1, i2,
                 df_of(__dadd_rn(__dadd_rn(p1, dx1), -p1)), df_of(__dadd_rn(__dadd_rn(p2, dx2), -p2)),
                 c1, c2, df_of(__dadd_rn(__dadd_rn((double)j1, e1), -p1)),
                 df_of(__dadd_rn(__dadd_rn((double)j2, e2), -p2)), df_of(v3));

@@ -1,0 +1,56 @@
+"""FP64 pushes of particles whose charge, momentum or field lies outside what a pair of FP32
+numbers resolves: the units of charge, of a photon's momentum and of the field are the caller's.
+One step at a small iter_tol, which takes the push's increment form, against the oracle. Tolerance:
+1e-12 relative per step, as for every FP64 push (tests/parity.py); all results scale with the
+unit, so the same relative bound holds in each."""
+import numpy as np
+import pytest
+
+import workloads as W
+from oracle import oracle as O
+from paper_2511_17701_gb300.binding import J01
+from parity import gpu_from_oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def torch_cuda():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    return torch
+
+
+def particles(cfg, n, seed, umag):
+    rng = np.random.default_rng(seed)
+    pos = dict(i1=rng.integers(3, cfg["n_r"] - 2, n).astype(np.int32),
+               i2=rng.integers(1, cfg["n_theta"] - 1, n).astype(np.int32),
+               dx1=rng.random(n), dx2=rng.random(n))
+    uh = rng.standard_normal((3, n))
+    return pos, uh * umag / np.linalg.norm(uh, axis=0)
+
+
+@pytest.mark.parametrize("k", [-800, -130, -107, -80, 120, 127, 700])
+def test_charge_unit(torch_cuda, k):
+    """A charge 2^k times as large deposits 2^k times the current: every contribution exactly,
+    their sums up to the order of the additions (a few of them per node, 2^-53 each; the nodes'
+    sums of absolute values are the oracle's)."""
+    cfg = W.grid_config("wald64")
+    osim = O.OracleSim(cfg)
+    osim.init_fields(O.FIELD_WALD, 1.0)
+    n = 4000
+    pos, uh = particles(cfg, n, 3, 1.0)
+    osim.add_species(pos, uh, 0.1 * np.ones(n), 1.0, -0.2)
+    g = gpu_from_oracle(osim, iter_tol=1e-12, sort_every=0)
+    J = []
+    for scale in (1.0, 2.0 ** k):
+        g.set_planes(osim.F)
+        g.set_particles(0, osim.species[0].view(), 1.0, -0.2 * scale)
+        g.step(1)
+        J.append(g.planes()[J01:J01 + 3] / scale)
+    osim.predict()
+    osim.push(0)
+    osim.deposit()
+    assert np.abs(J[0]).max() > 0.0
+    assert np.all(np.abs(J[1] - J[0]) <= 2.0 ** -50 * osim.F[O.JA1:O.JA1 + 3])
