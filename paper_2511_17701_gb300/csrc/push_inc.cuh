@@ -159,6 +159,21 @@ __device__ __forceinline__ void inc_deposit(const GridP &g, const FieldPtrsT<dou
   add_scaled(J3 + k + NX + 1, xt, e);
 }
 
+// A massless particle's momentum has no scale: the step's equations keep their form under u -> c u.
+// The pairs take it in a unit, the power of two that brings its largest component to [1, 2)
+// (exactly). False: beyond 2^+-480, where FP64's squares end too.
+__device__ __forceinline__ bool photon_unit(double u[3], double &unit) {
+  int top = 0;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) top = max(top, __double2hiint(u[q]) & 0x7ff00000);
+  if (top < ((1023 - 480) << 20) || top > ((1023 + 480) << 20)) return false;
+  unit = __hiloint2double(top, 0);
+  const double down = __hiloint2double((2046 << 20) - top, 0);
+#pragma unroll
+  for (int q = 0; q < 3; ++q) u[q] *= down;
+  return true;
+}
+
 // The geodesic substep's increment (d0, d1) from u in FP64, where it is large against u (next to
 // the axes, where the metric changes by order one over a step): the FP64 map's image of the
 // point that the pairs found
@@ -191,7 +206,8 @@ __device__ __forceinline__ bool push_inc(const GridP &g, const FieldPtrsT<double
   const double dx1 = s.dx1[kp], dx2 = s.dx2[kp];
   const IncC k = inc_c(g);
   const DF o1 = df_of(dx1), o2 = df_of(dx2);
-  double un[3] = {s.u1[kp], s.u2[kp], s.u3[kp]};
+  double un[3] = {s.u1[kp], s.u2[kp], s.u3[kp]}, unit = 1.0;
+  if (!em && !photon_unit(un, unit)) return false;
   DF ud[3] = {df_of(un[0]), df_of(un[1]), df_of(un[2])};
   {
     const DF u[3] = {ud[0], ud[1], ud[2]};
@@ -313,6 +329,10 @@ __device__ __forceinline__ bool push_inc(const GridP &g, const FieldPtrsT<double
     p.gp = 0.0;
     double v1, v2;
     velocity64<false>(g, p, un, s.m2, v1, v2, v3);
+  }
+  if (!em) {
+#pragma unroll
+    for (int q = 0; q < 3; ++q) un[q] *= unit;
   }
   if (reflected) count(diag, DG_REFLECT);
   s.i1[kp] = j1; s.i2[kp] = j2; s.dx1[kp] = e1; s.dx2[kp] = e2;

@@ -9,7 +9,7 @@ import pytest
 import workloads as W
 from oracle import oracle as O
 from paper_2511_17701_gb300.binding import J01
-from parity import gpu_from_oracle
+from parity import assert_particles, gpu_from_oracle
 
 pytestmark = pytest.mark.gpu
 
@@ -54,3 +54,19 @@ def test_charge_unit(torch_cuda, k):
     osim.deposit()
     assert np.abs(J[0]).max() > 0.0
     assert np.all(np.abs(J[1] - J[0]) <= 2.0 ** -50 * osim.F[O.JA1:O.JA1 + 3])
+
+
+@pytest.mark.parametrize("umag", [1e30, 1e3, 1e-3, 1e-14, 1e-18, 1e-30])
+def test_photon_momentum_unit(torch_cuda, umag):
+    cfg = W.grid_config("wald64")
+    osim = O.OracleSim(cfg)
+    osim.init_fields(O.FIELD_WALD, 1.0)
+    n = 4000
+    pos, uh = particles(cfg, n, 5, umag)
+    osim.add_species(pos, uh, 0.1 * np.ones(n), 1.0, 0.0, massless=True)
+    g = gpu_from_oracle(osim, iter_tol=1e-12, massless=[0])
+    osim.predict()
+    g.predict()
+    osim.push(0)
+    g.push(0)
+    assert_particles(g.get_particles(0), osim.species[0].view())
