@@ -220,7 +220,10 @@ __device__ __forceinline__ bool push_inc(const GridP &g, const FieldPtrsT<double
     }
     DF eD[3], eB[3];
     Strong w;
-    bool weak = !em || __all_sync(__activemask(), inc_small(g, F, tb, i1, i2, s.f_qm));
+    // (far outside this range of q/m the force's factors, not the force, leave FP32's range)
+    const float qm = fabsf(s.f_qm);
+    bool weak = !em || (((qm >= 0x1p-60f && qm <= 0x1p30f) || s.qm == 0.0) &&
+                        __all_sync(__activemask(), inc_small(g, F, tb, i1, i2, s.f_qm)));
     if (em && weak) {
       IncLerp l;
       inc_lerp(i1, i2, o1, o2, l);

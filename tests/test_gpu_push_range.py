@@ -70,3 +70,19 @@ def test_photon_momentum_unit(torch_cuda, umag):
     osim.push(0)
     g.push(0)
     assert_particles(g.get_particles(0), osim.species[0].view())
+
+
+@pytest.mark.parametrize("B0,qm", [(1e-22, 1e20), (1e-27, 1e24), (1e-35, 1e35), (1e25, 1e-25)])
+def test_field_unit(torch_cuda, B0, qm):
+    cfg = W.grid_config("wald64")
+    osim = O.OracleSim(cfg)
+    osim.init_fields(O.FIELD_WALD, B0)
+    n = 4000
+    pos, uh = particles(cfg, n, 7, 0.3)
+    osim.add_species(pos, uh, 0.1 * np.ones(n), qm, 0.2)
+    g = gpu_from_oracle(osim, iter_tol=1e-12)
+    osim.predict()
+    g.predict()
+    osim.push(0)
+    g.push(0)
+    assert_particles(g.get_particles(0), osim.species[0].view())
