@@ -6,8 +6,8 @@
 namespace {
 
 // An FP32 estimate of whether a Boris half step stays below INC_MAX for a momentum of order 1
-// (fields of one node, no interpolation): where it does not, the warp takes both half steps in
-// FP64 at once. Only speed depends on it.
+// (fields of one node, no interpolation): where it does not, both half steps are taken in FP64
+// at once, without trying the pairs first.
 __device__ __forceinline__ bool inc_small(const GridP &g, const FieldPtrsT<double> &F,
                                           const PushTables &tb, int i1, int i2, float f_qm) {
   const float r = __ldg(tb.r + i1 + G_), s = __ldg(tb.s + i2 + G_), c = __ldg(tb.c + i2 + G_);
@@ -220,10 +220,12 @@ __device__ __forceinline__ bool push_inc(const GridP &g, const FieldPtrsT<double
     }
     DF eD[3], eB[3];
     Strong w;
-    // (far outside this range of q/m the force's factors, not the force, leave FP32's range)
+    // (far outside this range of q/m the force's factors, not the force, leave FP32's range). The
+    // two forms round differently, so each particle decides for itself: a vote of the warp would
+    // make its bits depend on the particles beside it.
     const float qm = fabsf(s.f_qm);
     bool weak = !em || (((qm >= 0x1p-60f && qm <= 0x1p30f) || s.qm == 0.0) &&
-                        __all_sync(__activemask(), inc_small(g, F, tb, i1, i2, s.f_qm)));
+                        inc_small(g, F, tb, i1, i2, s.f_qm));
     if (em && weak) {
       IncLerp l;
       inc_lerp(i1, i2, o1, o2, l);
