@@ -337,6 +337,7 @@ __device__ __noinline__ void step_jacobian(const GridP &g, const FieldPtrsT<doub
 // ---------------------------------------------------------------------------------
 constexpr int INC_MIN_ITER = 16;   // iteration counts below are taken literally (general form)
 constexpr float INC_ADJ_TOL = 1e-16f;
+constexpr IncLimit ADJ_LIMIT = {0x1p-8f, 0x1p-4f};  // increments up to 1/16 of max(|u|, 1/4)
 
 struct AdjStep {
   int i1, i2;
@@ -384,20 +385,21 @@ __device__ __forceinline__ bool adj_inc_step(const GridP &g, const FieldPtrsT<do
     a.eD[q] = scale * a.eD1[q];
     a.u[q] = df_of(st[3 + q]);
   }
-  if (!inc_boris(a.L, a.eD, a.eB, a.u, du)) return false;
+  if (!inc_boris(a.L, a.eD, a.eB, a.u, ADJ_LIMIT, du)) return false;
 #pragma unroll
   for (int q = 0; q < 3; ++q) a.u1[q] = a.u[q] + du[q];
   GeoInc<DF> m;
   geo_inc_setup(k, a.L, a.u1, 1.0f, m);
-  if (geo_inc_solve<false>(m, a.L.G.H33.hi * a.u[2].hi * a.u[2].hi, n_iter, INC_ADJ_TOL, a.dg[0],
-                           a.dg[1]) != GEO_SMALL)
+  float rho;
+  if (geo_inc_solve<false>(m, a.L.G.H33.hi * a.u[2].hi * a.u[2].hi, n_iter, INC_ADJ_TOL,
+                           ADJ_LIMIT, a.dg[0], a.dg[1], rho) != GEO_SMALL)
     return false;
   du[0] = du[0] + a.dg[0];
   du[1] = du[1] + a.dg[1];
   a.u2[0] = a.u[0] + du[0];
   a.u2[1] = a.u[1] + du[1];
   a.u2[2] = a.u1[2];
-  if (!inc_boris(a.L, a.eD, a.eB, a.u2, du)) return false;
+  if (!inc_boris(a.L, a.eD, a.eB, a.u2, ADJ_LIMIT, du)) return false;
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
     a.un[q] = a.u[q] + du[q];

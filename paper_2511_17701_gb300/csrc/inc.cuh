@@ -4,19 +4,19 @@
 //
 // GB300 executes 2 FP64 operations per clock and SM against 128 FP32 ones, and the FP64
 // routine (push64) needs ~560 of them per particle. But everything a step computes for the
-// momentum ends in an increment that is a small part of u: u^{n+1} = u^n + du. An increment
-// of relative size eps, computed in pairs of floats (dfloat.cuh, relative error ~2^-48),
-// leaves an error of eps 2^-48 in u, which for eps <= 2^-4 is at or below what the FP64
-// routine's own rounding leaves (3e-16 of |u| rms). So the metric and its derivatives at x^n, the tetrads, the field interpolation,
-// both Boris half steps and the geodesic substep are evaluated in float pairs, as
+// momentum ends in an increment that is mostly a small part of u: u^{n+1} = u^n + du. An
+// increment of at most 2^-5 of |u|, computed in pairs of floats (dfloat.cuh, relative error
+// ~2^-48), leaves an error of 2^-53 in u, below what the FP64 routine's own rounding leaves
+// (3e-16 of |u| rms). So the metric and its derivatives at x^n, the tetrads, the field
+// interpolation, both Boris half steps and the geodesic substep are evaluated in float pairs, as
 // increments, and u^n + du is formed in FP64 by one addition per component. The coordinate
 // substep is not small against the offset it changes: its result is, as in push64, one FP64
 // evaluation of the map at the predictor's point.
 //
-// Where a Boris half step turns or kicks the momentum by more than INC_MAX of itself (strong
-// fields) both are taken in FP64, the rest as above. A particle that the
-// bounds behind this do not cover (a reflection off an axis, an iteration that the predictor
-// does not resolve, values outside the range of FP32) is left to push64, untouched.
+// A half step or a geodesic substep that changes the momentum by more than INC_MAX of it (strong
+// fields, cold particles, the rows on the axes) is taken in FP64, the rest as above. A particle
+// that the bounds behind this do not cover (an iteration that the predictor does not resolve,
+// values outside the range of FP32) is left to push64, untouched.
 //
 // Measured: a step of the 2048^2 workload (134 M particles) 173.6 -> 66.3 ms, of the 512^2 one
 // (16.8 M) 21.0 -> 9.35 ms. One push against 113-bit arithmetic, six grids from 64^2 to 2048^2
@@ -28,11 +28,27 @@
 
 namespace {
 
-constexpr float INC_MAX = 0x1p-4f;   // largest |increment| / |u| of a Boris half step in pairs
-constexpr float INC_GEO = 0x1p-4f;   // the same of the geodesic substep
-// increments are measured against 1/4 (a velocity of c/4) where |u| is less: what the rest of
-// a step sees of such a momentum is its absolute error, here below 2^-54
-constexpr float INC_UU = 0x1p-4f;
+// The largest |increment| / |u| of a Boris half step or the geodesic substep that pairs take: 2^-5
+// of a relative error of about 2^-48 is 2^-53 of u. Measured, |u| = 0.1 on 64^2 in a field that
+// kicks most particles by about that: 3.9e-16 of |u| rms, 2.3e-15 at most (the FP64 routine with
+// its iterations run to rounding: 3.7e-16, 1.2e-15); |u| = 1e-3:
+// 5.3e-16 and 5.7e-15 (5.4e-16, 6.2e-15).
+// Massless particles, whose FP64 push rounds less (no half steps: 6.9e-17), take half of it.
+// floor: where |u|^2 is less than this, it is taken as this (0: never).
+constexpr float INC_MAX = 0x1p-5f;
+struct IncLimit {
+  float r2, floor;  // the ratio's square, the floor
+};
+__device__ __forceinline__ IncLimit inc_limit(float times2) {  // times sqrt(times2)
+  return {times2 * INC_MAX * INC_MAX, 0.0f};
+}
+// below this, squared, the pairs' own floor of 2^-149 would show in an increment that is not
+// exactly zero
+constexpr float INC_UU = 0x1p-100f;
+__device__ __forceinline__ bool inc_within(IncLimit lim, float dd, float uu) {
+  const float w = fmaxf(uu, lim.floor);
+  return dd <= lim.r2 * w && w >= INC_UU;
+}
 constexpr float INC_E = 0.055f;      // largest |offset of xi| of the radial series
 constexpr float INC_D = 0.035f;      // largest |offset of theta| of the angular series
 constexpr int INC_ROWS = 64;          // rows from either axis with theta as map_theta rounds it
@@ -251,12 +267,13 @@ __device__ __forceinline__ void geo_inc_setup(const IncC &k, const Local<M> &L, 
 // G + M J r with r = G - d and M = (I - J)^{-1}, leave an error of |J| 2^-24 |r|, far below the
 // pairs' rounding of d. n_iter, tol: the method's iterations and what they have to come within
 // (inc_converges), else the method's iterations themselves are run, in pairs (LITERAL). h33:
-// h^33 u_3^2. Returns GEO_SMALL; GEO_LARGE where the increment is above INC_GEO, and the point
-// (n0, n1) whose image the result is to be; GEO_NONE: not resolved.
+// h^33 u_3^2. Returns GEO_SMALL; GEO_LARGE where the increment is beyond lim, and the point
+// (n0, n1), within the pairs' rounding of the fixed point, that FP64 evaluations have to start
+// from, with the contraction rho there; GEO_NONE: not resolved.
 enum { GEO_NONE = 0, GEO_SMALL, GEO_LARGE };
 template <bool LITERAL>
 __device__ __forceinline__ int geo_inc_solve(const GeoInc<DF> &m, float h33, int n_iter, float tol,
-                                             DF &n0, DF &n1) {
+                                             IncLimit lim, DF &n0, DF &n1, float &rho) {
   const GeoInc<float> mf = {m.u0.hi,  m.u1.hi,  m.c0.hi,  m.c1.hi,  m.e1.hi,    m.e2.hi,   m.f1.hi,
                             m.f2.hi,  m.D1a.hi, m.D1b.hi, m.D2a.hi, m.D2b.hi,   m.hdt.hi,  m.H11.hi,
                             m.H22.hi, m.d1H11.hi, m.d1H22.hi, m.d2H11.hi, m.d2H22.hi};
@@ -282,27 +299,27 @@ __device__ __forceinline__ int geo_inc_solve(const GeoInc<DF> &m, float h33, int
   const float us = fmaxf(fabsf(m.u0.hi), fabsf(m.u1.hi));
   // (a NaN anywhere makes one of the comparisons false)
   const float ds = fmaxf(fabsf(n0.hi), fabsf(n1.hi));
-  DF l0 = n0, l1 = n1;  // the iterate before the last
+  bool fixed = true;
+  rho = spectral_radius(J);
   if (!(fabsf(r0) + fabsf(r1) <= fmaf(0x1p-16f, ds, 0x1p-40f) &&
         inc_converges(first, J, n_iter, tol, us))) {
     // (an iteration that does not contract amplifies the pairs' rounding as well as FP64's)
-    if (!LITERAL || !(spectral_radius(J) < 0.5f)) return GEO_NONE;
+    if (!LITERAL || !(rho < 0.5f)) return GEO_NONE;
     n0 = n1 = DF(0.0f);
+    fixed = false;
 #pragma unroll 1
-    for (int it = 0; it < n_iter; ++it) {
-      l0 = n0;
-      l1 = n1;
+    for (int it = 0; it < n_iter && !fixed; ++it) {
+      const DF l0 = n0, l1 = n1;
       geo_inc_apply(m, l0, l1, n0, n1);
-      if (n0.hi == l0.hi && n0.lo == l0.lo && n1.hi == l1.hi && n1.lo == l1.lo) break;
+      fixed = n0.hi == l0.hi && n0.lo == l0.lo && n1.hi == l1.hi && n1.lo == l1.lo;
     }
   }
   // the increment and the momentum as lengths in the tetrad frame, squared (h^13 aside)
   const float dd = fmaf(mf.H11 * n0.hi, n0.hi, mf.H22 * n1.hi * n1.hi);
   const float uu = fmaf(mf.u0, fmaf(mf.H11, mf.u0, mf.c1), fmaf(mf.H22 * mf.u1, mf.u1, h33));
-  if (dd <= INC_GEO * INC_GEO * fmaxf(uu, INC_UU)) return GEO_SMALL;
-  n0 = l0;
-  n1 = l1;
-  return dd < 0x1p60f ? GEO_LARGE : GEO_NONE;
+  const bool none = n0.hi == 0.0f && n1.hi == 0.0f;
+  if (none || inc_within(lim, dd, uu)) return GEO_SMALL;
+  return fixed && dd < 0x1p60f ? GEO_LARGE : GEO_NONE;
 }
 
 // One Boris half step's increment of the covariant u, added to du (u = u^n + du in pairs):
@@ -328,14 +345,15 @@ __device__ __forceinline__ void inc_boris_core(const Local<M> &L, const R eD[3],
   du[1] = fma_(L.sh22, x[1], du[1]);
   du[2] = fma_(L.sh33, x[2], du[2]);
 }
-// False: the increment is above INC_MAX of |u| (of 1/4, where |u| is less).
+// False: the increment is beyond lim.
 __device__ __forceinline__ bool inc_boris(const Local<DF> &L, const DF eD[3], const DF eB[3],
-                                          const DF u[3], DF du[3]) {
+                                          const DF u[3], IncLimit lim, DF du[3]) {
   DF h[3], x[3];
   inc_boris_core(L, eD, eB, u, du, h, x);
   const float xx = fmaf(x[0].hi, x[0].hi, fmaf(x[1].hi, x[1].hi, x[2].hi * x[2].hi));
   const float hh = fmaf(h[0].hi, h[0].hi, fmaf(h[1].hi, h[1].hi, h[2].hi * h[2].hi));
-  return xx <= INC_MAX * INC_MAX * fmaxf(hh, INC_UU) && hh < 0x1p60f;
+  const bool none = fabsf(x[0].hi) + fabsf(x[1].hi) + fabsf(x[2].hi) == 0.0f;
+  return (none || inc_within(lim, xx, hh)) && hh < 0x1p60f;
 }
 
 // bilinear interpolation in pairs at the cell-relative offsets (o1, o2) of cell (i1, i2) for

@@ -72,6 +72,8 @@ __device__ __forceinline__ void strong_frame(const GridP &g, const FieldPtrsT<do
     o[2] = e * fma(w.k13, v[0], w.sh33 * v[2]);
   }
 }
+// (u + hat_cov(x) with the half step's change x in that frame, not hat_cov(cov_hat(u) + x): the two
+// maps' roundings then enter with the change, not with u)
 __device__ __forceinline__ void strong_boris(const Strong &w, double u[3]) {
   const double m0 = fma(w.sH11, fma(-w.m13, u[2], u[0]), w.eD[0]);
   const double m1 = fma(w.rh22, u[1], w.eD[1]), m2 = fma(w.rh33, u[2], w.eD[2]);
@@ -80,12 +82,12 @@ __device__ __forceinline__ void strong_boris(const Strong &w, double u[3]) {
   const double sf = 2.0 * rcp_nr(fma(t0, t0, fma(t1, t1, fma(t2, t2, 1.0))));
   const double p0 = fma(m1, t2, fma(-m2, t1, m0)), p1 = fma(m2, t0, fma(-m0, t2, m1));
   const double p2 = fma(m0, t1, fma(-m1, t0, m2));
-  const double h0 = fma(sf, fma(p1, t2, -(p2 * t1)), m0 + w.eD[0]);
-  const double h1 = fma(sf, fma(p2, t0, -(p0 * t2)), m1 + w.eD[1]);
-  const double h2 = fma(sf, fma(p0, t1, -(p1 * t0)), m2 + w.eD[2]);
-  u[0] = fma(h0, w.rH11, w.k13 * h2);
-  u[1] = w.sh22 * h1;
-  u[2] = w.sh33 * h2;
+  const double x0 = fma(sf, fma(p1, t2, -(p2 * t1)), 2.0 * w.eD[0]);
+  const double x1 = fma(sf, fma(p2, t0, -(p0 * t2)), 2.0 * w.eD[1]);
+  const double x2 = fma(sf, fma(p0, t1, -(p1 * t0)), 2.0 * w.eD[2]);
+  u[0] = u[0] + fma(x0, w.rH11, w.k13 * x2);
+  u[1] = fma(w.sh22, x1, u[1]);
+  u[2] = fma(w.sh33, x2, u[2]);
 }
 
 // floor of t in (-2, 2), on the integer pipe
@@ -174,12 +176,13 @@ __device__ __forceinline__ bool photon_unit(double u[3], double &unit) {
   return true;
 }
 
-// The geodesic substep's increment (d0, d1) from u in FP64, where it is large against u (next to
-// the axes, where the metric changes by order one over a step): the FP64 map's image of the
-// point that the pairs found
+// The geodesic substep in FP64 from the increment (d0, d1) that the pairs found, where it is large
+// against u (cold particles, and next to the axes, where the metric changes by order one over a
+// step): evaluations of the FP64 map until the pairs' error in it, below 2^-46 of the increment,
+// has contracted (by rho each) to FP64's rounding.
 __device__ __forceinline__ void strong_geodesic(const GridP &g, const PushTables &tb, int i1,
                                                 int i2, double dx1, double dx2, double m2,
-                                                DF d0, DF d1, double u[3]) {
+                                                DF d0, DF d1, float rho, double u[3]) {
   Pt<double> p;
   inc_point64(g, tb, i1, i2, dx1, dx2, __dadd_rn((double)i2, dx2), p.r, p.s, p.c);
   p.f = g.dxi * p.r;
@@ -189,7 +192,16 @@ __device__ __forceinline__ void strong_geodesic(const GridP &g, const PushTables
   Local<double> L;
   local_full<false>(g, p, L, false);
   const GeoMap<double> m(g, L, u, m2);
-  m.apply(u[0] + df_to_double(d0), u[1] + df_to_double(d1), u[0], u[1]);
+  double t0 = u[0] + df_to_double(d0), t1 = u[1] + df_to_double(d1);
+#pragma unroll 1
+  for (float left = 1.0f; left > 0x1p-9f; left *= rho) {
+    double n0, n1;
+    m.apply(t0, t1, n0, n1);
+    t0 = n0;
+    t1 = n1;
+  }
+  u[0] = t0;
+  u[1] = t1;
 }
 
 // One particle in the increment form; false: nothing stored, push64 has to take it. Loops that
@@ -243,7 +255,7 @@ __device__ __forceinline__ bool push_inc(const GridP &g, const FieldPtrsT<double
         eB[q] = e * eB[q];
         eD[q] = e * eD[q];
       }
-      weak = inc_boris(L, eD, eB, u, du);
+      weak = inc_boris(L, eD, eB, u, inc_limit(1.0f), du);
     }
     if (!weak) {
       strong_frame(g, F, tb, i1, i2, dx1, dx2, s.qm, w);
@@ -259,9 +271,11 @@ __device__ __forceinline__ bool push_inc(const GridP &g, const FieldPtrsT<double
       GeoInc<DF> m;
       geo_inc_setup(k, L, ud, em ? 1.0f : 0.0f, m);
       DF d0, d1;
+      float rho;
       // in the axis rows the result is the method's to rounding, as push64's is there
       const int found = geo_inc_solve<true>(m, L.G.H33.hi * ud[2].hi * ud[2].hi, g.n_iter,
-                                            axis ? 0x1p-54f : g.f_iter_tol, d0, d1);
+                                            axis ? 0x1p-54f : g.f_iter_tol,
+                                            inc_limit(em ? 1.0f : 0.25f), d0, d1, rho);
       if (found == GEO_NONE) return false;
       if (found == GEO_LARGE) {
 #pragma unroll
@@ -269,16 +283,16 @@ __device__ __forceinline__ bool push_inc(const GridP &g, const FieldPtrsT<double
           un[q] += df_to_double(du[q]);
           du[q] = DF(0.0f);
         }
-        strong_geodesic(g, tb, i1, i2, dx1, dx2, s.m2, d0, d1, un);
+        strong_geodesic(g, tb, i1, i2, dx1, dx2, s.m2, d0, d1, rho, un);
       } else {
         du[0] = du[0] + d0;
         du[1] = du[1] + d1;
       }
     }
-    if (em && weak) {
+    if (em && weak) {  // (twice the bound, so that a particle next to it need not start over)
 #pragma unroll
       for (int q = 0; q < 3; ++q) ud[q] = df_of(un[q]) + du[q];
-      if (!inc_boris(L, eD, eB, ud, du)) return false;
+      if (!inc_boris(L, eD, eB, ud, inc_limit(4.0f), du)) return false;
     }
 #pragma unroll
     for (int q = 0; q < 3; ++q) un[q] += df_to_double(du[q]);
