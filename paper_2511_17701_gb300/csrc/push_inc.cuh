@@ -114,19 +114,35 @@ __device__ __forceinline__ void add_scaled(double *p, DF v, int e) {
 }
 
 // deposit64 in pairs, relative to the start cell: the end points a, b are the positions as
-// deposit64 rounds them (absolute coordinates: a multiple of their last place, at most 48
-// bits, so a pair holds them exactly), the rest of its ~70 FP64 operations is in pairs. The
-// pairs' 2^-47 is below that rounding's share of a move. (i, j): the start cell, (c1, c2): the
-// end cell relative to it.
+// deposit64 rounds them (absolute coordinates). From row or column 16 on they are multiples of
+// 2^-48, which a pair holds exactly; before that they have up to 53 bits, so the lengths of the
+// move's two parts, which the fluxes are proportional to, are differences formed in FP64 (with
+// differences of pairs the flux of a move of 3e-3 cells in the first cells was off by up to 1e-12
+// of itself). The rest of deposit64's ~70 FP64 operations is in pairs: their 2^-47 is at or below
+// the rounding's share of a move. (i, j): the start cell, (c1, c2): the end cell relative to it.
+__device__ __forceinline__ void inc_parts(double a, double b, int c, DF &first, DF &second) {
+  if (c == 0) {
+    first = second = df_scale(df_of(b - a), 0.5f);
+  } else {
+    const double r = c > 0 ? 1.0 : (double)(c + 1);
+    first = df_of(r - a);
+    second = df_of(b - r);
+  }
+}
 __device__ __forceinline__ void inc_deposit(const GridP &g, const FieldPtrsT<double> &F,
-                                            double charge, DF idt, int i, int j, DF a1, DF a2,
-                                            int c1, int c2, DF b1, DF b2, DF v3) {
+                                            double charge, DF idt, int i, int j, double xa1,
+                                            double xa2, int c1, int c2, double xb1, double xb2,
+                                            DF v3) {
   const int qh = __double2hiint(charge);
   const bool some = (qh << 1) != 0;
   const int e = some ? (qh & 0x7ff00000) - 0x3ff00000 : 0;  // q = 2^e times its fraction
   const DF q = df_of(__hiloint2double(some ? qh - e : qh, __double2loint(charge)));
   const int NX = g.NX;
   const DF qi = q * idt;
+  const DF a1 = df_of(xa1), a2 = df_of(xa2), b1 = df_of(xb1), b2 = df_of(xb2);
+  DF p1, l1, p2, l2;  // the parts' lengths in the start cell, in the end cell
+  inc_parts(xa1, xb1, c1, p1, l1);
+  inc_parts(xa2, xb2, c2, p2, l2);
   const DF m1 = df_scale(a1 + b1, 0.5f), m2 = df_scale(a2 + b2, 0.5f);
   // the relay point: the midpoint clamped to the two cells' common range
   const DF r1 = c1 == 0 ? m1 : DF(c1 > 0 ? 1.0f : (float)(c1 + 1));
@@ -134,7 +150,7 @@ __device__ __forceinline__ void inc_deposit(const GridP &g, const FieldPtrsT<dou
   const int64_t ka = sidx(g, i, j), kb = sidx(g, i + c1, j + c2);
   double *J1 = F.J[0], *J2 = F.J[1], *J3 = F.J[2];
   {
-    const DF F1 = qi * (r1 - a1), F2 = qi * (r2 - a2);
+    const DF F1 = qi * p1, F2 = qi * p2;
     const DF t = F1 * df_scale(a2 + r2, 0.5f), s = F2 * df_scale(a1 + r1, 0.5f);
     add_scaled(J1 + ka, F1 - t, e);
     add_scaled(J1 + ka + NX, t, e);
@@ -142,7 +158,7 @@ __device__ __forceinline__ void inc_deposit(const GridP &g, const FieldPtrsT<dou
     add_scaled(J2 + ka + 1, s, e);
   }
   {
-    const DF F1 = qi * (b1 - r1), F2 = qi * (b2 - r2);
+    const DF F1 = qi * l1, F2 = qi * l2;
     const DF t = F1 * (df_scale(r2 + b2, 0.5f) + DF(-(float)c2));
     const DF s = F2 * (df_scale(r1 + b1, 0.5f) + DF(-(float)c1));
     add_scaled(J1 + kb, F1 - t, e);
@@ -362,9 +378,9 @@ __device__ __forceinline__ bool push_inc(const GridP &g, const FieldPtrsT<double
   if (DEPOSIT) {
     const double p1 = i1, p2 = i2;
     inc_deposit(g, F, s.qc * s.w[kp], df_of(g.idt), i1, i2,
-                df_of(__dadd_rn(__dadd_rn(p1, dx1), -p1)), df_of(__dadd_rn(__dadd_rn(p2, dx2), -p2)),
-                c1, c2, df_of(__dadd_rn(__dadd_rn((double)j1, e1), -p1)),
-                df_of(__dadd_rn(__dadd_rn((double)j2, e2), -p2)), df_of(v3));
+                __dadd_rn(__dadd_rn(p1, dx1), -p1), __dadd_rn(__dadd_rn(p2, dx2), -p2), c1, c2,
+                __dadd_rn(__dadd_rn((double)j1, e1), -p1), __dadd_rn(__dadd_rn((double)j2, e2), -p2),
+                df_of(v3));
   }
   return true;
 }

@@ -9,7 +9,7 @@ import pytest
 import workloads as W
 from oracle import oracle as O
 from paper_2511_17701_gb300.binding import J01
-from parity import assert_particles, gpu_from_oracle
+from parity import assert_particles, gpu_from_oracle, oracle_state
 
 pytestmark = pytest.mark.gpu
 
@@ -86,3 +86,42 @@ def test_field_unit(torch_cuda, B0, qm):
     osim.push(0)
     g.push(0)
     assert_particles(g.get_particles(0), osim.species[0].view())
+
+
+def test_small_moves_next_to_the_corner(torch_cuda):
+    """The flux of one slow particle in the first cells, where positions carry up to 53 bits: J^1
+    and J^2 summed over their two nodes against the oracle. Both sides take end points rounded to
+    absolute positions below 4 (2^-51 apart where they round differently) and a midpoint rounded
+    by 2^-52, each times q / dt."""
+    cfg = W.grid_config("wald64", metric="ks0", a=0.0, r_min=3.0, r_max=30.0, r_absorb=27.0)
+    rng = np.random.default_rng(17)
+    sim = None
+    for _ in range(60):
+        osim = O.OracleSim(cfg)
+        osim.init_fields(O.FIELD_WALD, 0.0)
+        pos = dict(i1=rng.integers(1, 4, 1).astype(np.int32), i2=rng.integers(2, 4, 1).astype(np.int32),
+                   dx1=rng.uniform(0.6, 0.9, 1), dx2=rng.uniform(0.6, 0.9, 1))
+        osim.add_species(pos, 1e-3 * rng.standard_normal((3, 1)), np.ones(1), 0.0, 1.0)
+        sp = osim.species[0]
+        if sim is None:
+            sim = gpu_from_oracle(osim, iter_tol=1e-16, sort_every=0)
+        sim.set_particles(0, sp.view(), sp.qm, sp.qc)
+        q = float(sp.view()["w"][0])
+        osim.predict()
+        osim.push(0)
+        osim.deposit()
+        sim.step(1)
+        for c in range(2):
+            flux = float(sim.plane(J01 + c).sum()), float(osim.F[O.J1 + c].sum())
+            assert abs(flux[0] - flux[1]) <= 2.0 ** -50 * q / osim.dt, (c, flux)
+
+
+def test_continuity(torch_cuda):
+    """Full steps of the increment form conserve charge as those of the general push do
+    (tests/test_gpu_charge.py, the same bound)."""
+    g = gpu_from_oracle(oracle_state(W.grid_config("wald64")), iter_tol=1e-12)
+    for _ in range(3):
+        g.step(1)
+        res, drho, _, scale = g.charge_check(after_step=True)
+        assert drho > 1e-3
+        assert res / scale < 1e-13, (res, drho, scale)
