@@ -232,8 +232,14 @@ __device__ __forceinline__ bool push_inc(const GridP &g, const FieldPtrsT<double
   if (DEPOSIT && !inc_charge(s.qc * s.w[kp])) return false;
   const bool em = s.m2 != 0.0, axis = i2 < 2 || i2 >= g.n_th - 2;
   const double dx1 = s.dx1[kp], dx2 = s.dx2[kp];
-  const IncC k = inc_c(g);
   const DF o1 = df_of(dx1), o2 = df_of(dx2);
+  // Next to theta = pi an absolute position x2 ~ n_theta has a last place of up to n_theta 2^-52
+  // cells, and dphi/dt, ~ 1/d^2 at a distance of d cells, follows a position rounded the other way
+  // by twice that over d. Within n_theta 2^-10 cells of the axis (an angle of pi / 1024), where it
+  // is above 2^-41 = 4.5e-13 of dphi/dt, push64's own sequence of roundings is kept.
+  const float pole = (float)g.n_th * 0x1p-10f;
+  if (axis && (float)(g.n_th - i2) - o2.hi < pole) return false;
+  const IncC k = inc_c(g);
   double un[3] = {s.u1[kp], s.u2[kp], s.u3[kp]}, unit = 1.0;
   if (!em && !photon_unit(un, unit)) return false;
   DF ud[3] = {df_of(un[0]), df_of(un[1]), df_of(un[2])};
@@ -345,12 +351,8 @@ __device__ __forceinline__ bool push_inc(const GridP &g, const FieldPtrsT<double
     reflected = true;
   }
   if (axis) {
-    // Close to the axis theta = pi dphi/dt (~ 1 / distance^2) follows every rounding of absolute
-    // positions that large: within n_theta 2^-10 cells of it, where that would show at ~1e-12,
-    // push64's own sequence of roundings is kept
-    const float far = (float)g.n_th * 0x1p-10f;
-    const float d0 = (float)(g.n_th - i2) - o2.hi, d1 = (float)(g.n_th - j2) - f32_trunc(e2);
-    if (fminf(d0, d1) < far) return false;
+    // (ends next to theta = pi: see above)
+    if ((float)(g.n_th - j2) - f32_trunc(e2) < pole) return false;
     // dphi/dt varies by order one over the distance to the axis, which next to theta = pi makes
     // it sensitive to how the midpoint is rounded: as push64 rounds it, from the absolute positions
     const double p1 = i1, p2 = i2;

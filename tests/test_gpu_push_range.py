@@ -125,3 +125,29 @@ def test_continuity(torch_cuda):
         res, drho, _, scale = g.charge_check(after_step=True)
         assert drho > 1e-3
         assert res / scale < 1e-13, (res, drho, scale)
+
+
+@pytest.mark.parametrize("n_theta", [48, 64, 1024, 2048])
+@pytest.mark.parametrize("massless", [False, True])
+def test_rows_on_the_axes(torch_cuda, n_theta, massless):
+    """The two rows next to each axis, among them particles closer to theta = pi than
+    n_theta 2^-10 cells, which the general routine keeps, and ones on either side of that."""
+    cfg = W.grid_config("wald64", n_theta=n_theta)
+    osim = O.OracleSim(cfg)
+    osim.init_fields(O.FIELD_WALD, 1.0)
+    rng = np.random.default_rng(23)
+    n = 4000
+    near = n_theta * 2.0 ** -10
+    d = np.where(rng.random(n) < 0.5, rng.uniform(0.0, 2.0, n), near * rng.uniform(0.5, 1.5, n))
+    d = np.clip(d, 0.02, 1.98)
+    x2 = np.where(rng.random(n) < 0.7, n_theta - d, d)
+    pos = dict(i1=rng.integers(3, cfg["n_r"] - 2, n).astype(np.int32), i2=np.floor(x2).astype(np.int32),
+               dx1=rng.random(n), dx2=x2 - np.floor(x2))
+    uh = rng.standard_normal((3, n))
+    osim.add_species(pos, uh / np.linalg.norm(uh, axis=0), 0.1 * np.ones(n), 1.0, 0.2, massless=massless)
+    g = gpu_from_oracle(osim, iter_tol=1e-12, massless=[0] if massless else [])
+    osim.predict()
+    g.predict()
+    osim.push(0)
+    g.push(0)
+    assert_particles(g.get_particles(0), osim.species[0].view())
