@@ -214,10 +214,9 @@ GRPIC_API size_t grpic_arena_bytes(const grpic_ctx *ctx);
 /* (Memory and stream management, no counterpart in the paper.)
  * Binds the caller-owned device arena (>= grpic_arena_bytes, 256-byte aligned)
  * and the CUDA stream (cudaStream_t, NULL = legacy default) on the current device.
- * The first bind also creates up to two internal streams and event pairs (no device
- * memory): the mixed push forks its guard-zone kernels onto them, small FP64 pushes of every
- * other species run there, and both join the bound stream before returning, so callers see
- * one stream.
+ * With GRPIC_MIXED the first bind also creates two internal streams and event pairs (no device
+ * memory): the push forks its guard-zone kernels onto them, one species on each in turn, and
+ * joins them back to the bound stream before returning, so callers see one stream.
  * Errors: GRPIC_ENOMEM (too small), GRPIC_EINVAL (misaligned), GRPIC_ECUDA. */
 GRPIC_API grpic_status grpic_bind(grpic_ctx *ctx, void *arena, size_t bytes, void *stream);
 
@@ -508,9 +507,9 @@ typedef struct {
   double predict_ms, sort_ms, push_ms, deposit_ms, advance_ms;
   int64_t push_calls;   /* particle-kernel launches timed in push_ms                 */
   int64_t launches;     /* kernels launched by the library since the last reset      */
-  double kernel_ms;     /* the main push kernel alone (FP64: k_push; mixed: the FP32
-                           kernel, which runs beside the guard kernels), summed over
-                           push_calls launches                                        */
+  double kernel_ms;     /* the main push kernel alone (FP64: k_push, or k_push_inc and
+                           k_push_rest together; mixed: the FP32 kernel, which runs
+                           beside the guard kernels), summed over push_calls launches */
   double inject_ms;     /* grpic_inject                                               */
 } grpic_timing;
 

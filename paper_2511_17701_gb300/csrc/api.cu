@@ -74,8 +74,7 @@ struct grpic_ctx {
   size_t need = 0;
   char *arena = nullptr;
   cudaStream_t stream = nullptr;
-  // species k's guard kernels (mixed push), or its whole push where that is small, on side[k % 2]
-  cudaStream_t side[2] = {};
+  cudaStream_t side[2] = {};  // species k's guard kernels (mixed push) run on side[k % 2]
   cudaEvent_t ev_fork[GRPIC_MAX_SPECIES] = {}, ev_done[GRPIC_MAX_SPECIES] = {};
   cudaEvent_t ev_class[GRPIC_MAX_SPECIES] = {};
   // grpic_step_host: copy streams, events and pinned counts, created on its first call;
@@ -269,7 +268,7 @@ cudaError_t do_push(grpic_ctx *c, FieldPtrsT<T> &F, int k, bool deposit, int sta
   const std::pair<cudaEvent_t, cudaEvent_t> *kt =
       push_main_stage(stage) ? next_events(c, PH_KERNEL) : nullptr;
   const PushStreams ps{c->stream, c->side[k & 1], c->ev_fork[k], c->ev_done[k], c->ev_class[k],
-                       kt ? kt->first : nullptr, kt ? kt->second : nullptr, stage, (k & 1) != 0};
+                       kt ? kt->first : nullptr, kt ? kt->second : nullptr, stage};
   const int tr = c->cfg.tile_r, tt = c->cfg.tile_theta;
   const int ntr = (c->g.n_r + tr - 1) / tr, ntt = (c->g.n_th + tt - 1) / tt;
   TileInfo ti{};
@@ -297,9 +296,7 @@ cudaError_t do_push(grpic_ctx *c, FieldPtrsT<T> &F, int k, bool deposit, int sta
 }
 // the main stream waits for the guard kernels of species k (mixed path)
 cudaError_t join_push(grpic_ctx *c, int k) {
-  // an event that this push has not recorded is left alone (a stream capture would refuse it)
-  if (!c->mixed && !push_apart((k & 1) != 0, c->sp[k].n_bound)) return cudaSuccess;
-  return cudaStreamWaitEvent(c->stream, c->ev_done[k], 0);
+  return c->mixed ? cudaStreamWaitEvent(c->stream, c->ev_done[k], 0) : cudaSuccess;
 }
 template <typename T>
 cudaError_t do_zero_J(grpic_ctx *c, FieldPtrsT<T> &F) {
@@ -548,13 +545,11 @@ grpic_status grpic_bind(grpic_ctx *ctx, void *arena, size_t bytes, void *stream)
       sp.tiles_valid = false;
     }
   }
-  // the guard kernels are the longer chain: higher priority (FP64 runs of one species need no
-  // stream, others the second)
-  if (!ctx->side[1] && (ctx->mixed || ctx->cfg.n_species > 1)) {
+  if (ctx->mixed && !ctx->side[1]) {  // the guard kernels are the longer chain: higher priority
     int lo = 0, hi = 0;
     CK(cudaDeviceGetStreamPriorityRange(&lo, &hi));
-    if (ctx->mixed) CK(cudaStreamCreateWithPriority(&ctx->side[0], cudaStreamNonBlocking, hi));
-    CK(cudaStreamCreateWithPriority(&ctx->side[1], cudaStreamNonBlocking, hi));
+    for (cudaStream_t &st : ctx->side)
+      if (!st) CK(cudaStreamCreateWithPriority(&st, cudaStreamNonBlocking, hi));
     for (int s = 0; s < GRPIC_MAX_SPECIES; ++s) {
       CK(cudaEventCreateWithFlags(&ctx->ev_fork[s], cudaEventDisableTiming));
       CK(cudaEventCreateWithFlags(&ctx->ev_done[s], cudaEventDisableTiming));
@@ -959,7 +954,6 @@ grpic_status host_species(grpic_ctx *ctx, int k, const HostIO &io, bool sort_now
     {
       PhaseTimer t(ctx, PH_PUSH);
       if (ctx->mixed) CK(do_push(ctx, ctx->F32, k, true));
-      else if (C == 1) CK(do_push(ctx, ctx->F64, k, true));
       else CK(push_range(ctx, k, a, b - a, cn + c));
       ++ctx->push_calls;
     }

@@ -417,16 +417,11 @@ __host__ __device__ inline bool push_classify_stage(int s) {
 __host__ __device__ inline bool push_guard_kernels_stage(int s) {
   return s == PUSH_ALL || s == PUSH_GUARD || s == PUSH_GUARD_KERNELS;
 }
-// whether an FP64 push that may run apart does: fewer particles than fill the GPU
-inline bool push_apart(bool may, int64_t n_bound) {
-  return may && n_bound > 0 && n_bound < (1 << 18);
-}
 struct PushStreams {
   cudaStream_t main, side;
   cudaEvent_t fork, done, classified;  // side after main; guard kernels done; classify done
   cudaEvent_t t0, t1;  // when not null: recorded on `main` around the main push kernel
   int stage = PUSH_ALL;
-  bool apart = false;  // FP64: a small push may run on `side` (forked and recorded as above)
 };
 
 template <typename T>

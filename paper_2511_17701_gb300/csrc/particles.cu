@@ -1796,40 +1796,27 @@ cudaError_t push_impl(const GridP &g, const FieldPtrsT<T> &F, SpeciesDevT<T> s,
   }
   if constexpr (sizeof(T) == 8) {
     if (!main_stage) return cudaSuccess;  // the FP64 path has no guard stage
-    // a push of fewer warps than the GPU holds runs beside that of the species before it: on
-    // 64^2 cells (1024 warps a species) the two took 2 x 95 us one behind the other
-    cudaStream_t st = ps.main;
-    if (push_apart(ps.apart, n_bound)) {
-      cudaError_t e;
-      st = ps.side;
-      if ((e = cudaEventRecord(ps.fork, ps.main)) != cudaSuccess) return e;
-      if ((e = cudaStreamWaitEvent(st, ps.fork, 0)) != cudaSuccess) return e;
-    }
-    if (ps.t0) cudaEventRecord(ps.t0, st);
+    if (ps.t0) cudaEventRecord(ps.t0, ps.main);
     const int b = blocks_for(n_bound);
     if (!Q && inc_applies(g)) {
       const bool small = n_bound < (1 << 19);
       const int br = blocks_for(small ? n_bound : (n_bound + 7) / 8);
       if (deposit) {
-        k_push_inc<true><<<b, TPB, 0, st>>>(g, F, tb, s, diag);
-        if (small) k_push_rest<true, 1><<<br, TPB, 0, st>>>(g, F, tb, s, diag);
-        else k_push_rest<true, 8><<<br, TPB, 0, st>>>(g, F, tb, s, diag);
+        k_push_inc<true><<<b, TPB, 0, ps.main>>>(g, F, tb, s, diag);
+        if (small) k_push_rest<true, 1><<<br, TPB, 0, ps.main>>>(g, F, tb, s, diag);
+        else k_push_rest<true, 8><<<br, TPB, 0, ps.main>>>(g, F, tb, s, diag);
       } else {
-        k_push_inc<false><<<b, TPB, 0, st>>>(g, F, tb, s, diag);
-        if (small) k_push_rest<false, 1><<<br, TPB, 0, st>>>(g, F, tb, s, diag);
-        else k_push_rest<false, 8><<<br, TPB, 0, st>>>(g, F, tb, s, diag);
+        k_push_inc<false><<<b, TPB, 0, ps.main>>>(g, F, tb, s, diag);
+        if (small) k_push_rest<false, 1><<<br, TPB, 0, ps.main>>>(g, F, tb, s, diag);
+        else k_push_rest<false, 8><<<br, TPB, 0, ps.main>>>(g, F, tb, s, diag);
       }
       COUNT_LAUNCH(1);
     } else if (deposit) {
-      k_push<true, Q><<<b, TPB, 0, st>>>(g, F, tb, s, diag);
+      k_push<true, Q><<<b, TPB, 0, ps.main>>>(g, F, tb, s, diag);
     } else {
-      k_push<false, Q><<<b, TPB, 0, st>>>(g, F, tb, s, diag);
+      k_push<false, Q><<<b, TPB, 0, ps.main>>>(g, F, tb, s, diag);
     }
-    if (ps.t1) cudaEventRecord(ps.t1, st);
-    if (st != ps.main) {
-      const cudaError_t e = cudaEventRecord(ps.done, st);
-      if (e != cudaSuccess) return e;
-    }
+    if (ps.t1) cudaEventRecord(ps.t1, ps.main);
     COUNT_LAUNCH(1);
   } else {
     cudaError_t e;
