@@ -375,6 +375,12 @@ __device__ __forceinline__ bool adj_inc_step(const GridP &g, const FieldPtrsT<do
   }
   vec_hat(a.L, a.V, a.eB1);
   vec_hat(a.L, a.V + 3, a.eD1);
+  // the gradient by the amplitude is proportional to the planes' own values, whatever they are:
+  // they have to be clear of the range where a pair loses its low half (2^-74)
+  float top = 0.0f;
+#pragma unroll
+  for (int q = 0; q < 6; ++q) top = fmaxf(top, fabsf(a.V[q].hi));
+  if (!(top == 0.0f || (top >= 0x1p-30f && top <= 0x1p40f))) return false;
   const DF e = df_scale(qm * a.L.alpha * k.dt, 0.25f);
   DF du[3] = {DF(0.0f), DF(0.0f), DF(0.0f)};
 #pragma unroll
@@ -782,10 +788,15 @@ int adj_blocks(int64_t n, int tpb) {
 }  // namespace
 
 // Whether the increment form may take steps: rows away from the axes clear of the
-// small-angle clamp, and an iteration limit that is one (the general form takes a small one
-// literally).
-static bool adj_inc_applies(const GridP &g, int n_iter) {
-  return n_iter >= INC_MIN_ITER && g.small_angle < g.dth;
+// small-angle clamp, an iteration limit that is one (the general form takes a small one
+// literally), and a charge-to-mass ratio, an amplitude and a time step whose products with
+// values of order 1 stay far inside a pair's range (2^-126, 2^128).
+static bool adj_inc_applies(const GridP &g, int n_iter, double qm, double scale) {
+  const auto in_range = [](double x) {
+    return x == 0.0 || (fabs(x) >= 0x1p-40 && fabs(x) <= 0x1p30);
+  };
+  return n_iter >= INC_MIN_ITER && g.small_angle < g.dth && in_range(qm) && in_range(scale) &&
+         g.dt >= 0x1p-40 && g.dt <= 0x1p30;
 }
 
 cudaError_t launch_adjoint_forward(const GridP &g, const FieldPtrsT<double> &F,
@@ -793,7 +804,7 @@ cudaError_t launch_adjoint_forward(const GridP &g, const FieldPtrsT<double> &F,
                                    int n_steps, int every, int n_iter, const double *st0,
                                    double *out, double *ckpt, cudaStream_t st) {
   if (n <= 0) return cudaGetLastError();
-  const auto kernel = adj_inc_applies(g, n_iter) ? k_adj_forward<true> : k_adj_forward<false>;
+  const auto kernel = adj_inc_applies(g, n_iter, qm, scale) ? k_adj_forward<true> : k_adj_forward<false>;
   kernel<<<adj_blocks(n, TPB_ADJ), TPB_ADJ, 0, st>>>(g, F, tb, n, qm, scale, n_steps, every,
                                                      n_iter, st0, out, ckpt);
   COUNT_LAUNCH(1);
@@ -807,7 +818,7 @@ cudaError_t launch_adjoint_backward(const GridP &g, const FieldPtrsT<double> &F,
                                     double *gscale_pp, double *gscale_sum, double *scratch,
                                     cudaStream_t st) {
   if (n <= 0) return cudaMemsetAsync(gscale_sum, 0, sizeof(double), st);
-  const auto kernel = adj_inc_applies(g, n_iter) ? k_adj_backward<true> : k_adj_backward<false>;
+  const auto kernel = adj_inc_applies(g, n_iter, qm, scale) ? k_adj_backward<true> : k_adj_backward<false>;
   kernel<<<adj_blocks(n, TPB_BWD), TPB_BWD, 0, st>>>(g, F, tb, n, qm, scale, gfac, n_steps, every,
                                                      n_iter, ckpt, gout, gin, gscale_pp, scratch);
   k_sum<<<1, 1024, 0, st>>>(gscale_pp, n, gscale_sum);
