@@ -18,8 +18,9 @@
 // are recomputed and kept in scratch memory for the reverse sweep.
 //
 // Both passes run a step in the increment form of inc.cuh where it applies: the state's
-// increment and J - 1, which are small against the state and 1, in pairs of floats, added in
-// FP64. The general FP64 form (step_values, step_jacobian) takes the rest.
+// increment and the derivatives by x1, x2, which are small against the state and 1, in pairs of
+// floats, added in FP64; those by u_1, u_2, u_3 and the scale in FP64. The general FP64 form
+// (step_values, step_jacobian) takes the rest.
 #include "dual.cuh"
 #include "grpic_internal.cuh"
 #include "inc.cuh"
@@ -330,10 +331,11 @@ __device__ __noinline__ void step_jacobian(const GridP &g, const FieldPtrsT<doub
 // A step in the increment form. GB300's FP64 pipe bounded both passes (~1800 FP64 operations
 // per particle-step forward, ~5500 backward, most of them exp and sincos per iterate and the
 // metric's derivatives in duals); here FP64 is left with one or two evaluations of the
-// coordinate map and the additions to the state. 65,536 orbits on 512^2, 100 steps forward and
-// back: 107 -> 29 ms, the gradients' error against FP64 references as before (4.3e-15, 4.2e-15).
-// The backward kernel waits for instructions and for its pair arithmetic at 8 warps per SM
-// (255 registers, spills).
+// coordinate map, the additions to the state and, backward, the derivatives along the momentum
+// and the scale (~900 operations). 65,536 orbits on 512^2, 100 steps forward and back: 107 -> 38
+// ms (28 ms with all derivatives in pairs, whose errors were larger: see the scratch layout below).
+// The backward kernel waits for instructions, FP64 results and its pair arithmetic at 8 warps per
+// SM (255 registers, spills).
 // ---------------------------------------------------------------------------------
 constexpr int INC_MIN_ITER = 16;   // iteration counts below are taken literally (general form)
 constexpr float INC_ADJ_TOL = 1e-16f;
@@ -342,11 +344,11 @@ constexpr IncLimit ADJ_LIMIT = {0x1p-8f, 0x1p-4f};  // increments up to 1/16 of 
 struct AdjStep {
   int i1, i2;
   DF o1, o2;            // x^n in its cell
+  double dx[2];         // the same
   DF r, s, c;           // there
   Local<DF> L;
   DF V[6];              // B, D at x^n, unit amplitude
-  DF eB1[3], eD1[3];    // e B, e D in the tetrad frame at unit amplitude, e = qm alpha dt/4
-  DF eB[3], eD[3];      // at the amplitude
+  DF eB[3], eD[3];      // e B, e D in the tetrad frame at the amplitude, e = qm alpha dt/4
   DF u[3], u1[3], dg[2], u2[3], un[3];  // u^n, after the first EM half step, the geodesic
                         // substep's increment, after it, u^{n+1}
   double u64[3], x64[2], v3, mid[2];    // u^{n+1}, x^{n+1}, dphi/dt; the midpoint's offsets
@@ -362,6 +364,8 @@ __device__ __forceinline__ bool adj_inc_step(const GridP &g, const FieldPtrsT<do
   a.i2 = (int)f2;
   if (!(a.i1 >= 0 && a.i1 < g.n_r && a.i2 >= 2 && a.i2 < g.n_th - 2)) return false;
   const double dx1 = st[0] - f1, dx2 = st[1] - f2;
+  a.dx[0] = dx1;
+  a.dx[1] = dx2;
   a.o1 = df_of(dx1);
   a.o2 = df_of(dx2);
   if (!inc_point_n(g, k, tb, a.i1, a.i2, dx2, a.o1, a.o2, a.r, a.s, a.c)) return false;
@@ -373,22 +377,20 @@ __device__ __forceinline__ bool adj_inc_step(const GridP &g, const FieldPtrsT<do
     const int h1 = q == 1 || q == 2 || q == 3, h2 = q == 0 || q == 2 || q == 4;
     a.V[q] = inc_interp(q < 3 ? F.B[q] : F.D[q - 3], g.NX, l, h1, h2);
   }
-  vec_hat(a.L, a.V, a.eB1);
-  vec_hat(a.L, a.V + 3, a.eD1);
+  vec_hat(a.L, a.V, a.eB);
+  vec_hat(a.L, a.V + 3, a.eD);
   // the gradient by the amplitude is proportional to the planes' own values, whatever they are:
   // they have to be clear of the range where a pair loses its low half (2^-74)
   float top = 0.0f;
 #pragma unroll
   for (int q = 0; q < 6; ++q) top = fmaxf(top, fabsf(a.V[q].hi));
   if (!(top == 0.0f || (top >= 0x1p-30f && top <= 0x1p40f))) return false;
-  const DF e = df_scale(qm * a.L.alpha * k.dt, 0.25f);
+  const DF es = scale * df_scale(qm * a.L.alpha * k.dt, 0.25f);
   DF du[3] = {DF(0.0f), DF(0.0f), DF(0.0f)};
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
-    a.eB1[q] = e * a.eB1[q];
-    a.eD1[q] = e * a.eD1[q];
-    a.eB[q] = scale * a.eB1[q];
-    a.eD[q] = scale * a.eD1[q];
+    a.eB[q] = es * a.eB[q];
+    a.eD[q] = es * a.eD[q];
     a.u[q] = df_of(st[3 + q]);
   }
   if (!inc_boris(a.L, a.eD, a.eB, a.u, ADJ_LIMIT, du)) return false;
@@ -433,20 +435,23 @@ __device__ __forceinline__ D2F adj_interp_d(const double *__restrict__ pl, int N
   return D2F(V, fma_(l.w2[h2], xy, x0), fma_(l.w1[h1], xy, y0));
 }
 
-// The momentum's derivative along two directions: du' of u^{n+1} - u^n for metric values L, u
-// and the fields with their derivatives. K: the geodesic substep's (I - A)^{-1}.
+// The momentum's derivative along x1, x2: du' of u^{n+1} - u^n for metric values L and fields with
+// their derivatives. K: the geodesic substep's (I - A)^{-1}.
 __device__ __forceinline__ void adj_momentum_d(const IncC &k, const Local<D2F> &L, const D2F eD[3],
-                                               const D2F eB[3], const D2F u[3], const AdjStep &a,
+                                               const D2F eB[3], const AdjStep &a,
                                                const DF K[2][2], D2F du[3]) {
-  D2F h[3], x[3], v[3] = {u[0], u[1], u[2]};
+  D2F h[3], x[3], v[3];
 #pragma unroll
-  for (int q = 0; q < 3; ++q) du[q] = D2F(0.0f);
+  for (int q = 0; q < 3; ++q) {
+    v[q] = D2F(a.u[q]);
+    du[q] = D2F(0.0f);
+  }
 #pragma unroll 1
   for (int half = 0;; ++half) {
     inc_boris_core(L, eD, eB, v, du, h, x);
     if (half) return;
 #pragma unroll
-    for (int q = 0; q < 3; ++q) v[q] = D2F(a.u1[q], u[q].d0 + du[q].d0, u[q].d1 + du[q].d1);
+    for (int q = 0; q < 3; ++q) v[q] = D2F(a.u1[q], du[q].d0, du[q].d1);
     GeoInc<D2F> m;
     geo_inc_setup(k, L, v, 1.0f, m);
     D2F n0, n1;
@@ -457,7 +462,7 @@ __device__ __forceinline__ void adj_momentum_d(const IncC &k, const Local<D2F> &
     du[1].d0 = du[1].d0 + fma_(K[1][0], n0.d0, K[1][1] * n1.d0);
     du[1].d1 = du[1].d1 + fma_(K[1][0], n0.d1, K[1][1] * n1.d1);
 #pragma unroll
-    for (int q = 0; q < 3; ++q) v[q] = D2F(a.u2[q], u[q].d0 + du[q].d0, u[q].d1 + du[q].d1);
+    for (int q = 0; q < 3; ++q) v[q] = D2F(a.u2[q], du[q].d0, du[q].d1);
   }
 }
 
@@ -472,25 +477,108 @@ __device__ __forceinline__ void adj_inv(const DF A[2][2], DF K[2][2]) {
 }
 
 // A step's derivatives in scratch memory: entry (row, column) of rows x1, x2, phi, u1, u2, u3
-// and columns x1, x2, u1, u2, u3, scale at w[(row * JC + column) n], either J - 1 as pairs (lo,
-// hi) or J as doubles; which one is the lowest bit of entry (0, 0): clear for pairs, set for
-// doubles (half an ulp of that one entry).
+// and columns x1, x2, u1, u2, u3, scale at w[(row * JC + column) n], either J - 1, as pairs (lo,
+// hi) in the first two columns and as doubles in the others, or J as doubles; which one is the
+// lowest bit of entry (0, 0): clear for J - 1, set for J (half an ulp of that one entry).
+//
+// Why two types: of J - 1 the first two columns are small (1e-3 where J has a 1), so pairs leave
+// less of J than FP64 does. The others hold entries that are the whole of J (dt dV/du, the
+// rotation between u_1, u_2 and u_3, the fields for the scale), of which pairs kept 2^-47, a part
+// of it (the grid's constants, the fields) the same in every step: on 200^2, 30 steps, |u| up to
+// 0.5, the gradients' rms errors against 80-bit arithmetic were 2.7e-15 (u1), 1.8e-15 (u2), 3.4e-15
+// (scale) where FP64 throughout has 1.5e-15, 1.3e-15, 1.1e-15; now 4.5e-16, 5.4e-16, 4.4e-16.
+__device__ __forceinline__ constexpr bool adj_is64(int c) { return c >= 2; }
 __device__ __forceinline__ float2 adj_pack(DF a, bool first) {
   return make_float2(first ? __uint_as_float(__float_as_uint(a.lo) & ~1u) : a.lo, a.hi);
 }
 
+// dV_j / du_k of the coordinate velocities at the midpoint in FP64 (adj_inc_jacobian's Vu)
+__device__ __forceinline__ void adj_vu64(const GridP &g, const PushTables &tb, const AdjStep &a,
+                                         double V[3][3]) {
+  double r, s, c;
+  inc_point64(g, tb, a.i1, a.i2, a.mid[0], a.mid[1], __dadd_rn((double)a.i2, a.mid[1]), r, s, c);
+  const double *u = a.u64;
+  const double s2 = s * s, r2 = r * r, f = g.dxi * r;
+  const double Sig = fma(g.a2, c * c, r2), M2r = g.M2 * r, S2 = Sig + M2r;
+  const double Rr = r2 + g.a2, A = fma(Rr, Rr, -(g.a2 * s2 * (Rr - M2r)));
+  const double fs = f * s2, iQ = rcp_nr(S2 * fs), T = iQ * S2, fi = T * s2, AS = A * (iQ * fs);
+  const double w0 = u[0] * fi, au = g.a * u[2], I = fma(AS, w0, au), kk = g.ig2 * u[1];
+  const double is2 = T * f, z = u[2] * is2, X = fma(w0, I + au, fma(kk, u[1], u[2] * z));
+  const double G = rsqrt(S2 * (Sig + X)), iN = G * G * S2, P0 = fi * I, P2 = fma(g.a, w0, z);
+  const double q0 = P0 * iN, q1 = kk * iN, q2 = P2 * iN;
+  V[0][0] = G * fma(fi * fi, AS, -(q0 * P0));
+  V[1][1] = G * fma(-q1, kk, g.ig2);
+  V[2][2] = G * fma(-q2, P2, is2);
+  V[0][1] = V[1][0] = -(G * (q0 * kk));
+  V[0][2] = V[2][0] = G * fma(g.a, fi, -(q0 * P2));
+  V[1][2] = V[2][1] = -(G * (q1 * P2));
+}
+__device__ __forceinline__ void cross64(const double a[3], const double b[3], double o[3]) {
+  o[0] = fma(a[1], b[2], -(a[2] * b[1]));
+  o[1] = fma(a[2], b[0], -(a[0] * b[2]));
+  o[2] = fma(a[0], b[1], -(a[1] * b[0]));
+}
+// A Boris half step from u in FP64 (inc_boris_core), what its derivatives need of it: m = h + e D,
+// t = e B / gamma, p = m + m x t, c = p x t, s = 2 / (1 + t^2)
+struct HalfStep {
+  double m[3], t[3], p[3], c[3], ig, sf;
+};
+__device__ __forceinline__ void adj_half64(const Strong &w, double scale, const double u[3],
+                                           HalfStep &h) {
+  h.m[0] = fma(scale, w.eD[0], w.sH11 * fma(-w.m13, u[2], u[0]));
+  h.m[1] = fma(scale, w.eD[1], w.rh22 * u[1]);
+  h.m[2] = fma(scale, w.eD[2], w.rh33 * u[2]);
+  h.ig = rsqrt(fma(h.m[0], h.m[0], fma(h.m[1], h.m[1], fma(h.m[2], h.m[2], 1.0))));
+  double x[3];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) h.t[q] = scale * w.eB[q] * h.ig;
+  h.sf = 2.0 * rcp_nr(fma(h.t[0], h.t[0], fma(h.t[1], h.t[1], fma(h.t[2], h.t[2], 1.0))));
+  cross64(h.m, h.t, x);
+#pragma unroll
+  for (int q = 0; q < 3; ++q) h.p[q] = h.m[q] + x[q];
+  cross64(h.p, h.t, h.c);
+}
+// its derivative: of the increment, added to dw, along a direction that changes u by du and the
+// scale by ds
+__device__ __forceinline__ void adj_half64_d(const Strong &w, const HalfStep &h, double scale,
+                                             const double du[3], double ds, double dw[3]) {
+  double md[3] = {w.sH11 * fma(-w.m13, du[2], du[0]), w.rh22 * du[1], w.rh33 * du[2]};
+  double td[3], pd[3], x[3], y[3];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) md[q] = fma(ds, w.eD[q], md[q]);
+  const double a = -(h.ig * h.ig) * fma(h.m[0], md[0], fma(h.m[1], md[1], h.m[2] * md[2]));
+  const double b = h.ig * ds;  // t' = t a + e B b
+#pragma unroll
+  for (int q = 0; q < 3; ++q) td[q] = fma(h.t[q], a, w.eB[q] * b);
+  const double sd = -(h.sf * h.sf) * fma(h.t[0], td[0], fma(h.t[1], td[1], h.t[2] * td[2]));
+  cross64(md, h.t, x);
+  cross64(h.m, td, y);
+#pragma unroll
+  for (int q = 0; q < 3; ++q) pd[q] = md[q] + (x[q] + y[q]);
+  cross64(pd, h.t, x);
+  cross64(h.p, td, y);
+#pragma unroll
+  for (int q = 0; q < 3; ++q) x[q] = fma(sd, h.c[q], fma(h.sf, x[q] + y[q], 2.0 * ds * w.eD[q]));
+  dw[0] += fma(x[0], w.rH11, w.k13 * x[2]);
+  dw[1] = fma(w.sh22, x[1], dw[1]);
+  dw[2] = fma(w.sh33, x[2], dw[2]);
+}
+
 __device__ __forceinline__ void adj_inc_jacobian(const GridP &g, const FieldPtrsT<double> &F,
-                                                 const PushTables &tb, const IncC &k, DF scale,
-                                                 DF qm, const AdjStep &a, double *wd, int64_t n) {
+                                                 const PushTables &tb, const IncC &k,
+                                                 const double st[6], double scale64, double qm64,
+                                                 DF scale, DF qm, const AdjStep &a, double *wd,
+                                                 int64_t n) {
   float2 *w = reinterpret_cast<float2 *>(wd);
+  const DF zero(0.0f);
   // the coordinate map's velocity (inc_velocity's grouping) at the midpoint: its derivatives
-  // along x (Vx) and along u (Vu): with P_j = half of dX/du_j, V_j + beta_j = G P_j and
+  // along x (Vx) and along u (Vu, FP64): with P_j = half of dX/du_j, V_j + beta_j = G P_j and
   // dV_j/du_k = G (c_jk - P_j P_k / N), N = m2 Sigma + X
-  DF Vx[3][2], Vu[3][3], Mx[2][2];
+  DF Vx[3][2], N[2][2];
   {
     DF r, s, c;
     inc_point(k, tb, a.i1, a.i2, df_of(a.mid[0]), df_of(a.mid[1]), r, s, c);
-    const D2F R(r, k.dxi * r, DF(0.0f)), S(s, DF(0.0f), c * k.dth), C(c, DF(0.0f), -(s * k.dth));
+    const D2F R(r, k.dxi * r, zero), S(s, zero, c * k.dth), C(c, zero, -(s * k.dth));
     const D2F s2 = S * S, r2 = R * R, f = k.dxi * R;
     const D2F Sig = fma_(k.a2, C * C, r2), M2r = df_scale(k.M * R, 2.0f), S2 = Sig + M2r;
     const D2F Rr = r2 + k.a2, A = fma_(Rr, Rr, -(k.a2 * s2 * (Rr - M2r)));
@@ -505,33 +593,39 @@ __device__ __forceinline__ void adj_inc_jacobian(const GridP &g, const FieldPtrs
     Vx[0][0] = V0.d0; Vx[0][1] = V0.d1;
     Vx[1][0] = V1.d0; Vx[1][1] = V1.d1;
     Vx[2][0] = V2.d0; Vx[2][1] = V2.d1;
-    const DF iN = G.v * G.v * S2.v;
-    const DF q0 = P0.v * iN, q1 = kk * iN, q2 = P2.v * iN;
-    Vu[0][0] = G.v * (fi.v * fi.v * AS.v - q0 * P0.v);
-    Vu[1][1] = G.v * (k.ig2 - q1 * kk);
-    Vu[2][2] = G.v * (is2.v - q2 * P2.v);
-    Vu[0][1] = Vu[1][0] = -(G.v * (q0 * kk));
-    Vu[0][2] = Vu[2][0] = G.v * (k.a * fi.v - q0 * P2.v);
-    Vu[1][2] = Vu[2][1] = -(G.v * (q1 * P2.v));
     const DF h = df_scale(k.dt, 0.5f);
     const DF B[2][2] = {{h * Vx[0][0], h * Vx[0][1]}, {h * Vx[1][0], h * Vx[1][1]}};
+    // N = (I - B)^{-1} - I = (I - B)^{-1} B
+    DF Mx[2][2];
     adj_inv(B, Mx);
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+      for (int p = 0; p < 2; ++p) N[q][p] = fma_(Mx[q][0], B[0][p], Mx[q][1] * B[1][p]);
   }
+  double Vu[3][3];
+  adj_vu64(g, tb, a, Vu);
+  // the geodesic substep: (I - A)^{-1}, and its change along u_1, u_2, u_3 (P)
   DF K[2][2];
+  double P[2][3];
   {
     GeoInc<DF> m;
     geo_inc_setup(k, a.L, a.u1, 1.0f, m);
-    DF A[2][2];
+    DF A[2][2], d3[2];
     geo_inc_jacobian(m, a.dg[0], a.dg[1], A);
+    geo_inc_d3(a.L, m, a.u1[2], a.dg[0], a.dg[1], d3);
     adj_inv(A, K);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+#pragma unroll
+      for (int p = 0; p < 2; ++p)
+        P[q][p] = df_to_double(df_scale(fma_(K[q][0], A[0][p], K[q][1] * A[1][p]), 2.0f));
+      P[q][2] = df_to_double(fma_(K[q][0], d3[0], K[q][1] * d3[1]));
+    }
   }
-  // Three pairs of columns, (x1, x2), (u1, u2), (u3, scale), through one copy of the code: the
-  // kernel waits for instructions more than for anything else, so that the metric's derivatives
-  // ride along as zeros in the second and third pass costs less than a second instance.
-  const DF zero(0.0f), one(1.0f);
-  Local<D2F> L;
-  D2F eB[3], eD[3];
-  {  // x1, x2: metric, tetrads and fields move
+  {  // x1, x2: metric, tetrads and fields move; pairs
+    Local<D2F> L;
+    D2F eB[3], eD[3];
     const D2F R(a.r, k.dxi * a.r, zero), S(a.s, zero, a.c * k.dth), C(a.c, zero, -(a.s * k.dth));
     inc_local(k, R, S, C, L);
     IncLerp l;
@@ -550,49 +644,73 @@ __device__ __forceinline__ void adj_inc_jacobian(const GridP &g, const FieldPtrs
       eB[q] = e * eB[q];
       eD[q] = e * eD[q];
     }
-  }
-#pragma unroll 1
-  for (int pass = 0; pass < 3; ++pass) {
-    const DF s0 = pass == 1 ? one : zero, s2 = pass == 2 ? one : zero;
-    if (pass == 1) {
-      D2F *m = reinterpret_cast<D2F *>(&L);
-      for (int q = 0; q < (int)(sizeof(L) / sizeof(D2F)); ++q) m[q].d0 = m[q].d1 = zero;
-    }
-    if (pass > 0)
-#pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        eB[q].d0 = eD[q].d0 = zero;
-        eB[q].d1 = s2 * a.eB1[q];
-        eD[q].d1 = s2 * a.eD1[q];
-      }
-    // seeds of the first and second direction of the pass: u1, u2; u3, scale
-    const D2F u[3] = {D2F(a.u[0], s0, zero), D2F(a.u[1], zero, s0), D2F(a.u[2], s2, zero)};
     D2F du[3];
-    adj_momentum_d(k, L, eD, eB, u, a, K, du);
+    adj_momentum_d(k, L, eD, eB, a, K, du);
+    const DF u64[3] = {df_of(Vu[0][0]), df_of(Vu[1][1]), df_of(Vu[2][2])};
+    const DF x01 = df_of(Vu[0][1]), x02 = df_of(Vu[0][2]), x12 = df_of(Vu[1][2]);
 #pragma unroll 1
-    for (int d = 0; d < 2; ++d) {
-      // the increments' derivatives from that of u^{n+1} (seed + du') and of x^n (xs)
-      const int col = 2 * pass + d;
-      DF w3[3], p[3], v[3];
+    for (int col = 0; col < 2; ++col) {
+      DF w3[3], x[3], f[3];
 #pragma unroll
       for (int q = 0; q < 3; ++q) {
-        w3[q] = d ? du[q].d1 : du[q].d0;
-        p[q] = (d ? u[q].d1 : u[q].d0) + w3[q];
+        w3[q] = col ? du[q].d1 : du[q].d0;
+        x[q] = col ? Vx[q][1] : Vx[q][0];
       }
-      const DF xs0 = col == 0 ? one : zero, xs1 = col == 1 ? one : zero;
-#pragma unroll
-      for (int q = 0; q < 3; ++q)
-        v[q] = fma_(Vu[q][0], p[0], fma_(Vu[q][1], p[1], fma_(Vu[q][2], p[2],
-               fma_(Vx[q][0], xs0, Vx[q][1] * xs1))));
-      const DF y0 = k.dt * fma_(Mx[0][0], v[0], Mx[0][1] * v[1]);
-      const DF y1 = k.dt * fma_(Mx[1][0], v[0], Mx[1][1] * v[1]);
+      f[0] = fma_(u64[0], w3[0], fma_(x01, w3[1], fma_(x02, w3[2], x[0])));
+      f[1] = fma_(x01, w3[0], fma_(u64[1], w3[1], fma_(x12, w3[2], x[1])));
+      f[2] = fma_(x02, w3[0], fma_(x12, w3[1], fma_(u64[2], w3[2], x[2])));
+      const DF y0 = k.dt * (f[0] + fma_(N[0][0], f[0], N[0][1] * f[1]));
+      const DF y1 = k.dt * (f[1] + fma_(N[1][0], f[0], N[1][1] * f[1]));
       // dphi/dt moves with the midpoint, x + y/2
-      const DF ph = k.dt * (v[2] + df_scale(fma_(Vx[2][0], y0, Vx[2][1] * y1), 0.5f));
+      const DF ph = k.dt * (f[2] + df_scale(fma_(Vx[2][0], y0, Vx[2][1] * y1), 0.5f));
       const DF o[6] = {y0, y1, ph, w3[0], w3[1], w3[2]};
 #pragma unroll
       for (int q = 0; q < 6; ++q)
         w[(int64_t)(q * JC + col) * n] = adj_pack(o[q], q == 0 && col == 0);
     }
+  }
+  // u_1, u_2, u_3 and the scale: the metric's values alone, in FP64
+  Strong sw;
+  strong_frame(g, F.B, F.D, tb, a.i1, a.i2, a.dx[0], a.dx[1], qm64, sw);
+  HalfStep h[2];
+  {
+    const double u0[3] = {st[3], st[4], st[5]};
+    adj_half64(sw, scale64, u0, h[0]);
+    double u2[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) u2[q] = df_to_double(a.u2[q]);
+    adj_half64(sw, scale64, u2, h[1]);
+  }
+  double Nx[2][2], Vp[2];
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    Nx[q][0] = df_to_double(N[q][0]);
+    Nx[q][1] = df_to_double(N[q][1]);
+    Vp[q] = 0.5 * df_to_double(Vx[2][q]);
+  }
+#pragma unroll 1
+  for (int col = 2; col < JC; ++col) {
+    const double s[3] = {col == 2 ? 1.0 : 0.0, col == 3 ? 1.0 : 0.0, col == 4 ? 1.0 : 0.0};
+    const double ds = col == 5 ? 1.0 : 0.0;
+    double dw[3] = {0.0, 0.0, 0.0}, d[3];
+    adj_half64_d(sw, h[0], scale64, s, ds, dw);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) d[q] = s[q] + dw[q];
+    dw[0] += fma(P[0][0], d[0], fma(P[0][1], d[1], P[0][2] * d[2]));
+    dw[1] += fma(P[1][0], d[0], fma(P[1][1], d[1], P[1][2] * d[2]));
+#pragma unroll
+    for (int q = 0; q < 2; ++q) d[q] = s[q] + dw[q];
+    adj_half64_d(sw, h[1], scale64, d, ds, dw);
+    double f[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) d[q] = s[q] + dw[q];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) f[q] = fma(Vu[q][0], d[0], fma(Vu[q][1], d[1], Vu[q][2] * d[2]));
+    const double y0 = g.dt * (f[0] + fma(Nx[0][0], f[0], Nx[0][1] * f[1]));
+    const double y1 = g.dt * (f[1] + fma(Nx[1][0], f[0], Nx[1][1] * f[1]));
+    const double o[6] = {y0, y1, g.dt * (f[2] + fma(Vp[0], y0, Vp[1] * y1)), dw[0], dw[1], dw[2]};
+#pragma unroll
+    for (int q = 0; q < 6; ++q) wd[(int64_t)(q * JC + col) * n] = o[q];
   }
 }
 
@@ -607,7 +725,7 @@ __device__ __forceinline__ bool adj_advance(const GridP &g, const FieldPtrsT<dou
     if (adj_inc_step(g, F, tb, k, st, scale_df, qm_df, n_iter, a)) {
       const bool ok = a.x64[0] >= 0.0 && a.x64[0] < g.n_r && a.x64[1] >= 0.0 && a.x64[1] <= g.n_th;
       if (!ok) return false;
-      if (w) adj_inc_jacobian(g, F, tb, k, scale_df, qm_df, a, w, n);
+      if (w) adj_inc_jacobian(g, F, tb, k, st, scale, qm, scale_df, qm_df, a, w, n);
       st[0] = a.x64[0];
       st[1] = a.x64[1];
       st[2] = fma(g.dt, a.v3, st[2]);
@@ -659,8 +777,8 @@ __global__ void __launch_bounds__(TPB_ADJ) k_adj_forward(
 }
 
 // lambda <- J^T lambda and the scale's derivative. With J - 1 in pairs: lambda += (J - 1)^T
-// lambda, the products in pairs on lambda scaled by the power of two that brings its largest
-// entry near 1 (any magnitude keeps its bits), the sums in FP64.
+// lambda, the pairs' products in pairs on lambda scaled by the power of two that brings its
+// largest entry near 1 (any magnitude keeps its bits), the others and the sums in FP64.
 __device__ __forceinline__ void adj_reverse(const double *w, int64_t n, double lam[6],
                                             double &gs) {
   // inputs x1, x2, u1, u2, u3 are state rows 0, 1, 3, 4, 5; phi passes through
@@ -685,30 +803,35 @@ __device__ __forceinline__ void adj_reverse(const double *w, int64_t n, double l
   DF l[6];
 #pragma unroll
   for (int q = 0; q < 6; ++q) l[q] = df_of(lam[q] * down);
-  DF nl[JC];
-#pragma unroll
-  for (int c = 0; c < JC; ++c) nl[c] = DF(0.0f);
+  DF nl[2] = {DF(0.0f), DF(0.0f)};
+  double nd[JC] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
 #pragma unroll
   for (int r = 0; r < 6; ++r)
 #pragma unroll
     for (int c = 0; c < JC; ++c) {
-      const float2 v = reinterpret_cast<const float2 *>(w)[(int64_t)(r * JC + c) * n];
-      nl[c] = fma_(DF(v.y, v.x), l[r], nl[c]);
+      const double *e = w + (int64_t)(r * JC + c) * n;
+      if (adj_is64(c)) {
+        nd[c] = fma(*e, lam[r], nd[c]);
+      } else {
+        const float2 v = *reinterpret_cast<const float2 *>(e);
+        nl[c] = fma_(DF(v.y, v.x), l[r], nl[c]);
+      }
     }
   const bool lost = top == 0x7ffu;  // infinities and NaN stay such
 #pragma unroll
-  for (int c = 0; c < 5; ++c)
-    lam[row[c]] = lost ? lam[row[c]] + NAN : fma(df_to_double(nl[c]), up, lam[row[c]]);
-  gs = lost ? NAN : fma(df_to_double(nl[5]), up, gs);
+  for (int c = 0; c < 2; ++c) nd[c] = df_to_double(nl[c]) * up;
+#pragma unroll
+  for (int c = 0; c < 5; ++c) lam[row[c]] += lost ? NAN : nd[c];
+  gs += lost ? NAN : nd[5];
 }
 
-// The step's code (about 20,000 instructions) is larger than the instruction caches: warps that
-// wander through it apart from one another fetch it once each, and most of their time went to
-// waiting for instructions (7.0 of 10.9 cycles between issues). The barrier before each step
+// The step's code is larger than the instruction caches: warps that wander through it apart from
+// one another fetch it once each, and most of their time went to waiting for instructions (7.0 of
+// 10.9 cycles between issues, with all derivatives in pairs). The barrier before each step
 // keeps a block's warps together, so that a fetch serves all of them; every thread reaches it,
-// particles or none. Together with one copy of the Jacobian's code for all columns: 39.6 ->
-// 31.0 ms for 65,536 orbits, 100 steps forward and back, events around repeated passes; 1 x 256,
-// 2 x 256 and 4 x 128 threads per SM measured 1 to 8% slower. Barriers inside the step as well
+// particles or none. Together with one copy of the Jacobian's code for all columns that gave 39.6
+// -> 31.0 ms for 65,536 orbits, 100 steps forward and back, events around repeated passes; 1 x
+// 256, 2 x 256 and 4 x 128 threads per SM measured 1 to 8% slower. Barriers inside the step as well
 // took twice as long (what a step keeps across them goes to local memory).
 #ifndef GRPIC_ADJ_BWD_TPB
 #define GRPIC_ADJ_BWD_TPB 128

@@ -225,6 +225,20 @@ __device__ __forceinline__ void geo_inc_jacobian(const GeoInc<R> &m, R d0, R d1,
   J[1][0] = half_(m.D2b - fma_(g0, m.D2a, fma_(a0, k2, ha * (twice_(m.d2H11 * b0) + m.f2))));
   J[1][1] = -half_(fma_(g1, m.D2a, fma_(a1, k2, ha * twice_(m.d2H22 * b1))));
 }
+// the map's derivative by u_3 (through c0, c1, e1, e2, f1, f2 of geo_inc_setup)
+__device__ __forceinline__ void geo_inc_d3(const Local<DF> &L, const GeoInc<DF> &m, DF u3, DF d0,
+                                           DF d1, DF d[2]) {
+  const DF b0 = m.u0 + half_(d0), b1 = m.u1 + half_(d1), b1s = b1 * b1;
+  const DF q = fma_(b0, fma_(m.H11, b0, m.c1), fma_(m.H22, b1s, m.c0));
+  const DF ig = rsqrt_(q), ha = m.hdt * ig;
+  const DF k1 = fma_(b0, fma_(m.d1H11, b0, m.e2), fma_(m.d1H22, b1s, m.e1));
+  const DF k2 = fma_(b0, fma_(m.d2H11, b0, m.f2), fma_(m.d2H22, b1s, m.f1));
+  const DF dq = fma_(L.G.H33, u3, L.G.H13 * b0);        // half of dq/du_3
+  const DF dg = ig * dq, dh = -(ha * ig * ig * dq);      // of gamma_bar, ha
+  const DF g1 = twice_(fma_(L.d1H33, u3, L.d1H13 * b0)), g2 = twice_(fma_(L.d2H33, u3, L.d2H13 * b0));
+  d[0] = -fma_(dg, m.D1a, fma_(dh, k1, ha * g1));
+  d[1] = -fma_(dg, m.D2a, fma_(dh, k2, ha * g2));
+}
 // whether the method's n_iter iterations come within a tenth of tol of the fixed point
 // (method_converges on FP32 values)
 __device__ __forceinline__ bool inc_converges(float d1, const float J[2][2], int n_iter, float tol,
@@ -446,6 +460,54 @@ __device__ __forceinline__ void inc_point64(const GridP &g, const PushTables &tb
   }
 }
 
+// The tetrad and the fields in it (times e = qm alpha dt/4) at x^n in FP64: for the half steps in
+// strong fields, and the adjoint's derivative by the amplitude
+struct Strong {
+  double rH11, sH11, rh22, sh22, rh33, sh33, k13, m13, eB[3], eD[3];
+};
+__device__ __forceinline__ void strong_frame(const GridP &g, double *const B[3],
+                                             double *const D[3], const PushTables &tb, int i1,
+                                             int i2, double dx1, double dx2, double qm,
+                                             Strong &w) {
+  double r, s, c;
+  inc_point64(g, tb, i1, i2, dx1, dx2, __dadd_rn((double)i2, dx2), r, s, c);
+  const double s2 = s * s, r2 = r * r, f = g.dxi * r;
+  const double Sig = fma(g.a2, c * c, r2), M2r = g.M2 * r, S2 = Sig + M2r;
+  const double Rr = r2 + g.a2, A = fma(Rr, Rr, -(g.a2 * s2 * (Rr - M2r)));
+  const double rSig = rsqrt(Sig), rS2 = rsqrt(S2), rA = rsqrt(A);
+  const double ifs = rcp_nr(f * s), qSig = Sig * rSig, qA = A * rA;
+  w.rH11 = f * qSig * (S2 * rS2) * rA;
+  w.sH11 = ifs * s * (rSig * rS2) * qA;
+  w.rh22 = rSig * (g.ig2 * g.dth);
+  w.sh22 = qSig * g.dth;
+  w.rh33 = qSig * rA * (ifs * f);
+  w.sh33 = s * rSig * qA;
+  const double faS = f * g.a * S2;
+  w.k13 = -(faS * (s * rSig) * rA);
+  w.m13 = -(faS * (rA * rA));
+  const double e = 0.25 * qm * (qSig * rS2) * g.dt;  // half of qm alpha dt/2
+  const bool l1 = lt_pos(dx1, 0.5) || dx1 == 0.0, l2 = lt_pos(dx2, 0.5) || dx2 == 0.0;
+  const double w1[2] = {dx1, l1 ? dx1 + 0.5 : dx1 - 0.5}, w2[2] = {dx2, l2 ? dx2 + 0.5 : dx2 - 0.5};
+  double V[6];
+#pragma unroll 1
+  for (int q = 0; q < 6; ++q) {  // one copy of the code
+    const int h1 = q == 1 || q == 2 || q == 3, h2 = q == 0 || q == 2 || q == 4;
+    const double *pl = q < 3 ? B[q] : D[q - 3];
+    const double *p = pl + sidx(g, i1 - (h1 && l1 ? 1 : 0), i2 - (h2 && l2 ? 1 : 0));
+    const double p00 = __ldg(p), p10 = __ldg(p + 1), p01 = __ldg(p + g.NX), p11 = __ldg(p + g.NX + 1);
+    const double a1 = h1 ? w1[1] : w1[0], a2 = h2 ? w2[1] : w2[0];
+    const double x = fma(a1, p10 - p00, p00), y = fma(a1, p11 - p01, p01);
+    V[q] = fma(a2, y - x, x);
+  }
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const double *v = V + 3 * q;
+    double *o = q ? w.eD : w.eB;
+    o[0] = e * (v[0] * w.rH11);
+    o[1] = e * (w.sh22 * v[1]);
+    o[2] = e * fma(w.k13, v[0], w.sh33 * v[2]);
+  }
+}
 // The FP64 evaluation of the map t -> dx + dt V((x^n + t)/2) that the result comes from, in
 // inc_velocity's grouping: ~80 FP64 operations.
 __device__ __forceinline__ void inc_coord64(const GridP &g, const PushTables &tb, int i1, int i2,

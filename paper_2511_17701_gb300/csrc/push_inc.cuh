@@ -26,52 +26,7 @@ __device__ __forceinline__ bool inc_small(const GridP &g, const FieldPtrsT<doubl
   return e * e * (BB + DD) <= INC_MAX * INC_MAX;
 }
 
-// The tetrad, the fields in it and the Boris half steps in FP64, for strong fields
-struct Strong {
-  double rH11, sH11, rh22, sh22, rh33, sh33, k13, m13, eB[3], eD[3];
-};
-__device__ __forceinline__ void strong_frame(const GridP &g, const FieldPtrsT<double> &F,
-                                             const PushTables &tb, int i1, int i2, double dx1,
-                                             double dx2, double qm, Strong &w) {
-  double r, s, c;
-  inc_point64(g, tb, i1, i2, dx1, dx2, __dadd_rn((double)i2, dx2), r, s, c);
-  const double s2 = s * s, r2 = r * r, f = g.dxi * r;
-  const double Sig = fma(g.a2, c * c, r2), M2r = g.M2 * r, S2 = Sig + M2r;
-  const double Rr = r2 + g.a2, A = fma(Rr, Rr, -(g.a2 * s2 * (Rr - M2r)));
-  const double rSig = rsqrt(Sig), rS2 = rsqrt(S2), rA = rsqrt(A);
-  const double ifs = rcp_nr(f * s), qSig = Sig * rSig, qA = A * rA;
-  w.rH11 = f * qSig * (S2 * rS2) * rA;
-  w.sH11 = ifs * s * (rSig * rS2) * qA;
-  w.rh22 = rSig * (g.ig2 * g.dth);
-  w.sh22 = qSig * g.dth;
-  w.rh33 = qSig * rA * (ifs * f);
-  w.sh33 = s * rSig * qA;
-  const double faS = f * g.a * S2;
-  w.k13 = -(faS * (s * rSig) * rA);
-  w.m13 = -(faS * (rA * rA));
-  const double e = 0.25 * qm * (qSig * rS2) * g.dt;  // half of qm alpha dt/2
-  const bool l1 = lt_pos(dx1, 0.5) || dx1 == 0.0, l2 = lt_pos(dx2, 0.5) || dx2 == 0.0;
-  const double w1[2] = {dx1, l1 ? dx1 + 0.5 : dx1 - 0.5}, w2[2] = {dx2, l2 ? dx2 + 0.5 : dx2 - 0.5};
-  double V[6];
-#pragma unroll 1
-  for (int q = 0; q < 6; ++q) {  // one copy of the code: see push_inc
-    const int h1 = q == 1 || q == 2 || q == 3, h2 = q == 0 || q == 2 || q == 4;
-    const double *pl = q < 3 ? F.Bn[q] : F.D[q - 3];
-    const double *p = pl + sidx(g, i1 - (h1 && l1 ? 1 : 0), i2 - (h2 && l2 ? 1 : 0));
-    const double p00 = __ldg(p), p10 = __ldg(p + 1), p01 = __ldg(p + g.NX), p11 = __ldg(p + g.NX + 1);
-    const double a1 = h1 ? w1[1] : w1[0], a2 = h2 ? w2[1] : w2[0];
-    const double x = fma(a1, p10 - p00, p00), y = fma(a1, p11 - p01, p01);
-    V[q] = fma(a2, y - x, x);
-  }
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    const double *v = V + 3 * q;
-    double *o = q ? w.eD : w.eB;
-    o[0] = e * (v[0] * w.rH11);
-    o[1] = e * (w.sh22 * v[1]);
-    o[2] = e * fma(w.k13, v[0], w.sh33 * v[2]);
-  }
-}
+// A Boris half step in FP64, for strong fields
 // (u + hat_cov(x) with the half step's change x in that frame, not hat_cov(cov_hat(u) + x): the two
 // maps' roundings then enter with the change, not with u)
 __device__ __forceinline__ void strong_boris(const Strong &w, double u[3]) {
@@ -280,7 +235,7 @@ __device__ __forceinline__ bool push_inc(const GridP &g, const FieldPtrsT<double
       weak = inc_boris(L, eD, eB, u, inc_limit(1.0f), du);
     }
     if (!weak) {
-      strong_frame(g, F, tb, i1, i2, dx1, dx2, s.qm, w);
+      strong_frame(g, F.Bn, F.D, tb, i1, i2, dx1, dx2, s.qm, w);
       strong_boris(w, un);
 #pragma unroll
       for (int q = 0; q < 3; ++q) ud[q] = df_of(un[q]);
