@@ -823,13 +823,13 @@ __device__ __forceinline__ void zigzag32(const GridP &g, const Move32 &m, float 
 __device__ __forceinline__ void zigzag_df(const GridP &g, DF q, int i, int j, DF a1, DF a2, int c1,
                                           int c2, DF b1, DF b2, DF v3, float c[3][4],
                                           int cell[3]) {
-  const DF qi = q * df_of(g.idt);
+  const DF idt = df_of(g.idt);
   const DF m1 = df_scale(a1 + b1, 0.5f), m2 = df_scale(a2 + b2, 0.5f);
   const DF r1 = c1 == 0 ? m1 : DF(c1 > 0 ? 1.0f : (float)(c1 + 1));
   const DF r2 = c2 == 0 ? m2 : DF(c2 > 0 ? 1.0f : (float)(c2 + 1));
 #pragma unroll
   for (int seg = 0; seg < 2; ++seg) {
-    const DF F1 = qi * (seg ? b1 - r1 : r1 - a1), F2 = qi * (seg ? b2 - r2 : r2 - a2);
+    const DF F1 = q * (seg ? b1 - r1 : r1 - a1) * idt, F2 = q * (seg ? b2 - r2 : r2 - a2) * idt;
     const DF W1 = seg ? df_scale(r1 + b1, 0.5f) + DF(-(float)c1) : df_scale(a1 + r1, 0.5f);
     const DF W2 = seg ? df_scale(r2 + b2, 0.5f) + DF(-(float)c2) : df_scale(a2 + r2, 0.5f);
     const DF t = F1 * W2, v = F2 * W1;
@@ -1136,6 +1136,16 @@ __device__ __forceinline__ bool push_axis(const GridP &g, const FieldPtrsT<float
     local_guard<Q>(g, p, L);
   }
   DF Bh[3], Dh[3], uh[3], u[3] = {DF(s.u1[k]), DF(s.u2[k]), DF(s.u3[k])};
+  // a massless particle's momentum has no scale, but its squares leave FP32's range: in the unit
+  // of the power of two next to its largest component (exactly; push_inc.cuh's photon_unit)
+  int unit = 0;
+  if (!em) {
+    const float top = fmaxf(fabsf(u[0].hi), fmaxf(fabsf(u[1].hi), fabsf(u[2].hi)));
+    unit = min(max((int)(__float_as_uint(top) >> 23) - 127, -120), 120);
+    const float down = __uint_as_float((unsigned)(127 - unit) << 23);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) u[q] = df_scale(u[q], down);
+  }
   const DF hq = df_scale(df_of(s.qm) * L.alpha * dt, 0.5f);
   if (em) {
     DF V[3] = {interp_axis(F.Bn[0], g.NX, i1, i2, dx1, dx2, false, true),
@@ -1203,7 +1213,8 @@ __device__ __forceinline__ bool push_axis(const GridP &g, const FieldPtrsT<float
     count(diag, DG_REFLECT);
   }
   s.i1[k] = j1; s.i2[k] = j2; s.dx1[k] = e1.hi; s.dx2[k] = e2.hi;
-  s.u1[k] = u[0].hi; s.u2[k] = u[1].hi; s.u3[k] = u[2].hi;
+  const float back = __uint_as_float((unsigned)(127 + unit) << 23);
+  s.u1[k] = u[0].hi * back; s.u2[k] = u[1].hi * back; s.u3[k] = u[2].hi * back;
   if (j1 < 0) { s.tag[k] = 2; count(diag, DG_LEFT_INNER); }
   else if (j1 >= g.n_r) { s.tag[k] = 2; count(diag, DG_LEFT_OUTER); }
   // step 11: phi at the midpoint of x^n and the final x^{n+1}
@@ -1215,7 +1226,7 @@ __device__ __forceinline__ bool push_axis(const GridP &g, const FieldPtrsT<float
   const DF v3 = rsqrt_(o.opz * gamma2_df(o, u, m2)) * fma_(o.H13, u[0], o.H33 * u[2]);
   s.phi[k] = fma_(dt, v3, DF(s.phi[k])).hi;
   if (!(j1 >= -G_ && j1 <= g.n_r)) return false;
-  zigzag_df(g, df_of(s.qc) * DF(s.w[k]), i1, i2, o1, o2, c1, c2, b1, b2, v3, c, cell);
+  zigzag_df(g, df_of(s.qc * (double)s.w[k]), i1, i2, o1, o2, c1, c2, b1, b2, v3, c, cell);
   return true;
 }
 
