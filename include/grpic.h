@@ -146,8 +146,9 @@ typedef struct {
                            (rho < 1 the contraction of the iteration), in fewer FP64
                            operations. On the plain log-r grid the momentum's increments (steps
                            2 to 9) are formed in pairs of FP32 numbers (48 bits) where they are
-                           small against the momentum and added in FP64, which leaves a smaller
-                           error than FP64 throughout. Must be below 1e-6                      */
+                           at most 2^-5 of the momentum (larger ones in FP64) and added in
+                           FP64, which leaves errors of FP64's own size or smaller. Must be
+                           below 1e-6                                                          */
   double r0, h0;        /* quasi-spherical Kerr-Schild grid (App. A): r = r0 + exp(xi), xi
                            uniform in x1 (r0 < r_min); theta = eta + 2 h0 eta (pi - 2 eta)
                            (pi - eta) / pi^2, eta uniform in x2 (-1/2 < h0 < 1; h0 > 0 puts

@@ -904,7 +904,7 @@ __global__ void __launch_bounds__(1024) k_sum(const double *__restrict__ x, int6
 
 int adj_blocks(int64_t n, int tpb) {
   int64_t b = (n + tpb - 1) / tpb;
-  const int64_t cap = 152 * 32;
+  const int64_t cap = N_SM * 32;
   return (int)(b < 1 ? 1 : (b > cap ? cap : b));
 }
 

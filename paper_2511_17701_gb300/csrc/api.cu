@@ -1006,8 +1006,8 @@ grpic_status step_once(grpic_ctx *ctx, const HostIO *io) {
     PhaseTimer t(ctx, PH_PUSH);  // fused push + deposit of every species
     if (ctx->mixed) CK(do_zero_J(ctx, ctx->F32));
     else CK(do_zero_J(ctx, ctx->F64));
-    // mixed: the guard stages of all species first, so that their FP64 kernels (the longer
-    // chain, on the side stream) run beside all the FP32 kernels instead of trailing the last
+    // mixed: the guard stages of all species first, so that their kernels (the longer chains,
+    // on the side streams) run beside all the FP32 kernels instead of trailing the last
     if (ctx->mixed)
       for (int k = 0; k < ctx->cfg.n_species; ++k)
         if (ctx->sp[k].loaded)

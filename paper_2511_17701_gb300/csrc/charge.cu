@@ -99,7 +99,7 @@ cudaError_t launch_charge_rho(const GridP &g, SpeciesDevT<T> s, int64_t n_bound,
                               cudaStream_t st) {
   if (n_bound <= 0) return cudaGetLastError();
   int64_t b = (n_bound + TPB_Q - 1) / TPB_Q;
-  if (b > 152 * 32) b = 152 * 32;
+  if (b > N_SM * 32) b = N_SM * 32;
   k_rho<T><<<(int)b, TPB_Q, 0, st>>>(g, s, rho_prev, rho_new, rho_abs);
   COUNT_LAUNCH(1);
   return cudaGetLastError();
@@ -113,7 +113,7 @@ cudaError_t launch_continuity(const GridP &g, const T *J1, const T *J2, const do
   if (e != cudaSuccess) return e;
   const int64_t nodes = (int64_t)(g.n_r + 3) * (g.n_th + 1);
   int64_t b = (nodes + TPB_Q - 1) / TPB_Q;
-  if (b > 152 * 8) b = 152 * 8;
+  if (b > N_SM * 8) b = N_SM * 8;
   k_continuity<T><<<(int)b, TPB_Q, 0, st>>>(g, J1, J2, rho_prev, rho_new, rho_abs, out);
   COUNT_LAUNCH(1);
   return cudaGetLastError();

@@ -1,10 +1,12 @@
-// dfloat.cuh -- unevaluated sums of two floats ("double-float", about 48 significant bits)
-// for the FP64 pusher's predictor: GB300's FP64 pipe bounds that kernel while its FP32 pipe
-// and instruction issue are mostly idle, so a predictor step carried in pairs of FP32 numbers
-// (Dekker's and Knuth's error-free transformations: the rounding error of an FP32 sum is
-// recovered with two-sum, that of a product with one fused multiply-add) lands within about
-// 1e-14 of the FP64 fixed point at FP32-pipe cost. Only start points come from here: every
-// result the pusher stores is an FP64 evaluation checked in FP64.
+// dfloat.cuh -- unevaluated sums of two floats ("double-float", about 48 significant bits).
+// GB300's FP64 pipe bounds the FP64 pusher while its FP32 pipe and instruction issue are mostly
+// idle, so work carried in pairs of FP32 numbers (Dekker's and Knuth's error-free
+// transformations: the rounding error of an FP32 sum is recovered with two-sum, that of a product
+// with one fused multiply-add) costs it little. Two kinds of use: a predictor that lands within
+// about 1e-14 of an FP64 fixed point, whose result is an FP64 evaluation checked in FP64; and
+// quantities whose 2^-48 is enough because they are a small part of what they are added to in
+// FP64 (inc.cuh) or are rounded to FP32 (the mixed path's guard zones). A pair has FP32's range of
+// exponents: what is outside about 2^-74 to 2^128 has to be kept from it (df_of).
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -98,9 +100,9 @@ __device__ __forceinline__ DF rsqrt_(DF x) { return df_rsqrt(x); }
 
 // a double split into a pair on the integer pipe: hi its leading 24 bits (truncated), lo
 // the next 24 of the remaining 29 (rounded by the integer-to-float conversion), so the pair
-// holds the double to about 2^-48 of itself; zero, subnormals, values below about 2^-100 in
-// the low part and non-finite values keep only hi (the predictor needs their leading bits
-// only)
+// holds the double to about 2^-48 of itself. Below 2^-74 the low part is left out (24 bits), below
+// 2^-126 the result is zero, from 2^128 on infinite: callers for which that matters test or scale
+// the double first (inc_charge, photon_unit).
 __device__ __forceinline__ DF df_of(double x) {
   const unsigned hi32 = (unsigned)__double2hiint(x), lo32 = (unsigned)__double2loint(x);
   const unsigned sign = hi32 & 0x80000000u, ex = (hi32 >> 20) & 0x7ffu;

@@ -10,7 +10,7 @@ namespace {
 constexpr int TPB = 256;
 
 // ---------------------------------------------------------------------------------
-// Coefficient tables of the field solver, FieldTab (grpic_internal.cuh): per component of
+// Coefficient tables of the field solver, T_... (grpic_internal.cuh): per component of
 // Eqs. (discretized-auxE), (discretized-auxH) the factor of every field value that enters it
 // (alpha h_ii; alpha sqrt(h~) h_13 / (2 sqrt(h~)) and sqrt(h~ h) beta^1 / (2 sqrt(h~)) of both
 // neighbours of an average), and dt / sqrt(h) of the curls, each formed in FP64 and rounded
@@ -660,7 +660,7 @@ __global__ void k_zero(T *p, int64_t n) {
 
 int blocks_for(int64_t n) {
   int64_t b = (n + TPB - 1) / TPB;
-  if (b > 152 * 32) b = 152 * 32;
+  if (b > N_SM * 32) b = N_SM * 32;
   return (int)(b < 1 ? 1 : b);
 }
 
@@ -693,13 +693,13 @@ void axis(const GridP &g, T *const p[3], int isB, cudaStream_t st) {
 }
 
 // Blocks covering ni x nj points: TPBX x TPBY, or 32 x 2 on grids that would not give every SM
-// two of those (64^2 points were 19 blocks, 8 warps of FP64 work on each of 19 SMs); rows beyond
-// the grid's limit in y are taken by the kernels' row loop
+// two of those (64^2 cells were 34 or 36 blocks, 8 warps of FP64 work on each of as many SMs);
+// rows beyond the grid's limit in y are taken by the kernels' row loop
 struct Tiles {
   dim3 grid, block;
 };
 Tiles tiles_for(int ni, int nj) {
-  const bool few = (int64_t)ni * nj < 2 * 152 * TPBX * TPBY;
+  const bool few = (int64_t)ni * nj < 2 * N_SM * TPBX * TPBY;
   const int bx = few ? 32 : TPBX, by = few ? 2 : TPBY, ny = (nj + by - 1) / by;
   return {dim3((ni + bx - 1) / bx, ny > 65535 ? 65535 : ny), dim3(bx, by)};
 }

@@ -23,7 +23,7 @@ namespace {
 
 constexpr int FT_X = 64, FT_Y = 32, F_MAXP = 8, F_TPB = 512;
 // The output tile of a block: FT_X x FT_Y, or FS_X x FS_Y on grids whose large tiles would leave
-// most SMs without one (64^2 points: 9 blocks, 22 us for 4 passes, of which all but the few SMs
+// most SMs without one (64^2 cells: 18 blocks, 22 us for 4 passes, of which all but the few SMs
 // in use see nothing); the small tiles' halo costs more arithmetic in all, but on idle SMs.
 constexpr int FS_X = 16, FS_Y = 8, FS_TPB = 128;
 
@@ -132,7 +132,7 @@ cudaError_t filter_chunk(const GridP &g, const FilterPlanes<T> &fp, int n_comp, 
     attr = true;
   }
   const int64_t large = (int64_t)((g.NX + FT_X - 1) / FT_X) * ((g.NY + FT_Y - 1) / FT_Y) * n_comp;
-  const bool few = large < 152;
+  const bool few = large < N_SM;
   const int tx = few ? FS_X : FT_X, ty = few ? FS_Y : FT_Y;
   const dim3 grid((g.NX + tx - 1) / tx, (g.NY + ty - 1) / ty, n_comp);
   k_filter<T><<<grid, few ? FS_TPB : F_TPB, filter_smem<T>(tx, ty, P), st>>>(g, fp, P, tx, ty);

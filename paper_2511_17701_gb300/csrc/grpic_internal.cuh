@@ -14,6 +14,7 @@
 #include "../../include/grpic.h"
 
 #define G_ GRPIC_GHOSTS
+constexpr int N_SM = 152;  // of a GB300: the unit of grid sizes and of "fills the GPU"
 #define GRPIC_PI 3.14159265358979323846
 
 // Grid and step parameters passed by value to every kernel.
@@ -372,11 +373,11 @@ struct PushTables {
   const float2 *r_df, *s_df, *c_df;
   const float2 *t1_df, *t2_df;  // the quasi-spherical theta offset's t1, t2 as pairs
   int guard_ilo, guard_ihi;  // cells guard_ilo <= i1 < guard_ihi (around the horizon) and
-  int guard_j;               // within guard_j of an axis evaluate the metric in FP64
+  int guard_j;               // within guard_j of an axis evaluate the metric in float pairs
 };
 
-// The guard particles of one species for the current push (mixed path): zone 1 (FP64
-// metric) indices ascending from idx[0], zone 2 (the cell rows on the axes, FP64 routine)
+// The guard particles of one species for the current push (mixed path): zone 1 (metric in
+// pairs) indices ascending from idx[0], zone 2 (the cell rows on the axes, all in pairs)
 // descending from idx[cap - 1], counted in count[0], count[1]; bit k of mask marks particle
 // k as listed (written only by the classification, read by the FP32 kernel).
 struct GuardList {
@@ -400,11 +401,12 @@ struct TileInfo {
 };
 constexpr int TILE_HALO = 6;  // cells of the window beyond the tile on every side
 
-// Streams of one push: the classification and the FP64-pipe-bound guard kernels run on
+// Streams of one push: the classification and the guard kernel of the mixed path run on
 // `side`, forked from `main` by `fork`; `done` is recorded on `side` after them and the
-// caller makes `main` wait on it before anything reads the currents or the particles.
-// which part of a push to launch: the mixed path's guard stage (classify, then the FP64
-// guard kernels, all on `side`) and its main FP32 kernel (on `main`, after the classify) can
+// caller makes `main` wait on it before anything reads the currents or the particles. (FP64
+// pushes run on `main` alone.)
+// which part of a push to launch: the mixed path's guard stage (classify, then the guard
+// kernel, both on `side`) and its main FP32 kernel (on `main`, after the classify) can
 // be issued separately, so that the guard stages of all species start before the first FP32
 // kernel
 // stages of a mixed push: PUSH_GUARD = PUSH_CLASSIFY then PUSH_GUARD_KERNELS (side stream),

@@ -18,10 +18,10 @@
 // that the bounds behind this do not cover (an iteration that the predictor does not resolve,
 // values outside the range of FP32) is left to push64, untouched.
 //
-// Measured: a step of the 2048^2 workload (134 M particles) 173.6 -> 66.3 ms, of the 512^2 one
-// (16.8 M) 21.0 -> 9.35 ms. One push against 113-bit arithmetic, six grids from 64^2 to 2048^2
-// (60,000 particles each): rms errors of u 4.7-8.0e-17 of its rms (push64: 2.5-3.3e-16), of the
-// offsets 2.4-4.6e-17 (2.4-5.5e-17).
+// Measured: a step of the 2048^2 workload (134 M particles) 173.6 -> 70.5 ms, of the 512^2 one
+// (16.8 M) 21.0 -> 9.8 ms. One push against 80-bit arithmetic, 20,000 particles with |u| = 1, the
+// iterations run to rounding: rms errors of |u| 1.1e-16 on 64^2, 5.8e-17 on 512^2 (push64:
+// 3.6e-16 on both), of the offsets 2.6e-17 to 3.6e-17 (2.8e-17 to 4.3e-17).
 #pragma once
 #include "dual_df.cuh"
 #include "refine.cuh"
@@ -52,7 +52,8 @@ __device__ __forceinline__ bool inc_within(IncLimit lim, float dd, float uu) {
 constexpr float INC_E = 0.055f;      // largest |offset of xi| of the radial series
 constexpr float INC_D = 0.035f;      // largest |offset of theta| of the angular series
 constexpr int INC_ROWS = 64;          // rows from either axis with theta as map_theta rounds it
-constexpr float INC_R = 1024.0f;     // largest r: r^-8 and its low parts stay in FP32's range
+constexpr float INC_R = 1024.0f;     // largest r: the metric's smallest products, ~ r^-6 dxi^-2, keep
+                                     // their low parts in FP32's range
 
 __device__ __forceinline__ DF df2(const float2 v) { return DF(v.x, v.y); }
 
@@ -235,7 +236,8 @@ __device__ __forceinline__ void geo_inc_d3(const Local<DF> &L, const GeoInc<DF> 
   const DF k2 = fma_(b0, fma_(m.d2H11, b0, m.f2), fma_(m.d2H22, b1s, m.f1));
   const DF dq = fma_(L.G.H33, u3, L.G.H13 * b0);        // half of dq/du_3
   const DF dg = ig * dq, dh = -(ha * ig * ig * dq);      // of gamma_bar, ha
-  const DF g1 = twice_(fma_(L.d1H33, u3, L.d1H13 * b0)), g2 = twice_(fma_(L.d2H33, u3, L.d2H13 * b0));
+  const DF g1 = twice_(fma_(L.d1H33, u3, L.d1H13 * b0));
+  const DF g2 = twice_(fma_(L.d2H33, u3, L.d2H13 * b0));
   d[0] = -fma_(dg, m.D1a, fma_(dh, k1, ha * g1));
   d[1] = -fma_(dg, m.D2a, fma_(dh, k2, ha * g2));
 }
@@ -533,8 +535,9 @@ __device__ __forceinline__ void inc_coord64(const GridP &g, const PushTables &tb
 
 // The coordinate substep (n_iter, tol: the method's iterations and what they have to come
 // within; FINE: the FP64 evaluations stop once what is left, the contraction times the last
-// update, is below 2^-55, else once the update is within tol): as coord_refined (FP32 predictor, one step in pairs, FP64
-// evaluations until the stop rule holds), the FP32 and pair maps in inc_velocity's grouping.
+// update, is below 2^-55, else once the update is within tol): as coord_refined (FP32 predictor,
+// one step in pairs, FP64 evaluations until the stop rule holds), the FP32 and pair maps in
+// inc_velocity's grouping.
 template <bool FINE>
 __device__ __forceinline__ bool inc_coord(const GridP &g, const IncC &k, const PushTables &tb,
                                           int n_iter, float tol, int i1, int i2, double dx1, double dx2, DF o1, DF o2,

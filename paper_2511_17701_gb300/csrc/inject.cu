@@ -241,7 +241,7 @@ __global__ void k_inj_cursor(int64_t *cursor, int64_t v) { *cursor = v; }
 
 int blocks_of(int64_t n, int tpb) {
   int64_t b = (n + tpb - 1) / tpb;
-  return (int)(b < 152 * 16 ? (b > 0 ? b : 1) : 152 * 16);
+  return (int)(b < N_SM * 16 ? (b > 0 ? b : 1) : N_SM * 16);
 }
 
 }  // namespace

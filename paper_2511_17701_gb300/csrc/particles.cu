@@ -1,11 +1,13 @@
 // particles.cu -- the GR particle pusher (Sec. 3.1 of arXiv:2511.17701) and the
 // charge-conserving conformal current deposit (Sec. 3.2), one thread per particle.
 //
-// FP64 path: the double-precision pipe, not HBM, bounds the kernel on GB300 (every
-// particle-step evaluates the metric up to n_iter + 2 times). Mixed path: FP32 state,
-// fields and arithmetic; for particles within a few cells of the horizon or an axis the
-// metric, lapse and shift are evaluated in pairs of floats (and rounded), in a second kernel. Particle state is SoA; consecutive threads read consecutive elements,
-// and field gathers hit L1/L2 because the particles are kept sorted by cell.
+// FP64 path: the general routine (push64, here) evaluates the metric up to n_iter + 2 times per
+// particle in FP64, whose pipe, not HBM, bounds it on GB300; on the plain grid with iter_tol > 0
+// the increment form (push_inc.cuh) takes most particles, the routine the rest. Mixed path: FP32
+// state, fields and arithmetic; for particles within a few cells of the horizon or an axis the
+// metric, lapse and shift are evaluated in pairs of floats (and rounded), in the rows on the axes
+// the whole push, in a second kernel. Particle state is SoA; consecutive threads read consecutive
+// elements, and field gathers hit L1/L2 because the particles are kept sorted by cell.
 #include "grpic_internal.cuh"
 #include "pusher.cuh"
 #include "refine.cuh"
@@ -1268,11 +1270,12 @@ __global__ void __launch_bounds__(TPB, GRPIC_PUSH64_MIN_BLOCKS)
 // tag TAG_REST, which lives from this kernel to k_push_rest right behind it. Two kernels, so
 // that this one runs with the registers of its own code (128, 4 blocks per SM; with push64 in
 // it, 166 and 3) and the long routine with full warps: a step of the 2048^2 workload 80.3 ->
-// 66.3 ms, of the 512^2 one 11.0 -> 9.35 ms, of the 512^2 monopole problem, whose Boris half
-// steps are taken in FP64, 5.94 -> 4.18 ms. What bounds it: 124 FP64 instructions and ~7500
-// others per warp overlap to about half of either pipe's peak; between them warps wait for FP64
-// results, for instructions (the code is 14,000 instructions) and for their own pair arithmetic.
-// 5 and 6 blocks per SM (96, 80 registers) measured within 1% of 4.
+// 70.5 ms, of the 512^2 one 11.0 -> 9.8 ms, of the 512^2 monopole problem, whose Boris half
+// steps are taken in FP64, 5.95 -> 4.6 ms. What bounds it: about 120 FP64 operations and 9000
+// instructions per warp of particles overlap to about half of either pipe's peak; between them
+// warps wait for FP64 results, for instructions (straight-line code, larger than the instruction
+// caches) and for their own pair arithmetic. 5 and 6 blocks per SM (96, 80 registers) measured
+// within 1% of 4.
 constexpr uint8_t TAG_REST = 3;
 #ifndef GRPIC_PUSH_INC_MIN_BLOCKS
 #define GRPIC_PUSH_INC_MIN_BLOCKS 4
@@ -1768,7 +1771,7 @@ __global__ void k_push_tables(GridP g, PushTables tb) {
 
 int blocks_for(int64_t n) {
   int64_t b = (n + TPB - 1) / TPB;
-  const int64_t cap = 152 * 64;
+  const int64_t cap = N_SM * 64;
   if (b > cap) b = cap;
   return (int)(b < 1 ? 1 : b);
 }
@@ -1849,7 +1852,7 @@ cudaError_t push_impl(const GridP &g, const FieldPtrsT<T> &F, SpeciesDevT<T> s,
     if (kernels_stage) {
       // a few one-warp blocks per SM: the guard kernel runs beside the FP32 kernel, to which it
       // leaves the registers
-      constexpr int gb = 152 * GRPIC_GUARD_BLOCKS_PER_SM, ab = 152 * GRPIC_AXIS_BLOCKS_PER_SM;
+      constexpr int gb = N_SM * GRPIC_GUARD_BLOCKS_PER_SM, ab = N_SM * GRPIC_AXIS_BLOCKS_PER_SM;
       if (deposit) k_push_guard<true, Q><<<gb + ab, 32, 0, ps.side>>>(g, F, s, tb, gl, ab, diag);
       else k_push_guard<false, Q><<<gb + ab, 32, 0, ps.side>>>(g, F, s, tb, gl, ab, diag);
       if ((e = cudaEventRecord(ps.done, ps.side)) != cudaSuccess) return e;
@@ -1871,7 +1874,7 @@ cudaError_t push_impl(const GridP &g, const FieldPtrsT<T> &F, SpeciesDevT<T> s,
                                       (int)smem)) != cudaSuccess) return e;
     }
     if (tiled && ti.tma) {  // the padded copy the tensor copies read
-      k_pad_fields<<<152 * 8, 256, 0, ps.main>>>(F, ti.pad, g.NX, g.NY, ti.NXp);
+      k_pad_fields<<<N_SM * 8, 256, 0, ps.main>>>(F, ti.pad, g.NX, g.NY, ti.NXp);
       COUNT_LAUNCH(1);
     }
     if (ps.t0) cudaEventRecord(ps.t0, ps.main);

@@ -281,7 +281,7 @@ __global__ void k_set_n(int64_t *n_dev, const unsigned long long *alive) {
 
 int grid_for(int64_t n, int tpb) {
   int64_t b = (n + tpb - 1) / tpb;
-  if (b > 152 * 64) b = 152 * 64;
+  if (b > N_SM * 64) b = N_SM * 64;
   return (int)(b < 1 ? 1 : b);
 }
 

@@ -53,7 +53,7 @@ extern "C" GRPIC_API grpic_status grpic_sum_bins_add(const double *x, int64_t n,
   if (cudaPeekAtLastError() != cudaSuccess) return GRPIC_ECUDA;  // not this call's error
   if (n == 0) return GRPIC_OK;
   int64_t blocks = (n + SUM_TPB - 1) / SUM_TPB;
-  if (blocks > 4 * 152) blocks = 4 * 152;
+  if (blocks > 4 * N_SM) blocks = 4 * N_SM;
   k_sum_bins<<<(int)blocks, SUM_TPB, 0, static_cast<cudaStream_t>(stream)>>>(
       x, n, reinterpret_cast<unsigned long long *>(bins));
   COUNT_LAUNCH(1);
