@@ -479,7 +479,8 @@ __device__ __forceinline__ void adj_inv(const DF A[2][2], DF K[2][2]) {
 // A step's derivatives in scratch memory: entry (row, column) of rows x1, x2, phi, u1, u2, u3
 // and columns x1, x2, u1, u2, u3, scale at w[(row * JC + column) n], either J - 1, as pairs (lo,
 // hi) in the first two columns and as doubles in the others, or J as doubles; which one is the
-// lowest bit of entry (0, 0): clear for J - 1, set for J (half an ulp of that one entry).
+// lowest bit of entry (phi, scale), a double in both: clear for J - 1, set for J. (An entry that
+// is near 1 would not do: half an ulp of it, always upwards, is in every step's product.)
 //
 // Why two types: of J - 1 the first two columns are small (1e-3 where J has a 1), so pairs leave
 // less of J than FP64 does. The others hold entries that are the whole of J (dt dV/du, the
@@ -488,8 +489,10 @@ __device__ __forceinline__ void adj_inv(const DF A[2][2], DF K[2][2]) {
 // 0.5, the gradients' rms errors against 80-bit arithmetic were 2.7e-15 (u1), 1.8e-15 (u2), 3.4e-15
 // (scale) where FP64 throughout has 1.5e-15, 1.3e-15, 1.1e-15; now 4.5e-16, 5.4e-16, 4.4e-16.
 __device__ __forceinline__ constexpr bool adj_is64(int c) { return c >= 2; }
-__device__ __forceinline__ float2 adj_pack(DF a, bool first) {
-  return make_float2(first ? __uint_as_float(__float_as_uint(a.lo) & ~1u) : a.lo, a.hi);
+constexpr int ADJ_FORM = 2 * JC + 5;  // that entry
+__device__ __forceinline__ double adj_form(double x, bool general) {
+  const long long b = __double_as_longlong(x);
+  return __longlong_as_double(general ? b | 1ll : b & ~1ll);
 }
 
 // dV_j / du_k of the coordinate velocities at the midpoint in FP64 (adj_inc_jacobian's Vu)
@@ -666,7 +669,7 @@ __device__ __forceinline__ void adj_inc_jacobian(const GridP &g, const FieldPtrs
       const DF o[6] = {y0, y1, ph, w3[0], w3[1], w3[2]};
 #pragma unroll
       for (int q = 0; q < 6; ++q)
-        w[(int64_t)(q * JC + col) * n] = adj_pack(o[q], q == 0 && col == 0);
+        w[(int64_t)(q * JC + col) * n] = make_float2(o[q].lo, o[q].hi);
     }
   }
   // u_1, u_2, u_3 and the scale: the metric's values alone, in FP64
@@ -708,7 +711,8 @@ __device__ __forceinline__ void adj_inc_jacobian(const GridP &g, const FieldPtrs
     for (int q = 0; q < 3; ++q) f[q] = fma(Vu[q][0], d[0], fma(Vu[q][1], d[1], Vu[q][2] * d[2]));
     const double y0 = g.dt * (f[0] + fma(Nx[0][0], f[0], Nx[0][1] * f[1]));
     const double y1 = g.dt * (f[1] + fma(Nx[1][0], f[0], Nx[1][1] * f[1]));
-    const double o[6] = {y0, y1, g.dt * (f[2] + fma(Vp[0], y0, Vp[1] * y1)), dw[0], dw[1], dw[2]};
+    const double ph = g.dt * (f[2] + fma(Vp[0], y0, Vp[1] * y1));
+    const double o[6] = {y0, y1, col == 5 ? adj_form(ph, false) : ph, dw[0], dw[1], dw[2]};
 #pragma unroll
     for (int q = 0; q < 6; ++q) wd[(int64_t)(q * JC + col) * n] = o[q];
   }
@@ -744,7 +748,7 @@ __device__ __forceinline__ bool adj_advance(const GridP &g, const FieldPtrsT<dou
     step_jacobian(g, F, st, scale, qm, sv, fr, J);
     for (int r = 0; r < 6; ++r)
       for (int c = 0; c < JC; ++c) w[(int64_t)(r * JC + c) * n] = J[r][c];
-    w[0] = __longlong_as_double(__double_as_longlong(J[0][0]) | 1ll);
+    w[(int64_t)ADJ_FORM * n] = adj_form(J[2][5], true);
   }
   st[0] = sv.xn[0]; st[1] = sv.xn[1]; st[2] = sv.phin;
   st[3] = sv.un[0]; st[4] = sv.un[1]; st[5] = sv.un[2];
@@ -783,7 +787,7 @@ __device__ __forceinline__ void adj_reverse(const double *w, int64_t n, double l
                                             double &gs) {
   // inputs x1, x2, u1, u2, u3 are state rows 0, 1, 3, 4, 5; phi passes through
   const int row[5] = {0, 1, 3, 4, 5};
-  if (__double_as_longlong(w[0]) & 1ll) {
+  if (__double_as_longlong(w[(int64_t)ADJ_FORM * n]) & 1ll) {
     double nl[JC] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
     for (int r = 0; r < 6; ++r)
 #pragma unroll
