@@ -330,88 +330,120 @@ __device__ __noinline__ void step_jacobian(const GridP &g, const FieldPtrsT<doub
 // ---------------------------------------------------------------------------------
 // A step in the increment form. GB300's FP64 pipe bounded both passes (~1800 FP64 operations
 // per particle-step forward, ~5500 backward, most of them exp and sincos per iterate and the
-// metric's derivatives in duals); here FP64 is left with one or two evaluations of the
-// coordinate map, the additions to the state and, backward, the derivatives along the momentum
-// and the scale (~900 operations). 65,536 orbits on 512^2, 100 steps forward and back: 107 -> 38
-// ms (28 ms with all derivatives in pairs, whose errors were larger: see the scratch layout below).
-// The backward kernel waits for instructions, FP64 results and its pair arithmetic at 8 warps per
-// SM (255 registers, spills).
+// metric's derivatives in duals); here FP64 is left with the half steps (250 operations with the
+// fields and tetrads), one or two evaluations of the coordinate map, the additions to the state
+// and, backward, the derivatives along the momentum and the scale (~600). 65,536 orbits on
+// 512^2, 100 steps forward and back: 107 -> 39 ms (28 ms with the half steps and all derivatives
+// in pairs, whose errors were larger: see ADJ_MAX and the scratch layout below). The backward
+// kernel waits for instructions, FP64 results and its pair arithmetic at 8 warps per SM (255
+// registers, spills).
 // ---------------------------------------------------------------------------------
 constexpr int INC_MIN_ITER = 16;   // iteration counts below are taken literally (general form)
 constexpr float INC_ADJ_TOL = 1e-16f;
-constexpr IncLimit ADJ_LIMIT = {0x1p-8f, 0x1p-4f};  // increments up to 1/16 of max(|u|, 1/4)
+// Half steps and geodesic maps up to this (the turn and the kick of a half step; the map's
+// contraction): beyond, the derivatives by x1, x2 in pairs, whose errors are about 1e-14 of the
+// entries, leave more than the general form's rounding (200^2, 20 steps, half steps that turn the
+// momentum by 0.04: the gradient by x1 off by 3.1e-15 of its rms, the general form's by 8.8e-16;
+// at 0.005 7.0e-16 and 9.9e-16).
+constexpr float ADJ_MAX = 0x1p-7f;
+
+// A Boris half step from u in FP64 (inc_boris_core) and what its derivatives need of it: m = h + e
+// D, t = e B / gamma, p = m + m x t, c = p x t, sf = 2 / (1 + t^2)
+struct HalfStep {
+  double m[3], t[3], p[3], c[3], ig, sf;
+};
+__device__ __forceinline__ void cross64(const double a[3], const double b[3], double o[3]) {
+  o[0] = fma(a[1], b[2], -(a[2] * b[1]));
+  o[1] = fma(a[2], b[0], -(a[0] * b[2]));
+  o[2] = fma(a[0], b[1], -(a[1] * b[0]));
+}
+__device__ __forceinline__ void adj_half64(const Strong &w, double scale, double u[3],
+                                           HalfStep &h) {
+  h.m[0] = fma(scale, w.eD[0], w.sH11 * fma(-w.m13, u[2], u[0]));
+  h.m[1] = fma(scale, w.eD[1], w.rh22 * u[1]);
+  h.m[2] = fma(scale, w.eD[2], w.rh33 * u[2]);
+  h.ig = rsqrt(fma(h.m[0], h.m[0], fma(h.m[1], h.m[1], fma(h.m[2], h.m[2], 1.0))));
+  double x[3];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) h.t[q] = scale * w.eB[q] * h.ig;
+  h.sf = 2.0 * rcp_nr(fma(h.t[0], h.t[0], fma(h.t[1], h.t[1], fma(h.t[2], h.t[2], 1.0))));
+  cross64(h.m, h.t, x);
+#pragma unroll
+  for (int q = 0; q < 3; ++q) h.p[q] = h.m[q] + x[q];
+  cross64(h.p, h.t, h.c);
+#pragma unroll
+  for (int q = 0; q < 3; ++q) x[q] = fma(h.sf, h.c[q], 2.0 * scale * w.eD[q]);
+  u[0] += fma(x[0], w.rH11, w.k13 * x[2]);
+  u[1] = fma(w.sh22, x[1], u[1]);
+  u[2] = fma(w.sh33, x[2], u[2]);
+}
 
 struct AdjStep {
   int i1, i2;
   DF o1, o2;            // x^n in its cell
-  double dx[2];         // the same
   DF r, s, c;           // there
   Local<DF> L;
-  DF V[6];              // B, D at x^n, unit amplitude
-  DF eB[3], eD[3];      // e B, e D in the tetrad frame at the amplitude, e = qm alpha dt/4
+  Strong w;             // tetrad and fields (unit amplitude) at x^n
+  HalfStep h[2];
   DF u[3], u1[3], dg[2], u2[3], un[3];  // u^n, after the first EM half step, the geodesic
                         // substep's increment, after it, u^{n+1}
   double u64[3], x64[2], v3, mid[2];    // u^{n+1}, x^{n+1}, dphi/dt; the midpoint's offsets
 };
 
-// The values of a step; false: not covered by the increment form.
+// The values of a step, the half steps in FP64; false: not covered by the increment form.
 __device__ __forceinline__ bool adj_inc_step(const GridP &g, const FieldPtrsT<double> &F,
                                              const PushTables &tb, const IncC &k,
-                                             const double st[6], DF scale, DF qm, int n_iter,
-                                             AdjStep &a) {
+                                             const double st[6], double scale, double qm,
+                                             int n_iter, AdjStep &a) {
   const double f1 = floor(st[0]), f2 = floor(st[1]);
   a.i1 = (int)f1;
   a.i2 = (int)f2;
   if (!(a.i1 >= 0 && a.i1 < g.n_r && a.i2 >= 2 && a.i2 < g.n_th - 2)) return false;
   const double dx1 = st[0] - f1, dx2 = st[1] - f2;
-  a.dx[0] = dx1;
-  a.dx[1] = dx2;
   a.o1 = df_of(dx1);
   a.o2 = df_of(dx2);
   if (!inc_point_n(g, k, tb, a.i1, a.i2, dx2, a.o1, a.o2, a.r, a.s, a.c)) return false;
   inc_local(k, a.r, a.s, a.c, a.L);
-  IncLerp l;
-  inc_lerp(a.i1, a.i2, a.o1, a.o2, l);
-#pragma unroll 1
-  for (int q = 0; q < 6; ++q) {
-    const int h1 = q == 1 || q == 2 || q == 3, h2 = q == 0 || q == 2 || q == 4;
-    a.V[q] = inc_interp(q < 3 ? F.B[q] : F.D[q - 3], g.NX, l, h1, h2);
-  }
-  vec_hat(a.L, a.V, a.eB);
-  vec_hat(a.L, a.V + 3, a.eD);
-  // the gradient by the amplitude is proportional to the planes' own values, whatever they are:
-  // they have to be clear of the range where a pair loses its low half (2^-74)
-  float top = 0.0f;
+  strong_frame(g, F.B, F.D, tb, a.i1, a.i2, dx1, dx2, qm, a.w);
+  // the derivatives take the planes' own values in pairs, which have to be clear of the range
+  // where a pair loses its low half (2^-74)
+  if (!(a.w.top == 0.0f || (a.w.top >= 0x1p-30f && a.w.top <= 0x1p40f))) return false;
+  double u[3] = {st[3], st[4], st[5]};
+  float turn = 0.0f, kick = 0.0f, mm = 1.0f;
 #pragma unroll
-  for (int q = 0; q < 6; ++q) top = fmaxf(top, fabsf(a.V[q].hi));
-  if (!(top == 0.0f || (top >= 0x1p-30f && top <= 0x1p40f))) return false;
-  const DF es = scale * df_scale(qm * a.L.alpha * k.dt, 0.25f);
-  DF du[3] = {DF(0.0f), DF(0.0f), DF(0.0f)};
+  for (int q = 0; q < 3; ++q) a.u[q] = df_of(u[q]);
+  adj_half64(a.w, scale, u, a.h[0]);
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
-    a.eB[q] = es * a.eB[q];
-    a.eD[q] = es * a.eD[q];
-    a.u[q] = df_of(st[3 + q]);
+    const float t = f32_trunc(a.h[0].t[q]), d = f32_trunc(scale * a.w.eD[q]);
+    const float m = f32_trunc(a.h[0].m[q]);
+    turn = fmaf(t, t, turn);
+    kick = fmaf(d, d, kick);
+    mm = fmaf(m, m, mm);
+    a.u1[q] = df_of(u[q]);
   }
-  if (!inc_boris(a.L, a.eD, a.eB, a.u, ADJ_LIMIT, du)) return false;
-#pragma unroll
-  for (int q = 0; q < 3; ++q) a.u1[q] = a.u[q] + du[q];
+  // (a NaN anywhere makes one of the comparisons false)
+  if (!(4.0f * turn <= ADJ_MAX * ADJ_MAX && 4.0f * kick <= ADJ_MAX * ADJ_MAX * mm && mm < 0x1p60f))
+    return false;
   GeoInc<DF> m;
   geo_inc_setup(k, a.L, a.u1, 1.0f, m);
   float rho;
-  if (geo_inc_solve<false>(m, a.L.G.H33.hi * a.u[2].hi * a.u[2].hi, n_iter, INC_ADJ_TOL,
-                           ADJ_LIMIT, a.dg[0], a.dg[1], rho) != GEO_SMALL)
-    return false;
-  du[0] = du[0] + a.dg[0];
-  du[1] = du[1] + a.dg[1];
-  a.u2[0] = a.u[0] + du[0];
-  a.u2[1] = a.u[1] + du[1];
-  a.u2[2] = a.u1[2];
-  if (!inc_boris(a.L, a.eD, a.eB, a.u2, ADJ_LIMIT, du)) return false;
+  const int found = geo_inc_solve<false>(m, a.L.G.H33.hi * a.u1[2].hi * a.u1[2].hi, n_iter,
+                                         INC_ADJ_TOL, 0.0625f, a.dg[0], a.dg[1], rho);
+  if (found == GEO_NONE || !(rho <= ADJ_MAX)) return false;
+  if (found == GEO_LARGE) {
+    strong_geodesic(g, tb, a.i1, a.i2, dx1, dx2, 1.0, a.dg[0], a.dg[1], rho, u);
+  } else {
+    u[0] += df_to_double(a.dg[0]);
+    u[1] += df_to_double(a.dg[1]);
+  }
+#pragma unroll
+  for (int q = 0; q < 3; ++q) a.u2[q] = df_of(u[q]);
+  adj_half64(a.w, scale, u, a.h[1]);
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
-    a.un[q] = a.u[q] + du[q];
-    a.u64[q] = st[3 + q] + df_to_double(du[q]);
+    a.u64[q] = u[q];
+    a.un[q] = df_of(u[q]);
   }
   double t1, t2;
   if (!inc_coord<true>(g, k, tb, n_iter, INC_ADJ_TOL, a.i1, a.i2, dx1, dx2, a.o1, a.o2, a.u64,
@@ -424,15 +456,15 @@ __device__ __forceinline__ bool adj_inc_step(const GridP &g, const FieldPtrsT<do
   return finite64(a.u64[0]) && finite64(a.u64[1]) && finite64(a.u64[2]);
 }
 
-// a field component at x^n with its derivatives along x1, x2 (V: its value)
+// a field component at x^n with its derivatives along x1, x2
 __device__ __forceinline__ D2F adj_interp_d(const double *__restrict__ pl, int NX, const IncLerp &l,
-                                            int h1, int h2, DF V) {
+                                            int h1, int h2) {
   const double *p = pl + (int64_t)(l.j[h2] + G_) * NX + (l.i[h1] + G_);
   const DF p00 = df_of(__ldg(p)), p10 = df_of(__ldg(p + 1));
   const DF p01 = df_of(__ldg(p + NX)), p11 = df_of(__ldg(p + NX + 1));
   const DF x0 = p10 - p00, x1 = p11 - p01, y0 = p01 - p00;
-  const DF xy = x1 - x0;
-  return D2F(V, fma_(l.w2[h2], xy, x0), fma_(l.w1[h1], xy, y0));
+  const DF xy = x1 - x0, a = fma_(l.w1[h1], x0, p00), b = fma_(l.w1[h1], x1, p01);
+  return D2F(fma_(l.w2[h2], b - a, a), fma_(l.w2[h2], xy, x0), fma_(l.w1[h1], xy, y0));
 }
 
 // The momentum's derivative along x1, x2: du' of u^{n+1} - u^n for metric values L and fields with
@@ -516,34 +548,9 @@ __device__ __forceinline__ void adj_vu64(const GridP &g, const PushTables &tb, c
   V[0][2] = V[2][0] = G * fma(g.a, fi, -(q0 * P2));
   V[1][2] = V[2][1] = -(G * (q1 * P2));
 }
-__device__ __forceinline__ void cross64(const double a[3], const double b[3], double o[3]) {
-  o[0] = fma(a[1], b[2], -(a[2] * b[1]));
-  o[1] = fma(a[2], b[0], -(a[0] * b[2]));
-  o[2] = fma(a[0], b[1], -(a[1] * b[0]));
-}
-// A Boris half step from u in FP64 (inc_boris_core), what its derivatives need of it: m = h + e D,
-// t = e B / gamma, p = m + m x t, c = p x t, s = 2 / (1 + t^2)
-struct HalfStep {
-  double m[3], t[3], p[3], c[3], ig, sf;
-};
-__device__ __forceinline__ void adj_half64(const Strong &w, double scale, const double u[3],
-                                           HalfStep &h) {
-  h.m[0] = fma(scale, w.eD[0], w.sH11 * fma(-w.m13, u[2], u[0]));
-  h.m[1] = fma(scale, w.eD[1], w.rh22 * u[1]);
-  h.m[2] = fma(scale, w.eD[2], w.rh33 * u[2]);
-  h.ig = rsqrt(fma(h.m[0], h.m[0], fma(h.m[1], h.m[1], fma(h.m[2], h.m[2], 1.0))));
-  double x[3];
-#pragma unroll
-  for (int q = 0; q < 3; ++q) h.t[q] = scale * w.eB[q] * h.ig;
-  h.sf = 2.0 * rcp_nr(fma(h.t[0], h.t[0], fma(h.t[1], h.t[1], fma(h.t[2], h.t[2], 1.0))));
-  cross64(h.m, h.t, x);
-#pragma unroll
-  for (int q = 0; q < 3; ++q) h.p[q] = h.m[q] + x[q];
-  cross64(h.p, h.t, h.c);
-}
-// its derivative: of the increment, added to dw, along a direction that changes u by du and the
-// scale by ds
-__device__ __forceinline__ void adj_half64_d(const Strong &w, const HalfStep &h, double scale,
+// A half step's derivative: of the increment, added to dw, along a direction that changes u by du
+// and the scale by ds
+__device__ __forceinline__ void adj_half64_d(const Strong &w, const HalfStep &h,
                                              const double du[3], double ds, double dw[3]) {
   double md[3] = {w.sH11 * fma(-w.m13, du[2], du[0]), w.rh22 * du[1], w.rh33 * du[2]};
   double td[3], pd[3], x[3], y[3];
@@ -568,10 +575,8 @@ __device__ __forceinline__ void adj_half64_d(const Strong &w, const HalfStep &h,
 }
 
 __device__ __forceinline__ void adj_inc_jacobian(const GridP &g, const FieldPtrsT<double> &F,
-                                                 const PushTables &tb, const IncC &k,
-                                                 const double st[6], double scale64, double qm64,
-                                                 DF scale, DF qm, const AdjStep &a, double *wd,
-                                                 int64_t n) {
+                                                 const PushTables &tb, const IncC &k, DF scale,
+                                                 DF qm, const AdjStep &a, double *wd, int64_t n) {
   float2 *w = reinterpret_cast<float2 *>(wd);
   const DF zero(0.0f);
   // the coordinate map's velocity (inc_velocity's grouping) at the midpoint: its derivatives
@@ -637,7 +642,7 @@ __device__ __forceinline__ void adj_inc_jacobian(const GridP &g, const FieldPtrs
 #pragma unroll 1
     for (int q = 0; q < 6; ++q) {
       const int h1 = q == 1 || q == 2 || q == 3, h2 = q == 0 || q == 2 || q == 4;
-      V[q] = adj_interp_d(q < 3 ? F.B[q] : F.D[q - 3], g.NX, l, h1, h2, a.V[q]);
+      V[q] = adj_interp_d(q < 3 ? F.B[q] : F.D[q - 3], g.NX, l, h1, h2);
     }
     vec_hat(L, V, eB);
     vec_hat(L, V + 3, eD);
@@ -673,17 +678,6 @@ __device__ __forceinline__ void adj_inc_jacobian(const GridP &g, const FieldPtrs
     }
   }
   // u_1, u_2, u_3 and the scale: the metric's values alone, in FP64
-  Strong sw;
-  strong_frame(g, F.B, F.D, tb, a.i1, a.i2, a.dx[0], a.dx[1], qm64, sw);
-  HalfStep h[2];
-  {
-    const double u0[3] = {st[3], st[4], st[5]};
-    adj_half64(sw, scale64, u0, h[0]);
-    double u2[3];
-#pragma unroll
-    for (int q = 0; q < 3; ++q) u2[q] = df_to_double(a.u2[q]);
-    adj_half64(sw, scale64, u2, h[1]);
-  }
   double Nx[2][2], Vp[2];
 #pragma unroll
   for (int q = 0; q < 2; ++q) {
@@ -696,14 +690,14 @@ __device__ __forceinline__ void adj_inc_jacobian(const GridP &g, const FieldPtrs
     const double s[3] = {col == 2 ? 1.0 : 0.0, col == 3 ? 1.0 : 0.0, col == 4 ? 1.0 : 0.0};
     const double ds = col == 5 ? 1.0 : 0.0;
     double dw[3] = {0.0, 0.0, 0.0}, d[3];
-    adj_half64_d(sw, h[0], scale64, s, ds, dw);
+    adj_half64_d(a.w, a.h[0], s, ds, dw);
 #pragma unroll
     for (int q = 0; q < 3; ++q) d[q] = s[q] + dw[q];
     dw[0] += fma(P[0][0], d[0], fma(P[0][1], d[1], P[0][2] * d[2]));
     dw[1] += fma(P[1][0], d[0], fma(P[1][1], d[1], P[1][2] * d[2]));
 #pragma unroll
     for (int q = 0; q < 2; ++q) d[q] = s[q] + dw[q];
-    adj_half64_d(sw, h[1], scale64, d, ds, dw);
+    adj_half64_d(a.w, a.h[1], d, ds, dw);
     double f[3];
 #pragma unroll
     for (int q = 0; q < 3; ++q) d[q] = s[q] + dw[q];
@@ -726,10 +720,10 @@ __device__ __forceinline__ bool adj_advance(const GridP &g, const FieldPtrsT<dou
                                             double st[6], double *w, int64_t n) {
   if (INC) {
     AdjStep a;
-    if (adj_inc_step(g, F, tb, k, st, scale_df, qm_df, n_iter, a)) {
+    if (adj_inc_step(g, F, tb, k, st, scale, qm, n_iter, a)) {
       const bool ok = a.x64[0] >= 0.0 && a.x64[0] < g.n_r && a.x64[1] >= 0.0 && a.x64[1] <= g.n_th;
       if (!ok) return false;
-      if (w) adj_inc_jacobian(g, F, tb, k, st, scale, qm, scale_df, qm_df, a, w, n);
+      if (w) adj_inc_jacobian(g, F, tb, k, scale_df, qm_df, a, w, n);
       st[0] = a.x64[0];
       st[1] = a.x64[1];
       st[2] = fma(g.dt, a.v3, st[2]);

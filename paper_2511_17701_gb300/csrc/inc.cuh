@@ -34,20 +34,13 @@ namespace {
 // its iterations run to rounding: 3.7e-16, 1.2e-15); |u| = 1e-3:
 // 5.3e-16 and 5.7e-15 (5.4e-16, 6.2e-15).
 // Massless particles, whose FP64 push rounds less (no half steps: 6.9e-17), take half of it.
-// floor: where |u|^2 is less than this, it is taken as this (0: never).
 constexpr float INC_MAX = 0x1p-5f;
-struct IncLimit {
-  float r2, floor;  // the ratio's square, the floor
-};
-__device__ __forceinline__ IncLimit inc_limit(float times2) {  // times sqrt(times2)
-  return {times2 * INC_MAX * INC_MAX, 0.0f};
-}
 // below this, squared, the pairs' own floor of 2^-149 would show in an increment that is not
 // exactly zero
 constexpr float INC_UU = 0x1p-100f;
-__device__ __forceinline__ bool inc_within(IncLimit lim, float dd, float uu) {
-  const float w = fmaxf(uu, lim.floor);
-  return dd <= lim.r2 * w && w >= INC_UU;
+// whether an increment of square dd is within sqrt(times2) INC_MAX of a momentum of square uu
+__device__ __forceinline__ bool inc_within(float times2, float dd, float uu) {
+  return dd <= times2 * (INC_MAX * INC_MAX) * uu && uu >= INC_UU;
 }
 constexpr float INC_E = 0.055f;      // largest |offset of xi| of the radial series
 constexpr float INC_D = 0.035f;      // largest |offset of theta| of the angular series
@@ -283,13 +276,13 @@ __device__ __forceinline__ void geo_inc_setup(const IncC &k, const Local<M> &L, 
 // G + M J r with r = G - d and M = (I - J)^{-1}, leave an error of |J| 2^-24 |r|, far below the
 // pairs' rounding of d. n_iter, tol: the method's iterations and what they have to come within
 // (inc_converges), else the method's iterations themselves are run, in pairs (LITERAL). h33:
-// h^33 u_3^2. Returns GEO_SMALL; GEO_LARGE where the increment is beyond lim, and the point
+// h^33 u_3^2. Returns GEO_SMALL; GEO_LARGE where the increment is beyond the bound, and the point
 // (n0, n1), within the pairs' rounding of the fixed point, that FP64 evaluations have to start
 // from, with the contraction rho there; GEO_NONE: not resolved.
 enum { GEO_NONE = 0, GEO_SMALL, GEO_LARGE };
 template <bool LITERAL>
 __device__ __forceinline__ int geo_inc_solve(const GeoInc<DF> &m, float h33, int n_iter, float tol,
-                                             IncLimit lim, DF &n0, DF &n1, float &rho) {
+                                             float times2, DF &n0, DF &n1, float &rho) {
   const GeoInc<float> mf = {m.u0.hi,  m.u1.hi,  m.c0.hi,  m.c1.hi,  m.e1.hi,    m.e2.hi,   m.f1.hi,
                             m.f2.hi,  m.D1a.hi, m.D1b.hi, m.D2a.hi, m.D2b.hi,   m.hdt.hi,  m.H11.hi,
                             m.H22.hi, m.d1H11.hi, m.d1H22.hi, m.d2H11.hi, m.d2H22.hi};
@@ -334,7 +327,7 @@ __device__ __forceinline__ int geo_inc_solve(const GeoInc<DF> &m, float h33, int
   const float dd = fmaf(mf.H11 * n0.hi, n0.hi, mf.H22 * n1.hi * n1.hi);
   const float uu = fmaf(mf.u0, fmaf(mf.H11, mf.u0, mf.c1), fmaf(mf.H22 * mf.u1, mf.u1, h33));
   const bool none = n0.hi == 0.0f && n1.hi == 0.0f;
-  if (none || inc_within(lim, dd, uu)) return GEO_SMALL;
+  if (none || inc_within(times2, dd, uu)) return GEO_SMALL;
   return fixed && dd < 0x1p60f ? GEO_LARGE : GEO_NONE;
 }
 
@@ -361,15 +354,15 @@ __device__ __forceinline__ void inc_boris_core(const Local<M> &L, const R eD[3],
   du[1] = fma_(L.sh22, x[1], du[1]);
   du[2] = fma_(L.sh33, x[2], du[2]);
 }
-// False: the increment is beyond lim.
+// False: the increment is beyond the bound (inc_within).
 __device__ __forceinline__ bool inc_boris(const Local<DF> &L, const DF eD[3], const DF eB[3],
-                                          const DF u[3], IncLimit lim, DF du[3]) {
+                                          const DF u[3], float times2, DF du[3]) {
   DF h[3], x[3];
   inc_boris_core(L, eD, eB, u, du, h, x);
   const float xx = fmaf(x[0].hi, x[0].hi, fmaf(x[1].hi, x[1].hi, x[2].hi * x[2].hi));
   const float hh = fmaf(h[0].hi, h[0].hi, fmaf(h[1].hi, h[1].hi, h[2].hi * h[2].hi));
   const bool none = fabsf(x[0].hi) + fabsf(x[1].hi) + fabsf(x[2].hi) == 0.0f;
-  return (none || inc_within(lim, xx, hh)) && hh < 0x1p60f;
+  return (none || inc_within(times2, xx, hh)) && hh < 0x1p60f;
 }
 
 // bilinear interpolation in pairs at the cell-relative offsets (o1, o2) of cell (i1, i2) for
@@ -466,6 +459,7 @@ __device__ __forceinline__ void inc_point64(const GridP &g, const PushTables &tb
 // strong fields, and the adjoint's derivative by the amplitude
 struct Strong {
   double rH11, sH11, rh22, sh22, rh33, sh33, k13, m13, eB[3], eD[3];
+  float top;  // the largest of the planes' values there
 };
 __device__ __forceinline__ void strong_frame(const GridP &g, double *const B[3],
                                              double *const D[3], const PushTables &tb, int i1,
@@ -491,6 +485,7 @@ __device__ __forceinline__ void strong_frame(const GridP &g, double *const B[3],
   const bool l1 = lt_pos(dx1, 0.5) || dx1 == 0.0, l2 = lt_pos(dx2, 0.5) || dx2 == 0.0;
   const double w1[2] = {dx1, l1 ? dx1 + 0.5 : dx1 - 0.5}, w2[2] = {dx2, l2 ? dx2 + 0.5 : dx2 - 0.5};
   double V[6];
+  w.top = 0.0f;
 #pragma unroll 1
   for (int q = 0; q < 6; ++q) {  // one copy of the code
     const int h1 = q == 1 || q == 2 || q == 3, h2 = q == 0 || q == 2 || q == 4;
@@ -500,6 +495,7 @@ __device__ __forceinline__ void strong_frame(const GridP &g, double *const B[3],
     const double a1 = h1 ? w1[1] : w1[0], a2 = h2 ? w2[1] : w2[0];
     const double x = fma(a1, p10 - p00, p00), y = fma(a1, p11 - p01, p01);
     V[q] = fma(a2, y - x, x);
+    w.top = fmaxf(w.top, fabsf(f32_trunc(V[q])));
   }
 #pragma unroll
   for (int q = 0; q < 2; ++q) {
@@ -510,6 +506,34 @@ __device__ __forceinline__ void strong_frame(const GridP &g, double *const B[3],
     o[2] = e * fma(w.k13, v[0], w.sh33 * v[2]);
   }
 }
+// The geodesic substep in FP64 from the increment (d0, d1) that the pairs found, where it is large
+// against u (cold particles, and next to the axes, where the metric changes by order one over a
+// step): evaluations of the FP64 map until the pairs' error in it, below 2^-46 of the increment,
+// has contracted (by rho each) to FP64's rounding.
+__device__ __forceinline__ void strong_geodesic(const GridP &g, const PushTables &tb, int i1,
+                                                int i2, double dx1, double dx2, double m2,
+                                                DF d0, DF d1, float rho, double u[3]) {
+  Pt<double> p;
+  inc_point64(g, tb, i1, i2, dx1, dx2, __dadd_rn((double)i2, dx2), p.r, p.s, p.c);
+  p.f = g.dxi * p.r;
+  p.gg = g.dth;
+  p.igg = g.ig2;
+  p.gp = 0.0;
+  Local<double> L;
+  local_full<false>(g, p, L, false);
+  const GeoMap<double> m(g, L, u, m2);
+  double t0 = u[0] + df_to_double(d0), t1 = u[1] + df_to_double(d1);
+#pragma unroll 1
+  for (float left = 1.0f; left > 0x1p-9f; left *= rho) {
+    double n0, n1;
+    m.apply(t0, t1, n0, n1);
+    t0 = n0;
+    t1 = n1;
+  }
+  u[0] = t0;
+  u[1] = t1;
+}
+
 // The FP64 evaluation of the map t -> dx + dt V((x^n + t)/2) that the result comes from, in
 // inc_velocity's grouping: ~80 FP64 operations.
 __device__ __forceinline__ void inc_coord64(const GridP &g, const PushTables &tb, int i1, int i2,

@@ -147,34 +147,6 @@ __device__ __forceinline__ bool photon_unit(double u[3], double &unit) {
   return true;
 }
 
-// The geodesic substep in FP64 from the increment (d0, d1) that the pairs found, where it is large
-// against u (cold particles, and next to the axes, where the metric changes by order one over a
-// step): evaluations of the FP64 map until the pairs' error in it, below 2^-46 of the increment,
-// has contracted (by rho each) to FP64's rounding.
-__device__ __forceinline__ void strong_geodesic(const GridP &g, const PushTables &tb, int i1,
-                                                int i2, double dx1, double dx2, double m2,
-                                                DF d0, DF d1, float rho, double u[3]) {
-  Pt<double> p;
-  inc_point64(g, tb, i1, i2, dx1, dx2, __dadd_rn((double)i2, dx2), p.r, p.s, p.c);
-  p.f = g.dxi * p.r;
-  p.gg = g.dth;
-  p.igg = g.ig2;
-  p.gp = 0.0;
-  Local<double> L;
-  local_full<false>(g, p, L, false);
-  const GeoMap<double> m(g, L, u, m2);
-  double t0 = u[0] + df_to_double(d0), t1 = u[1] + df_to_double(d1);
-#pragma unroll 1
-  for (float left = 1.0f; left > 0x1p-9f; left *= rho) {
-    double n0, n1;
-    m.apply(t0, t1, n0, n1);
-    t0 = n0;
-    t1 = n1;
-  }
-  u[0] = t0;
-  u[1] = t1;
-}
-
 // One particle in the increment form; false: nothing stored, push64 has to take it. Loops that
 // the compiler would unroll stay loops: the code is straight-line and long, and warps waited
 // for its instructions (17% of their time with every copy unrolled).
@@ -232,7 +204,7 @@ __device__ __forceinline__ bool push_inc(const GridP &g, const FieldPtrsT<double
         eB[q] = e * eB[q];
         eD[q] = e * eD[q];
       }
-      weak = inc_boris(L, eD, eB, u, inc_limit(1.0f), du);
+      weak = inc_boris(L, eD, eB, u, 1.0f, du);
     }
     if (!weak) {
       strong_frame(g, F.Bn, F.D, tb, i1, i2, dx1, dx2, s.qm, w);
@@ -252,7 +224,7 @@ __device__ __forceinline__ bool push_inc(const GridP &g, const FieldPtrsT<double
       // in the axis rows the result is the method's to rounding, as push64's is there
       const int found = geo_inc_solve<true>(m, L.G.H33.hi * ud[2].hi * ud[2].hi, g.n_iter,
                                             axis ? 0x1p-54f : g.f_iter_tol,
-                                            inc_limit(em ? 1.0f : 0.25f), d0, d1, rho);
+                                            em ? 1.0f : 0.25f, d0, d1, rho);
       if (found == GEO_NONE) return false;
       if (found == GEO_LARGE) {
 #pragma unroll
@@ -269,7 +241,7 @@ __device__ __forceinline__ bool push_inc(const GridP &g, const FieldPtrsT<double
     if (em && weak) {  // (twice the bound, so that a particle next to it need not start over)
 #pragma unroll
       for (int q = 0; q < 3; ++q) ud[q] = df_of(un[q]) + du[q];
-      if (!inc_boris(L, eD, eB, ud, inc_limit(4.0f), du)) return false;
+      if (!inc_boris(L, eD, eB, ud, 4.0f, du)) return false;
     }
 #pragma unroll
     for (int q = 0; q < 3; ++q) un[q] += df_to_double(du[q]);
