@@ -59,19 +59,19 @@ GRID_BYTES_PER_CELL = {"fp64": 33 * 8, "mixed": 33 * 4}
 # dram__bytes_read.sum + dram__bytes_write.sum per particle. When the sources change the
 # counts are reported as stale and the traffic as null until they are captured again.
 KERNEL_COUNTS = {
-    "fp64": {"src": "96d18af130762614",
+    "fp64": {"src": "e486abea1a01dc40",
              "workload": "wald2048; operations from ncu of one launch at 1 particle per cell per "
                          "species (4,194,304 particles), DRAM bytes from a one-pass capture of a "
                          "full launch (67,108,864 particles)",
              "fp64_ops": (197766875 + 168165888 + 146903855) / 4194304,
              "flop": (197766875 + 168165888 + 2 * 146903855) / 4194304,
-             "dram_bytes": (4711499008 + 3860228864) / 67108864},
-    "mixed": {"src": "96d18af130762614",
+             "dram_bytes": (4713322496 + 3860807936) / 67108864},
+    "mixed": {"src": "e486abea1a01dc40",
               "workload": "wald2048; warp instructions from ncu of one launch at 1 particle per "
                           "cell per species, DRAM bytes from a one-pass capture of a full launch "
                           "(67,108,864 particles)",
               "warp_inst": 163906694 / 4194304,
-              "dram_bytes": (2646780928 + 2362233088) / 67108864},
+              "dram_bytes": (2646268160 + 2362720000) / 67108864},
 }
 KERNEL_SOURCES = ("particles.cu", "push_inc.cuh", "inc.cuh", "refine.cuh", "pusher.cuh", "dfloat.cuh",
                   "grpic_internal.cuh")
